@@ -946,7 +946,7 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags
             for (int i = 0; i < kChunk; ++i) nd_peel_round<CT>(v, r, s, P, st);
         }
         if ((rc = nd_check_launch("peel round"))) break;
-        cudaMemcpyAsync(hdone, &P.ctl->done, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+        cudaMemcpyAsync(hdone, &P.ctl->h.done, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
         if ((rc = nd_sync(c, "peel round"))) break;
         if (*hdone) break;
         if (++chunks > max_chunks) {
@@ -967,20 +967,20 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags
             else if (h.err & 2) rc = nd_set_error(ND_ETIMEOUT, "peel: round cap reached");
             else if (h.err & 4) rc = nd_set_error(ND_EINTERNAL, "peel: empty round (inconsistent state)");
             else if (h.err & 16) rc = nd_set_error(ND_EINTERNAL, "peel: an r-subset of a listed s-clique is not in the index");
-            else if (h.finished != n_r) rc = nd_set_error(ND_EINTERNAL, "peel: finished %lld of %lld",
-                                                          (long long)h.finished, (long long)n_r);
-            po.rho = h.t;
-            po.max_core = n_r ? h.k : 0;
+            else if (h.h.finished != n_r) rc = nd_set_error(ND_EINTERNAL, "peel: finished %lld of %lld",
+                                                          (long long)h.h.finished, (long long)n_r);
+            po.rho = h.h.t;
+            po.max_core = n_r ? h.h.k : 0;
             if (looped && !persistent_launches)  // graph nodes executed: every iteration (rho + 1), plus advance and refill phases
-                nd_note_launches((int64_t)(h.t + 1) * nd_peel_nodes_per_round(r, s, contract) +
-                                 3 * (int64_t)h.advances + 4 * (int64_t)h.refills);
+                nd_note_launches((int64_t)(h.h.t + 1) * nd_peel_nodes_per_round(r, s, contract) +
+                                 3 * (int64_t)h.h.advances + 4 * (int64_t)h.h.refills);
             po.listed = (int64_t)h.listed;
             po.decs = (int64_t)h.decs;
             for (int i = 0; i < 7; ++i) po.phase_ms[i] = persistent_launches ? 1e-6 * (double)h.ph_ns[i] : 0.0;
-            po.contractions = h.contractions;
-            po.advances = h.advances;
-            po.refills = h.refills;
-            if (h.k > INT32_MAX && !rc) rc = nd_set_error(ND_EOVERFLOW, "a core number exceeds 2^31-1");
+            po.contractions = h.h.contractions;
+            po.advances = h.h.advances;
+            po.refills = h.h.refills;
+            if (h.h.k > INT32_MAX && !rc) rc = nd_set_error(ND_EOVERFLOW, "a core number exceeds 2^31-1");
         }
     }
     if (!rc) {

@@ -35,6 +35,7 @@
 // first index i in [0, n) with a[i] >= x (n if none)
 __device__ __forceinline__ int64_t nd_lower_bound(const int32_t* __restrict__ a, int64_t n, int32_t x) {
     int64_t lo = 0, hi = n;
+#pragma unroll 1
     while (lo < hi) {
         int64_t mid = (lo + hi) >> 1;
         if (__ldg(a + mid) < x)
@@ -255,55 +256,62 @@ struct GraphView {
 #define ND_HBINS 4096
 #define ND_MODE_ADV 1
 
-struct PeelCtl {
+// The part of the control block that a round's phases read: written by the serial steps between
+// phases and by the phases' appends, stable while a phase that reads it runs. The persistent kernel
+// copies it into shared memory after every barrier, so a phase starts without a chain of loads from
+// L2 (the copy is sizeof(PeelHot) / 16 loads of 16 bytes by one warp, all in flight at once).
+struct __align__(128) PeelHot {
     // loop state
     int32_t t;          // current round
     int32_t mode;       // ND_MODE_ADV when this round moves to a new level
     int32_t done;       // 1 once every r-clique is peeled
-    int32_t err;        // list overflow / inconsistency
     int32_t started;    // 0 before the first round
     int32_t wa, wn, wl; // ping-pong selectors of the A, N and L lists
     int32_t lmat;       // 0: L is implicitly 0..n_r-1
-    int32_t heavy;      // persistent kernel: this round has a heavy phase (set by a serial step)
-    int32_t sorta;      // persistent kernel: this round rebuilds A in id order (set by a serial step)
     int32_t heavy_split;// persistent kernel, (2,4): this round's heavy phase is split over the grid
+    int32_t sorta;      // persistent kernel: this round rebuilds A in id order (set by a serial step)
+    int32_t contract;   // graph contraction before this round's phases (set by the serial control step)
+    int32_t stage;      // persistent kernel: 0 start of the round, 3 selection of A, 1 Update, 2 heavy Update
+    unsigned int nA;    // |A| of a same-level round
     int64_t k;          // current level
     int64_t hi;         // bucket window: N holds every unpeeled r-clique with count < hi
     int64_t finished;   // r-cliques peeled so far
+    int64_t peeled_since;    // r-cliques peeled since the last contraction
     int64_t n_r;
     int64_t max_rounds; // round cap (ND_ETIMEOUT)
-    unsigned long long bar_timeout_ns;  // persistent kernel: longest wait at one grid barrier
-    int32_t drop_block; // persistent kernel, test of the barrier bound: the last block leaves at once
-    int32_t contract;   // graph contraction before this round's phases (set by the serial control step)
     int64_t contract_every;  // contract once this many r-cliques were peeled since the last one (0: never)
-    int64_t peeled_since;    // r-cliques peeled since the last contraction
-    int64_t contractions;    // contractions run
-    int32_t contract_shift;  // compact a row that lost at least len >> shift entries (0: any loss)
-    int32_t pad3;
-    // list sizes
-    unsigned int nA;    // |A| of a same-level round
+    // list sizes, counted up by the phases
     unsigned int cntA;  // |A| written by adv_select
-    unsigned int nNext; // next round's A (r-cliques that fell to <= k during this round)
     unsigned int nN;    // |N| (current)
     unsigned int nN2;   // |N'| being written this round (advance rounds)
     unsigned int nL;    // |L|
     unsigned int nL2;   // |L'| being written by refill
     unsigned int nH;    // r-cliques of this round's A deferred to the heavy Update kernel
-    unsigned int upd_next;  // next unassigned position of A in this round's Update (dynamic chunks)
-    unsigned int upd_pad;
     unsigned long long minN;  // min count over unpeeled members of N (adv_min)
     unsigned long long gmin;  // min count over unpeeled r-cliques (refill)
+    unsigned int nNext; // next round's A (r-cliques that fell to <= k during this round)
+    unsigned int upd_next;  // next unassigned position of A in this round's Update (dynamic chunks)
+    int64_t contractions;    // contractions run
+    int64_t advances, refills;
+};
+static_assert(sizeof(PeelHot) == 256, "two lines of 128 bytes");
+
+struct PeelCtl {
+    PeelHot h;
+    int32_t err;        // list overflow / inconsistency
+    int32_t contract_shift;  // compact a row that lost at least len >> shift entries (0: any loss)
+    int32_t drop_block; // persistent kernel, test of the barrier bound: the last block leaves at once
+    unsigned long long bar_timeout_ns;  // persistent kernel: longest wait at one grid barrier
     // grid barrier of the persistent peel kernel: arrivals since the launch, and the arrival
-    // count up to which blocks have been released
-    unsigned long long bar_arrive;
-    unsigned long long bar_gen;
+    // count up to which blocks have been released (lines of their own: one is written by every
+    // block, the other read by every block)
+    __align__(128) unsigned long long bar_arrive;
+    __align__(128) unsigned long long bar_gen;
     // statistics
-    unsigned long long listed;
+    __align__(128) unsigned long long listed;
     unsigned long long decs;
-    long long advances, refills;
     // persistent kernel: nanoseconds per phase between barriers, as seen by block 0
     unsigned long long ph_ns[7];  // [6]: graph contraction
-    unsigned long long ph_last;
     unsigned long long hist[ND_HBINS];
 };
 

@@ -52,13 +52,24 @@ constexpr int kThreads = 256;
 
 __device__ __forceinline__ int64_t gwarp() { return ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; }
 __device__ __forceinline__ int64_t nwarps() { return ((int64_t)gridDim.x * blockDim.x) >> 5; }
-__device__ __forceinline__ int64_t gthread() { return (int64_t)blockIdx.x * blockDim.x + threadIdx.x; }
-__device__ __forceinline__ int64_t nthreads() { return (int64_t)gridDim.x * blockDim.x; }
 
-__device__ __forceinline__ int64_t knew_of(const PeelCtl* c) {
-    unsigned long long mn = c->minN != ULLONG_MAX ? c->minN : c->gmin;
-    int64_t m = mn == ULLONG_MAX ? c->k : (int64_t)mn;
-    return m > c->k ? m : c->k;
+// The grid's warps and threads as a phase numbers them. Neighbouring warp numbers lie in different
+// blocks, so that a handful of r-cliques spreads over the SMs.
+struct Team {
+    unsigned warp, nwarps;
+    unsigned block, nblocks;
+    __device__ __forceinline__ int64_t thread() const { return (int64_t)block * blockDim.x + threadIdx.x; }
+    __device__ __forceinline__ int64_t nthreads() const { return (int64_t)nblocks * blockDim.x; }
+};
+
+__device__ __forceinline__ Team grid_team() {
+    return Team{(threadIdx.x >> 5) * gridDim.x + blockIdx.x, (blockDim.x >> 5) * gridDim.x, blockIdx.x, gridDim.x};
+}
+
+__device__ __forceinline__ int64_t knew_of(const PeelHot& s) {
+    unsigned long long mn = s.minN != ULLONG_MAX ? s.minN : s.gmin;
+    int64_t m = mn == ULLONG_MAX ? s.k : (int64_t)mn;
+    return m > s.k ? m : s.k;
 }
 
 // a[i] for a two-entry pointer array without dynamic indexing (which would copy the kernel
@@ -102,8 +113,8 @@ __device__ __forceinline__ void unmark_a(const PeelView<CT>& P, int32_t x) {
 // ctl->err and is reported by the host)
 __device__ __forceinline__ unsigned clampn(unsigned v, uint32_t cap) { return v < cap ? v : cap; }
 
-__device__ __forceinline__ bool need_refill(const PeelCtl* c) {
-    return !c->done && (c->mode & ND_MODE_ADV) && c->minN == ULLONG_MAX;
+__device__ __forceinline__ bool need_refill(const PeelHot& s) {
+    return !s.done && (s.mode & ND_MODE_ADV) && s.minN == ULLONG_MAX;
 }
 
 __device__ __forceinline__ unsigned long long block_min(unsigned long long v) {
@@ -128,37 +139,21 @@ __device__ __forceinline__ unsigned long long block_min(unsigned long long v) {
 __global__ void k_init(PeelCtl* c, int64_t n_r, int64_t max_rounds, unsigned long long barrier_ns, int drop_block,
                        int64_t contract_every, int contract_shift) {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
-        c->bar_timeout_ns = barrier_ns;
-        c->drop_block = drop_block;
-        c->contract = 0;
-        c->contract_every = contract_every;
-        c->contract_shift = contract_shift;
-        c->peeled_since = 0;
-        c->contractions = 0;
-        c->t = 0;
-        c->mode = 0;
-        c->done = 0;
+        PeelHot h = {};
+        h.n_r = n_r;
+        h.max_rounds = max_rounds;
+        h.contract_every = contract_every;
+        h.minN = h.gmin = ULLONG_MAX;
+        c->h = h;
         c->err = 0;
-        c->started = 0;
-        c->wa = c->wn = c->wl = 0;
-        c->lmat = 0;
-        c->heavy = 0;
-        c->sorta = 0;
-        for (int i = 0; i < 7; ++i) c->ph_ns[i] = 0;
-        c->ph_last = 0;
-        c->k = 0;
-        c->hi = 0;
-        c->finished = 0;
-        c->n_r = n_r;
-        c->max_rounds = max_rounds;
-        c->nA = c->cntA = c->nNext = c->nN = c->nN2 = c->nL = c->nL2 = c->nH = 0;
-        c->upd_next = 0;
-        c->minN = c->gmin = ULLONG_MAX;
-        c->listed = 0;
-        c->decs = 0;
+        c->contract_shift = contract_shift;
+        c->drop_block = drop_block;
+        c->bar_timeout_ns = barrier_ns;
         c->bar_arrive = 0;
         c->bar_gen = 0;
-        c->advances = c->refills = 0;
+        c->listed = 0;
+        c->decs = 0;
+        for (int i = 0; i < 7; ++i) c->ph_ns[i] = 0;
     }
 }
 
@@ -172,76 +167,78 @@ __global__ void k_ctl(PeelCtl* c, int64_t* round_size, int64_t* round_level, int
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     ctl_step(c, round_size, round_level, round_cap);
     if (use_cond) {
-        cudaGraphSetConditional(h_loop, c->done ? 0u : 1u);
-        cudaGraphSetConditional(h_adv, (!c->done && (c->mode & ND_MODE_ADV)) ? 1u : 0u);
+        cudaGraphSetConditional(h_loop, c->h.done ? 0u : 1u);
+        cudaGraphSetConditional(h_adv, (!c->h.done && (c->h.mode & ND_MODE_ADV)) ? 1u : 0u);
     }
 }
 
 // IF condition of the refill phase: the window N holds no unpeeled r-clique
 __global__ void k_set_refill(PeelCtl* c, cudaGraphConditionalHandle h_refill) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) cudaGraphSetConditional(h_refill, need_refill(c) ? 1u : 0u);
+    if (threadIdx.x == 0 && blockIdx.x == 0) cudaGraphSetConditional(h_refill, need_refill(c->h) ? 1u : 0u);
+}
+
+// The control step on a copy of the hot state.
+__device__ __forceinline__ void ctl_next(PeelHot& s, int* err, int64_t* round_size, int64_t* round_level,
+                                         int64_t round_cap) {
+    if (s.started) {
+        const bool adv = s.mode & ND_MODE_ADV;
+        const unsigned nA = adv ? s.cntA : s.nA;
+        if (adv) {
+            s.k = knew_of(s);
+            s.nN = s.nN2;
+            s.wn ^= 1;
+            s.advances++;
+        }
+        if (s.t < round_cap) {
+            round_size[s.t] = nA;
+            round_level[s.t] = s.k;
+        }
+        s.finished += nA;
+        s.peeled_since += nA;
+        s.t += 1;
+        if (s.finished >= s.n_r) {
+            s.done = 1;
+            return;
+        }
+        // an empty round cannot happen in a consistent state (4); the round cap (2)
+        if (nA == 0 || s.t >= s.max_rounds) {
+            atomicOr(err, nA == 0 ? 4 : 2);
+            s.done = 1;
+            return;
+        }
+    } else {
+        s.started = 1;
+        if (s.n_r == 0) {
+            s.done = 1;
+            return;
+        }
+    }
+    s.nH = 0;
+    s.upd_next = 0;
+    // graph contraction (Section 5.6) once enough r-cliques were peeled since the previous one
+    s.contract = s.contract_every > 0 && s.peeled_since >= s.contract_every;
+    if (s.contract) {
+        s.peeled_since = 0;
+        s.contractions++;
+    }
+    if (s.nNext > 0) {
+        s.wa ^= 1;
+        s.nA = s.nNext;
+        s.nNext = 0;
+        s.mode = 0;
+    } else {
+        s.mode = ND_MODE_ADV;
+        s.nA = 0;
+        s.cntA = 0;
+        s.nN2 = 0;
+        s.minN = ULLONG_MAX;
+        s.gmin = ULLONG_MAX;
+    }
 }
 
 __device__ void ctl_step(PeelCtl* c, int64_t* round_size, int64_t* round_level, int64_t round_cap) {
-    if (c->done) return;
-    if (c->started) {
-        bool adv = c->mode & ND_MODE_ADV;
-        unsigned nA = adv ? c->cntA : c->nA;
-        if (adv) {
-            c->k = knew_of(c);
-            c->nN = c->nN2;
-            c->wn ^= 1;
-            c->advances++;
-        }
-        if (c->t < round_cap) {
-            round_size[c->t] = nA;
-            round_level[c->t] = c->k;
-        }
-        c->finished += nA;
-        c->peeled_since += nA;
-        c->t += 1;
-        if (c->finished >= c->n_r) {
-            c->done = 1;
-            return;
-        }
-        if (nA == 0) {  // an empty round cannot happen in a consistent state
-            c->err |= 4;
-            c->done = 1;
-            return;
-        }
-        if (c->t >= c->max_rounds) {
-            c->err |= 2;
-            c->done = 1;
-            return;
-        }
-    } else {
-        c->started = 1;
-        if (c->n_r == 0) {
-            c->done = 1;
-            return;
-        }
-    }
-    c->nH = 0;
-    c->upd_next = 0;
-    // graph contraction (Section 5.6) once enough r-cliques were peeled since the previous one
-    c->contract = c->contract_every > 0 && c->peeled_since >= c->contract_every;
-    if (c->contract) {
-        c->peeled_since = 0;
-        c->contractions++;
-    }
-    if (c->nNext > 0) {
-        c->wa ^= 1;
-        c->nA = c->nNext;
-        c->nNext = 0;
-        c->mode = 0;
-    } else {
-        c->mode = ND_MODE_ADV;
-        c->nA = 0;
-        c->cntA = 0;
-        c->nN2 = 0;
-        c->minN = ULLONG_MAX;
-        c->gmin = ULLONG_MAX;
-    }
+    if (c->h.done) return;
+    ctl_next(c->h, &c->err, round_size, round_level, round_cap);
 }
 
 // Dense buckets: the new level is the first non-empty bucket at or above k, found by the
@@ -252,13 +249,12 @@ __device__ void ctl_step(PeelCtl* c, int64_t* round_size, int64_t* round_level, 
 // that bucket lies inside the window (count < hi) it is the window's minimum; else the window
 // has no unpeeled member and is refilled as usual.
 template <typename CT>
-__device__ void dense_min(const PeelView<CT>& P) {
-    PeelCtl* c = P.ctl;
+__device__ __noinline__ void dense_min(const PeelView<CT>& P, const PeelHot& s) {
     if (blockIdx.x != 0) return;
     __shared__ unsigned long long s_found;
     if (threadIdx.x == 0) s_found = ULLONG_MAX;
     __syncthreads();
-    int64_t lo = c->k, span = 1;
+    int64_t lo = s.k, span = 1;
     unsigned long long got = ULLONG_MAX;
     while (lo < P.bmax) {
         int64_t hi = lo + span < P.bmax ? lo + span : P.bmax;
@@ -274,21 +270,20 @@ __device__ void dense_min(const PeelView<CT>& P) {
         lo = hi;
         span *= 2;
     }
-    if (threadIdx.x == 0 && got != ULLONG_MAX && (int64_t)got < c->hi) c->minN = got;
+    if (threadIdx.x == 0 && got != ULLONG_MAX && (int64_t)got < s.hi) P.ctl->h.minN = got;
 }
 
 template <typename CT>
-__device__ void phase_adv_min(const PeelView<CT>& P) {
-    PeelCtl* c = P.ctl;
-    if (c->done || !(c->mode & ND_MODE_ADV)) return;
+__device__ __noinline__ void phase_adv_min(const PeelView<CT>& P, const PeelHot& s, const Team& T) {
+    if (s.done || !(s.mode & ND_MODE_ADV)) return;
     if (P.bcnt) {
-        dense_min(P);
+        dense_min(P, s);
         return;
     }
-    const int32_t* N = pick(P.N, c->wn);
-    unsigned n = clampn(c->nN, P.cap);
+    const int32_t* N = pick(P.N, s.wn);
+    unsigned n = clampn(s.nN, P.cap);
     unsigned long long mn = ULLONG_MAX;
-    for (int64_t i = gthread(); i < n; i += nthreads()) {
+    for (int64_t i = T.thread(); i < n; i += T.nthreads()) {
         int32_t R = N[i];
         if (P.rnd[R] == ND_UNPEELED) {
             unsigned long long v = (unsigned long long)P.cnt[R];
@@ -296,66 +291,67 @@ __device__ void phase_adv_min(const PeelView<CT>& P) {
         }
     }
     mn = block_min(mn);
-    if (threadIdx.x == 0 && mn != ULLONG_MAX) atomicMin(&c->minN, mn);
+    if (threadIdx.x == 0 && mn != ULLONG_MAX) atomicMin(&P.ctl->h.minN, mn);
 }
 
 // refill 1/4: compact L into L' (alive only), global minimum count, clear the histogram
 template <typename CT>
-__device__ void phase_refill_scan(const PeelView<CT>& P) {
+__device__ __noinline__ void phase_refill_scan(const PeelView<CT>& P, const PeelHot& s, const Team& T) {
+    if (!need_refill(s)) return;
     PeelCtl* c = P.ctl;
-    if (!need_refill(c)) return;
-    for (int64_t i = gthread(); i < ND_HBINS; i += nthreads()) c->hist[i] = 0;
-    const int32_t* L = pick(P.L, c->wl);
-    int32_t* L2 = pick(P.L, c->wl ^ 1);
-    int64_t n = c->lmat ? (int64_t)clampn(c->nL, P.cap) : c->n_r;
+    for (int64_t i = T.thread(); i < ND_HBINS; i += T.nthreads()) c->hist[i] = 0;
+    const int32_t* L = pick(P.L, s.wl);
+    int32_t* L2 = pick(P.L, s.wl ^ 1);
+    const int32_t lmat = s.lmat;
+    int64_t n = lmat ? (int64_t)clampn(s.nL, P.cap) : s.n_r;
     unsigned long long mn = ULLONG_MAX;
     // grid-stride in whole-warp steps so that appends aggregate per warp
-    for (int64_t base = gthread() - (threadIdx.x & 31); base < n; base += nthreads()) {
+    for (int64_t base = T.thread() - (threadIdx.x & 31); base < n; base += T.nthreads()) {
         int64_t i = base + (threadIdx.x & 31);
         if (i < n) {
-            int32_t R = c->lmat ? L[i] : (int32_t)i;
+            int32_t R = lmat ? L[i] : (int32_t)i;
             if (P.rnd[R] == ND_UNPEELED) {
                 unsigned long long v = (unsigned long long)P.cnt[R];
                 mn = v < mn ? v : mn;
-                nd_append(&c->nL2, L2, P.cap, R, &c->err);
+                nd_append(&c->h.nL2, L2, P.cap, R, &c->err);
             }
         }
     }
     mn = block_min(mn);
-    if (threadIdx.x == 0 && mn != ULLONG_MAX) atomicMin(&c->gmin, mn);
+    if (threadIdx.x == 0 && mn != ULLONG_MAX) atomicMin(&c->h.gmin, mn);
 }
 
 // refill 2/4: histogram of count - gmin over L'
 template <typename CT>
-__device__ void phase_refill_hist(const PeelView<CT>& P) {
-    PeelCtl* c = P.ctl;
-    if (!need_refill(c)) return;
+__device__ __noinline__ void phase_refill_hist(const PeelView<CT>& P, const PeelHot& s, const Team& T) {
+    if (!need_refill(s)) return;
     __shared__ unsigned int h[ND_HBINS];
     for (int i = threadIdx.x; i < ND_HBINS; i += blockDim.x) h[i] = 0;
     __syncthreads();
-    const int32_t* L2 = pick(P.L, c->wl ^ 1);
-    unsigned n = clampn(c->nL2, P.cap);
-    unsigned long long g0 = c->gmin;
-    for (int64_t i = gthread(); i < n; i += nthreads()) {
+    const int32_t* L2 = pick(P.L, s.wl ^ 1);
+    unsigned n = clampn(s.nL2, P.cap);
+    unsigned long long g0 = s.gmin;
+    for (int64_t i = T.thread(); i < n; i += T.nthreads()) {
         unsigned long long d = (unsigned long long)P.cnt[L2[i]] - g0;
         atomicAdd(&h[d < ND_HBINS - 1 ? d : ND_HBINS - 1], 1u);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < ND_HBINS; i += blockDim.x)
-        if (h[i]) atomicAdd(&c->hist[i], (unsigned long long)h[i]);
+        if (h[i]) atomicAdd(&P.ctl->hist[i], (unsigned long long)h[i]);
 }
 
-// refill 3/4 (one block; any multiple of 32 threads dividing ND_HBINS): choose hi so that the
-// window holds about 1/16 of the unpeeled r-cliques (at least 16384), swap L <- L', clear N
-__device__ void phase_refill_pick(PeelCtl* c) {
-    if (!need_refill(c)) return;
+// refill 3/4: the bound hi of a window that holds about 1/16 of the unpeeled r-cliques (at least
+// 16384). Every thread of the block calls it (a multiple of 32 threads dividing ND_HBINS) and gets
+// the same answer; the persistent kernel has every block work it out for itself, because one thread
+// walking the bins waits for L2 up to 4096 times (0.5 ms, as long as a small graph's whole peel).
+__device__ __noinline__ int64_t refill_bound(const PeelCtl* c, const PeelHot& s) {
     __shared__ unsigned long long part[1024];
     __shared__ int best;
     const int nt = blockDim.x;
     const int per = ND_HBINS / nt;
-    unsigned long long s = 0;
-    for (int j = 0; j < per; ++j) s += c->hist[threadIdx.x * per + j];
-    part[threadIdx.x] = s;
+    unsigned long long sum = 0;
+    for (int j = 0; j < per; ++j) sum += c->hist[threadIdx.x * per + j];
+    part[threadIdx.x] = sum;
     if (threadIdx.x == 0) best = ND_HBINS - 1;
     __syncthreads();
     // inclusive scan of part[0..nt) (Hillis-Steele)
@@ -365,7 +361,7 @@ __device__ void phase_refill_pick(PeelCtl* c) {
         part[threadIdx.x] += y;
         __syncthreads();
     }
-    unsigned long long alive = c->nL2;
+    unsigned long long alive = s.nL2;
     unsigned long long target = alive / 16;
     if (target < 16384) target = 16384;
     unsigned long long run = threadIdx.x ? part[threadIdx.x - 1] : 0;
@@ -377,74 +373,56 @@ __device__ void phase_refill_pick(PeelCtl* c) {
         }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int b = best;
-        c->hi = (b >= ND_HBINS - 1) ? LLONG_MAX : (int64_t)c->gmin + b + 1;
-        c->wl ^= 1;
-        c->nL = c->nL2;
-        c->nL2 = 0;
-        c->lmat = 1;
-        c->nN = 0;
-        c->refills++;
-    }
+    const int b = best;
     __syncthreads();
+    return b >= ND_HBINS - 1 ? LLONG_MAX : (int64_t)s.gmin + b + 1;
 }
 
-__global__ void k_refill_pick(PeelCtl* c) { phase_refill_pick(c); }
+// the refilled window's bound, and L <- L'
+__device__ __forceinline__ void refill_apply(PeelHot& s, int64_t hi) {
+    s.hi = hi;
+    s.wl ^= 1;
+    s.nL = s.nL2;
+    s.nL2 = 0;
+    s.lmat = 1;
+    s.refills++;
+}
 
-// The same choice made by one thread (the serial part of a grid barrier).
-__device__ void refill_pick_serial(PeelCtl* c) {
-    unsigned long long alive = c->nL2;
-    unsigned long long target = alive / 16;
-    if (target < 16384) target = 16384;
-    unsigned long long run = 0;
-    int b = ND_HBINS - 1;
-    for (int i = 0; i < ND_HBINS; ++i) {
-        run += c->hist[i];
-        if (run >= target) {
-            b = i;
-            break;
-        }
+__global__ void k_refill_pick(PeelCtl* c) {
+    if (!need_refill(c->h)) return;
+    const int64_t hi = refill_bound(c, c->h);
+    if (threadIdx.x == 0) {
+        refill_apply(c->h, hi);
+        c->h.nN = 0;
     }
-    c->hi = (b >= ND_HBINS - 1) ? LLONG_MAX : (int64_t)c->gmin + b + 1;
-    c->wl ^= 1;
-    c->nL = c->nL2;
-    c->nL2 = 0;
-    c->lmat = 1;
-    c->nN = 0;
-    c->refills++;
 }
 
-// refill 4/4: N = { R in L : count < hi }
+// refill 4/4: N = { R in list : count < hi }
 template <typename CT>
-__device__ void phase_refill_select(const PeelView<CT>& P) {
+__device__ __noinline__ void phase_refill_select(const PeelView<CT>& P, const int32_t* L, unsigned n, int32_t* N, int64_t hi,
+                                    const Team& T) {
     PeelCtl* c = P.ctl;
-    if (!need_refill(c)) return;
-    const int32_t* L = pick(P.L, c->wl);
-    int32_t* N = pick(P.N, c->wn);
-    unsigned n = clampn(c->nL, P.cap);
-    int64_t hi = c->hi;
-    for (int64_t base = gthread() - (threadIdx.x & 31); base < n; base += nthreads()) {
+    for (int64_t base = T.thread() - (threadIdx.x & 31); base < n; base += T.nthreads()) {
         int64_t i = base + (threadIdx.x & 31);
         if (i < n) {
             int32_t R = L[i];
-            if ((int64_t)P.cnt[R] < hi) nd_append(&c->nN, N, P.cap, R, &c->err);
+            if ((int64_t)P.cnt[R] < hi) nd_append(&c->h.nN, N, P.cap, R, &c->err);
         }
     }
 }
 
 // advance: k' = max(k, min over N); A = { R in N alive : count <= k' }; N' = the other alive
 template <typename CT>
-__device__ void phase_adv_select(const PeelView<CT>& P) {
+__device__ __noinline__ void phase_adv_select(const PeelView<CT>& P, const PeelHot& s, const Team& T) {
+    if (s.done || !(s.mode & ND_MODE_ADV)) return;
     PeelCtl* c = P.ctl;
-    if (c->done || !(c->mode & ND_MODE_ADV)) return;
-    int64_t kn = knew_of(c);
-    const int32_t* N = pick(P.N, c->wn);
-    int32_t* N2 = pick(P.N, c->wn ^ 1);
-    int32_t* A = pick(P.A, c->wa);
-    unsigned n = clampn(c->nN, P.cap);
-    int32_t t = c->t;
-    for (int64_t base = gthread() - (threadIdx.x & 31); base < n; base += nthreads()) {
+    int64_t kn = knew_of(s);
+    const int32_t* N = pick(P.N, s.wn);
+    int32_t* N2 = pick(P.N, s.wn ^ 1);
+    int32_t* A = pick(P.A, s.wa);
+    unsigned n = clampn(s.nN, P.cap);
+    int32_t t = s.t;
+    for (int64_t base = T.thread() - (threadIdx.x & 31); base < n; base += T.nthreads()) {
         int64_t i = base + (threadIdx.x & 31);
         if (i < n) {
             int32_t R = N[i];
@@ -455,9 +433,9 @@ __device__ void phase_adv_select(const PeelView<CT>& P) {
                     P.core[R] = (int32_t)kn;
                     if (P.et_rnd) set_tri_round(P, R, t);
                     mark_a(P, R);
-                    nd_append(&c->cntA, A, P.cap, R, &c->err);
+                    nd_append(&c->h.cntA, A, P.cap, R, &c->err);
                 } else {
-                    nd_append(&c->nN2, N2, P.cap, R, &c->err);
+                    nd_append(&c->h.nN2, N2, P.cap, R, &c->err);
                 }
             }
         }
@@ -471,10 +449,9 @@ __device__ void phase_adv_select(const PeelView<CT>& P) {
 // <= its own position. Edges of the current round stay: the owner rule needs them. Runs at the
 // start of a round, between barriers, so no Update reads the rows meanwhile.
 template <typename CT>
-__device__ void phase_contract(const GraphView& g, const PeelView<CT>& P) {
-    PeelCtl* c = P.ctl;
-    if (c->done || !c->contract) return;
-    const int32_t t = c->t, shift = c->contract_shift;
+__device__ __noinline__ void phase_contract(const GraphView& g, const PeelView<CT>& P, const PeelHot& s) {
+    if (s.done || !s.contract) return;
+    const int32_t t = s.t, shift = P.ctl->contract_shift;
     const int lane = threadIdx.x & 31;
     for (int64_t v = gwarp(); v < g.n; v += nwarps()) {
         const int64_t b = g.rp[v];
@@ -512,7 +489,7 @@ __device__ void phase_contract(const GraphView& g, const PeelView<CT>& P) {
 }
 
 template <typename CT>
-__global__ void k_contract(GraphView g, PeelView<CT> P) { phase_contract(g, P); }
+__global__ void k_contract(GraphView g, PeelView<CT> P) { phase_contract(g, P, P.ctl->h); }
 
 // The same for the (3,4) triangle lists L(e): an entry is lost when its triangle was peeled in an
 // earlier round (its tag); a list that lost at least len_prev >> contract_shift entries since the
@@ -523,10 +500,9 @@ __global__ void k_contract(GraphView g, PeelView<CT> P) { phase_contract(g, P); 
 // when a < w < c, yz when w < a). The hash tables keep every entry: a lookup of a removed entry
 // finds its earlier tag, so the candidate is dropped as before.
 template <typename CT>
-__device__ void phase_contract34(const GraphView& g, const PeelView<CT>& P) {
-    PeelCtl* c = P.ctl;
-    if (c->done || !c->contract) return;
-    const int32_t t = c->t, shift = c->contract_shift;
+__device__ __noinline__ void phase_contract34(const GraphView& g, const PeelView<CT>& P, const PeelHot& s) {
+    if (s.done || !s.contract) return;
+    const int32_t t = s.t, shift = P.ctl->contract_shift;
     const int lane = threadIdx.x & 31;
     for (int64_t e = gwarp(); e < g.m; e += nwarps()) {
         const int64_t b = g.et_rp[e];
@@ -568,24 +544,28 @@ __device__ void phase_contract34(const GraphView& g, const PeelView<CT>& P) {
 }
 
 template <typename CT>
-__global__ void k_contract34(GraphView g, PeelView<CT> P) { phase_contract34(g, P); }
+__global__ void k_contract34(GraphView g, PeelView<CT> P) { phase_contract34(g, P, P.ctl->h); }
 
 template <typename CT>
-__global__ void k_adv_min(PeelView<CT> P) { phase_adv_min(P); }
+__global__ void k_adv_min(PeelView<CT> P) { phase_adv_min(P, P.ctl->h, grid_team()); }
 template <typename CT>
-__global__ void k_refill_scan(PeelView<CT> P) { phase_refill_scan(P); }
+__global__ void k_refill_scan(PeelView<CT> P) { phase_refill_scan(P, P.ctl->h, grid_team()); }
 template <typename CT>
-__global__ void k_refill_hist(PeelView<CT> P) { phase_refill_hist(P); }
+__global__ void k_refill_hist(PeelView<CT> P) { phase_refill_hist(P, P.ctl->h, grid_team()); }
 template <typename CT>
-__global__ void k_refill_select(PeelView<CT> P) { phase_refill_select(P); }
+__global__ void k_refill_select(PeelView<CT> P) {
+    const PeelHot& s = P.ctl->h;
+    if (!need_refill(s)) return;
+    phase_refill_select(P, pick(P.L, s.wl), clampn(s.nL, P.cap), pick(P.N, s.wn), s.hi, grid_team());
+}
 template <typename CT>
-__global__ void k_adv_select(PeelView<CT> P) { phase_adv_select(P); }
+__global__ void k_adv_select(PeelView<CT> P) { phase_adv_select(P, P.ctl->h, grid_team()); }
 
 // Rebuild A in ascending id order from the membership bitmap (persistent kernel, large rounds):
 // each block owns a fixed range of bitmap words; pass 1 counts its members, the serial step of the
 // barrier turns the per-block counts (hist[0 .. gridDim)) into offsets, pass 2 writes the ids.
-__device__ __forceinline__ void sort_range(const PeelCtl* c, int64_t& w0, int64_t& w1) {
-    int64_t nwords = (c->n_r + 31) >> 5;
+__device__ __forceinline__ void sort_range(const PeelHot& s, int64_t& w0, int64_t& w1) {
+    int64_t nwords = (s.n_r + 31) >> 5;
     int64_t per = (nwords + gridDim.x - 1) / gridDim.x;
     w0 = (int64_t)blockIdx.x * per;
     w1 = w0 + per < nwords ? w0 + per : nwords;
@@ -621,10 +601,10 @@ __device__ unsigned block_excl_sum(unsigned v, unsigned& excl) {
 }
 
 template <typename CT>
-__device__ void phase_sort_count(const PeelView<CT>& P) {
+__device__ __noinline__ void phase_sort_count(const PeelView<CT>& P, const PeelHot& s) {
     PeelCtl* c = P.ctl;
     int64_t w0, w1;
-    sort_range(c, w0, w1);
+    sort_range(s, w0, w1);
     unsigned cnt = 0, excl;
     for (int64_t w = w0 + threadIdx.x; w < w1; w += blockDim.x) cnt += __popc(P.abits[w]);
     unsigned total = block_excl_sum(cnt, excl);
@@ -636,10 +616,10 @@ __device__ void phase_sort_count(const PeelView<CT>& P) {
 // before it in this block (recounted from the bitmap, which the count pass left in L2); inside the
 // slice a warp scan places 32 words at a time, with no block-wide barrier per step.
 template <typename CT>
-__device__ void phase_sort_write(const PeelView<CT>& P) {
+__device__ __noinline__ void phase_sort_write(const PeelView<CT>& P, const PeelHot& s) {
     PeelCtl* c = P.ctl;
     int64_t w0, w1;
-    sort_range(c, w0, w1);
+    sort_range(s, w0, w1);
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int64_t per = (w1 - w0 + nw - 1) / nw;
@@ -654,7 +634,7 @@ __device__ void phase_sort_write(const PeelView<CT>& P) {
     const unsigned blocks_before = block_excl_sum(prior, excl);
     block_excl_sum(lane == 0 ? cnt : 0u, excl);
     unsigned long long at = (unsigned long long)blocks_before + __shfl_sync(full, excl, 0);
-    int32_t* A = pick(P.A, c->wa);
+    int32_t* A = pick(P.A, s.wa);
     for (int64_t base = a; base < b; base += 32) {
         const int64_t w = base + lane;
         uint32_t bits = w < b ? P.abits[w] : 0u;
@@ -679,33 +659,26 @@ __device__ void phase_sort_write(const PeelView<CT>& P) {
 // ------------------------------------------------------------------------------------
 // Update
 
+// What an Update phase works with: the view (in the kernel's parameters), a copy of it in shared
+// memory for what is called out of line, and the round's state.
 template <typename CT>
 struct RoundEnv {
-    PeelView<CT> P;
+    const PeelView<CT>& P;
+    const PeelView<CT>* Q;
+    const PeelHot* s;
     int32_t t;
     int64_t k, hi;
-    const int32_t* A;
-    unsigned nA;
-    int32_t* next;
-    int32_t* Ncur;
-    unsigned int* ncnt;
 };
 
 template <typename CT>
-__device__ __forceinline__ RoundEnv<CT> round_env(const PeelView<CT>& P) {
-    PeelCtl* c = P.ctl;
-    RoundEnv<CT> E;
-    E.P = P;
-    bool adv = c->mode & ND_MODE_ADV;
-    E.t = c->t;
-    E.k = adv ? knew_of(c) : c->k;
-    E.hi = c->hi;
-    E.A = pick(P.A, c->wa);
-    E.nA = clampn(adv ? c->cntA : c->nA, P.cap);
-    E.next = pick(P.A, c->wa ^ 1);
-    E.Ncur = adv ? pick(P.N, c->wn ^ 1) : pick(P.N, c->wn);
-    E.ncnt = adv ? &c->nN2 : &c->nN;
-    return E;
+__device__ __forceinline__ RoundEnv<CT> round_env(const PeelView<CT>& P, const PeelView<CT>* Q, const PeelHot* s) {
+    return RoundEnv<CT>{P, Q, s, s->t, (s->mode & ND_MODE_ADV) ? knew_of(*s) : s->k, s->hi};
+}
+
+// |A| and A of the round
+template <typename CT>
+__device__ __forceinline__ unsigned round_nA(const PeelView<CT>& P, const PeelHot& s) {
+    return clampn((s.mode & ND_MODE_ADV) ? s.cntA : s.nA, P.cap);
 }
 
 // per-thread statistics of one Update phase
@@ -714,27 +687,37 @@ struct UpdCounters {
     unsigned long long decs = 0;    // count decrements applied
 };
 
-// What a decrement of r-clique x from o to o - 1 implies: x falls to <= k (it is the next
-// round's A: its round, core number and index tags are written now) and/or below the bucket
-// window (it joins N).
+// What a decrement of r-clique x from o to o - 1 implies: at o = k + 1 x falls to k (it is the next
+// round's A: its round, core number and index tags are written now), at o = hi it falls below the
+// bucket window's bound and joins N. Most decrements do neither, and so the rest is out of
+// line, with its pointers in shared memory, and costs the loops around it no registers.
 template <typename CT>
-__device__ __forceinline__ void after_dec(const RoundEnv<CT>& E, int32_t x, int64_t o) {
+__device__ __noinline__ void after_dec_rest(const PeelView<CT>* Q, const PeelHot* s, int32_t x, int64_t o, int64_t k) {
+    PeelCtl* c = Q->ctl;
     // dense buckets: a count above k + 1 moves down one bucket; at k + 1 the r-clique is scheduled
     // now and leaves the buckets; at or below k it was scheduled already
-    if (E.P.bcnt && o > E.k) {
-        atomicSub(&E.P.bcnt[o], 1u);
-        if (o > E.k + 1) atomicAdd(&E.P.bcnt[o - 1], 1u);
+    if (Q->bcnt && o > k) {
+        atomicSub(&Q->bcnt[o], 1u);
+        if (o > k + 1) atomicAdd(&Q->bcnt[o - 1], 1u);
     }
-    if (o > E.k && o - 1 <= E.k) {
-        E.P.rnd[x] = E.t + 1;
-        E.P.core[x] = (int32_t)E.k;
-        if (E.P.et_rnd) set_tri_round(E.P, x, E.t + 1);
-        mark_a(E.P, x);
-        nd_append(&E.P.ctl->nNext, E.next, E.P.cap, x, &E.P.ctl->err);
+    if (o == k + 1) {
+        const int32_t t1 = s->t + 1;
+        Q->rnd[x] = t1;
+        Q->core[x] = (int32_t)k;
+        if (Q->et_rnd) set_tri_round(*Q, x, t1);
+        mark_a(*Q, x);
+        nd_append(&c->h.nNext, s->wa ? Q->A[0] : Q->A[1], Q->cap, x, &c->err);
     }
-    if (o >= E.hi && o - 1 < E.hi) nd_append(E.ncnt, E.Ncur, E.P.cap, x, &E.P.ctl->err);
+    if (o == s->hi) {
+        const bool adv = s->mode & ND_MODE_ADV;
+        nd_append(adv ? &c->h.nN2 : &c->h.nN, s->wn ^ (adv ? 1 : 0) ? Q->N[1] : Q->N[0], Q->cap, x, &c->err);
+    }
 }
 
+template <typename CT>
+__device__ __forceinline__ void after_dec(const RoundEnv<CT>& E, int32_t x, int64_t o) {
+    if (o == E.k + 1 || o == E.hi || E.P.bcnt) after_dec_rest(E.Q, E.s, x, o, E.k);
+}
 
 // Whether a member of a destroyed S with round tag r has its count decremented on the device: not
 // if it is in A (r = t), and not if it was already pushed into the next round's A during this
@@ -767,14 +750,18 @@ __device__ __forceinline__ void update_func(const RoundEnv<CT>& E, int32_t R, co
     }
 }
 
-__device__ __forceinline__ void add_counters(PeelCtl* c, UpdCounters k) {
+// A phase's counters, summed over the warp, to `listed` and `decs` (the control block's, or in the
+// persistent kernel the block's own in shared memory, which reach the control block once at the end:
+// two same-address atomics per warp and round cost as much as a short round's Update).
+__device__ __forceinline__ void add_counters(unsigned long long* listed, unsigned long long* decs, UpdCounters k) {
+    if (!__any_sync(0xffffffffu, (k.listed | k.decs) != 0)) return;
     for (int o = 16; o > 0; o >>= 1) {
         k.listed += __shfl_down_sync(0xffffffffu, k.listed, o);
         k.decs += __shfl_down_sync(0xffffffffu, k.decs, o);
     }
     if ((threadIdx.x & 31) == 0) {
-        if (k.listed) atomicAdd(&c->listed, k.listed);
-        if (k.decs) atomicAdd(&c->decs, k.decs);
+        if (k.listed) atomicAdd(listed, k.listed);
+        if (k.decs) atomicAdd(decs, k.decs);
     }
 }
 
@@ -806,6 +793,19 @@ __device__ __forceinline__ void run_all(const GraphView& g, const RoundEnv<CT>& 
     for (int64_t j = j0; j < n0; j += dj) U::cand(g, E, R, q, j, k);
 }
 
+// R is left to the heavy phase; false if its list is full. Called by a whole warp.
+template <typename CT>
+__device__ __noinline__ bool defer_heavy(const PeelView<CT>* Q, int32_t R) {
+    int queued = 0;
+    if ((threadIdx.x & 31) == 0) {
+        const unsigned slot = atomicAdd(&Q->ctl->h.nH, 1u);
+        if (slot < Q->hcap) {
+            Q->H[slot] = R;
+            queued = 1;
+        }
+    }
+    return __shfl_sync(0xffffffffu, queued, 0);
+}
 
 // (1,2): R = v; S = {v, w} for every neighbour w.
 template <typename CT>
@@ -835,6 +835,7 @@ struct Upd13 {
     __device__ static void cand(const GraphView& g, const RoundEnv<CT>& E, int32_t v, const Q& q, int64_t j,
                                 UpdCounters& k) {
         int32_t w = g.col[q.b[0] + j];
+#pragma unroll 1
         for (int64_t jx = g.dg_rp[w]; jx < g.dg_rp[w + 1]; ++jx) {
             int32_t x = g.dg_col[jx];
             if (nd_find(g.col + q.b[0], q.n[0], x) < 0) continue;
@@ -952,6 +953,7 @@ struct Upd24 {
         int64_t xb = u_drives ? ub : vb, xn = u_drives ? un : vn;
         int64_t yb = u_drives ? vb : ub, yn = u_drives ? vn : un;
         int cnt = 0;
+#pragma unroll 1
         for (int64_t p0 = 0; p0 < xn; p0 += 32) {
             int64_t p = p0 + lane;
             int64_t q = -1;
@@ -976,6 +978,7 @@ struct Upd24 {
         __syncwarp();
         // exclusive prefix of the out-degrees (cnt <= kI24 < 128: at most four 32-wide chunks)
         int32_t carry = 0;
+#pragma unroll 1
         for (int c0 = 0; c0 < cnt; c0 += 32) {
             int i = c0 + lane;
             int32_t d = i < cnt ? st.pre[i] : 0, inc = d;
@@ -988,6 +991,7 @@ struct Upd24 {
         }
         if (lane == 0) st.pre[cnt] = carry;
         __syncwarp();
+#pragma unroll 1
         for (int32_t p = lane; p < carry; p += 32) pair(g, E, R, st, cnt, p, k);
         __syncwarp();
     }
@@ -1040,7 +1044,8 @@ struct Upd24 {
         // exclusive prefix of the out-degrees (one warp; the totals fit int32: at most m)
         if (wid == 0) {
             int32_t carry = 0;
-            for (int c0 = 0; c0 < cnt; c0 += 32) {
+    #pragma unroll 1
+        for (int c0 = 0; c0 < cnt; c0 += 32) {
                 int i = c0 + lane;
                 int32_t d = i < cnt ? st.pre[i] : 0, inc = d;
                 for (int o = 1; o < 32; o <<= 1) {
@@ -1109,33 +1114,37 @@ struct Upd34 {
         lists34(g, P, R, q);
         return q.n[0];
     }
-    // the triangle R + w of list x (w's entry in L(e_x)) and its round; false when w is not there
+    // the triangle R + w of list x, which has no table (w's entry in L(e_x)), and its round; false
+    // when w is not there
     template <typename Q>
-    __device__ static bool look(const GraphView& g, const RoundEnv<CT>& E, const Q& q, int x, int32_t w,
-                                int32_t& id, int32_t& r) {
-        if (q.h[x] >= 0) {
-            if (!nd_hash_find(E.P.htab + q.h[x], q.hk[x], w, id, r)) return false;
-        } else {
-            int64_t i = nd_find(g.et_w + q.b[x], q.n[x], w);
-            if (i < 0) return false;
-            r = E.P.et_rnd[q.b[x] + i];
-            id = g.et_t[q.b[x] + i];
-        }
+    __device__ static bool bisect(const GraphView& g, const RoundEnv<CT>& E, const Q& q, int x, int32_t w,
+                                  int32_t& id, int32_t& r) {
+        int64_t i = nd_find(g.et_w + q.b[x], q.n[x], w);
+        if (i < 0) return false;
+        r = E.P.et_rnd[q.b[x] + i];
+        id = g.et_t[q.b[x] + i];
         return true;
     }
     // S = R + w, w = entry j of list 0. Only the owner (smallest id of S's members in A) applies
     // S, so R stops as soon as a member in A with a smaller id is known: first the entry's own
-    // triangle (read along the list), then the ones found in lists 1 and 2.
+    // triangle (read along the list), then the ones found in lists 1 and 2. The entry's three words
+    // are loaded together and so are the first slots of both tables: one trip to L2 each.
     template <typename Q>
     __device__ static void cand(const GraphView& g, const RoundEnv<CT>& E, int32_t R, const Q& q, int64_t j,
                                 UpdCounters& k) {
-        int32_t r0 = E.P.et_rnd[q.b[0] + j];
+        const int32_t r0 = E.P.et_rnd[q.b[0] + j], id0 = g.et_t[q.b[0] + j], w = g.et_w[q.b[0] + j];
         if (r0 < E.t) return;
-        int32_t id0 = g.et_t[q.b[0] + j];
         if (r0 == E.t && id0 < R) return;
-        int32_t w = g.et_w[q.b[0] + j], id1, r1, id2, r2;
-        if (!look(g, E, q, 1, w, id1, r1) || r1 < E.t || (r1 == E.t && id1 < R)) return;
-        if (!look(g, E, q, 2, w, id2, r2) || r2 < E.t || (r2 == E.t && id2 < R)) return;
+        const NdHashSlot *t1 = E.P.htab + q.h[1], *t2 = E.P.htab + q.h[2];
+        uint32_t s1 = 0, s2 = 0;
+        int4 p1, p2;
+        if (q.h[1] >= 0) p1 = *reinterpret_cast<const int4*>(t1 + (s1 = nd_hash_slot(w, q.hk[1])));
+        if (q.h[2] >= 0) p2 = *reinterpret_cast<const int4*>(t2 + (s2 = nd_hash_slot(w, q.hk[2])));
+        int32_t id1, r1, id2, r2;
+        if (q.h[1] >= 0 ? !nd_hash_resolve(t1, q.hk[1], w, s1, p1, id1, r1) : !bisect(g, E, q, 1, w, id1, r1)) return;
+        if (r1 < E.t || (r1 == E.t && id1 < R)) return;
+        if (q.h[2] >= 0 ? !nd_hash_resolve(t2, q.hk[2], w, s2, p2, id2, r2) : !bisect(g, E, q, 2, w, id2, r2)) return;
+        if (r2 < E.t || (r2 == E.t && id2 < R)) return;
         k.listed++;
         // issue the decrements before looking at any result (the atomics overlap in flight)
         int64_t o0 = dec_live(r0, E.t) ? nd_atomic_dec(&E.P.cnt[id0]) : 0;
@@ -1180,7 +1189,7 @@ struct Upd34 {
             hk = q.hk[1] | (q.hk[2] << 8);
             paired = h1 >= 0 && h2 >= 0;
             if (n0 > heavy) {
-                unsigned slot = atomicAdd(&E.P.ctl->nH, 1u);
+                unsigned slot = atomicAdd(&E.P.ctl->h.nH, 1u);
                 if (slot < E.P.hcap) {
                     E.P.H[slot] = R;
                     n0 = 0;  // the heavy phase lists it
@@ -1189,6 +1198,7 @@ struct Upd34 {
         }
         int qn = 0;
         unsigned todo = __ballot_sync(full, paired && n0 > 0);
+#pragma unroll 1
         while (todo) {
             const int sl = __ffs(todo) - 1;
             todo &= todo - 1;
@@ -1202,6 +1212,7 @@ struct Upd34 {
                 i0 = g.et_t[bs + j];
                 w0 = g.et_w[bs + j];
             }
+#pragma unroll 1
             for (int64_t off = 0; off < ns; off += 32) {
                 const int64_t jn = off + 32 + lane;
                 int32_t r1 = -1, i1 = 0, w1 = 0;
@@ -1236,12 +1247,14 @@ struct Upd34 {
         }
         // triangles with a list that is not hashed: one at a time, per candidate
         unsigned rest = __ballot_sync(full, !paired && n0 > 0);
+#pragma unroll 1
         while (rest) {
             const int sl = __ffs(rest) - 1;
             rest &= rest - 1;
             const int32_t Rs = __shfl_sync(full, R, sl);
             Prep q;
             lists34(g, E.P, Rs, q);
+#pragma unroll 1
             for (int64_t jj = lane; jj < q.n[0]; jj += 32) cand(g, E, Rs, q, jj, k);
         }
     }
@@ -1372,20 +1385,34 @@ struct heavy_work<U, decltype((void)U::kHeavyWork)> {
     static constexpr int64_t value = U::kHeavyWork;
 };
 
-// Update hands out A to warps in chunks taken from a counter that the round's control step resets:
-// a warp that finishes early takes more, so the round ends when the work ends rather than when the
-// unluckiest warp of a static assignment does. A chunk holds about nA / (16 warps) r-cliques (at
-// least 1), so a round costs about 16 counter updates per warp however large A is.
-__device__ __forceinline__ unsigned update_chunk(unsigned nA) {
-    unsigned long long w = (unsigned long long)nwarps() * 16ull;
-    unsigned long long c = nA / w;
-    return c ? (unsigned)c : 1u;
+// Update hands out A to warps in chunks. The first chunk of each warp is its own by number; the
+// others come from a counter that the round's control step resets, so that a warp that finishes
+// early takes more and the round ends when the work ends rather than when the unluckiest warp of a
+// static assignment does. A chunk holds about nA / (16 warps) r-cliques (at least 1), so a round costs
+// about 16 counter updates per warp however large A is, and none when A has no more than one chunk
+// for each warp: 4,864 warps asking one counter take longer than a short round's work.
+__device__ __forceinline__ unsigned update_chunk(unsigned nA, const Team& T) {
+    unsigned c = nA / (T.nwarps * 16u);
+    return c ? c : 1u;
 }
 
-__device__ __forceinline__ unsigned take_chunk(PeelCtl* c, unsigned chunk) {
+__device__ __forceinline__ unsigned next_chunk(PeelCtl* c, unsigned nA, unsigned chunk, const Team& T) {
+    const unsigned first = T.nwarps * chunk;  // at most nA / 4 + nwarps
+    if (first >= nA) return nA;
     unsigned i0 = 0;
-    if ((threadIdx.x & 31) == 0) i0 = atomicAdd(&c->upd_next, chunk);
-    return __shfl_sync(0xffffffffu, i0, 0);
+    if ((threadIdx.x & 31) == 0) i0 = atomicAdd(&c->h.upd_next, chunk);
+    return first + __shfl_sync(0xffffffffu, i0, 0);
+}
+
+// A round with fewer r-cliques than half the warps shares each among 2^shift of them (at most 128):
+// a round lasts as long as its longest r-clique, and one warp takes a chain of half a dozen to twenty
+// dependent accesses, at 0.35 us each, for every 32 candidates.
+// Measured against one warp each: (2,3) on a Chung-Lu graph of 200,001 vertices and 2.4 M edges, Update
+// 5.2 + heavy phase 2.3 ms before, 4.8 + 0.1 ms after; (3,4) on R-MAT scale 18, 490 -> 430 ms.
+__device__ __forceinline__ unsigned split_shift(unsigned nA, const Team& T) {
+    if (nA == 0 || nA > T.nwarps / 2) return 0;
+    const unsigned shift = 31 - __clz(T.nwarps / nA);
+    return shift < 7 ? shift : 7;
 }
 
 // the heavy-phase threshold of this decomposition: a tuned value if given (capped by what a warp's
@@ -1398,87 +1425,118 @@ __device__ __forceinline__ int64_t heavy_limit(const PeelView<CT>& P) {
 }
 
 template <typename CT, typename U>
-__device__ void phase_update(const GraphView& g, const PeelView<CT>& P) {
-    if (P.ctl->done) return;
-    RoundEnv<CT> E = round_env(P);
-    const unsigned full = 0xffffffffu;
+__device__ __forceinline__ void phase_update(const GraphView& g, const PeelView<CT>& P, const PeelView<CT>* Q,
+                                             const PeelHot& s, const Team& T, unsigned long long* listed,
+                                             unsigned long long* decs) {
+    if (s.done) return;
+    const RoundEnv<CT> E = round_env(P, Q, &s);
+    const int32_t* A = pick(P.A, s.wa);
+    const unsigned nA = round_nA(P, s);
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     UpdCounters k;
-    if constexpr (is_staged<U>::value) {
-        // one warp per r-clique, I staged in the warp's shared memory
-        __shared__ int32_t s_w[kMaxWarpsPerBlock][kI24], s_x[kMaxWarpsPerBlock][kI24],
-            s_y[kMaxWarpsPerBlock][kI24], s_b[kMaxWarpsPerBlock][kI24], s_p[kMaxWarpsPerBlock][kI24 + 1];
-        const unsigned chunk = update_chunk(E.nA);
-        for (unsigned i0 = take_chunk(P.ctl, chunk); i0 < E.nA; i0 = take_chunk(P.ctl, chunk))
-        for (unsigned i = i0; i < i0 + chunk && i < E.nA; ++i) {
-            int32_t R = E.A[i];
-            if (lane == 0) unmark_a(P, R);
-            if (U::work(g, R) > heavy_limit<U>(P)) {
-                int queued = 0;
-                if (lane == 0) {
-                    unsigned slot = atomicAdd(&P.ctl->nH, 1u);
-                    if (slot < P.hcap) {
-                        P.H[slot] = R;
-                        queued = 1;
-                    }
+    if constexpr (!is_staged<U>::value) {
+        const unsigned shift = split_shift(nA, T);
+        if (shift) {
+            // fewer r-cliques than half the warps: 2^shift warps share each one, 32 candidates each in turn
+            const unsigned i = T.warp >> shift, part = T.warp & ((1u << shift) - 1u);
+            if (i < nA) {
+                const int32_t R = A[i];
+                Prep q;
+                int64_t n0 = U::prep(g, P, R, q), j0 = part * 32 + lane, dj = (int64_t)32 << shift;
+                if (part == 0 && lane == 0) unmark_a(P, R);
+                if (n0 > heavy_limit<U>(P) << shift) {
+                    // one of the warps hands it over; with no room there it lists all of it itself
+                    if (part != 0 || defer_heavy(Q, R)) n0 = 0;
+                    j0 = lane;
+                    dj = 32;
                 }
-                if (__shfl_sync(full, queued, 0)) continue;
-                // the staged warp path holds at most kI24 entries; the list is sized to hold every
-                // r-clique for staged functors, so this is unreachable
-                if (lane == 0) atomicOr(&P.ctl->err, 1);
-                continue;
+#pragma unroll 1
+                for (int64_t j = j0; j < n0; j += dj) U::cand(g, E, R, q, j, k);
             }
-            Stage24 stg{s_w[wid], s_x[wid], s_y[wid], s_b[wid], s_p[wid]};
-            U::run_warp(g, E, R, k, stg);
+            add_counters(listed, decs, k);
+            return;
         }
-    } else if constexpr (is_queued<U>::value) {
+    }
+    if constexpr (is_queued<U>::value) {
         // groups of up to 32 r-cliques per warp with a queue of live candidates (Upd34::run_group);
         // chunks of at most 32, about nA / (4 warps) each, so that small rounds still spread
         __shared__ int32_t s_qw[kMaxWarpsPerBlock][U::kQueue], s_qi[kMaxWarpsPerBlock][U::kQueue],
             s_qm[kMaxWarpsPerBlock][U::kQueue];
-        unsigned long long per = (unsigned long long)nwarps() * 4ull;
-        unsigned chunk = (unsigned)(E.nA / per);
+        unsigned chunk = nA / (T.nwarps * 4u);
         chunk = chunk < 1u ? 1u : (chunk > 32u ? 32u : chunk);
         const int64_t heavy = heavy_limit<U>(P);
-        for (unsigned i0 = take_chunk(P.ctl, chunk); i0 < E.nA; i0 = take_chunk(P.ctl, chunk)) {
-            int nG = (int)(E.nA - i0 < chunk ? E.nA - i0 : chunk);
-            U::run_group(g, E, E.A + i0, nG, heavy, k, s_qw[wid], s_qi[wid], s_qm[wid]);
+#pragma unroll 1
+        for (unsigned i0 = T.warp * chunk; i0 < nA; i0 = next_chunk(P.ctl, nA, chunk, T)) {
+            int nG = (int)(nA - i0 < chunk ? nA - i0 : chunk);
+            U::run_group(g, E, A + i0, nG, heavy, k, s_qw[wid], s_qi[wid], s_qm[wid]);
         }
     } else {
-        // one warp per r-clique: its lanes read the driving list coalesced
-        const unsigned chunk = update_chunk(E.nA);
-        for (unsigned i0 = take_chunk(P.ctl, chunk); i0 < E.nA; i0 = take_chunk(P.ctl, chunk))
-        for (unsigned i = i0; i < i0 + chunk && i < E.nA; ++i) {
-            int32_t R = E.A[i];
-            if (lane == 0) unmark_a(P, R);
-            Prep q;
-            int64_t n0 = U::prep(g, P, R, q);
-            if (n0 > heavy_limit<U>(P)) {
-                int queued = 0;
-                if (lane == 0) {
-                    unsigned slot = atomicAdd(&P.ctl->nH, 1u);
-                    if (slot < P.hcap) {
-                        P.H[slot] = R;
-                        queued = 1;
+        // staged variants: one warp per r-clique, I in the warp's shared memory; in a round with at most
+        // two r-cliques per block, one block each, I in the memory of all its warps (or, too long for that,
+        // left to the heavy phase): a warp needs some 25 dependent accesses to stage I and 5 more for
+        // every 32 pairs. (2,4) on a Chung-Lu graph of 500,009 vertices with 500 communities: Update
+        // 68 -> 36 ms, heavy phase 56 -> 43 ms
+        constexpr int kCap = is_staged<U>::value ? kMaxWarpsPerBlock * kI24 : 1;
+        constexpr int kOwn = is_staged<U>::value ? kI24 : 1;
+        __shared__ int32_t s_w[kCap], s_x[kCap], s_y[kCap], s_b[kCap], s_p[kCap + kMaxWarpsPerBlock];
+        if constexpr (is_staged<U>::value) {
+            if (nA <= 2 * T.nblocks) {
+                Stage24 stg{s_w, s_x, s_y, s_b, s_p};
+#pragma unroll 1
+                for (unsigned i = T.block; i < nA; i += T.nblocks) {
+                    const int32_t R = A[i];
+                    if (threadIdx.x == 0) unmark_a(P, R);
+                    if (U::work(g, R) > (int64_t)(blockDim.x >> 5) * kI24) {
+                        if (threadIdx.x < 32 && !defer_heavy(Q, R) && lane == 0) atomicOr(&P.ctl->err, 1);
+                        continue;
                     }
+                    U::run_block(g, E, R, k, stg);
                 }
-                if (__shfl_sync(full, queued, 0)) continue;
+                add_counters(listed, decs, k);
+                return;
             }
-            for (int64_t j = lane; j < n0; j += 32) U::cand(g, E, R, q, j, k);
         }
+        const unsigned chunk = update_chunk(nA, T);
+#pragma unroll 1
+        for (unsigned i0 = T.warp * chunk; i0 < nA; i0 = next_chunk(P.ctl, nA, chunk, T))
+#pragma unroll 1
+            for (unsigned i = i0; i < i0 + chunk && i < nA; ++i) {
+                const int32_t R = A[i];
+                if (lane == 0) unmark_a(P, R);
+                if constexpr (is_staged<U>::value) {
+                    if (U::work(g, R) > heavy_limit<U>(P)) {
+                        // the staged warp path holds at most kI24 entries; the heavy list holds every
+                        // r-clique for staged functors, so it is never full
+                        if (!defer_heavy(Q, R) && lane == 0) atomicOr(&P.ctl->err, 1);
+                        continue;
+                    }
+                    const int at = wid * kOwn;
+                    Stage24 stg{s_w + at, s_x + at, s_y + at, s_b + at, s_p + wid * (kOwn + 1)};
+                    U::run_warp(g, E, R, k, stg);
+                } else {
+                    // one warp per r-clique: its lanes read the driving list coalesced
+                    Prep q;
+                    int64_t n0 = U::prep(g, P, R, q);
+                    if (n0 > heavy_limit<U>(P) && defer_heavy(Q, R)) continue;
+#pragma unroll 1
+                    for (int64_t j = lane; j < n0; j += 32) U::cand(g, E, R, q, j, k);
+                }
+            }
     }
-    add_counters(P.ctl, k);
+    add_counters(listed, decs, k);
 }
 
+// The heavy phase: one block per heavy r-clique, its threads striding the driving list, so that heavy
+// r-cliques run side by side, each over many threads.
 template <typename CT, typename U>
-__device__ void phase_update_heavy(const GraphView& g, const PeelView<CT>& P) {
-    if (P.ctl->done) return;
-    unsigned nH = clampn(P.ctl->nH, P.hcap);
+__device__ __forceinline__ void phase_update_heavy(const GraphView& g, const PeelView<CT>& P, const PeelView<CT>* Q,
+                                                   const PeelHot& s, unsigned long long* listed,
+                                                   unsigned long long* decs) {
+    if (s.done) return;
+    unsigned nH = clampn(s.nH, P.hcap);
     if (nH == 0) return;
-    RoundEnv<CT> E = round_env(P);
+    const RoundEnv<CT> E = round_env(P, Q, &s);
     UpdCounters k;
-    // one block per heavy r-clique, its threads striding the driving list: heavy r-cliques run
-    // side by side, each over many threads
     if constexpr (is_staged<U>::value) {
         // blocks below hslices own a scratch slice of 5 * (hstage + 1) int32 and share the list
         unsigned ns = (unsigned)P.hslices < gridDim.x ? (unsigned)P.hslices : gridDim.x;
@@ -1491,7 +1549,7 @@ __device__ void phase_update_heavy(const GraphView& g, const PeelView<CT>& P) {
     } else {
         for (unsigned h = blockIdx.x; h < nH; h += gridDim.x) run_all<U>(g, E, P.H[h], threadIdx.x, blockDim.x, k);
     }
-    add_counters(P.ctl, k);
+    add_counters(listed, decs, k);
 }
 
 // (2,4) heavy phase split over the grid (persistent kernel, when the round's heavy edges fit the
@@ -1501,10 +1559,10 @@ __device__ void phase_update_heavy(const GraphView& g, const PeelView<CT>& P) {
 // of any heavy edge. A round whose few heavy edges used to occupy a few blocks spreads them over
 // all of them.
 template <typename CT, typename U>
-__device__ void phase_heavy_stage(const GraphView& g, const PeelView<CT>& P) {
-    if (P.ctl->done) return;
-    unsigned nH = clampn(P.ctl->nH, P.hcap);
-    RoundEnv<CT> E = round_env(P);
+__device__ __forceinline__ void phase_heavy_stage(const GraphView& g, const PeelView<CT>& P, const PeelView<CT>* Q, const PeelHot& s) {
+    if (s.done) return;
+    unsigned nH = clampn(s.nH, P.hcap);
+    const RoundEnv<CT> E = round_env(P, Q, &s);
     const int64_t c = P.hstage + 1;
     for (unsigned b = blockIdx.x; b < nH; b += gridDim.x) {
         int32_t* base = P.hscratch + (int64_t)b * 5 * c;
@@ -1519,13 +1577,15 @@ __device__ void phase_heavy_stage(const GraphView& g, const PeelView<CT>& P) {
 }
 
 template <typename CT, typename U>
-__device__ void phase_heavy_pairs(const GraphView& g, const PeelView<CT>& P) {
-    if (P.ctl->done) return;
-    unsigned nH = clampn(P.ctl->nH, P.hcap);
-    RoundEnv<CT> E = round_env(P);
+__device__ __forceinline__ void phase_heavy_pairs(const GraphView& g, const PeelView<CT>& P, const PeelView<CT>* Q, const PeelHot& s,
+                                  unsigned long long* listed, unsigned long long* decs) {
+    if (s.done) return;
+    unsigned nH = clampn(s.nH, P.hcap);
+    const RoundEnv<CT> E = round_env(P, Q, &s);
     UpdCounters k;
     const int64_t c = P.hstage + 1, T = P.hpre[nH];
-    for (int64_t p = gthread(); p < T; p += nthreads()) {
+    const Team G = grid_team();
+    for (int64_t p = G.thread(); p < T; p += G.nthreads()) {
         unsigned lo = 0, hi = nH;  // the last edge whose offset is <= p
         while (hi - lo > 1) {
             unsigned mid = (lo + hi) >> 1;
@@ -1538,13 +1598,23 @@ __device__ void phase_heavy_pairs(const GraphView& g, const PeelView<CT>& P) {
         Stage24 stg{base, base + c, base + 2 * c, base + 3 * c, base + 4 * c};
         U::pair(g, E, P.H[lo], stg, P.hcnt[lo], (int32_t)(p - P.hpre[lo]), k);
     }
-    add_counters(P.ctl, k);
+    add_counters(listed, decs, k);
 }
 
 template <typename CT, typename U>
-__global__ void k_update(GraphView g, PeelView<CT> P) { phase_update<CT, U>(g, P); }
+__global__ void k_update(GraphView g, PeelView<CT> P) {
+    __shared__ PeelView<CT> Q;
+    if (threadIdx.x == 0) Q = P;
+    __syncthreads();
+    phase_update<CT, U>(g, P, &Q, P.ctl->h, grid_team(), &P.ctl->listed, &P.ctl->decs);
+}
 template <typename CT, typename U>
-__global__ void k_update_heavy(GraphView g, PeelView<CT> P) { phase_update_heavy<CT, U>(g, P); }
+__global__ void k_update_heavy(GraphView g, PeelView<CT> P) {
+    __shared__ PeelView<CT> Q;
+    if (threadIdx.x == 0) Q = P;
+    __syncthreads();
+    phase_update_heavy<CT, U>(g, P, &Q, P.ctl->h, &P.ctl->listed, &P.ctl->decs);
+}
 
 // ------------------------------------------------------------------------------------
 // The whole peeling loop in one cooperative launch (every block resident at once), with a grid
@@ -1567,9 +1637,15 @@ __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long
     return v;
 }
 
-__device__ __forceinline__ int ld_acquire_i32(const int* p) {
+__device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ int ld_relaxed_i32(const int* p) {
     int v;
-    asm volatile("ld.acquire.gpu.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    asm volatile("ld.relaxed.gpu.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
 
@@ -1584,186 +1660,251 @@ __device__ __forceinline__ void st_release_u64(unsigned long long* p, unsigned l
     asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-// Grid barrier. The block that arrives last runs serial() in its thread 0 (it sees every write
-// made before the barrier) and then releases the others, so a control step costs no extra
-// barrier. Arrival is an acquire-release RMW and the release a release store; waiting blocks poll
-// with an acquire load, so all writes before the barrier are visible after it. The wait is
-// bounded by the global timer: after ctl->bar_timeout_ns (kBarrierTimeoutNs by default), or once
-// another block gave up, a block sets ctl->err bit 8 and the function returns false.
-template <typename F>
-__device__ bool grid_barrier(PeelCtl* c, unsigned long long& target, F serial) {
-    __shared__ int ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        target += gridDim.x;
-        unsigned long long old = atom_add_acq_rel_u64(&c->bar_arrive, 1ull);
-        int good = 1;
-        if (old + 1 == target) {
-            serial();
-            st_release_u64(&c->bar_gen, target);
-        } else {
-            unsigned long long t0 = globaltimer();
-            const unsigned long long limit = c->bar_timeout_ns;
-            while (ld_acquire_u64(&c->bar_gen) < target) {
-                if ((ld_acquire_i32(&c->err) & 8) || globaltimer() - t0 > limit) {
-                    atomicOr(&c->err, 8);
-                    good = 0;
-                    break;
-                }
-                __nanosleep(20);
+// What the persistent kernel's blocks keep in shared memory between phases.
+struct LoopState {
+    PeelHot s;      // the round's state, copied from the control block after every barrier
+    PeelCtl* c;
+    unsigned long long target;  // arrivals after which the next grid barrier opens
+    unsigned long long listed, decs;  // this block's counters
+    unsigned long long last, in_round, ph_ns[7];  // block 0: time of the last barrier, of this round's Update, of each phase
+    int ok;
+    // for the serial steps
+    int64_t* round_size;
+    int64_t* round_level;
+    int64_t* round_ns;
+    int64_t round_cap;
+    int64_t* hpre;
+    unsigned sort_min;  // |A| from which a round sorts A (beyond cap: never)
+    unsigned cap;
+    int32_t hslices;
+};
+
+// The serial step that runs inside a barrier.
+enum Serial { kNothing, kRound, kAfterMin, kAfterSelect, kAfterUpdate, kContracted, kClearWindow, kRefilled, kHeavyScan };
+
+__device__ __forceinline__ void load_hot(LoopState* L) {
+    const unsigned lane = threadIdx.x & 31;
+    if (lane < sizeof(PeelHot) / 16)
+        reinterpret_cast<int4*>(&L->s)[lane] = reinterpret_cast<const int4*>(&L->c->h)[lane];
+}
+
+// The serial step, run by one warp between a barrier's last arrival and its release: it sees every
+// write made before the barrier. Everything the next phases branch on is decided here, so that every
+// block reads the same values. The state passes through shared memory: one round trip to L2 for all
+// of it.
+__device__ __noinline__ void serial_step(LoopState* L, int what, int64_t arg) {
+    load_hot(L);
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) {
+        PeelHot& s = L->s;
+        if (what == kRefilled) {
+            refill_apply(s, arg);
+        } else if (what == kClearWindow) {  // before the window is rebuilt
+            s.nN = 0;
+        } else if (what == kContracted) {
+            s.contract = 0;
+        } else if (what == kHeavyScan) {  // (2,4): the pair totals of the staged heavy edges become offsets
+            long long run = 0;
+            const unsigned nH = s.nH;
+#pragma unroll 1
+            for (unsigned b = 0; b < nH; ++b) {
+                long long v = L->hpre[b];
+                L->hpre[b] = run;
+                run += v;
             }
+            L->hpre[nH] = run;
+        } else if (what == kAfterMin) {
+            s.stage = 3;
+        } else if (what == kAfterUpdate && s.nH != 0) {
+            s.stage = 2;  // heavy r-cliques are waiting
+            s.heavy_split = L->hpre && s.nH <= (unsigned)L->hslices;
+        } else if (what != kNothing) {
+            if (what == kAfterSelect) {
+                s.stage = 1;
+            } else {
+                if (!s.done) ctl_next(s, &L->c->err, L->round_size, L->round_level, L->round_cap);
+                s.stage = s.mode & ND_MODE_ADV ? 0 : 1;
+            }
+            const unsigned nA = (s.mode & ND_MODE_ADV) ? s.cntA : s.nA;
+            s.sorta = s.stage == 1 && !s.done && nA >= L->sort_min && nA <= L->cap;
         }
-        ok = good;
+    }
+    __syncwarp();
+    const unsigned lane = threadIdx.x & 31;
+    if (lane < sizeof(PeelHot) / 16)
+        reinterpret_cast<int4*>(&L->c->h)[lane] = reinterpret_cast<const int4*>(&L->s)[lane];
+    __syncwarp();
+}
+
+// Grid barrier. The block that arrives last runs the serial step in its thread 0 and then releases
+// the others, so a control step costs no extra barrier. Arrival is an acquire-release RMW and the
+// release a release store; waiting blocks poll with relaxed loads and acquire once they are released,
+// so all writes before the barrier are visible after it (an acquire per poll empties the L1 cache
+// under the other block of the SM, which may still be working). Then the first warp copies the round's state into shared memory. The
+// wait is bounded by the global timer: after ctl->bar_timeout_ns (kBarrierTimeoutNs by default), or
+// once another block gave up (looked at every 64 polls), a block sets ctl->err bit 8 and the function
+// returns false. An empty barrier takes 1.75 us on 304 blocks (0.9 us on 8, 1.6 us on 16), the serial
+// step another 0.7: short rounds are bound by their own chains of accesses, at 0.35 us each, and not by
+// the barrier, and letting one block run them alone with block barriers gained nothing measurable.
+__device__ __noinline__ bool grid_barrier(LoopState* L, int what, int64_t arg = 0) {
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        PeelCtl* c = L->c;
+        unsigned long long target = 0;
+        int last = 0;
+        if (threadIdx.x == 0) {
+            target = L->target + gridDim.x;
+            L->target = target;
+            last = atom_add_acq_rel_u64(&c->bar_arrive, 1ull) + 1 == target;
+            L->ok = 1;
+        }
+        last = __shfl_sync(0xffffffffu, last, 0);
+        if (last) {
+            serial_step(L, what, arg);
+            if (threadIdx.x == 0) st_release_u64(&c->bar_gen, target);
+        } else {
+            if (threadIdx.x == 0) {
+                unsigned long long t0 = 0;
+#pragma unroll 1
+                for (unsigned polls = 0; ld_relaxed_u64(&c->bar_gen) < target; ++polls) {
+                    if ((polls & 63) == 63) {
+                        const unsigned long long now = globaltimer();
+                        if (!t0) t0 = now;
+                        if ((ld_relaxed_i32(&c->err) & 8) || now - t0 > c->bar_timeout_ns) {
+                            atomicOr(&c->err, 8);
+                            L->ok = 0;
+                            break;
+                        }
+                    }
+                    __nanosleep(20);
+                }
+                ld_acquire_u64(&c->bar_gen);
+            }
+            __syncwarp();
+            load_hot(L);
+        }
     }
     __syncthreads();
-    return ok != 0;
+    return L->ok != 0;
 }
 
-struct NoSerial {
-    __device__ void operator()() const {}
-};
-
-// whether the round about to run its Update sorts A first (decided only in serial steps, so every
-// block reads the same value after the barrier)
-template <typename CT>
-__device__ __forceinline__ void decide_sort(PeelCtl* c, const PeelView<CT>* P) {
-    unsigned nA = (c->mode & ND_MODE_ADV) ? c->cntA : c->nA;
-    c->sorta = P->abits && !c->done && nA >= P->sort_min && nA <= P->cap;
+// Block 0 books the time since the previous barrier to the phase that just ended (and the Update
+// phases, 4 and 5, also to the round). Called by one thread.
+__device__ __noinline__ void book_phase(LoopState* L, int ph, int32_t round) {
+    const unsigned long long now = globaltimer(), d = now - L->last;
+    L->ph_ns[ph] += d;
+    L->last = now;
+    if (ph == 4 || ph == 5) {
+        L->in_round = ph == 4 ? d : L->in_round + d;
+        if (L->round_ns && round < L->round_cap) L->round_ns[round] = (int64_t)L->in_round;
+    }
 }
 
-template <typename CT>
-struct CtlSerial {
-    PeelCtl* c;
-    const PeelView<CT>* P;
-    __device__ void operator()() const {
-        ctl_step(c, P->round_size, P->round_level, P->round_cap);
-        decide_sort(c, P);  // same-level rounds; advance rounds decide after selecting A
-    }
-};
-
-template <typename CT>
-struct SortDecide {
-    PeelCtl* c;
-    const PeelView<CT>* P;
-    __device__ void operator()() const { decide_sort(c, P); }
-};
-
-// after the light Update: finish the round now unless heavy r-cliques are waiting
-template <typename CT>
-struct CtlUnlessHeavy {
-    PeelCtl* c;
-    const PeelView<CT>* P;
-    __device__ void operator()() const {
-        // the blocks branch on `heavy`, which only serial steps write: nH itself may already be
-        // growing in the next round's update by the time a slow block looks
-        c->heavy = c->nH != 0;
-        c->heavy_split = c->heavy && P->hpre && c->nH <= (unsigned)P->hslices;
-        if (!c->heavy) {
-            ctl_step(c, P->round_size, P->round_level, P->round_cap);
-            decide_sort(c, P);
-        }
-    }
-};
-
-struct PickSerial {
-    PeelCtl* c;
-    __device__ void operator()() const { refill_pick_serial(c); }
-};
-
-// (2,4) heavy phase split over the grid: the pair totals of the staged heavy edges become offsets
-template <typename CT>
-struct HeavyScan {
-    PeelCtl* c;
-    const PeelView<CT>* P;
-    __device__ void operator()() const {
-        unsigned nH = c->nH;
-        long long run = 0;
-        for (unsigned b = 0; b < nH; ++b) {
-            long long v = P->hpre[b];
-            P->hpre[b] = run;
-            run += v;
-        }
-        P->hpre[nH] = run;
-    }
-};
-
-// One round: [advance: min over N; (refill: compact + min, histogram, pick, select); select A]
+// One round: [advance: min over N; (refill: compact + min, histogram, bound and select); select A]
 // Update (light, one warp per r-clique), then the heavy r-cliques if any. The control step runs
-// as the serial part of the round's last barrier; a same-level round costs one barrier.
+// as the serial part of the round's last barrier; a same-level round costs one barrier. What comes
+// next (s.stage) is decided in serial steps only, so every block takes the same branch.
 template <typename CT, typename U, bool k34>
 __global__ void __launch_bounds__(512, 2) k_peel_loop(GraphView g, PeelView<CT> P) {
+    __shared__ LoopState L;
+    __shared__ PeelView<CT> Q;  // for the phases that are called out of line
+    __shared__ GraphView h;
     PeelCtl* c = P.ctl;
-    unsigned long long target = 0;
-    bool timer = blockIdx.x == 0 && threadIdx.x == 0;
-    int32_t tr = 0;  // the round being run
-    // block 0 books the time since the previous barrier to the phase that just ended (and the
-    // Update phases also to the round)
-    auto book = [&](int ph) {
-        if (timer) {
-            unsigned long long now = globaltimer(), d = now - c->ph_last;
-            c->ph_ns[ph] += d;
-            c->ph_last = now;
-            if ((ph == 4 || ph == 5) && P.round_ns && tr < P.round_cap) P.round_ns[tr] += (int64_t)d;
-        }
+    const PeelHot& s = L.s;
+    const bool timer = blockIdx.x == 0 && threadIdx.x == 0;
+    if (threadIdx.x == 0) {
+        Q = P;
+        h = g;
+        L.c = c;
+        L.target = 0;
+        L.listed = L.decs = 0;
+        L.round_size = P.round_size;
+        L.round_level = P.round_level;
+        L.round_cap = P.round_cap;
+        L.hpre = P.hpre;
+        L.sort_min = P.abits ? P.sort_min : 0xffffffffu;
+        L.cap = P.cap;
+        L.hslices = P.hslices;
+        L.round_ns = P.round_ns;
+        L.last = L.in_round = 0;
+        for (int i = 0; i < 7; ++i) L.ph_ns[i] = 0;
+    }
+    auto book = [&](int ph, int32_t round) {
+        if (timer) book_phase(&L, ph, round);
     };
     // test of the barrier bound (ND_LIMIT_DROP_BLOCK): one block never arrives, so the others give
     // up after bar_timeout_ns and the call reports ND_ETIMEOUT
     if (c->drop_block && blockIdx.x == gridDim.x - 1) return;
-    if (!grid_barrier(c, target, CtlSerial<CT>{c, &P})) return;  // set up round 0
-    if (timer) c->ph_last = globaltimer();
+    if (!grid_barrier(&L, kRound)) return;  // set up round 0
+    if (timer) L.last = globaltimer();
     for (;;) {
-        if (c->done) return;  // every block reads the same value after the barrier
-        tr = c->t;
-        if (c->contract) {  // written only by serial steps
+        if (s.done) break;
+        const Team T = grid_team();
+        const int32_t tr = s.t;  // the round being run
+        if (s.contract && s.stage != 2) {
             if constexpr (k34)
-                phase_contract34(g, P);
+                phase_contract34(h, Q, s);
             else
-                phase_contract(g, P);
-            if (!grid_barrier(c, target, NoSerial{})) return;
-            book(6);
+                phase_contract(h, Q, s);
+            if (!grid_barrier(&L, kContracted)) return;
+            book(6, tr);
+            continue;
         }
-        if (c->mode & ND_MODE_ADV) {
-            phase_adv_min(P);
-            if (!grid_barrier(c, target, NoSerial{})) return;
-            book(0);
-            if (need_refill(c)) {
-                phase_refill_scan(P);
-                if (!grid_barrier(c, target, NoSerial{})) return;
-                phase_refill_hist(P);
-                if (!grid_barrier(c, target, PickSerial{c})) return;
-                phase_refill_select(P);
-                if (!grid_barrier(c, target, NoSerial{})) return;
-                book(1);
+        if (s.stage == 0) {
+            phase_adv_min(Q, s, T);
+            if (!grid_barrier(&L, kAfterMin)) return;
+            book(0, tr);
+            continue;
+        }
+        if (s.stage == 3) {
+            if (need_refill(s)) {
+                phase_refill_scan(Q, s, T);
+                if (!grid_barrier(&L, kNothing)) return;
+                phase_refill_hist(Q, s, T);
+                if (!grid_barrier(&L, kClearWindow)) return;
+                const int64_t hi = refill_bound(c, s);
+                phase_refill_select(Q, pick(P.L, s.wl ^ 1), clampn(s.nL2, P.cap), pick(P.N, s.wn), hi, T);
+                if (!grid_barrier(&L, kRefilled, hi)) return;
+                book(1, tr);
             }
-            phase_adv_select(P);
-            if (!grid_barrier(c, target, SortDecide<CT>{c, &P})) return;
-            book(2);
+            phase_adv_select(Q, s, T);
+            if (!grid_barrier(&L, kAfterSelect)) return;
+            book(2, tr);
+            continue;
         }
-        if (c->sorta) {
-            phase_sort_count(P);
-            if (!grid_barrier(c, target, NoSerial{})) return;
-            phase_sort_write(P);
-            if (!grid_barrier(c, target, NoSerial{})) return;
-            book(3);
-        }
-        phase_update<CT, U>(g, P);
-        if (!grid_barrier(c, target, CtlUnlessHeavy<CT>{c, &P})) return;
-        book(4);
-        if (c->heavy) {
-            if constexpr (is_staged<U>::value) {
-                if (c->heavy_split) {  // written only by serial steps
-                    phase_heavy_stage<CT, U>(g, P);
-                    if (!grid_barrier(c, target, HeavyScan<CT>{c, &P})) return;
-                    phase_heavy_pairs<CT, U>(g, P);
-                    if (!grid_barrier(c, target, CtlSerial<CT>{c, &P})) return;
-                    book(5);
-                    continue;
-                }
+        if (s.stage == 1) {
+            if (s.sorta) {
+                phase_sort_count(Q, s);
+                if (!grid_barrier(&L, kNothing)) return;
+                phase_sort_write(Q, s);
+                if (!grid_barrier(&L, kNothing)) return;
+                book(3, tr);
             }
-            phase_update_heavy<CT, U>(g, P);
-            if (!grid_barrier(c, target, CtlSerial<CT>{c, &P})) return;
-            book(5);
+            phase_update<CT, U>(g, P, &Q, s, T, &L.listed, &L.decs);
+            if (!grid_barrier(&L, kAfterUpdate)) return;
+            book(4, tr);
+            continue;
         }
+        if constexpr (is_staged<U>::value) {
+            if (s.heavy_split) {
+                phase_heavy_stage<CT, U>(g, P, &Q, s);
+                if (!grid_barrier(&L, kHeavyScan)) return;
+                phase_heavy_pairs<CT, U>(g, P, &Q, s, &L.listed, &L.decs);
+                if (!grid_barrier(&L, kRound)) return;
+                book(5, tr);
+                continue;
+            }
+        }
+        phase_update_heavy<CT, U>(g, P, &Q, s, &L.listed, &L.decs);
+        if (!grid_barrier(&L, kRound)) return;
+        book(5, tr);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (L.listed) atomicAdd(&c->listed, L.listed);
+        if (L.decs) atomicAdd(&c->decs, L.decs);
+        if (timer)
+            for (int i = 0; i < 7; ++i) c->ph_ns[i] = L.ph_ns[i];
     }
 }
 
