@@ -700,15 +700,79 @@ static int build_tri_hash(nd_graph* g, DBuf& hoff, DBuf& htab, DBuf& hpos) {
     return nd_check_launch("triangle hash");
 }
 
+// Incidence lists of the s-cliques, read by the peel (nd_inc.cu).
+struct IncBufs {
+    DBuf off, list, row, dead, status;
+    int32_t stride = 0;
+    int64_t n_s = 0;
+};
+
+static void free_inc(nd_ctx* c, IncBufs& b) {
+    for (DBuf* x : {&b.off, &b.list, &b.row, &b.dead, &b.status}) nd_free(c, *x);
+}
+
+// Which decompositions are peeled from incidence lists. (1,2) has them in the CSR itself. (2,3) keeps
+// the adjacency rows, whose contraction (Section 5.6) its statistics report; so does a (3,4) run that is
+// asked to contract before every round. The lists are an accelerator and must leave room for others,
+// hence the bound; the (3,4) lists of R-MAT graphs from scale 17 on, for instance, are over it, and
+// their s-cliques are listed again by Update.
+constexpr int64_t kIncBytes = (int64_t)16 << 30;
+
+static bool wants_inc(int r, int s, int flags, int64_t n_s) {
+    if ((r == 1 && s == 2) || (r == 2 && s == 3) || (flags & ND_CONTRACT_ALWAYS)) return false;
+    return n_s < UINT32_MAX && n_s <= kIncBytes / (4 * (nd_inc_stride(r, s) + binom64(s, r)));
+}
+
+static int build_inc(nd_graph* g, int r, int s, const DBuf& cnt, int w, int64_t n_r, int64_t n_s, IncBufs& b) {
+    nd_ctx* c = g->ctx;
+    cudaStream_t st = c->stream;
+    b.stride = nd_inc_stride(r, s);
+    b.n_s = n_s;
+    const int64_t entries = n_s * binom64(s, r);
+    DBuf cursor, tmp;
+    int rc = ND_OK;
+    if ((rc = nd_alloc(c, b.off, 8 * (n_r + 1))) || (rc = nd_alloc(c, cursor, 8 * (n_r + 1))) ||
+        (rc = nd_alloc(c, tmp, nd_scan_tmp_bytes(n_r))) || (rc = nd_alloc(c, b.list, 4 * std::max<int64_t>(entries, 1))) ||
+        (rc = nd_alloc(c, b.row, 4 * b.stride * std::max<int64_t>(n_s, 1))) ||
+        (rc = nd_alloc(c, b.dead, 4 * ((n_s + 31) / 32 + 1))) || (rc = nd_alloc(c, b.status, 16))) {
+        nd_free(c, cursor);
+        nd_free(c, tmp);
+        free_inc(c, b);
+        return rc;
+    }
+    if (w == 8)
+        nd_scan_i64((const int64_t*)cnt.p, (int64_t*)b.off.p, n_r, tmp.p, st);
+    else
+        nd_scan_i32((const int32_t*)cnt.p, (int64_t*)b.off.p, n_r, tmp.p, st);
+    cudaMemcpyAsync(cursor.p, b.off.p, 8 * (n_r + 1), cudaMemcpyDeviceToDevice, st);
+    cudaMemsetAsync(b.dead.p, 0, b.dead.bytes, st);
+    cudaMemsetAsync(b.status.p, 0, b.status.bytes, st);
+    IncFill F;
+    F.cursor = (unsigned long long*)cursor.p;
+    F.list = (uint32_t*)b.list.p;
+    F.row = (int32_t*)b.row.p;
+    F.stride = b.stride;
+    F.status = (unsigned int*)b.status.p;
+    F.n_s = n_s;
+    F.entries = entries;
+    nd_inc_fill(nd_view(g), r, s, n_r, F, st);
+    rc = nd_check_launch("incidence lists");
+    nd_free(c, cursor);
+    nd_free(c, tmp);
+    if (rc) free_inc(c, b);
+    return rc;
+}
+
 template <typename CT>
-static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags, PeelOut& po) {
+static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags, PeelOut& po,
+                    const IncBufs* inc = nullptr) {
     nd_ctx* c = g->ctx;
     cudaStream_t st = c->stream;
     int64_t cap = std::max<int64_t>(n_r, 1);
     int64_t rcap = std::min<int64_t>(n_r, (int64_t)1 << 22) + 1;
     // (2,4) stages N(u) ∩ N(v) of every heavy edge: its heavy list holds every edge (the light
     // path cannot take one back) and each heavy-phase block gets a slice of 5 * (hstage + 1) int32
-    bool staged = r == 2 && s == 4;
+    bool staged = r == 2 && s == 4 && !inc;
     int64_t hcap = staged ? cap : std::min<int64_t>(cap, (int64_t)1 << 20);
     int64_t hstage = 0, hslices = 0;
     int rc = ND_OK;
@@ -727,7 +791,8 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags
     // (2,3) graph contraction (Section 5.6): compacted copies of the rows and their lengths
     bool contract = r == 2 && s == 3 && !(flags & ND_CONTRACT_OFF);
     // (3,4): the same for the triangle lists (compacted copies of the lists and entry offsets)
-    bool contract34 = r == 3 && s == 4 && !(flags & ND_CONTRACT_OFF);
+    const bool lists34 = r == 3 && s == 4 && !inc;
+    bool contract34 = lists34 && !(flags & ND_CONTRACT_OFF);
     // dense buckets (Section 4.2 Discussion): one bucket per count value up to the largest count
     bool dense = flags & ND_DENSE_BUCKETS;
     int64_t bmax = 0;
@@ -748,9 +813,9 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags
     if ((rc = nd_alloc(c, ctl, sizeof(PeelCtl))) || (rc = nd_alloc(c, A0, 4 * cap)) || (rc = nd_alloc(c, A1, 4 * cap)) ||
         (rc = nd_alloc(c, N0, 4 * cap)) || (rc = nd_alloc(c, N1, 4 * cap)) || (rc = nd_alloc(c, L0, 4 * cap)) ||
         (rc = nd_alloc(c, L1, 4 * cap)) || (rc = nd_alloc(c, H, 4 * hcap)) || (rc = nd_alloc(c, rs, 8 * rcap)) ||
-        (rc = nd_alloc(c, rl, 8 * rcap)) || (rc = nd_alloc(c, rt, 8 * rcap)) || (r == 3 && s == 4 && (rc = nd_alloc(c, etr, 4 * std::max<int64_t>(3 * g->n3, 1)))) ||
+        (rc = nd_alloc(c, rl, 8 * rcap)) || (rc = nd_alloc(c, rt, 8 * rcap)) || (lists34 && (rc = nd_alloc(c, etr, 4 * std::max<int64_t>(3 * g->n3, 1)))) ||
         (staged && (rc = nd_alloc(c, hsc, 4 * 5 * (hstage + 1) * hslices))) ||
-        (rc = nd_alloc(c, abits, r == 3 ? 4 * ((cap + 31) / 32) : 4)) ||
+        (rc = nd_alloc(c, abits, r == 3 && !inc ? 4 * ((cap + 31) / 32) : 4)) ||
         (contract && ((rc = nd_alloc(c, ccol, 4 * std::max<int64_t>(g->nnz, 1))) ||
                       (rc = nd_alloc(c, cpos, 4 * std::max<int64_t>(g->nnz, 1))) ||
                       (rc = nd_alloc(c, clen, 4 * std::max<int64_t>(g->n, 1))) ||
@@ -782,9 +847,9 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags
     P.hpre = staged ? (int64_t*)hpre.p : nullptr;
     P.hstage = hstage;
     P.hslices = (int32_t)hslices;
-    // id-order rebuilds of A pay off for triangles (their lists are long); edges and vertices
-    // skip them
-    P.abits = r == 3 ? (uint32_t*)abits.p : nullptr;
+    // id-order rebuilds of A pay off for triangles (their lists are long); edges and vertices, and
+    // what is peeled from incidence lists, skip them
+    P.abits = r == 3 && !inc ? (uint32_t*)abits.p : nullptr;
     // a round sorts A when it holds at least 1/8192 of the r-cliques (and 2048): then the two
     // passes over the bitmap cost little next to the Update they make cache-friendly
     P.sort_min = (uint32_t)std::max<int64_t>(n_r / 8192, 2048);
@@ -803,7 +868,7 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags
     P.hoff = nullptr;
     P.htab = nullptr;
     P.hpos = nullptr;
-    if (r == 3 && s == 4) {
+    if (lists34) {
         // the hash directory, when the decomposition built one (nd_decompose_dev, (3,4))
         P.hoff = (const int64_t*)g->hoff.p;
         P.htab = (NdHashSlot*)g->htab.p;
@@ -822,6 +887,11 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags
     P.bcnt = nullptr;
     P.bmax = 0;
     P.heavy_work = c->tune_heavy[r * 8 + s];
+    P.inc_off = inc ? (const int64_t*)inc->off.p : nullptr;
+    P.inc_list = inc ? (const uint32_t*)inc->list.p : nullptr;
+    P.inc_row = inc ? (const int32_t*)inc->row.p : nullptr;
+    P.inc_dead = inc ? (uint32_t*)inc->dead.p : nullptr;
+    P.inc_stride = inc ? inc->stride : 0;
     if (dense) {
         P.bcnt = (unsigned int*)bcnt.p;
         P.bmax = bmax;
@@ -874,7 +944,7 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags
         contract_shift = always ? 0 : 2;
     }
     nd_peel_init(P.ctl, n_r, max_rounds, st, (uint64_t)c->barrier_ns, (c->limit_flags & ND_LIMIT_DROP_BLOCK) ? 1 : 0,
-                 contract_every, contract_shift);
+                 contract_every, contract_shift, inc ? (const unsigned int*)inc->status.p : nullptr, inc ? inc->n_s : 0);
     bool looped = false;
     int persistent_launches = 0;
     bool want_persistent = (flags & ND_PEEL_PERSISTENT) || !(flags & (ND_NO_GRAPH | ND_PEEL_LOOP_GRAPH));
@@ -1037,7 +1107,22 @@ int nd_decompose_dev(nd_graph* g, int r, int s, int count_width, int flags, Peel
     unsigned long long tot = 0;
     if (!rc) rc = sum_counts(g, cnt, w, n_r, &tot);
     cudaEventRecord(e3, c->stream);
-    if (!rc) rc = (w == 8) ? run_peel<int64_t>(g, r, s, cnt, n_r, flags, po) : run_peel<int32_t>(g, r, s, cnt, n_r, flags, po);
+    const int64_t n_s = (int64_t)(tot / (unsigned long long)binom64(s, r));
+    IncBufs inc;
+    bool use_inc = !rc && wants_inc(r, s, flags, n_s);
+    if (use_inc) {
+        rc = build_inc(g, r, s, cnt, w, n_r, n_s, inc);
+        if (rc == ND_ENOMEM) {
+            use_inc = false;
+            rc = ND_OK;
+        }
+        if (use_inc)
+            for (DBuf* b : {&g->hoff, &g->htab, &g->hpos}) nd_free(c, *b);  // the lists replace it
+    }
+    if (!rc)
+        rc = (w == 8) ? run_peel<int64_t>(g, r, s, cnt, n_r, flags, po, use_inc ? &inc : nullptr)
+                      : run_peel<int32_t>(g, r, s, cnt, n_r, flags, po, use_inc ? &inc : nullptr);
+    free_inc(c, inc);
     cudaEventRecord(e2, c->stream);
     if (!rc) rc = nd_sync(c, "nd_decompose");
     float tc = 0, tp = 0, th = 0;
@@ -1055,7 +1140,7 @@ int nd_decompose_dev(nd_graph* g, int r, int s, int count_width, int flags, Peel
     for (DBuf* b : {&g->hoff, &g->htab, &g->hpos}) nd_free(c, *b);
     if (rc) return rc;
     S.n_r = n_r;
-    S.n_s = (int64_t)(tot / (unsigned long long)binom64(s, r));
+    S.n_s = n_s;
     S.rho = po.rho;
     S.max_core = po.max_core;
     S.listed = po.listed;

@@ -372,6 +372,14 @@ struct PeelView {
     int32_t* ltp;
     int32_t* llen;
     int32_t* lprev;
+    // incidence lists (NULL: Update lists the s-cliques of each r-clique again): the s-cliques of r-clique R are
+    // inc_list[inc_off[R] .. inc_off[R+1]); s-clique S has its r-subsets' ids in inc_row[S * inc_stride ..]
+    // (stride a multiple of 4, filled up with -1) and bit S of inc_dead set once it is destroyed
+    const int64_t* inc_off;
+    const uint32_t* inc_list;
+    const int32_t* inc_row;
+    uint32_t* inc_dead;
+    int32_t inc_stride;
     // driving-list length above which Update defers an r-clique to the heavy phase (0: the
     // variant's built-in threshold)
     int64_t heavy_work;
@@ -392,6 +400,7 @@ void nd_set_capturing(bool on);
 // out[0..n] = exclusive scan of in[0..n), out[n] = total. tmp: nd_scan_tmp_bytes(n) bytes.
 size_t nd_scan_tmp_bytes(int64_t n);
 void nd_scan_i64(const int64_t* in, int64_t* out, int64_t n, void* tmp, cudaStream_t st);
+void nd_scan_i32(const int32_t* in, int64_t* out, int64_t n, void* tmp, cudaStream_t st);
 void nd_fill_i32(int32_t* p, int32_t v, int64_t n, cudaStream_t st);
 void nd_iota_i32(int32_t* p, int64_t n, cudaStream_t st);
 // *out = max over a[0..n) (int64 device scalar, must be pre-set to 0)
@@ -430,6 +439,19 @@ void nd_tri_hash_fill(const GraphView& g, const int64_t* hoff, NdHashSlot* tab, 
 // blocks of the (2,4) heavy phase that hold a scratch slice; the others skip the phase
 int nd_peel_heavy_slices();
 
+// Incidence lists of the s-cliques (nd_inc.cu), what filling them writes: cursor[R] starts at the first
+// place of R's list; status[0] counts the s-cliques, status[1] is set when one has no room.
+struct IncFill {
+    unsigned long long* cursor;
+    uint32_t* list;
+    int32_t* row;
+    int32_t stride;
+    unsigned int* status;
+    int64_t n_s, entries;
+};
+int nd_inc_stride(int r, int s);
+void nd_inc_fill(const GraphView& g, int r, int s, int64_t n_r, const IncFill& F, cudaStream_t st);
+
 // counting (nd_count.cu): counts into cnt (CT = int32_t or int64_t), zero-initialised
 template <typename CT>
 void nd_count_launch(const GraphView& g, int r, int s, CT* cnt, int64_t n_r, cudaStream_t st);
@@ -448,8 +470,10 @@ template <typename CT>
 cudaError_t nd_peel_persistent(const GraphView& g, int r, int s, const PeelView<CT>& P, cudaStream_t st);
 // barrier_ns 0: the default bound (60 s); drop_block: see ND_LIMIT_DROP_BLOCK; contract_every /
 // contract_shift: graph contraction schedule (0: off)
+// inc_status / n_s: the counters of the incidence lists (NULL without) and what they have to show
 void nd_peel_init(PeelCtl* ctl, int64_t n_r, int64_t max_rounds, cudaStream_t st, uint64_t barrier_ns = 0,
-                  int drop_block = 0, int64_t contract_every = 0, int contract_shift = 2);
+                  int drop_block = 0, int64_t contract_every = 0, int contract_shift = 2,
+                  const unsigned int* inc_status = nullptr, int64_t n_s = 0);
 // row lengths len[v] = rp[v+1] - rp[v] (int32) into two arrays
 void nd_row_len(const int64_t* rp, int32_t n, int32_t* a, int32_t* b, cudaStream_t st);
 // dense buckets: bcnt[cnt[R]] += 1 for every R < n_r (bcnt zeroed by the caller)

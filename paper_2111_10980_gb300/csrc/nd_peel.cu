@@ -31,6 +31,8 @@
 //     warp applies S's effect, subtracting exactly 1 from every r-subset not in A. The paper
 //     has each of the a members of A subtract 1/a; the owner rule gives the same total (1 per
 //     live S and surviving member) with integer atomics and without double counting.
+// With incidence lists (nd_inc.cu; the default but for (1,2), (2,3) and very many s-cliques) the s-cliques
+// are not listed again: the first peeled member of S to set S's bit applies S's effect (UpdInc).
 // Warps take A in dynamic chunks; r-cliques with long driving lists go to a heavy phase that
 // gives each a block ((2,4) in the persistent kernel: stage per block, then the pairs of all
 // heavy edges over the whole grid).
@@ -137,15 +139,18 @@ __device__ __forceinline__ unsigned long long block_min(unsigned long long v) {
 }
 
 __global__ void k_init(PeelCtl* c, int64_t n_r, int64_t max_rounds, unsigned long long barrier_ns, int drop_block,
-                       int64_t contract_every, int contract_shift) {
+                       int64_t contract_every, int contract_shift, const unsigned int* inc_status, int64_t n_s) {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         PeelHot h = {};
         h.n_r = n_r;
         h.max_rounds = max_rounds;
         h.contract_every = contract_every;
         h.minN = h.gmin = ULLONG_MAX;
+        // incidence lists that do not hold every s-clique once are not peeled
+        const bool bad = inc_status && (inc_status[1] || (int64_t)inc_status[0] != n_s);
+        h.done = bad;
         c->h = h;
-        c->err = 0;
+        c->err = bad ? 16 : 0;
         c->contract_shift = contract_shift;
         c->drop_block = drop_block;
         c->bar_timeout_ns = barrier_ns;
@@ -1357,6 +1362,52 @@ struct UpdGen {
     }
 };
 
+// Any (r,s) with incidence lists: the candidates are the s-cliques of R's list. The first of S's peeled
+// members to set S's bit destroys it, so nothing has to be looked up: no intersection, no r-clique
+// ids, no owner rule. A chain of five accesses (offsets, list, row and bit, counts, append) instead of
+// up to twenty-five bounds a short round. kVec: int4 words of a row (0: as the stride says).
+template <typename CT, int kVec>
+struct UpdInc {
+    static constexpr bool kInc = true;
+    __device__ static int64_t prep(const GraphView&, const PeelView<CT>& P, int32_t R, Prep& q) {
+        q.b[0] = P.inc_off[R];
+        q.n[0] = P.inc_off[R + 1] - q.b[0];
+        return q.n[0];
+    }
+    template <typename Q>
+    __device__ static void cand(const GraphView&, const RoundEnv<CT>& E, int32_t R, const Q& q, int64_t j,
+                                UpdCounters& k) {
+        const uint32_t S = E.P.inc_list[q.b[0] + j], bit = 1u << (S & 31);
+        const int nv = kVec ? kVec : E.P.inc_stride >> 2;
+        const int4* row = reinterpret_cast<const int4*>(E.P.inc_row + (int64_t)S * E.P.inc_stride);
+        int4 v[kVec ? kVec : 1];
+        v[0] = row[0];
+#pragma unroll
+        for (int i = 1; i < (kVec ? kVec : 1); ++i) v[i] = row[i];
+        if (atomicOr(&E.P.inc_dead[S >> 5], bit) & bit) return;
+        k.listed++;
+#pragma unroll
+        for (int i = 0; i < nv; ++i) {
+            if (!kVec && i) v[0] = row[i];
+            const int4 w = v[kVec ? i : 0];
+            const int32_t x[4] = {w.x, w.y, w.z, w.w};
+            int32_t r[4];
+            int64_t o[4];
+            // members of A (round t) keep their counts; one that was already put into the next round
+            // (t + 1) may lose one more, which nobody reads
+#pragma unroll
+            for (int m = 0; m < 4; ++m) r[m] = x[m] >= 0 && x[m] != R ? E.P.rnd[x[m]] : E.t;
+#pragma unroll
+            for (int m = 0; m < 4; ++m) o[m] = dec_live(r[m], E.t) ? nd_atomic_dec(&E.P.cnt[x[m]]) : 0;
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                k.decs += r[m] != E.t;
+                if (dec_live(r[m], E.t)) after_dec(E, x[m], o[m]);
+            }
+        }
+    }
+};
+
 template <typename U, typename = void>
 struct is_staged {
     static constexpr bool value = false;
@@ -1931,9 +1982,10 @@ int peel_blocks() { return nd_sm_count() * 4; }
 int nd_peel_heavy_slices() { return nd_sm_count() * 2; }
 
 void nd_peel_init(PeelCtl* ctl, int64_t n_r, int64_t max_rounds, cudaStream_t st, uint64_t barrier_ns,
-                  int drop_block, int64_t contract_every, int contract_shift) {
+                  int drop_block, int64_t contract_every, int contract_shift, const unsigned int* inc_status,
+                  int64_t n_s) {
     ND_K(k_init<<<1, 32, 0, st>>>(ctl, n_r, max_rounds, barrier_ns ? barrier_ns : kBarrierTimeoutNs, drop_block,
-                                  contract_every, contract_shift));
+                                  contract_every, contract_shift, inc_status, n_s));
 }
 
 template <typename CT>
@@ -1974,7 +2026,18 @@ void nd_peel_adv_select(const PeelView<CT>& P, cudaStream_t st) {
 template <typename CT>
 void nd_peel_update(const GraphView& g, int r, int s, const PeelView<CT>& P, cudaStream_t st) {
     int nb = peel_blocks();
-    if (r == 1 && s == 2) {
+    if (P.inc_off) {
+        if (P.inc_stride == 4) {
+            ND_K(k_update<CT, UpdInc<CT, 1>><<<nb, kThreads, 0, st>>>(g, P));
+            ND_K(k_update_heavy<CT, UpdInc<CT, 1>><<<nb, kThreads, 0, st>>>(g, P));
+        } else if (P.inc_stride == 8) {
+            ND_K(k_update<CT, UpdInc<CT, 2>><<<nb, kThreads, 0, st>>>(g, P));
+            ND_K(k_update_heavy<CT, UpdInc<CT, 2>><<<nb, kThreads, 0, st>>>(g, P));
+        } else {
+            ND_K(k_update<CT, UpdInc<CT, 0>><<<nb, kThreads, 0, st>>>(g, P));
+            ND_K(k_update_heavy<CT, UpdInc<CT, 0>><<<nb, kThreads, 0, st>>>(g, P));
+        }
+    } else if (r == 1 && s == 2) {
         ND_K(k_update<CT, Upd12<CT>><<<nb, kThreads, 0, st>>>(g, P));
         ND_K(k_update_heavy<CT, Upd12<CT>><<<nb, kThreads, 0, st>>>(g, P));
     } else if (r == 1 && s == 3) {
@@ -2113,6 +2176,11 @@ cudaError_t nd_peel_loop_graph(const GraphView& g, int r, int s, const PeelView<
 // cooperative launch is not possible.
 template <typename CT>
 cudaError_t nd_peel_persistent(const GraphView& g, int r, int s, const PeelView<CT>& P, cudaStream_t st) {
+    if (P.inc_off) {
+        if (P.inc_stride == 4) return launch_peel_loop<CT, UpdInc<CT, 1>, false>(g, P, st);
+        if (P.inc_stride == 8) return launch_peel_loop<CT, UpdInc<CT, 2>, false>(g, P, st);
+        return launch_peel_loop<CT, UpdInc<CT, 0>, false>(g, P, st);
+    }
     if (r == 1 && s == 2) return launch_peel_loop<CT, Upd12<CT>, false>(g, P, st);
     if (r == 1 && s == 3) return launch_peel_loop<CT, Upd13<CT>, false>(g, P, st);
     if (r == 2 && s == 3) return launch_peel_loop<CT, Upd23<CT>, false>(g, P, st);

@@ -44,7 +44,8 @@ __device__ int64_t block_excl_scan(int64_t v, int64_t* total) {
     return res;
 }
 
-__global__ void k_scan_tiles(const int64_t* __restrict__ in, int64_t n, int64_t* __restrict__ bsum) {
+template <typename T>
+__global__ void k_scan_tiles(const T* __restrict__ in, int64_t n, int64_t* __restrict__ bsum) {
     int64_t base = (int64_t)blockIdx.x * kScanTile;
     int64_t s = 0;
     for (int i = 0; i < kScanItems; ++i) {
@@ -70,7 +71,8 @@ __global__ void k_scan_sums(int64_t* bsum, int64_t nb) {
     if (threadIdx.x == 0) bsum[nb] = carry;
 }
 
-__global__ void k_scan_apply(const int64_t* __restrict__ in, int64_t* __restrict__ out, int64_t n,
+template <typename T>
+__global__ void k_scan_apply(const T* __restrict__ in, int64_t* __restrict__ out, int64_t n,
                              const int64_t* __restrict__ bsum, int64_t nb) {
     int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
     int64_t v[kScanItems];
@@ -167,14 +169,18 @@ size_t nd_scan_tmp_bytes(int64_t n) {
     return (size_t)(nb + 1) * sizeof(int64_t);
 }
 
-void nd_scan_i64(const int64_t* in, int64_t* out, int64_t n, void* tmp, cudaStream_t st) {
+template <typename T>
+static void scan(const T* in, int64_t* out, int64_t n, void* tmp, cudaStream_t st) {
     int64_t nb = (n + kScanTile - 1) / kScanTile;
     if (nb < 1) nb = 1;
     int64_t* bsum = static_cast<int64_t*>(tmp);
-    ND_K(k_scan_tiles<<<(unsigned)nb, kScanThreads, 0, st>>>(in, n, bsum));
+    ND_K(k_scan_tiles<T><<<(unsigned)nb, kScanThreads, 0, st>>>(in, n, bsum));
     ND_K(k_scan_sums<<<1, kScanThreads, 0, st>>>(bsum, nb));
-    ND_K(k_scan_apply<<<(unsigned)nb, kScanThreads, 0, st>>>(in, out, n, bsum, nb));
+    ND_K(k_scan_apply<T><<<(unsigned)nb, kScanThreads, 0, st>>>(in, out, n, bsum, nb));
 }
+
+void nd_scan_i64(const int64_t* in, int64_t* out, int64_t n, void* tmp, cudaStream_t st) { scan(in, out, n, tmp, st); }
+void nd_scan_i32(const int32_t* in, int64_t* out, int64_t n, void* tmp, cudaStream_t st) { scan(in, out, n, tmp, st); }
 
 void nd_fill_i32(int32_t* p, int32_t v, int64_t n, cudaStream_t st) {
     if (n <= 0) return;

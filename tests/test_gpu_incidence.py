@@ -1,0 +1,67 @@
+"""Peeling from incidence lists against peeling by listing the s-cliques again.
+
+The lists are an accelerator that a context without the memory for them does without: an allocator
+that refuses the large buffers sends the same decomposition down the other path. Both have to
+give the oracle's cores, rounds and statistics, for every row length C(s,r) (3 to 20) and its padding.
+"""
+import math
+
+import numpy as np
+import pytest
+
+import graphgen as gg
+import oracle as orc
+from test_gpu_parity import assert_parity
+
+pytestmark = pytest.mark.gpu
+
+RS = [(1, 3), (1, 4), (2, 4), (2, 5), (3, 4), (3, 5), (3, 6), (4, 5), (4, 6)]
+
+
+@pytest.fixture(scope="module")
+def nd():
+    import paper_2111_10980_gb300 as nd
+
+    nd.lib()
+    return nd
+
+
+@pytest.mark.parametrize("r,s", RS)
+def test_with_and_without_room_for_the_lists(nd, r, s):
+    import torch
+
+    # dense communities over a sparse graph, so that the rows are the largest buffer (next to the stages
+    # of the heavy edges when (2,4) lists its s-cliques again)
+    g = gg.with_planted(gg.chung_lu(1200, 6.0, 2.3, seed=91), 30 if (r, s) == (2, 4) else 12, 14, 20, 0.85, seed=92)
+    rows = 4 * ((math.comb(s, r) + 3) // 4 * 4) * orc.decompose(g, r, s).n_s
+    alloc, free = nd.torch_allocator_hooks(0)
+    for limit in (None, rows):
+        refused = []
+
+        def hook(nbytes, stream):
+            if limit is not None and nbytes >= limit:
+                refused.append(nbytes)
+                return 0
+            return alloc(nbytes, stream)
+
+        ctx = nd.nd_ctx_create(0, stream=torch.cuda.Stream())
+        nd.nd_ctx_set_allocator(ctx, hook, free)
+        try:
+            for flags in (0, nd.ND_PEEL_LOOP_GRAPH, nd.ND_NO_GRAPH):
+                assert_parity(nd, ctx, g, r, s, flags=flags)
+        finally:
+            nd.nd_ctx_destroy(ctx)
+        assert bool(refused) == (limit is not None)
+
+
+@pytest.mark.parametrize("r,s", RS)
+def test_no_s_clique(nd, r, s):
+    g = gg.path(50)
+    ctx = nd.nd_ctx_create(0)
+    try:
+        G = nd.nd_load_csr(ctx, g.rowptr, g.col)
+        core, rnd, st = nd.nd_decompose(G, r, s)
+        nd.nd_graph_free(G)
+        assert st["n_s"] == 0 and not np.any(core) and st["rho"] == (1 if st["n_r"] else 0)
+    finally:
+        nd.nd_ctx_destroy(ctx)
