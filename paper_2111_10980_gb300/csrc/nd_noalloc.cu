@@ -105,12 +105,17 @@ extern "C" int nd_kcore_noalloc(int32_t n, const int64_t* rowptr, const int32_t*
     v.rp = rowptr;
     v.col = col;
 
-    // count (degrees), then the same peeling rounds as nd_decompose(1, 2), launched one by one
+    // count (degrees), then the same peeling loop as nd_decompose(1, 2): one cooperative kernel, which
+    // needs no memory but the scratch; where that cannot be launched, its rounds launched one by one
+    // (nine launches each and a read-back every 32 rounds: 12.5 ms against 2.2 ms for 273 rounds on a
+    // Chung-Lu graph of 100,003 vertices)
     nd_count_launch<int32_t>(v, 1, 2, P.cnt, n, st);
     nd_fill_i32(P.rnd, ND_UNPEELED, n, st);
     nd_fill_i32(P.core, 0, n, st);
     nd_peel_init(P.ctl, n, (int64_t)n + 2, st);
     if ((rc = nd_check_launch("nd_kcore_noalloc"))) return rc;
+    const bool looped = nd_peel_persistent<int32_t>(v, 1, 2, P, st) == cudaSuccess;
+    if (!looped) cudaGetLastError();
     const int kChunk = 32;
     int64_t max_chunks = ((int64_t)n + 2) / kChunk + 4;
     // the head of the control block (pageable host memory: no pinned allocation)
@@ -121,7 +126,7 @@ extern "C" int nd_kcore_noalloc(int32_t n, const int64_t* rowptr, const int32_t*
     static_assert(offsetof(PeelCtl, err) == sizeof(PeelHot), "the head ends with err");
     constexpr size_t kHead = offsetof(PeelCtl, err) + sizeof(int32_t);
     for (int64_t chunk = 0;; ++chunk) {
-        for (int i = 0; i < kChunk; ++i) nd_peel_round<int32_t>(v, 1, 2, P, st);
+        for (int i = 0; !looped && i < kChunk; ++i) nd_peel_round<int32_t>(v, 1, 2, P, st);
         if ((rc = nd_check_launch("nd_kcore_noalloc"))) return rc;
         e = cudaMemcpyAsync(&head, P.ctl, kHead, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -129,10 +134,11 @@ extern "C" int nd_kcore_noalloc(int32_t n, const int64_t* rowptr, const int32_t*
             cudaGetLastError();
             return nd_set_error(ND_ECUDA, "nd_kcore_noalloc: %s", cudaGetErrorString(e));
         }
-        if (head.h.done) break;
+        if (looped || head.h.done) break;
         if (chunk + 1 > max_chunks)
             return nd_set_error(ND_ETIMEOUT, "nd_kcore_noalloc: peeling did not finish");
     }
+    if (head.err & 8) return nd_set_error(ND_ETIMEOUT, "nd_kcore_noalloc: a grid barrier of the peel kernel timed out");
     if (head.err & 1) return nd_set_error(ND_EINTERNAL, "nd_kcore_noalloc: a work list overflowed");
     if (head.err & 2) return nd_set_error(ND_ETIMEOUT, "nd_kcore_noalloc: round cap reached");
     if (head.err & 4) return nd_set_error(ND_EINTERNAL, "nd_kcore_noalloc: inconsistent peeling state");
