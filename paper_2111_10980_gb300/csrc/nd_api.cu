@@ -711,16 +711,15 @@ static void free_inc(nd_ctx* c, IncBufs& b) {
     for (DBuf* x : {&b.off, &b.list, &b.row, &b.dead, &b.status}) nd_free(c, *x);
 }
 
-// Which decompositions are peeled from incidence lists. (1,2) has them in the CSR itself. (2,3) keeps
-// the adjacency rows, whose contraction (Section 5.6) its statistics report; so does a (3,4) run that is
-// asked to contract before every round. The lists are an accelerator and must leave room for others,
+// Which decompositions are peeled from incidence lists. (1,2) has them in the CSR itself; a (3,4) run that
+// is asked to contract before every round contracts its triangle lists. The lists are an accelerator and must leave room for others,
 // hence the bound; the (3,4) lists of R-MAT graphs from scale 17 on, for instance, are over it, and
 // their s-cliques are listed again by Update.
 constexpr int64_t kIncBytes = (int64_t)16 << 30;
 
 static bool wants_inc(int r, int s, int flags, int64_t n_s) {
-    if ((r == 1 && s == 2) || (r == 2 && s == 3) || (flags & ND_CONTRACT_ALWAYS)) return false;
-    return n_s < UINT32_MAX && n_s <= kIncBytes / (4 * (nd_inc_stride(r, s) + binom64(s, r)));
+    if ((r == 1 && s == 2) || (r == 3 && s == 4 && (flags & ND_CONTRACT_ALWAYS))) return false;
+    return n_s < INT32_MAX && n_s <= kIncBytes / (4 * (nd_inc_stride(r, s) + binom64(s, r)));
 }
 
 static int build_inc(nd_graph* g, int r, int s, const DBuf& cnt, int w, int64_t n_r, int64_t n_s, IncBufs& b) {
@@ -729,12 +728,14 @@ static int build_inc(nd_graph* g, int r, int s, const DBuf& cnt, int w, int64_t 
     b.stride = nd_inc_stride(r, s);
     b.n_s = n_s;
     const int64_t entries = n_s * binom64(s, r);
+    IncFill F;
+    F.rows = nd_inc_rows(r, s, n_r, g->m, n_s, &F.run);
     DBuf cursor, tmp;
     int rc = ND_OK;
     if ((rc = nd_alloc(c, b.off, 8 * (n_r + 1))) || (rc = nd_alloc(c, cursor, 8 * (n_r + 1))) ||
         (rc = nd_alloc(c, tmp, nd_scan_tmp_bytes(n_r))) || (rc = nd_alloc(c, b.list, 4 * std::max<int64_t>(entries, 1))) ||
-        (rc = nd_alloc(c, b.row, 4 * b.stride * std::max<int64_t>(n_s, 1))) ||
-        (rc = nd_alloc(c, b.dead, 4 * ((n_s + 31) / 32 + 1))) || (rc = nd_alloc(c, b.status, 16))) {
+        (rc = nd_alloc(c, b.row, 4 * b.stride * F.rows)) ||
+        (rc = nd_alloc(c, b.dead, 4 * (F.rows / 32 + 1))) || (rc = nd_alloc(c, b.status, 16))) {
         nd_free(c, cursor);
         nd_free(c, tmp);
         free_inc(c, b);
@@ -747,13 +748,10 @@ static int build_inc(nd_graph* g, int r, int s, const DBuf& cnt, int w, int64_t 
     cudaMemcpyAsync(cursor.p, b.off.p, 8 * (n_r + 1), cudaMemcpyDeviceToDevice, st);
     cudaMemsetAsync(b.dead.p, 0, b.dead.bytes, st);
     cudaMemsetAsync(b.status.p, 0, b.status.bytes, st);
-    IncFill F;
     F.cursor = (unsigned long long*)cursor.p;
     F.list = (uint32_t*)b.list.p;
     F.row = (int32_t*)b.row.p;
-    F.stride = b.stride;
     F.status = (unsigned int*)b.status.p;
-    F.n_s = n_s;
     F.entries = entries;
     nd_inc_fill(nd_view(g), r, s, n_r, F, st);
     rc = nd_check_launch("incidence lists");
@@ -788,8 +786,10 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags
         hstage = g->edge_mindeg;
         hslices = nd_peel_heavy_slices();
     }
-    // (2,3) graph contraction (Section 5.6): compacted copies of the rows and their lengths
-    bool contract = r == 2 && s == 3 && !(flags & ND_CONTRACT_OFF);
+    // (2,3) graph contraction (Section 5.6): compacted copies of the rows and their lengths, or the
+    // lengths of the incidence lists
+    const bool contract23 = r == 2 && s == 3 && !(flags & ND_CONTRACT_OFF);
+    bool contract = contract23 && !inc, contract_inc = contract23 && inc;
     // (3,4): the same for the triangle lists (compacted copies of the lists and entry offsets)
     const bool lists34 = r == 3 && s == 4 && !inc;
     bool contract34 = lists34 && !(flags & ND_CONTRACT_OFF);
@@ -807,7 +807,7 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags
         ND_TRY(read_back(g, g->scal.p, &mx, "peel setup"));
         bmax = (int64_t)mx + 1;
     }
-    DBuf ctl, A0, A1, N0, N1, L0, L1, H, rs, rl, rt, etr, hsc, abits, ccol, cpos, clen, cprev, bcnt, hcnt, hpre, lw, lt,
+    DBuf ilen, iprev, ctl, A0, A1, N0, N1, L0, L1, H, rs, rl, rt, etr, hsc, abits, ccol, cpos, clen, cprev, bcnt, hcnt, hpre, lw, lt,
         ltp, llen, lprev;
     const int64_t nent = std::max<int64_t>(3 * g->n3, 1);
     if ((rc = nd_alloc(c, ctl, sizeof(PeelCtl))) || (rc = nd_alloc(c, A0, 4 * cap)) || (rc = nd_alloc(c, A1, 4 * cap)) ||
@@ -820,13 +820,14 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags
                       (rc = nd_alloc(c, cpos, 4 * std::max<int64_t>(g->nnz, 1))) ||
                       (rc = nd_alloc(c, clen, 4 * std::max<int64_t>(g->n, 1))) ||
                       (rc = nd_alloc(c, cprev, 4 * std::max<int64_t>(g->n, 1))))) ||
+        (contract_inc && ((rc = nd_alloc(c, ilen, 4 * cap)) || (rc = nd_alloc(c, iprev, 4 * cap)))) ||
         (dense && (rc = nd_alloc(c, bcnt, 4 * std::max<int64_t>(bmax, 1)))) ||
         (staged && ((rc = nd_alloc(c, hcnt, 4 * (hslices + 1))) || (rc = nd_alloc(c, hpre, 8 * (hslices + 1))))) ||
         (contract34 && ((rc = nd_alloc(c, lw, 4 * nent)) || (rc = nd_alloc(c, lt, 4 * nent)) ||
                         (rc = nd_alloc(c, ltp, 4 * nent)) || (rc = nd_alloc(c, llen, 4 * std::max<int64_t>(g->m, 1))) ||
                         (rc = nd_alloc(c, lprev, 4 * std::max<int64_t>(g->m, 1)))))) {
         for (DBuf* b : {&ctl, &A0, &A1, &N0, &N1, &L0, &L1, &H, &rs, &rl, &rt, &etr, &hsc, &abits, &ccol, &cpos, &clen,
-                        &cprev, &bcnt, &hcnt, &hpre, &lw, &lt, &ltp, &llen, &lprev})
+                        &cprev, &bcnt, &hcnt, &hpre, &lw, &lt, &ltp, &llen, &lprev, &ilen, &iprev})
             nd_free(c, *b);
         return rc;
     }
@@ -888,10 +889,11 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags
     P.bmax = 0;
     P.heavy_work = c->tune_heavy[r * 8 + s];
     P.inc_off = inc ? (const int64_t*)inc->off.p : nullptr;
-    P.inc_list = inc ? (const uint32_t*)inc->list.p : nullptr;
+    P.inc_list = inc ? (uint32_t*)inc->list.p : nullptr;
     P.inc_row = inc ? (const int32_t*)inc->row.p : nullptr;
     P.inc_dead = inc ? (uint32_t*)inc->dead.p : nullptr;
     P.inc_stride = inc ? inc->stride : 0;
+    P.inc_len = P.inc_prev = nullptr;
     if (dense) {
         P.bcnt = (unsigned int*)bcnt.p;
         P.bmax = bmax;
@@ -915,6 +917,14 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags
         v.col = P.ccol;
         v.pos2e = P.cpos;
         v.rlen = P.clen;
+        bool always = flags & ND_CONTRACT_ALWAYS;
+        contract_every = always ? 1 : std::max<int64_t>(2 * (int64_t)g->n, 1);
+        contract_shift = always ? 0 : 2;
+    }
+    if (contract_inc) {
+        P.inc_len = (int32_t*)ilen.p;
+        P.inc_prev = (int32_t*)iprev.p;
+        nd_row_len(P.inc_off, (int32_t)n_r, P.inc_len, P.inc_prev, st);
         bool always = flags & ND_CONTRACT_ALWAYS;
         contract_every = always ? 1 : std::max<int64_t>(2 * (int64_t)g->n, 1);
         contract_shift = always ? 0 : 2;
@@ -1042,7 +1052,7 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags
             po.rho = h.h.t;
             po.max_core = n_r ? h.h.k : 0;
             if (looped && !persistent_launches)  // graph nodes executed: every iteration (rho + 1), plus advance and refill phases
-                nd_note_launches((int64_t)(h.h.t + 1) * nd_peel_nodes_per_round(r, s, contract) +
+                nd_note_launches((int64_t)(h.h.t + 1) * nd_peel_nodes_per_round(r, s, contract || contract_inc || contract34) +
                                  3 * (int64_t)h.h.advances + 4 * (int64_t)h.h.refills);
             po.listed = (int64_t)h.listed;
             po.decs = (int64_t)h.decs;
@@ -1066,7 +1076,7 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags
         }
     }
     for (DBuf* b : {&ctl, &A0, &A1, &N0, &N1, &L0, &L1, &H, &rs, &rl, &rt, &etr, &hsc, &abits, &ccol, &cpos, &clen,
-                    &cprev, &bcnt, &hcnt, &hpre, &lw, &lt, &ltp, &llen, &lprev})
+                    &cprev, &bcnt, &hcnt, &hpre, &lw, &lt, &ltp, &llen, &lprev, &ilen, &iprev})
         nd_free(c, *b);
     return rc;
 }

@@ -376,10 +376,13 @@ struct PeelView {
     // inc_list[inc_off[R] .. inc_off[R+1]); s-clique S has its r-subsets' ids in inc_row[S * inc_stride ..]
     // (stride a multiple of 4, filled up with -1) and bit S of inc_dead set once it is destroyed
     const int64_t* inc_off;
-    const uint32_t* inc_list;
+    uint32_t* inc_list;
     const int32_t* inc_row;
     uint32_t* inc_dead;
     int32_t inc_stride;
+    // (2,3) with contraction: the lists' current lengths and those after the previous contraction; else NULL
+    int32_t* inc_len;
+    int32_t* inc_prev;
     // driving-list length above which Update defers an r-clique to the heavy phase (0: the
     // variant's built-in threshold)
     int64_t heavy_work;
@@ -440,16 +443,19 @@ void nd_tri_hash_fill(const GraphView& g, const int64_t* hoff, NdHashSlot* tab, 
 int nd_peel_heavy_slices();
 
 // Incidence lists of the s-cliques (nd_inc.cu), what filling them writes: cursor[R] starts at the first
-// place of R's list; status[0] counts the s-cliques, status[1] is set when one has no room.
+// place of R's list; status[0] counts the rows handed out, status[1] the s-cliques that got one, status[2]
+// is set when one has no room. Warps take rows in runs of `run`, so a few stay unused.
 struct IncFill {
     unsigned long long* cursor;
     uint32_t* list;
     int32_t* row;
-    int32_t stride;
     unsigned int* status;
-    int64_t n_s, entries;
+    int64_t rows, entries;
+    unsigned run;
 };
 int nd_inc_stride(int r, int s);
+// the rows to allocate for n_s s-cliques, and the length of a run
+int64_t nd_inc_rows(int r, int s, int64_t n_r, int64_t m, int64_t n_s, unsigned* run);
 void nd_inc_fill(const GraphView& g, int r, int s, int64_t n_r, const IncFill& F, cudaStream_t st);
 
 // counting (nd_count.cu): counts into cnt (CT = int32_t or int64_t), zero-initialised

@@ -2,20 +2,19 @@
 // Algorithm 1 (rec-list-cliques) on the oriented graph DG.
 //
 // Two kernel shapes, one per kind of (r,s):
-//   * s = r + 1  ((1,2), (2,3), (3,4)): the s-cliques containing R are R plus one vertex of
-//     I(R) = ∩_{v in R} N(v), so count[R] = |I(R)|. One warp per r-clique intersects the two
-//     shortest lists by merge path (or probes / bisects the longer one when it is much longer);
-//     the result is written once, with no atomics.
-//     For r = 3 the lists are the per-edge common-neighbour tables L(e) of the triangle index
-//     (|L(e)| is the edge's triangle support, far shorter than the vertex degrees).
-//   * s = r + 2  ((1,3), (2,4)): the s-cliques are listed once each over DG (Algorithm 1:
-//     I' = I ∩ N_DG(v) at each level) and add 1 to each of their C(s,r) r-subsets (Count-Func),
-//     with one aggregated atomic for an r-subset shared by a whole level: (1,3) one warp per
-//     lowest vertex; (2,4) one warp per lowest DG edge, the pairs of its last level spread over the
-//     lanes.
+//   * (1,2) reads the degrees; (3,4): count[R] = |I(R)|, the 4-cliques containing R being R plus one
+//     vertex of I(R) = ∩_{v in R} N(v). One warp per triangle intersects the two shortest lists by merge
+//     path (or probes / bisects the longer one when it is much longer); the result is written
+//     once, with no atomics. The lists are the per-edge common-neighbour tables L(e) of the triangle
+//     index (|L(e)| is the edge's triangle support, far shorter than the vertex degrees).
+//   * (1,3), (2,3), (2,4): the s-cliques are listed once each over DG (Algorithm 1: I' = I ∩ N_DG(v) at each
+//     level) and add 1 to each of their C(s,r) r-subsets (Count-Func), with one aggregated atomic for an
+//     r-subset shared by a whole level: triangles 32 DG edges to a warp, 4-cliques one warp per
+//     lowest DG edge, the pairs of its last level spread over the lanes.
 #include "nd_common.cuh"
 #include "nd_gen.cuh"
 #include "nd_quad24.cuh"
+#include "nd_tri.cuh"
 
 namespace {
 
@@ -43,31 +42,44 @@ __global__ void k_count12(GraphView g, CT* __restrict__ cnt) {
         cnt[v] = (CT)(g.rp[v + 1] - g.rp[v]);
 }
 
-// count[e] = |N(a) ∩ N(b)|
-template <typename CT>
-__global__ void k_count23(GraphView g, CT* __restrict__ cnt) {
-    int lane = threadIdx.x & 31;
-    for (int64_t e = gwarp(); e < g.m; e += nwarps()) {
-        int32_t a = g.eu[e], b = g.ev[e];
-        int64_t ab = g.rp[a], ae = g.rp[a + 1], bb = g.rp[b], be = g.rp[b + 1];
-        const int32_t *xs = g.col + ab, *ys = g.col + bb;
-        int64_t nx = ae - ab, ny = be - bb;
-        if (nx > ny) {
-            const int32_t* t = xs;
-            xs = ys;
-            ys = t;
-            int64_t tn = nx;
-            nx = ny;
-            ny = tn;
-        }
-        int c = 0;
-        if (nd_prefer_merge(nx, ny))
-            c = nd_merge_count(xs, (int)nx, ys, (int)ny);
-        else
-            for (int64_t i = lane; i < nx; i += 32) c += nd_find(ys, ny, xs[i]) >= 0 ? 1 : 0;
-        c = warp_sum(c);
-        if (lane == 0) cnt[e] = (CT)c;
+// (2,3) and (1,3): nd_tri.cuh lists the triangles of DG; each adds 1 to its edges or vertices. What the
+// triangles of one DG edge share is kept in shared memory and added once.
+template <typename CT, int R_>
+struct CountTri {
+    CT* cnt;
+    const int32_t* eid;
+    unsigned* own;  // the warp's triangles per edge
+    __device__ void begin(int slot) const {
+        own[slot] = 0;
+        __syncwarp();
     }
+    __device__ void tri(bool hit, int slot, int32_t, int32_t px, int32_t py, int32_t, int32_t, int32_t w) const {
+        if (!hit) return;
+        atomicAdd(&own[slot], 1u);
+        if (R_ == 1) {
+            nd_atomic_add(&cnt[w], 1);
+        } else {
+            nd_atomic_add(&cnt[eid[px]], 1);
+            nd_atomic_add(&cnt[eid[py]], 1);
+        }
+    }
+    __device__ void end(int slot, int32_t e, int32_t u, int32_t v) const {
+        const unsigned c = own[slot];
+        if (!c) return;
+        if (R_ == 1) {
+            nd_atomic_add(&cnt[u], c);
+            nd_atomic_add(&cnt[v], c);
+        } else {
+            nd_atomic_add(&cnt[e], c);
+        }
+    }
+};
+
+template <typename CT, int R_>
+__global__ void __launch_bounds__(kTriThreads) k_count_tri(GraphView g, CT* __restrict__ cnt) {
+    __shared__ unsigned s_own[kTriThreads];
+    CountTri<CT, R_> sink{cnt, g.dg_eid, s_own + (threadIdx.x & ~31u)};
+    tri_list(g, sink);
 }
 
 // count[t] = |L(ab) ∩ L(ac) ∩ L(bc)|. Any two of the lists already intersect to the common
@@ -113,32 +125,6 @@ __global__ void k_count34(GraphView g, CT* __restrict__ cnt) {
     }
 }
 
-// (1,3): every triangle (u, v, w) of DG (u -> v, u -> w, v -> w) adds 1 to u, v and w.
-template <typename CT>
-__global__ void k_count13(GraphView g, CT* __restrict__ cnt) {
-    int lane = threadIdx.x & 31;
-    for (int64_t u = gwarp(); u < g.n; u += nwarps()) {
-        int64_t ub = g.dg_rp[u], ue = g.dg_rp[u + 1];
-        int cu = 0;
-        for (int64_t jv = ub; jv < ue; ++jv) {
-            int32_t v = g.dg_col[jv];
-            int64_t vb = g.dg_rp[v], vn = g.dg_rp[v + 1] - vb;
-            int cv = 0;
-            for (int64_t i = ub + lane; i < ue; i += 32) {
-                int32_t w = g.dg_col[i];
-                if (nd_find(g.dg_col + vb, vn, w) >= 0) {
-                    nd_atomic_add(&cnt[w], 1);
-                    cv++;
-                }
-            }
-            cv = warp_sum(cv);
-            if (lane == 0 && cv) nd_atomic_add(&cnt[v], cv);
-            cu += cv;
-        }
-        if (lane == 0 && cu) nd_atomic_add(&cnt[u], cu);
-    }
-}
-
 // (2,4): nd_quad24.cuh lists the 4-cliques; each adds 1 to its six edges
 template <typename CT>
 struct Count24 {
@@ -146,7 +132,8 @@ struct Count24 {
     static constexpr bool kTally = true;
     __device__ void pair(int32_t e_wx) const { nd_atomic_add(&cnt[e_wx], 1); }
     __device__ void add(int32_t e, int64_t c) const { nd_atomic_add(&cnt[e], c); }
-    __device__ void clique(const int32_t (&e)[6]) const {
+    __device__ void clique(bool hit, const int32_t (&e)[6]) const {
+        if (!hit) return;
 #pragma unroll
         for (int i = 1; i < 6; ++i) nd_atomic_add(&cnt[e[i]], 1);
     }
@@ -154,7 +141,8 @@ struct Count24 {
 
 template <typename CT>
 __global__ void __launch_bounds__(kQuadThreads) k_count24_flat(GraphView g, CT* __restrict__ cnt) {
-    quad24_list(g, Count24<CT>{cnt});
+    Count24<CT> sink{cnt};
+    quad24_list(g, sink);
 }
 
 // Any other supported (r,s) ((1,4), (2,5), (3,5), (3,6), (4,5), (4,6)): one warp per r-clique R counts the
@@ -191,12 +179,13 @@ void nd_count_launch(const GraphView& g, int r, int s, CT* cnt, int64_t n_r, cud
     if (r == 1 && s == 2) {
         ND_K(k_count12<CT><<<blk, kThreads, 0, st>>>(g, cnt));
     } else if (r == 2 && s == 3) {
-        ND_K(k_count23<CT><<<blk, kThreads, 0, st>>>(g, cnt));
+        ND_K(k_zero<CT><<<blk, kThreads, 0, st>>>(cnt, n_r));
+        ND_K(k_count_tri<CT, 2><<<blocks_for_warps((g.m + 31) / 32), kTriThreads, 0, st>>>(g, cnt));
     } else if (r == 3 && s == 4) {
         ND_K(k_count34<CT><<<blk, kThreads, 0, st>>>(g, cnt));
     } else if (r == 1 && s == 3) {
         ND_K(k_zero<CT><<<blk, kThreads, 0, st>>>(cnt, n_r));
-        ND_K(k_count13<CT><<<blocks_for_warps(g.n), kThreads, 0, st>>>(g, cnt));
+        ND_K(k_count_tri<CT, 1><<<blocks_for_warps((g.m + 31) / 32), kTriThreads, 0, st>>>(g, cnt));
     } else if (r == 2 && s == 4) {
         ND_K(k_zero<CT><<<blk, kThreads, 0, st>>>(cnt, n_r));
         ND_K(k_count24_flat<CT><<<blocks_for_warps(g.m), kQuadThreads, 0, st>>>(g, cnt));

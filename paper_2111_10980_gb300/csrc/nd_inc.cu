@@ -10,10 +10,12 @@
 // Measured, count and peel with the lists' building, before and after: (2,4) on a Chung-Lu graph of
 // 500,009 vertices with 500 communities (8.4 M 4-cliques, 1,968 rounds) 87 -> 36 ms; (4,5) on a flat R-MAT
 // graph of 40,000 vertices, degeneracy order and all, 15.4 -> 12.1 ms; (3,4) on a Chung-Lu graph of a million
-// vertices (17 M 4-cliques) 64.0 -> 61.7 ms.
+// vertices (17 M 4-cliques) 64.0 -> 61.7 ms; (2,3) on R-MAT scale 20 (374 M triangles, 2,107 rounds) 208 ->
+// 144 ms, the fill 34 ms of it.
 #include "nd_common.cuh"
 #include "nd_gen.cuh"
 #include "nd_quad24.cuh"
+#include "nd_tri.cuh"
 
 namespace {
 
@@ -28,16 +30,17 @@ int blocks_for_warps(int64_t items) {
     return (int)(want < cap ? want : cap);
 }
 
-// one s-clique with members id[0..C): a row, and a place in each member's list
+// A warp's run of rows: F.run at a time from one counter (a counter update for every handful of matches is
+// what the first form of k_inc_tri waited for: 130 ms for the 374 M triangles of R-MAT scale 20).
+struct IncRun {
+    unsigned at = 0, left = 0, used = 0;
+};
+
+// row and list places of one s-clique
 template <int C>
-__device__ __forceinline__ void inc_put(const IncFill& F, const int32_t* id) {
-    const unsigned mask = __activemask();
-    const int lane = threadIdx.x & 31, leader = __ffs(mask) - 1;
-    unsigned base = 0;
-    if (lane == leader) base = atomicAdd(&F.status[0], (unsigned)__popc(mask));
-    const unsigned S = __shfl_sync(mask, base, leader) + __popc(mask & nd_lanemask_lt());
-    if (S >= F.n_s) {
-        F.status[1] = 1;
+__device__ __forceinline__ void inc_write(const IncFill& F, unsigned S, const int32_t* id) {
+    if (S >= F.rows) {
+        F.status[2] = 1;
         return;
     }
     unsigned long long at[C];
@@ -53,33 +56,87 @@ __device__ __forceinline__ void inc_put(const IncFill& F, const int32_t* id) {
         if ((int64_t)at[i] < F.entries)
             F.list[at[i]] = S;
         else
-            F.status[1] = 1;
+            F.status[2] = 1;
     }
 }
 
-// (1,3): every triangle (u, v, w) of DG, as k_count13 lists them
-__global__ void k_inc13(GraphView g, IncFill F) {
-    int lane = threadIdx.x & 31;
-    for (int64_t u = gwarp(); u < g.n; u += nwarps()) {
-        int64_t ub = g.dg_rp[u], ue = g.dg_rp[u + 1];
-        for (int64_t jv = ub; jv < ue; ++jv) {
-            int32_t v = g.dg_col[jv];
-            int64_t vb = g.dg_rp[v], vn = g.dg_rp[v + 1] - vb;
-            for (int64_t i = ub + lane; i < ue; i += 32) {
-                const int32_t id[3] = {(int32_t)u, v, g.dg_col[i]};
-                if (nd_find(g.dg_col + vb, vn, id[2]) >= 0) inc_put<3>(F, id);
-            }
-        }
+// The s-cliques of the lanes with hit set, members id[0..C). The whole warp calls it. F.run >= 32.
+template <int C>
+__device__ __forceinline__ void inc_put(const IncFill& F, IncRun& run, bool hit, const int32_t* id) {
+    const unsigned full = 0xffffffffu, mask = __ballot_sync(full, hit);
+    const unsigned n = __popc(mask), rank = __popc(mask & nd_lanemask_lt());
+    unsigned next = 0;
+    if (n > run.left) {
+        if ((threadIdx.x & 31) == 0) next = atomicAdd(&F.status[0], F.run);
+        next = __shfl_sync(full, next, 0);
     }
+    const unsigned S = rank < run.left ? run.at + rank : next + (rank - run.left);
+    if (n > run.left) {
+        run.at = next + (n - run.left);
+        run.left = F.run - (n - run.left);
+    } else {
+        run.at += n;
+        run.left -= n;
+    }
+    run.used += n;
+    if (hit) inc_write<C>(F, S, id);
+}
+
+__device__ __forceinline__ void inc_done(const IncFill& F, const IncRun& run) {
+    if ((threadIdx.x & 31) == 0 && run.used) atomicAdd(&F.status[1], run.used);
+}
+
+// The same from lanes that come as they find them: a row each from the counter
+template <int C>
+__device__ __forceinline__ void inc_put_any(const IncFill& F, const int32_t* id) {
+    const unsigned mask = __activemask();
+    const int lane = threadIdx.x & 31, leader = __ffs(mask) - 1;
+    unsigned base = 0;
+    if (lane == leader) {
+        base = atomicAdd(&F.status[0], (unsigned)__popc(mask));
+        atomicAdd(&F.status[1], (unsigned)__popc(mask));
+    }
+    inc_write<C>(F, __shfl_sync(mask, base, leader) + __popc(mask & nd_lanemask_lt()), id);
+}
+
+// (1,3), (2,3): every triangle of DG
+template <int R_>
+struct PutTri {
+    IncFill F;
+    const int32_t* eid;
+    IncRun run;
+    __device__ void begin(int) const {}
+    __device__ void tri(bool hit, int, int32_t e, int32_t px, int32_t py, int32_t u, int32_t v, int32_t w) {
+        int32_t id[3] = {u, v, w};
+        if (R_ == 2 && hit) {
+            id[0] = e;
+            id[1] = eid[px];
+            id[2] = eid[py];
+        }
+        inc_put<3>(F, run, hit, id);
+    }
+    __device__ void end(int, int32_t, int32_t, int32_t) const {}
+};
+
+template <int R_>
+__global__ void __launch_bounds__(kTriThreads) k_inc_tri(GraphView g, IncFill F) {
+    PutTri<R_> sink{F, g.dg_eid, IncRun{}};
+    tri_list(g, sink);
+    inc_done(F, sink.run);
 }
 
 struct Put24 {
     IncFill F;
+    IncRun run;
     static constexpr bool kTally = false;
-    __device__ void clique(const int32_t (&e)[6]) const { inc_put<6>(F, e); }
+    __device__ void clique(bool hit, const int32_t (&e)[6]) { inc_put<6>(F, run, hit, e); }
 };
 
-__global__ void __launch_bounds__(kQuadThreads) k_inc24(GraphView g, IncFill F) { quad24_list(g, Put24{F}); }
+__global__ void __launch_bounds__(kQuadThreads) k_inc24(GraphView g, IncFill F) {
+    Put24 sink{F, IncRun{}};
+    quad24_list(g, sink);
+    inc_done(F, sink.run);
+}
 
 // (3,4): every 4-clique from its lowest triangle (a < b < c): the vertices w > c of the shortest of the
 // triangle's three lists that the other two hold as well; each entry names its triangle
@@ -96,6 +153,7 @@ __device__ __forceinline__ bool inc_look(const GraphView& g, int32_t e, int64_t 
 
 __global__ void k_inc34(GraphView g, IncFill F) {
     int lane = threadIdx.x & 31;
+    IncRun run;
     for (int64_t t = gwarp(); t < g.n3; t += nwarps()) {
         int32_t e[3];
         int64_t b[3], n[3];
@@ -113,12 +171,19 @@ __global__ void k_inc34(GraphView g, IncFill F) {
         const int32_t e1 = d == 0 ? e[1] : e[0], e2 = d == 2 ? e[1] : e[2];
         const int64_t b1 = d == 0 ? b[1] : b[0], n1 = d == 0 ? n[1] : n[0];
         const int64_t b2 = d == 2 ? b[1] : b[2], n2 = d == 2 ? n[1] : n[2];
-        for (int64_t j = nd_lower_bound(g.et_w + bd, nd, c + 1) + lane; j < nd; j += 32) {
-            const int32_t w = g.et_w[bd + j];
-            int32_t id[4] = {(int32_t)t, g.et_t[bd + j], 0, 0};
-            if (inc_look(g, e1, b1, n1, w, id[2]) && inc_look(g, e2, b2, n2, w, id[3])) inc_put<4>(F, id);
+        for (int64_t j0 = nd_lower_bound(g.et_w + bd, nd, c + 1); j0 < nd; j0 += 32) {
+            const int64_t j = j0 + lane;
+            int32_t id[4] = {(int32_t)t, 0, 0, 0};
+            bool hit = false;
+            if (j < nd) {
+                const int32_t w = g.et_w[bd + j];
+                id[1] = g.et_t[bd + j];
+                hit = inc_look(g, e1, b1, n1, w, id[2]) && inc_look(g, e2, b2, n2, w, id[3]);
+            }
+            inc_put<4>(F, run, hit, id);
         }
     }
+    inc_done(F, run);
 }
 
 // Any other (r,s): every s-clique from the r-clique of its r lowest vertices, the others above them
@@ -141,10 +206,10 @@ __global__ void k_inc_gen(GraphView g, int64_t n_r, IncFill F) {
                 gen_merge<R_, S_>(v, Cv, Sv);
                 o[0] = (int32_t)id;
                 if (!gen_others<R_, S_>(g, v, Sv, o + 1)) {
-                    F.status[1] = 1;
+                    F.status[2] = 1;
                     return;
                 }
-                inc_put<C>(F, o);
+                inc_put_any<C>(F, o);
             });
     }
 }
@@ -157,13 +222,28 @@ int nd_inc_stride(int r, int s) {
     return (c + 3) / 4 * 4;
 }
 
+// the work items of a fill kernel, one per warp at a time
+static int64_t inc_items(int r, int s, int64_t n_r, int64_t m) {
+    return s == 3 ? (m + 31) / 32 : r == 2 && s == 4 ? m : n_r;
+}
+
+int64_t nd_inc_rows(int r, int s, int64_t n_r, int64_t m, int64_t n_s, unsigned* run) {
+    const int64_t warps = (int64_t)blocks_for_warps(inc_items(r, s, n_r, m)) * (kThreads / 32);
+    const int64_t share = n_s / (8 * warps);  // an eighth of a warp's share, so at most an eighth more rows
+    *run = (unsigned)(share < 32 ? 32 : share > 1024 ? 1024 : share);
+    return n_s + warps * *run;
+}
+
 void nd_inc_fill(const GraphView& g, int r, int s, int64_t n_r, const IncFill& F, cudaStream_t st) {
     if (n_r <= 0) return;
-    const int blk = blocks_for_warps(n_r);
+    const int blk = blocks_for_warps(inc_items(r, s, n_r, g.m));
+    static_assert(kTriThreads == kThreads && kQuadThreads == kThreads, "nd_inc_rows counts the warps");
     if (r == 1 && s == 3) {
-        ND_K(k_inc13<<<blocks_for_warps(g.n), kThreads, 0, st>>>(g, F));
+        ND_K(k_inc_tri<1><<<blk, kTriThreads, 0, st>>>(g, F));
+    } else if (r == 2 && s == 3) {
+        ND_K(k_inc_tri<2><<<blk, kTriThreads, 0, st>>>(g, F));
     } else if (r == 2 && s == 4) {
-        ND_K(k_inc24<<<blocks_for_warps(g.m), kQuadThreads, 0, st>>>(g, F));
+        ND_K(k_inc24<<<blk, kQuadThreads, 0, st>>>(g, F));
     } else if (r == 3 && s == 4) {
         ND_K(k_inc34<<<blk, kThreads, 0, st>>>(g, F));
     } else if (r == 1 && s == 4) {

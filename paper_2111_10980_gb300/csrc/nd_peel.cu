@@ -31,7 +31,7 @@
 //     warp applies S's effect, subtracting exactly 1 from every r-subset not in A. The paper
 //     has each of the a members of A subtract 1/a; the owner rule gives the same total (1 per
 //     live S and surviving member) with integer atomics and without double counting.
-// With incidence lists (nd_inc.cu; the default but for (1,2), (2,3) and very many s-cliques) the s-cliques
+// With incidence lists (nd_inc.cu; the default but for (1,2) and very many s-cliques) the s-cliques
 // are not listed again: the first peeled member of S to set S's bit applies S's effect (UpdInc).
 // Warps take A in dynamic chunks; r-cliques with long driving lists go to a heavy phase that
 // gives each a block ((2,4) in the persistent kernel: stage per block, then the pairs of all
@@ -147,7 +147,7 @@ __global__ void k_init(PeelCtl* c, int64_t n_r, int64_t max_rounds, unsigned lon
         h.contract_every = contract_every;
         h.minN = h.gmin = ULLONG_MAX;
         // incidence lists that do not hold every s-clique once are not peeled
-        const bool bad = inc_status && (inc_status[1] || (int64_t)inc_status[0] != n_s);
+        const bool bad = inc_status && (inc_status[2] || (int64_t)inc_status[1] != n_s);
         h.done = bad;
         c->h = h;
         c->err = bad ? 16 : 0;
@@ -547,6 +547,54 @@ __device__ __noinline__ void phase_contract34(const GraphView& g, const PeelView
         }
     }
 }
+
+// The same for the (2,3) incidence lists: a list's dead entries are the triangles with an edge peeled in an
+// earlier round. How many a list lost follows from the edge's count (its live triangles), so only the
+// lists that are compacted are read: a warp looks 32 edges over and then filters theirs one after
+// another, in place and in order. Edges that are peeled or scheduled are left alone: their lists are
+// read once more at most.
+template <typename CT>
+__device__ __noinline__ void phase_contract_inc(const PeelView<CT>& P, const PeelHot& s) {
+    if (s.done || !s.contract) return;
+    const unsigned full = 0xffffffffu;
+    const int32_t shift = P.ctl->contract_shift;
+    const int lane = threadIdx.x & 31;
+    for (int64_t R0 = gwarp() * 32; R0 < s.n_r; R0 += nwarps() * 32) {
+        const int64_t R = R0 + lane;
+        bool due = false;
+        if (R < s.n_r && P.rnd[R] == ND_UNPEELED) {
+            const int64_t prev = P.inc_prev[R], lost = prev - (int64_t)P.cnt[R], need = shift ? prev >> shift : 1;
+            due = lost > 0 && lost >= need;
+        }
+        unsigned todo = __ballot_sync(full, due);
+        while (todo) {
+            const int64_t Q = R0 + __ffs(todo) - 1;
+            todo &= todo - 1;
+            uint32_t* list = P.inc_list + P.inc_off[Q];
+            const int32_t len = P.inc_len[Q];
+            int32_t out = 0;
+            for (int32_t i0 = 0; i0 < len; i0 += 32) {
+                const int32_t i = i0 + lane;
+                uint32_t S = 0;
+                bool keep = false;
+                if (i < len) {
+                    S = list[i];
+                    keep = !(P.inc_dead[S >> 5] >> (S & 31) & 1u);
+                }
+                const unsigned mk = __ballot_sync(full, keep);
+                if (keep) list[out + __popc(mk & nd_lanemask_lt())] = S;
+                out += __popc(mk);
+            }
+            if (lane == 0) {
+                P.inc_len[Q] = out;
+                P.inc_prev[Q] = out;
+            }
+        }
+    }
+}
+
+template <typename CT>
+__global__ void k_contract_inc(PeelView<CT> P) { phase_contract_inc(P, P.ctl->h); }
 
 template <typename CT>
 __global__ void k_contract34(GraphView g, PeelView<CT> P) { phase_contract34(g, P, P.ctl->h); }
@@ -1371,13 +1419,22 @@ struct UpdInc {
     static constexpr bool kInc = true;
     __device__ static int64_t prep(const GraphView&, const PeelView<CT>& P, int32_t R, Prep& q) {
         q.b[0] = P.inc_off[R];
-        q.n[0] = P.inc_off[R + 1] - q.b[0];
+        q.n[0] = P.inc_len ? (int64_t)P.inc_len[R] : P.inc_off[R + 1] - q.b[0];
+        q.hk[0] = 0;
         return q.n[0];
     }
+    // A candidate of a shared round (q.hk[0], set by phase_update) goes the shortest way: the bit is claimed
+    // while the row is on its way, and all members but R lose one, those of A included (nobody reads their
+    // counts again), so no round tag is waited for. In a round with work for every warp what counts is
+    // traffic: the dead two thirds are dropped by a plain read of the bit, and members of A, or already in
+    // the next round's, keep their counts. Measured: R-MAT
+    // scale 20 (2,3), Update 79 ms with every candidate the first way, 57 ms with both.
     template <typename Q>
     __device__ static void cand(const GraphView&, const RoundEnv<CT>& E, int32_t R, const Q& q, int64_t j,
                                 UpdCounters& k) {
         const uint32_t S = E.P.inc_list[q.b[0] + j], bit = 1u << (S & 31);
+        const bool shared = q.hk[0];
+        if (!shared && (E.P.inc_dead[S >> 5] & bit)) return;
         const int nv = kVec ? kVec : E.P.inc_stride >> 2;
         const int4* row = reinterpret_cast<const int4*>(E.P.inc_row + (int64_t)S * E.P.inc_stride);
         int4 v[kVec ? kVec : 1];
@@ -1393,16 +1450,19 @@ struct UpdInc {
             const int32_t x[4] = {w.x, w.y, w.z, w.w};
             int32_t r[4];
             int64_t o[4];
-            // members of A (round t) keep their counts; one that was already put into the next round
-            // (t + 1) may lose one more, which nobody reads
 #pragma unroll
             for (int m = 0; m < 4; ++m) r[m] = x[m] >= 0 && x[m] != R ? E.P.rnd[x[m]] : E.t;
+            if (shared) {
 #pragma unroll
-            for (int m = 0; m < 4; ++m) o[m] = dec_live(r[m], E.t) ? nd_atomic_dec(&E.P.cnt[x[m]]) : 0;
+                for (int m = 0; m < 4; ++m) o[m] = x[m] >= 0 && x[m] != R ? nd_atomic_dec(&E.P.cnt[x[m]]) : E.k;
+            } else {
+#pragma unroll
+                for (int m = 0; m < 4; ++m) o[m] = dec_live(r[m], E.t) ? nd_atomic_dec(&E.P.cnt[x[m]]) : E.k;
+            }
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
                 k.decs += r[m] != E.t;
-                if (dec_live(r[m], E.t)) after_dec(E, x[m], o[m]);
+                after_dec(E, x[m], o[m]);
             }
         }
     }
@@ -1417,6 +1477,15 @@ struct is_staged<U, decltype((void)U::kStaged)> {
     static constexpr bool value = U::kStaged;
 };
 
+
+template <typename U, typename = void>
+struct is_inc {
+    static constexpr bool value = false;
+};
+template <typename U>
+struct is_inc<U, decltype((void)U::kInc)> {
+    static constexpr bool value = U::kInc;
+};
 
 template <typename U, typename = void>
 struct is_queued {
@@ -1494,6 +1563,7 @@ __device__ __forceinline__ void phase_update(const GraphView& g, const PeelView<
                 const int32_t R = A[i];
                 Prep q;
                 int64_t n0 = U::prep(g, P, R, q), j0 = part * 32 + lane, dj = (int64_t)32 << shift;
+                if constexpr (is_inc<U>::value) q.hk[0] = 1;
                 if (part == 0 && lane == 0) unmark_a(P, R);
                 if (n0 > heavy_limit<U>(P) << shift) {
                     // one of the warps hands it over; with no room there it lists all of it itself
@@ -1893,7 +1963,9 @@ __global__ void __launch_bounds__(512, 2) k_peel_loop(GraphView g, PeelView<CT> 
         const Team T = grid_team();
         const int32_t tr = s.t;  // the round being run
         if (s.contract && s.stage != 2) {
-            if constexpr (k34)
+            if constexpr (is_inc<U>::value)
+                phase_contract_inc(Q, s);
+            else if constexpr (k34)
                 phase_contract34(h, Q, s);
             else
                 phase_contract(h, Q, s);
@@ -1990,6 +2062,7 @@ void nd_peel_init(PeelCtl* ctl, int64_t n_r, int64_t max_rounds, cudaStream_t st
 
 template <typename CT>
 void nd_peel_contract(const GraphView& g, const PeelView<CT>& P, cudaStream_t st) {
+    if (P.inc_len) ND_K(k_contract_inc<CT><<<peel_blocks(), kThreads, 0, st>>>(P));
     if (P.ccol) ND_K(k_contract<CT><<<peel_blocks(), kThreads, 0, st>>>(g, P));
     if (P.lw) ND_K(k_contract34<CT><<<peel_blocks(), kThreads, 0, st>>>(g, P));
 }

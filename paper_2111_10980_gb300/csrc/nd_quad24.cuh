@@ -14,7 +14,8 @@ constexpr int kQuadThreads = 256;
 // tallies (kTally) gets w-x of every 4-clique, and at the end the numbers of u-w, v-w (the same for
 // both, kept in shared memory meanwhile) and u-v: one global atomic for each 4-clique instead of five
 // (R-MAT of 50,001 vertices, 131 M 4-cliques: the count call 7.0 -> 5.2 ms, with the vertex u read
-// from the edge instead of bisected). Another sink gets the six edges, u-v first.
+// from the edge instead of bisected). Another sink gets the six edges, u-v
+// first, from the whole warp, with each lane saying whether it has a 4-clique.
 // An edge whose I does not fit the stage (more than kC24 vertices) is listed by the lanes walking
 // out-lists instead; a tallying sink's clique() then adds to all but u-v.
 constexpr int kC24 = 128;
@@ -32,7 +33,7 @@ __device__ __forceinline__ int stage_find24(const int32_t* a, int n, int32_t x) 
 }
 
 template <typename Sink>
-__device__ void quad24_list(const GraphView& g, const Sink& sink) {
+__device__ __forceinline__ void quad24_list(const GraphView& g, Sink& sink) {
     constexpr int kWarpsPerBlock = kQuadThreads / 32;
     __shared__ int32_t s_w[kWarpsPerBlock][kC24], s_eu[kWarpsPerBlock][kC24], s_ev[kWarpsPerBlock][kC24],
         s_b[kWarpsPerBlock][kC24], s_p[kWarpsPerBlock][kC24 + 1];
@@ -83,26 +84,31 @@ __device__ void quad24_list(const GraphView& g, const Sink& sink) {
             }
             if (lane == 0) sp[c] = carry;
             __syncwarp();
-            for (int32_t p = lane; p < carry; p += 32) {
-                int a = 0, b = c;  // owner: the last i with sp[i] <= p
-                while (b - a > 1) {
-                    int mid = (a + b) >> 1;
-                    if (sp[mid] <= p)
-                        a = mid;
-                    else
-                        b = mid;
+            for (int32_t p0 = 0; p0 < carry; p0 += 32) {
+                const int32_t p = p0 + lane;
+                int a = 0, b = c, k = -1;  // owner a: the last i with sp[i] <= p
+                int64_t jx = 0;
+                if (p < carry) {
+                    while (b - a > 1) {
+                        int mid = (a + b) >> 1;
+                        if (sp[mid] <= p)
+                            a = mid;
+                        else
+                            b = mid;
+                    }
+                    jx = (int64_t)sb[a] + (p - sp[a]);
+                    k = stage_find24(sw, c, g.dg_col[jx]);
                 }
-                int64_t jx = (int64_t)sb[a] + (p - sp[a]);
-                int k = stage_find24(sw, c, g.dg_col[jx]);
-                if (k < 0) continue;
                 if constexpr (Sink::kTally) {
+                    if (k < 0) continue;
                     ++c_uv;
                     sink.pair(g.dg_eid[jx]);
                     atomicAdd(&s_c[wid][k], 1);
                     atomicAdd(&s_c[wid][a], 1);
                 } else {
-                    const int32_t e[6] = {e_uv, seu[k], sev[k], seu[a], sev[a], g.dg_eid[jx]};
-                    sink.clique(e);
+                    const bool hit = k >= 0;
+                    const int32_t e[6] = {e_uv, hit ? seu[k] : 0, hit ? sev[k] : 0, seu[a], sev[a], hit ? g.dg_eid[jx] : 0};
+                    sink.clique(hit, e);
                 }
             }
             if constexpr (Sink::kTally) {
@@ -117,20 +123,29 @@ __device__ void quad24_list(const GraphView& g, const Sink& sink) {
         } else {
             // I does not fit the stage: the lanes take the w of N_DG(u) ∩ N_DG(v) and walk their
             // out-lists, searching x in both lists
-            for (int64_t p = ub + lane; p < ue; p += 32) {
-                int32_t w = g.dg_col[p];
-                int64_t q = nd_find(g.dg_col + vb, vn, w);
-                if (q < 0) continue;
-                int32_t e_uw = g.dg_eid[p], e_vw = g.dg_eid[vb + q];
-                for (int64_t jx = g.dg_rp[w]; jx < g.dg_rp[w + 1]; ++jx) {
-                    int32_t x = g.dg_col[jx];
-                    int64_t pux = nd_find(g.dg_col + ub, ue - ub, x);
-                    if (pux < 0) continue;
-                    int64_t pvx = nd_find(g.dg_col + vb, vn, x);
-                    if (pvx < 0) continue;
-                    ++c_uv;
-                    const int32_t e[6] = {e_uv, g.dg_eid[ub + pux], g.dg_eid[vb + pvx], e_uw, e_vw, g.dg_eid[jx]};
-                    sink.clique(e);
+            for (int64_t p0 = ub; p0 < ue; p0 += 32) {
+                const int64_t p = p0 + lane;
+                const int32_t w = p < ue ? g.dg_col[p] : 0;
+                const int64_t q = p < ue ? nd_find(g.dg_col + vb, vn, w) : -1;
+                int64_t jx = q < 0 ? 0 : g.dg_rp[w];
+                const int64_t je = q < 0 ? 0 : g.dg_rp[w + 1];
+                const int32_t e_uw = q < 0 ? 0 : g.dg_eid[p], e_vw = q < 0 ? 0 : g.dg_eid[vb + q];
+                for (; __any_sync(full, jx < je); ++jx) {
+                    int64_t pux = -1, pvx = -1;
+                    if (jx < je) {
+                        const int32_t x = g.dg_col[jx];
+                        pux = nd_find(g.dg_col + ub, ue - ub, x);
+                        if (pux >= 0) pvx = nd_find(g.dg_col + vb, vn, x);
+                    }
+                    const bool hit = pvx >= 0;
+                    int32_t e[6] = {e_uv, 0, 0, e_uw, e_vw, 0};
+                    if (hit) {
+                        e[1] = g.dg_eid[ub + pux];
+                        e[2] = g.dg_eid[vb + pvx];
+                        e[5] = g.dg_eid[jx];
+                        ++c_uv;
+                    }
+                    sink.clique(hit, e);
                 }
             }
         }

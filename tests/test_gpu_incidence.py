@@ -15,7 +15,7 @@ from test_gpu_parity import assert_parity
 
 pytestmark = pytest.mark.gpu
 
-RS = [(1, 3), (1, 4), (2, 4), (2, 5), (3, 4), (3, 5), (3, 6), (4, 5), (4, 6)]
+RS = [(1, 3), (1, 4), (2, 3), (2, 4), (2, 5), (3, 4), (3, 5), (3, 6), (4, 5), (4, 6)]
 
 
 @pytest.fixture(scope="module")
@@ -32,7 +32,7 @@ def test_with_and_without_room_for_the_lists(nd, r, s):
 
     # dense communities over a sparse graph, so that the rows are the largest buffer (next to the stages
     # of the heavy edges when (2,4) lists its s-cliques again)
-    g = gg.with_planted(gg.chung_lu(1200, 6.0, 2.3, seed=91), 30 if (r, s) == (2, 4) else 12, 14, 20, 0.85, seed=92)
+    g = gg.with_planted(gg.chung_lu(1200, 6.0, 2.3, seed=91), 30 if r == 2 and s < 5 else 12, 14, 20, 0.85, seed=92)
     rows = 4 * ((math.comb(s, r) + 3) // 4 * 4) * orc.decompose(g, r, s).n_s
     alloc, free = nd.torch_allocator_hooks(0)
     for limit in (None, rows):
@@ -47,7 +47,7 @@ def test_with_and_without_room_for_the_lists(nd, r, s):
         ctx = nd.nd_ctx_create(0, stream=torch.cuda.Stream())
         nd.nd_ctx_set_allocator(ctx, hook, free)
         try:
-            for flags in (0, nd.ND_PEEL_LOOP_GRAPH, nd.ND_NO_GRAPH):
+            for flags in (0, nd.ND_CONTRACT_ALWAYS, nd.ND_CONTRACT_OFF, nd.ND_PEEL_LOOP_GRAPH, nd.ND_NO_GRAPH):
                 assert_parity(nd, ctx, g, r, s, flags=flags)
         finally:
             nd.nd_ctx_destroy(ctx)
