@@ -463,8 +463,8 @@ static int ensure_tri(nd_graph* g) {
     DBuf sigma, up, tmp;
     int rc = ND_OK;
     int64_t m = g->m;
-    if ((rc = nd_alloc(c, sigma, sizeof(int64_t) * std::max<int64_t>(m, 1))) ||
-        (rc = nd_alloc(c, up, sizeof(int64_t) * std::max<int64_t>(m, 1))) ||
+    if ((rc = nd_alloc(c, sigma, sizeof(int32_t) * std::max<int64_t>(m, 1))) ||
+        (rc = nd_alloc(c, up, sizeof(int32_t) * std::max<int64_t>(m, 1))) ||
         (rc = nd_alloc(c, tmp, nd_scan_tmp_bytes(m))) || (rc = nd_alloc(c, g->et_rp, sizeof(int64_t) * (m + 1))) ||
         (rc = nd_alloc(c, g->tbase, sizeof(int64_t) * (m + 1)))) {
         nd_free(c, sigma);
@@ -473,9 +473,11 @@ static int ensure_tri(nd_graph* g) {
         return rc;
     }
     GraphView v = nd_view(g);
-    nd_edge_support(v, (int64_t*)sigma.p, (int64_t*)up.p, st);
-    nd_scan_i64((const int64_t*)sigma.p, (int64_t*)g->et_rp.p, m, tmp.p, st);
-    nd_scan_i64((const int64_t*)up.p, (int64_t*)g->tbase.p, m, tmp.p, st);
+    cudaMemsetAsync(sigma.p, 0, sigma.bytes, st);
+    cudaMemsetAsync(up.p, 0, up.bytes, st);  // a failure surfaces at the launch check below
+    nd_edge_support(v, (int32_t*)sigma.p, (int32_t*)up.p, st);
+    nd_scan_i32((const int32_t*)sigma.p, (int64_t*)g->et_rp.p, m, tmp.p, st);
+    nd_scan_i32((const int32_t*)up.p, (int64_t*)g->tbase.p, m, tmp.p, st);
     int64_t tot[2] = {0, 0};
     rc = nd_check_launch("triangle index");
     if (!rc) rc = read_back(g, (int64_t*)g->et_rp.p + m, &tot[0], "triangle index");
@@ -494,12 +496,18 @@ static int ensure_tri(nd_graph* g) {
         (rc = nd_alloc(c, g->tri_pos, sizeof(int32_t) * std::max<int64_t>(3 * n3, 1))))
         return rc;
     g->n3 = n3;
+    ND_TRY(scalar_zero(g));
     v = nd_view(g);
     nd_edge_fill(v, (int64_t*)g->et_rp.p, (int64_t*)g->tbase.p, (int32_t*)g->et_w.p, (int32_t*)g->et_t.p,
-                 (int32_t*)g->tri_e.p, (int32_t*)g->tri_pos.p, st);
+                 (int32_t*)g->tri_e.p, (int32_t*)g->tri_pos.p, (int*)g->scal.p, st);
     v = nd_view(g);
     nd_edge_fill_tid(v, (int32_t*)g->et_t.p, (int32_t*)g->tri_pos.p, st);
+    int err = 0;
     ND_TRY(nd_check_launch("triangle index"));
+    ND_TRY(read_back(g, g->scal.p, &err, "triangle index"));
+    if (err)
+        return nd_set_error(ND_EINVAL, "the CSR is not a simple graph in ascending rows; load it with ND_VALIDATE for "
+                                       "details");
     g->have_tri = true;
     return ND_OK;
 }
@@ -700,26 +708,17 @@ static int build_tri_hash(nd_graph* g, DBuf& hoff, DBuf& htab, DBuf& hpos) {
     return nd_check_launch("triangle hash");
 }
 
-// Incidence lists of the s-cliques, read by the peel (nd_inc.cu).
-struct IncBufs {
-    DBuf off, list, row, dead, status;
-    int32_t stride = 0;
-    int64_t n_s = 0;
-};
-
-static void free_inc(nd_ctx* c, IncBufs& b) {
-    for (DBuf* x : {&b.off, &b.list, &b.row, &b.dead, &b.status}) nd_free(c, *x);
-}
-
 // Which decompositions are peeled from incidence lists. (1,2) has them in the CSR itself; a (3,4) run that
 // is asked to contract before every round contracts its triangle lists. The lists are an accelerator and must leave room for others,
-// hence the bound; the (3,4) lists of R-MAT graphs from scale 17 on, for instance, are over it, and
+// hence the bound (nd_ctx::inc_bytes); the (3,4) lists of R-MAT graphs from scale 17 on, for instance, are over it, and
 // their s-cliques are listed again by Update.
-constexpr int64_t kIncBytes = (int64_t)16 << 30;
-
-static bool wants_inc(int r, int s, int flags, int64_t n_s) {
+static bool wants_inc(const nd_ctx* c, int r, int s, int flags, int64_t n_s) {
     if ((r == 1 && s == 2) || (r == 3 && s == 4 && (flags & ND_CONTRACT_ALWAYS))) return false;
-    return n_s < INT32_MAX && n_s <= kIncBytes / (4 * (nd_inc_stride(r, s) + binom64(s, r)));
+    return n_s < INT32_MAX && n_s <= c->inc_bytes / (4 * (nd_inc_stride(r, s) + binom64(s, r)));
+}
+
+void nd_free_inc(nd_ctx* c, IncBufs& b) {
+    for (DBuf* x : {&b.off, &b.list, &b.row, &b.dead, &b.status}) nd_free(c, *x);
 }
 
 static int build_inc(nd_graph* g, int r, int s, const DBuf& cnt, int w, int64_t n_r, int64_t n_s, IncBufs& b) {
@@ -738,7 +737,7 @@ static int build_inc(nd_graph* g, int r, int s, const DBuf& cnt, int w, int64_t 
         (rc = nd_alloc(c, b.dead, 4 * (F.rows / 32 + 1))) || (rc = nd_alloc(c, b.status, 16))) {
         nd_free(c, cursor);
         nd_free(c, tmp);
-        free_inc(c, b);
+        nd_free_inc(c, b);
         return rc;
     }
     if (w == 8)
@@ -757,7 +756,42 @@ static int build_inc(nd_graph* g, int r, int s, const DBuf& cnt, int w, int64_t 
     rc = nd_check_launch("incidence lists");
     nd_free(c, cursor);
     nd_free(c, tmp);
-    if (rc) free_inc(c, b);
+    if (rc) nd_free_inc(c, b);
+    return rc;
+}
+
+// Counts the s-cliques of a prepared graph and builds their lists, for callers that read them without
+// peeling; *built stays false where nd_decompose would do without lists.
+int nd_build_inc(nd_graph* g, int r, int s, int64_t n_r, IncBufs& b, bool* built) {
+    nd_ctx* c = g->ctx;
+    *built = false;
+    if (r == 1 && s == 2) return ND_OK;
+    DBuf cnt;
+    int w = 0;
+    unsigned long long tot = 0;
+    unsigned int status[3] = {0, 0, 0};
+    int rc = nd_pick_width(g, r, s, 0, &w);
+    if (!rc && r == 3 && s == 4) {
+        rc = build_tri_hash(g, g->hoff, g->htab, g->hpos);
+        if (rc == ND_ENOMEM) {
+            for (DBuf* x : {&g->hoff, &g->htab, &g->hpos}) nd_free(c, *x);
+            rc = ND_OK;
+        }
+    }
+    if (!rc) rc = nd_count_into(g, r, s, w, n_r, cnt);
+    if (!rc) rc = sum_counts(g, cnt, w, n_r, &tot);
+    const int64_t n_s = (int64_t)(tot / (unsigned long long)binom64(s, r));
+    if (!rc && wants_inc(c, r, s, 0, n_s)) {
+        rc = build_inc(g, r, s, cnt, w, n_r, n_s, b);
+        if (!rc) rc = read_back(g, b.status.p, &status, "incidence lists");
+        if (!rc && (status[2] || status[1] != n_s))
+            rc = nd_set_error(ND_EINTERNAL, "incidence lists: %u of %lld s-cliques", status[1], (long long)n_s);
+        if (!rc) *built = true;
+    }
+    if (rc == ND_ENOMEM) rc = ND_OK;  // the lists are an accelerator
+    if (!*built) nd_free_inc(c, b);
+    nd_free(c, cnt);
+    for (DBuf* x : {&g->hoff, &g->htab, &g->hpos}) nd_free(c, *x);
     return rc;
 }
 
@@ -1119,7 +1153,7 @@ int nd_decompose_dev(nd_graph* g, int r, int s, int count_width, int flags, Peel
     cudaEventRecord(e3, c->stream);
     const int64_t n_s = (int64_t)(tot / (unsigned long long)binom64(s, r));
     IncBufs inc;
-    bool use_inc = !rc && wants_inc(r, s, flags, n_s);
+    bool use_inc = !rc && wants_inc(c, r, s, flags, n_s);
     if (use_inc) {
         rc = build_inc(g, r, s, cnt, w, n_r, n_s, inc);
         if (rc == ND_ENOMEM) {
@@ -1132,7 +1166,7 @@ int nd_decompose_dev(nd_graph* g, int r, int s, int count_width, int flags, Peel
     if (!rc)
         rc = (w == 8) ? run_peel<int64_t>(g, r, s, cnt, n_r, flags, po, use_inc ? &inc : nullptr)
                       : run_peel<int32_t>(g, r, s, cnt, n_r, flags, po, use_inc ? &inc : nullptr);
-    free_inc(c, inc);
+    nd_free_inc(c, inc);
     cudaEventRecord(e2, c->stream);
     if (!rc) rc = nd_sync(c, "nd_decompose");
     float tc = 0, tp = 0, th = 0;

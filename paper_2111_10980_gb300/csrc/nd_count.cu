@@ -53,7 +53,7 @@ struct CountTri {
         own[slot] = 0;
         __syncwarp();
     }
-    __device__ void tri(bool hit, int slot, int32_t, int32_t px, int32_t py, int32_t, int32_t, int32_t w) const {
+    __device__ void tri(bool hit, int slot, int32_t, int32_t px, int32_t py, bool, int32_t, int32_t, int32_t w) const {
         if (!hit) return;
         atomicAdd(&own[slot], 1u);
         if (R_ == 1) {

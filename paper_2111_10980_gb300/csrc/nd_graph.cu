@@ -14,6 +14,7 @@
 //     it), together with the triangle's canonical id; a triangle (a<b<c) gets id
 //     tbase[e(a,b)] + rank of c among the entries of L(a,b) greater than b.
 #include "nd_common.cuh"
+#include "nd_tri.cuh"
 
 namespace {
 
@@ -143,106 +144,125 @@ __global__ void k_dg_fill(GraphView g, const int32_t* __restrict__ key_hi, const
     }
 }
 
-// sigma[e] = |N(a) ∩ N(b)|, up[e] = |{w in N(a) ∩ N(b) : w > b}| for canonical edge e = (a,b)
-__global__ void k_edge_support(GraphView g, int64_t* __restrict__ sigma, int64_t* __restrict__ up) {
-    int lane = threadIdx.x & 31;
-    for (int64_t e = gwarp(); e < g.m; e += nwarps()) {
-        int32_t a = g.eu[e], b = g.ev[e];
-        int64_t ab = g.rp[a], ae = g.rp[a + 1], bb = g.rp[b], be = g.rp[b + 1];
-        const int32_t *xs = g.col + ab, *ys = g.col + bb;
-        int64_t nx = ae - ab, ny = be - bb;
-        if (nx > ny) {
-            const int32_t* t = xs;
-            xs = ys;
-            ys = t;
-            int64_t tn = nx;
-            nx = ny;
-            ny = tn;
-        }
-        int c = 0, cu = 0;
-        if (nd_prefer_merge(nx, ny)) {
-            const int ix = (int)nx, iy = (int)ny;
-            nd_merge_walk(xs, ix, ys, iy, nd_merge_run(xs, ix, ys, iy), [&](int, int, int32_t w) {
-                c++;
-                cu += w > b ? 1 : 0;
-            });
-        } else {
-            for (int64_t i = lane; i < nx; i += 32) {
-                int32_t w = xs[i];
-                if (nd_find(ys, ny, w) >= 0) {
-                    c++;
-                    cu += (w > b) ? 1 : 0;
-                }
-            }
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            c += __shfl_down_sync(0xffffffffu, c, o);
-            cu += __shfl_down_sync(0xffffffffu, cu, o);
-        }
-        if (lane == 0) {
-            sigma[e] = c;
-            up[e] = cu;
-        }
+// sigma[e] = |N(a) ∩ N(b)|, up[e] = |{w in N(a) ∩ N(b) : w > b}| for canonical edge e = (a,b): each triangle,
+// met once over DG, adds 1 to sigma of its edges and to up of the one without its largest vertex.
+// The numbers of u -> v itself are kept in shared memory and added once.
+struct SupportSink {
+    int32_t* sigma;
+    int32_t* up;
+    const int32_t* eid;
+    unsigned* own;  // per slot: triangles, then those with u -> v lowest
+    __device__ void begin(int slot) const {
+        own[slot] = 0;
+        own[slot + 32] = 0;
+        __syncwarp();
     }
+    __device__ void tri(bool hit, int slot, int32_t, int32_t px, int32_t py, bool of_u, int32_t u, int32_t v,
+                        int32_t w) const {
+        if (!hit) return;
+        const int32_t ex = eid[px], ey = eid[py];
+        atomicAdd(&own[slot], 1u);
+        atomicAdd(&sigma[ex], 1);
+        atomicAdd(&sigma[ey], 1);
+        if (w > u && w > v)
+            atomicAdd(&own[slot + 32], 1u);
+        else
+            atomicAdd(&up[(u > v) == of_u ? ey : ex], 1);  // the edge without the larger of u and v
+    }
+    __device__ void end(int slot, int32_t e, int32_t, int32_t) const {
+        if (own[slot]) atomicAdd(&sigma[e], (int)own[slot]);
+        if (own[slot + 32]) atomicAdd(&up[e], (int)own[slot + 32]);
+    }
+};
+
+__global__ void __launch_bounds__(kTriThreads) k_edge_support(GraphView g, int32_t* __restrict__ sigma,
+                                                              int32_t* __restrict__ up) {
+    __shared__ unsigned s_own[2 * kTriThreads];
+    SupportSink sink{sigma, up, g.dg_eid, s_own + 2 * (threadIdx.x & ~31u)};
+    tri_list(g, sink);
 }
 
 // Writes L(a,b) in ascending w with, per entry: the canonical triangle id when w > b, else
-// (temporarily) the id of edge (a,w); and the edges of every triangle whose lowest edge is e.
+// (temporarily) the id of edge (a,w); and the edges of every triangle whose lowest edge is e. Edges
+// without triangles, most of them in a sparse graph, cost a lane a look and not a warp an intersection
+// (Chung-Lu, a million vertices, 15 M edges: the index 28 -> 18 ms, 13 of them here). The rows of a CSR with duplicates do not give what DG
+// gave for sigma: nothing is written outside the edge's list then, and *err is set.
 __global__ void k_edge_fill(GraphView g, const int64_t* __restrict__ et_rp, const int64_t* __restrict__ tbase,
                             int32_t* __restrict__ et_w, int32_t* __restrict__ et_t, int32_t* __restrict__ tri_e,
-                            int32_t* __restrict__ tri_pos) {
-    int lane = threadIdx.x & 31;
-    for (int64_t e = gwarp(); e < g.m; e += nwarps()) {
-        int32_t a = g.eu[e], b = g.ev[e];
-        int64_t ab = g.rp[a], ae = g.rp[a + 1], bb = g.rp[b], be = g.rp[b + 1];
-        bool a_drives = (ae - ab) <= (be - bb);
-        int64_t xb = a_drives ? ab : bb, xe = a_drives ? ae : be;
-        int64_t yb = a_drives ? bb : ab, ye = a_drives ? be : ae;
-        int64_t out = et_rp[e];
-        int64_t sig = et_rp[e + 1] - out;
-        int64_t split_e = sig - (tbase[e + 1] - tbase[e]);
-        // writes common element w, found at driver position p and other-list position q, as entry
-        // `local` of L(a,b)
-        auto put = [&](int64_t local, int64_t p, int64_t q, int32_t w) {
-            int64_t pa = a_drives ? p : q;  // position of w in N(a)
-            int64_t pb = a_drives ? q : p;  // position of w in N(b)
-            int32_t e_aw = g.pos2e[pa], e_bw = g.pos2e[pb];
-            et_w[out + local] = w;
-            if (w > b) {
-                int64_t tid = tbase[e] + (local - split_e);
-                et_t[out + local] = (int32_t)tid;
-                tri_e[3 * tid + 0] = (int32_t)e;
-                tri_e[3 * tid + 1] = e_aw;
-                tri_e[3 * tid + 2] = e_bw;
-                tri_pos[3 * tid + 0] = (int32_t)local;
+                            int32_t* __restrict__ tri_pos, int* err) {
+    const int lane = threadIdx.x & 31;
+    const unsigned full = 0xffffffffu;
+    for (int64_t e0 = gwarp() * 32; e0 < g.m; e0 += nwarps() * 32) {
+        // each lane looks one edge over and sets it up; those with triangles are then taken one after another
+        const int64_t el = e0 + lane;
+        int32_t la = 0, lb = 0;
+        int64_t lab = 0, lae = 0, lbb = 0, lbe = 0, lout = 0, lsig = 0, ltb = 0, lup = 0;
+        if (el < g.m) {
+            lout = et_rp[el];
+            lsig = et_rp[el + 1] - lout;
+            if (lsig) {
+                la = g.eu[el], lb = g.ev[el];
+                lab = g.rp[la], lae = g.rp[la + 1], lbb = g.rp[lb], lbe = g.rp[lb + 1];
+                ltb = tbase[el], lup = tbase[el + 1] - ltb;
+            }
+        }
+        for (unsigned todo = __ballot_sync(full, lsig != 0); todo; todo &= todo - 1) {
+            const int src = __ffs(todo) - 1;
+            const int64_t e = e0 + src;
+            const int32_t b = __shfl_sync(full, lb, src);
+            const int64_t ab = __shfl_sync(full, lab, src), ae = __shfl_sync(full, lae, src);
+            const int64_t bb = __shfl_sync(full, lbb, src), be = __shfl_sync(full, lbe, src);
+            const int64_t out = __shfl_sync(full, lout, src), sig = __shfl_sync(full, lsig, src);
+            const int64_t tb = __shfl_sync(full, ltb, src), split_e = sig - __shfl_sync(full, lup, src);
+            const bool a_drives = (ae - ab) <= (be - bb);
+            const int64_t xb = a_drives ? ab : bb, xe = a_drives ? ae : be;
+            const int64_t yb = a_drives ? bb : ab, ye = a_drives ? be : ae;
+            // writes common element w, found at driver position p and other-list position q, as entry
+            // `local` of L(a,b)
+            auto put = [&](int64_t local, int64_t p, int64_t q, int32_t w) {
+                if (local >= sig || (w > b) != (local >= split_e)) return;  // no simple graph: reported below
+                int64_t pa = a_drives ? p : q;  // position of w in N(a)
+                int64_t pb = a_drives ? q : p;  // position of w in N(b)
+                int32_t e_aw = g.pos2e[pa], e_bw = g.pos2e[pb];
+                et_w[out + local] = w;
+                if (w > b) {
+                    int64_t tid = tb + (local - split_e);
+                    et_t[out + local] = (int32_t)tid;
+                    tri_e[3 * tid + 0] = (int32_t)e;
+                    tri_e[3 * tid + 1] = e_aw;
+                    tri_e[3 * tid + 2] = e_bw;
+                    tri_pos[3 * tid + 0] = (int32_t)local;
+                } else {
+                    et_t[out + local] = e_aw;
+                }
+            };
+            if (nd_prefer_merge(xe - xb, ye - yb)) {
+                // merge path: count this lane's matches, place them after the lower lanes' (exclusive
+                // scan), then walk the run again and write them
+                const int32_t *X = g.col + xb, *Y = g.col + yb;
+                const int nx = (int)(xe - xb), ny = (int)(ye - yb);
+                const NdMergeRun run = nd_merge_run(X, nx, Y, ny);
+                int cnt = 0;
+                nd_merge_walk(X, nx, Y, ny, run, [&](int, int, int32_t) { ++cnt; });
+                int inc = cnt;
+                for (int o = 1; o < 32; o <<= 1) {
+                    int y = __shfl_up_sync(0xffffffffu, inc, o);
+                    if (lane >= o) inc += y;
+                }
+                if (lane == 31 && inc != sig) atomicOr(err, 1);
+                int64_t local = inc - cnt;
+                nd_merge_walk(X, nx, Y, ny, run, [&](int i, int j, int32_t w) { put(local++, xb + i, yb + j, w); });
             } else {
-                et_t[out + local] = e_aw;
-            }
-        };
-        if (nd_prefer_merge(xe - xb, ye - yb)) {
-            // merge path: count this lane's matches, place them after the lower lanes' (exclusive
-            // scan), then walk the run again and write them
-            const int32_t *X = g.col + xb, *Y = g.col + yb;
-            const int nx = (int)(xe - xb), ny = (int)(ye - yb);
-            const NdMergeRun run = nd_merge_run(X, nx, Y, ny);
-            int cnt = 0;
-            nd_merge_walk(X, nx, Y, ny, run, [&](int, int, int32_t) { ++cnt; });
-            int inc = cnt;
-            for (int o = 1; o < 32; o <<= 1) {
-                int y = __shfl_up_sync(0xffffffffu, inc, o);
-                if (lane >= o) inc += y;
-            }
-            int64_t local = inc - cnt;
-            nd_merge_walk(X, nx, Y, ny, run, [&](int i, int j, int32_t w) { put(local++, xb + i, yb + j, w); });
-        } else {
-            int64_t pos = 0;
-            for (int64_t p0 = xb; p0 < xe; p0 += 32) {
-                int64_t p = p0 + lane;
-                int64_t q = -1;
-                if (p < xe) q = nd_find(g.col + yb, ye - yb, g.col[p]);
-                unsigned m = __ballot_sync(0xffffffffu, q >= 0);
-                if (q >= 0) put(pos + __popc(m & nd_lanemask_lt()), p, yb + q, g.col[p]);
-                pos += __popc(m);
+                int64_t pos = 0;
+                for (int64_t p0 = xb; p0 < xe; p0 += 32) {
+                    int64_t p = p0 + lane;
+                    int64_t q = -1;
+                    if (p < xe) q = nd_find(g.col + yb, ye - yb, g.col[p]);
+                    unsigned m = __ballot_sync(0xffffffffu, q >= 0);
+                    if (q >= 0) put(pos + __popc(m & nd_lanemask_lt()), p, yb + q, g.col[p]);
+                    pos += __popc(m);
+                }
+                if (lane == 0 && pos != sig) atomicOr(err, 1);
             }
         }
     }
@@ -251,20 +271,45 @@ __global__ void k_edge_fill(GraphView g, const int64_t* __restrict__ et_rp, cons
 // For entries of L(a,b) with w < b, the triangle {a,w,b} has b as its largest vertex, so its
 // lowest edge is (a,w) (or (w,a)); its id is tbase[e'] + rank of b among the upper entries of L(e').
 // The entry is the triangle's (a,c) entry when a < w, its (b,c) entry when w < a (slots 1, 2).
+// A warp takes the lower entries of 32 edges together, 32 at a time.
 __global__ void k_edge_fill_tid(GraphView g, int32_t* __restrict__ et_t, int32_t* __restrict__ tri_pos) {
-    int lane = threadIdx.x & 31;
-    for (int64_t e = gwarp(); e < g.m; e += nwarps()) {
-        int32_t a = g.eu[e], b = g.ev[e];
-        int64_t lo = g.et_rp[e], hi = g.et_rp[e + 1];
-        int64_t split_e = (hi - lo) - (g.tbase[e + 1] - g.tbase[e]);
-        for (int64_t j = lo + lane; j < lo + split_e; j += 32) {
-            int32_t e2 = et_t[j];
-            int64_t l2 = g.et_rp[e2], h2 = g.et_rp[e2 + 1];
-            int64_t s2 = (h2 - l2) - (g.tbase[e2 + 1] - g.tbase[e2]);
-            int64_t at = nd_lower_bound(g.et_w + l2, h2 - l2, b);
-            int64_t tid = g.tbase[e2] + (at - s2);
+    const int lane = threadIdx.x & 31;
+    const unsigned full = 0xffffffffu;
+    for (int64_t e0 = gwarp() * 32; e0 < g.m; e0 += nwarps() * 32) {
+        const int64_t e = e0 + lane;
+        int64_t lo = 0, low = 0;
+        int32_t a = 0, b = 0;
+        if (e < g.m) {
+            lo = g.et_rp[e];
+            low = g.et_rp[e + 1] - lo - (g.tbase[e + 1] - g.tbase[e]);
+            if (low) {
+                a = g.eu[e];
+                b = g.ev[e];
+            }
+        }
+        int64_t inc = low;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t y = __shfl_up_sync(full, inc, o);
+            if (lane >= o) inc += y;
+        }
+        const int64_t total = __shfl_sync(full, inc, 31), before = inc - low;
+        for (int64_t p0 = 0; p0 < total; p0 += 32) {
+            const int64_t p = p0 + lane;
+            int own = 0;  // the last lane with before <= p: the one whose entry it is
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (__shfl_sync(full, before, own + o) <= p) own += o;
+            const int64_t k = p - __shfl_sync(full, before, own), j = __shfl_sync(full, lo, own) + k;
+            const int32_t oa = __shfl_sync(full, a, own), ob = __shfl_sync(full, b, own);
+            if (p >= total) continue;
+            const int32_t e2 = et_t[j], w = g.et_w[j];
+            if ((uint32_t)e2 >= (uint64_t)g.m) continue;  // not filled (see k_edge_fill's err)
+            const int64_t l2 = g.et_rp[e2], h2 = g.et_rp[e2 + 1], t2 = g.tbase[e2];
+            const int64_t s2 = (h2 - l2) - (g.tbase[e2 + 1] - t2);
+            const int64_t at = nd_lower_bound(g.et_w + l2 + s2, h2 - l2 - s2, ob), tid = t2 + at;
+            if (at >= h2 - l2 - s2) continue;
             et_t[j] = (int32_t)tid;
-            tri_pos[3 * tid + (g.et_w[j] > a ? 1 : 2)] = (int32_t)(j - lo);
+            tri_pos[3 * tid + (w > oa ? 1 : 2)] = (int32_t)k;
         }
     }
 }
@@ -510,20 +555,20 @@ void nd_dg_fill(const GraphView& g, const int32_t* key_hi, int64_t* dg_rp, int32
     ND_K(k_dg_fill<<<blocks_for_warps(g.n), kThreads, 0, st>>>(g, key_hi, dg_rp, dg_col, dg_eid));
 }
 
-void nd_edge_support(const GraphView& g, int64_t* sigma, int64_t* up, cudaStream_t st) {
+void nd_edge_support(const GraphView& g, int32_t* sigma, int32_t* up, cudaStream_t st) {
     if (g.m <= 0) return;
-    ND_K(k_edge_support<<<blocks_for_warps(g.m), kThreads, 0, st>>>(g, sigma, up));
+    ND_K(k_edge_support<<<blocks_for_warps((g.m + 31) / 32), kTriThreads, 0, st>>>(g, sigma, up));
 }
 
 void nd_edge_fill(const GraphView& g, int64_t* et_rp, int64_t* tbase, int32_t* et_w, int32_t* et_t, int32_t* tri_e,
-                  int32_t* tri_pos, cudaStream_t st) {
+                  int32_t* tri_pos, int* err, cudaStream_t st) {
     if (g.m <= 0) return;
-    ND_K(k_edge_fill<<<blocks_for_warps(g.m), kThreads, 0, st>>>(g, et_rp, tbase, et_w, et_t, tri_e, tri_pos));
+    ND_K(k_edge_fill<<<blocks_for_warps((g.m + 31) / 32), kThreads, 0, st>>>(g, et_rp, tbase, et_w, et_t, tri_e, tri_pos, err));
 }
 
 void nd_edge_fill_tid(const GraphView& g, int32_t* et_t, int32_t* tri_pos, cudaStream_t st) {
     if (g.m <= 0) return;
-    ND_K(k_edge_fill_tid<<<blocks_for_warps(g.m), kThreads, 0, st>>>(g, et_t, tri_pos));
+    ND_K(k_edge_fill_tid<<<blocks_for_warps((g.m + 31) / 32), kThreads, 0, st>>>(g, et_t, tri_pos));
 }
 
 

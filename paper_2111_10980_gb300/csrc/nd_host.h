@@ -32,6 +32,7 @@ struct nd_ctx {
     int64_t barrier_ns = 0;
     int64_t count_limit = 0;
     int32_t limit_flags = 0;
+    int64_t inc_bytes = (int64_t)16 << 30;  // most device bytes of a decomposition's incidence lists
     void* stage = nullptr;  // pinned staging of batches (grown on demand)
     size_t stage_bytes = 0;
     // nd_ctx_set_tuning, indexed by r * 8 + s
@@ -78,6 +79,13 @@ struct PeelOut {
     std::vector<int64_t> sizes, levels, round_ns;
 };
 
+// Incidence lists of the s-cliques (nd_inc.cu).
+struct IncBufs {
+    DBuf off, list, row, dead, status;
+    int32_t stride = 0;
+    int64_t n_s = 0;
+};
+
 int nd_set_error(int code, const char* fmt, ...);
 int nd_alloc(nd_ctx* ctx, DBuf& b, size_t bytes);
 void nd_free(nd_ctx* ctx, DBuf& b);
@@ -87,4 +95,6 @@ GraphView nd_view(const nd_graph* g);
 int nd_prepare(nd_graph* g, int r, int s, int64_t* n_r, double* t_orient, double* t_index);
 int nd_pick_width(const nd_graph* g, int r, int s, int count_width, int* w);
 int nd_count_into(nd_graph* g, int r, int s, int w, int64_t n_r, DBuf& cnt);
+void nd_free_inc(nd_ctx* c, IncBufs& b);
+int nd_build_inc(nd_graph* g, int r, int s, int64_t n_r, IncBufs& b, bool* built);
 int nd_decompose_dev(nd_graph* g, int r, int s, int count_width, int flags, PeelOut& po, nd_stats* st);

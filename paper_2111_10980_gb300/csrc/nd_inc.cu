@@ -106,7 +106,7 @@ struct PutTri {
     const int32_t* eid;
     IncRun run;
     __device__ void begin(int) const {}
-    __device__ void tri(bool hit, int, int32_t e, int32_t px, int32_t py, int32_t u, int32_t v, int32_t w) {
+    __device__ void tri(bool hit, int, int32_t e, int32_t px, int32_t py, bool, int32_t u, int32_t v, int32_t w) {
         int32_t id[3] = {u, v, w};
         if (R_ == 2 && hit) {
             id[0] = e;

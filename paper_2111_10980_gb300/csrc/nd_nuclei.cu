@@ -4,8 +4,8 @@
 // in X_c; the connected nuclei at level c are the components of that relation. Components at a
 // higher level nest inside those of a lower one, so the levels together form the nucleus hierarchy.
 //
-// One warp per r-clique R of X_c lists the s-cliques containing R (the generic listing of
-// nd_gen.cuh); an s-clique whose r-subsets all lie in X_c is handled by its owner, the smallest id
+// One warp per r-clique R of X_c reads the s-cliques containing R from their incidence lists (nd_inc.cu),
+// or, without memory for those, lists them with nd_gen.cuh; an s-clique whose r-subsets all lie in X_c is handled by its owner, the smallest id
 // among them, which unites the others with itself in a union-find over r-clique ids. Unions hook
 // the larger root under the smaller with a compare-and-swap, so every link points to a smaller id,
 // roots end as the smallest id of their component, and finds halve paths without conflicting with
@@ -103,6 +103,51 @@ __global__ void k_nuclei_union(GraphView g, const int32_t* __restrict__ core, in
                 for (int i = 0; i < M; ++i) uf_union(parent, (int32_t)id, o[i], err);
             });
     }
+}
+
+// The same from the incidence lists: R's s-cliques and their members are read, not listed and looked up
+// ((2,3) hierarchy of R-MAT scale 16, 16 M triangles, 83 levels: 22.9 -> 7.4 ms, and 2.8 ms for counting and the lists).
+template <bool kBucket>
+__global__ void k_nuclei_union_inc(const int64_t* __restrict__ off, const uint32_t* __restrict__ list,
+                                   const int32_t* __restrict__ row, int stride, const int32_t* __restrict__ core,
+                                   int32_t level, const int32_t* __restrict__ ids, int64_t count, int32_t* parent,
+                                   int* err) {
+    const int lane = threadIdx.x & 31, nv = stride >> 2;
+    for (int64_t k = gwarp(); k < count; k += nwarps()) {
+        const int32_t id = kBucket ? ids[k] : (int32_t)k;
+        if (!kBucket && core[id] < level) continue;
+        const int64_t b = off[id], e = off[id + 1];
+        for (int64_t j = b + lane; j < e; j += 32) {
+            const int4* v = reinterpret_cast<const int4*>(row + (int64_t)list[j] * stride);
+            bool own = true;
+            for (int i = 0; i < nv && own; ++i) {
+                const int4 w = v[i];
+                const int32_t x[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    if (x[m] < 0) continue;
+                    const int32_t co = core[x[m]];
+                    own = own && co >= level && (x[m] >= id || (kBucket && co != level));
+                }
+            }
+            if (!own) continue;
+            for (int i = 0; i < nv; ++i) {
+                const int4 w = v[i];
+                const int32_t x[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                for (int m = 0; m < 4; ++m)
+                    if (x[m] >= 0 && x[m] != id) uf_union(parent, id, x[m], err);
+            }
+        }
+    }
+}
+
+template <bool kBucket>
+void launch_union_inc(const IncBufs& inc, const int32_t* core, int32_t level, const int32_t* ids, int64_t count,
+                      int32_t* parent, int* err, cudaStream_t st) {
+    ND_K(k_nuclei_union_inc<kBucket><<<blocks_for_warps(count), kThreads, 0, st>>>(
+        (const int64_t*)inc.off.p, (const uint32_t*)inc.list.p, (const int32_t*)inc.row.p, inc.stride, core, level, ids,
+        count, parent, err));
 }
 
 __global__ void k_nuclei_label(const int32_t* __restrict__ core, int32_t level, int64_t n_r, int32_t* parent,
@@ -282,7 +327,12 @@ extern "C" int nd_nuclei(nd_graph* g, int r, int s, const int32_t* core, int32_t
     cudaMemsetAsync(scal.p, 0, 64, st);
     nd_iota_i32((int32_t*)parent.p, n_r, st);
     GraphView v = nd_view(g);
-    if (n_r && !dispatch_union(r, s, false, v, cd, level, nullptr, n_r, (int32_t*)parent.p, (int*)scal.p, st))
+    IncBufs inc;
+    bool lists = false;
+    if (n_r) rc = nd_build_inc(g, r, s, n_r, inc, &lists);
+    if (!rc && lists)
+        launch_union_inc<false>(inc, cd, level, nullptr, n_r, (int32_t*)parent.p, (int*)scal.p, st);
+    else if (!rc && n_r && !dispatch_union(r, s, false, v, cd, level, nullptr, n_r, (int32_t*)parent.p, (int*)scal.p, st))
         rc = nd_set_error(ND_EINVAL, "nd_nuclei: (r,s) = (%d,%d) is not supported", r, s);
     if (!rc && n_r) {
         int64_t want = (n_r + 255) / 256, cap = (int64_t)nd_sm_count() * 8;
@@ -309,6 +359,7 @@ extern "C" int nd_nuclei(nd_graph* g, int r, int s, const int32_t* core, int32_t
         if (!rc) rc = nd_sync(c, "nd_nuclei");
     }
     if (!rc && n_comp_out) *n_comp_out = (int64_t)h.n;
+    nd_free_inc(c, inc);
     for (DBuf* b : {&dcore, &parent, &comp, &scal}) nd_free(c, *b);
     return rc;
 }
@@ -332,8 +383,11 @@ extern "C" int nd_hierarchy(nd_graph* g, int r, int s, const int32_t* core, int3
     enum { kCore, kParent, kComp, kRepTmp, kNodeRep, kNodeAt, kNodeRepAt, kParentRep, kOrder, kPR0, kPP0, kPR1, kPP1,
            kOutC, kOutL, kOutP, kScal, kHist, kN };
     DBuf b[kN];
+    IncBufs inc;
+    bool lists = false;
     auto release = [&]() {
         for (DBuf& x : b) nd_free(c, x);
+        nd_free_inc(c, inc);
     };
     for (int i = 0; i < kScal && !rc; ++i) {
         if ((i == kCore || i >= kOutC) && dev) continue;  // caller's device arrays are used directly
@@ -370,6 +424,10 @@ extern "C" int nd_hierarchy(nd_graph* g, int r, int s, const int32_t* core, int3
     if (lo_hi[0] < 0 || lo_hi[1] >= (1 << 26)) {
         release();
         return nd_set_error(ND_EINVAL, "nd_hierarchy: core numbers must lie in [0, 2^26) (got %d .. %d)", lo_hi[0], lo_hi[1]);
+    }
+    if ((rc = nd_build_inc(g, r, s, n_r, inc, &lists))) {
+        release();
+        return rc;
     }
     const int64_t nb = (int64_t)lo_hi[1] + 1;
     if ((rc = nd_alloc(c, b[kHist], 4 * nb))) {
@@ -408,7 +466,9 @@ extern "C" int nd_hierarchy(nd_graph* g, int r, int s, const int32_t* core, int3
         const int nxt = cur ^ 1;
         int32_t* nroot = I32(nxt ? kPR1 : kPR0);
         int32_t* nrep = I32(nxt ? kPP1 : kPP0);
-        if (!dispatch_union(r, s, true, v, cd, (int32_t)lv, ids, cnt, I32(kParent), sc, st)) {
+        if (lists)
+            launch_union_inc<true>(inc, cd, (int32_t)lv, ids, cnt, I32(kParent), sc, st);
+        else if (!dispatch_union(r, s, true, v, cd, (int32_t)lv, ids, cnt, I32(kParent), sc, st)) {
             rc = nd_set_error(ND_EINVAL, "nd_hierarchy: (r,s) = (%d,%d) is not supported", r, s);
             break;
         }

@@ -424,6 +424,13 @@ static void worker_loop(nd_server* sv, int w) {
                     ++it;
                 }
             }
+            // incidence lists, whose size is known only after counting, may take a part of what the
+            // budget leaves; it counts as used while the batch runs
+            if (sv->cfg.mem_budget) {
+                const size_t held = sv->used + est, spare = held < sv->cfg.mem_budget ? sv->cfg.mem_budget - held : 0;
+                ctx->inc_bytes = (int64_t)std::min<size_t>(spare / (2 * (size_t)sv->cfg.workers), (size_t)16 << 30);
+                est += (size_t)ctx->inc_bytes;
+            }
             sv->used += est;
             sv->running++;
         }

@@ -11,7 +11,7 @@ constexpr int kTriThreads = 256;
 // takes 32 at a time, whatever edges they belong to, so that the many edges with two or three
 // candidates fill its lanes as well as the few with thousands. The whole warp calls sink.tri() with each
 // lane's candidate: whether it is a triangle, the slot of u -> v among the 32 edges, its edge, the DG
-// positions of the other two edges and the vertices. sink.end() is called once per edge by the lane
+// positions of the other two edges (the first is u's if of_u), and the vertices. sink.end() is called once per edge by the lane
 // that set it up.
 //
 // Bound by the bisections' loads (L1 and L2) and, past them, by the sinks' atomics. Against one warp per edge
@@ -25,6 +25,7 @@ __device__ __forceinline__ void tri_list(const GraphView& g, Sink& sink) {
     for (int64_t j0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; j0 < g.m; j0 += nwarps * 32) {
         const int64_t j = j0 + lane;
         int32_t u = 0, v = 0, e = 0, xb = 0, xn = 0, yb = 0, yn = 0;  // DG positions are below m < 2^31
+        int32_t of_u = 0;
         if (j < g.m) {
             e = g.dg_eid[j];
             v = g.dg_col[j];
@@ -33,6 +34,7 @@ __device__ __forceinline__ void tri_list(const GraphView& g, Sink& sink) {
             const int32_t ub = (int32_t)g.dg_rp[u], un = (int32_t)g.dg_rp[u + 1] - ub;
             const int32_t vb = (int32_t)g.dg_rp[v], vn = (int32_t)g.dg_rp[v + 1] - vb;
             const bool u_drives = un <= vn;
+            of_u = u_drives;
             xb = u_drives ? ub : vb, xn = u_drives ? un : vn;
             yb = u_drives ? vb : ub, yn = u_drives ? vn : un;
         }
@@ -53,7 +55,7 @@ __device__ __forceinline__ void tri_list(const GraphView& g, Sink& sink) {
                 if (b <= p) own += o;
             }
             const int32_t oxb = __shfl_sync(full, xb, own), oyb = __shfl_sync(full, yb, own);
-            const int32_t oyn = __shfl_sync(full, yn, own);
+            const int32_t oyn = __shfl_sync(full, yn, own), oof = __shfl_sync(full, of_u, own);
             const int64_t ob = __shfl_sync(full, before, own);
             const int32_t ou = __shfl_sync(full, u, own), ov = __shfl_sync(full, v, own), oe = __shfl_sync(full, e, own);
             const int32_t px = oxb + (int32_t)(p - ob);
@@ -74,7 +76,7 @@ __device__ __forceinline__ void tri_list(const GraphView& g, Sink& sink) {
                 }
                 hit = lo < oyn && __ldg(ys + lo) == w;
             }
-            sink.tri(hit, own, oe, px, oyb + lo, ou, ov, w);
+            sink.tri(hit, own, oe, px, oyb + lo, oof != 0, ou, ov, w);
         }
         __syncwarp();
         if (j < g.m) sink.end(lane, e, u, v);
