@@ -258,10 +258,11 @@ struct GraphView {
 
 // The part of the control block that a round's phases read: written by the serial steps between
 // phases and by the phases' appends, stable while a phase that reads it runs. The persistent kernel
-// copies it into shared memory after every barrier, so a phase starts without a chain of loads from
-// L2 (the copy is sizeof(PeelHot) / 16 loads of 16 bytes by one warp, all in flight at once).
+// keeps a copy in every block's shared memory, so a phase starts without a chain of loads from L2.
+// The first line is the loop state, which only serial steps change (in the persistent kernel every
+// block's copy holds it, the control block only after a full serial step); the second holds the
+// counters of the phases; the third the counter that every scheduled r-clique adds to.
 struct __align__(128) PeelHot {
-    // loop state
     int32_t t;          // current round
     int32_t mode;       // ND_MODE_ADV when this round moves to a new level
     int32_t done;       // 1 once every r-clique is peeled
@@ -273,6 +274,8 @@ struct __align__(128) PeelHot {
     int32_t contract;   // graph contraction before this round's phases (set by the serial control step)
     int32_t stage;      // persistent kernel: 0 start of the round, 3 selection of A, 1 Update, 2 heavy Update
     unsigned int nA;    // |A| of a same-level round
+    int32_t contractions;    // contractions run
+    int32_t advances, refills;
     int64_t k;          // current level
     int64_t hi;         // bucket window: N holds every unpeeled r-clique with count < hi
     int64_t finished;   // r-cliques peeled so far
@@ -280,6 +283,7 @@ struct __align__(128) PeelHot {
     int64_t n_r;
     int64_t max_rounds; // round cap (ND_ETIMEOUT)
     int64_t contract_every;  // contract once this many r-cliques were peeled since the last one (0: never)
+    int64_t state_pad;
     // list sizes, counted up by the phases
     unsigned int cntA;  // |A| written by adv_select
     unsigned int nN;    // |N| (current)
@@ -287,14 +291,17 @@ struct __align__(128) PeelHot {
     unsigned int nL;    // |L|
     unsigned int nL2;   // |L'| being written by refill
     unsigned int nH;    // r-cliques of this round's A deferred to the heavy Update kernel
+    unsigned int upd_next;  // next unassigned position of A in this round's Update (dynamic chunks)
+    unsigned int count_pad;
     unsigned long long minN;  // min count over unpeeled members of N (adv_min)
     unsigned long long gmin;  // min count over unpeeled r-cliques (refill)
-    unsigned int nNext; // next round's A (r-cliques that fell to <= k during this round)
-    unsigned int upd_next;  // next unassigned position of A in this round's Update (dynamic chunks)
-    int64_t contractions;    // contractions run
-    int64_t advances, refills;
+    unsigned int count_pad2[20];
+    // next round's A (r-cliques that fell to <= k during this round), counted in nNext[t & 1]; the
+    // other one is 0 when round t begins
+    unsigned int nNext[2];
+    unsigned int next_pad[30];
 };
-static_assert(sizeof(PeelHot) == 256, "two lines of 128 bytes");
+static_assert(sizeof(PeelHot) == 384, "three lines of 128 bytes");
 
 struct PeelCtl {
     PeelHot h;

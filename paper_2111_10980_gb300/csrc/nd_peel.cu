@@ -185,7 +185,10 @@ __global__ void k_set_refill(PeelCtl* c, cudaGraphConditionalHandle h_refill) {
 // The control step on a copy of the hot state.
 __device__ __forceinline__ void ctl_next(PeelHot& s, int* err, int64_t* round_size, int64_t* round_level,
                                          int64_t round_cap) {
+    unsigned next = 0;
     if (s.started) {
+        next = s.nNext[s.t & 1];
+        s.nNext[s.t & 1] = 0;
         const bool adv = s.mode & ND_MODE_ADV;
         const unsigned nA = adv ? s.cntA : s.nA;
         if (adv) {
@@ -226,10 +229,9 @@ __device__ __forceinline__ void ctl_next(PeelHot& s, int* err, int64_t* round_si
         s.peeled_since = 0;
         s.contractions++;
     }
-    if (s.nNext > 0) {
+    if (next > 0) {
         s.wa ^= 1;
-        s.nA = s.nNext;
-        s.nNext = 0;
+        s.nA = next;
         s.mode = 0;
     } else {
         s.mode = ND_MODE_ADV;
@@ -759,7 +761,7 @@ __device__ __noinline__ void after_dec_rest(const PeelView<CT>* Q, const PeelHot
         Q->core[x] = (int32_t)k;
         if (Q->et_rnd) set_tri_round(*Q, x, t1);
         mark_a(*Q, x);
-        nd_append(&c->h.nNext, s->wa ? Q->A[0] : Q->A[1], Q->cap, x, &c->err);
+        nd_append(&c->h.nNext[s->t & 1], s->wa ? Q->A[0] : Q->A[1], Q->cap, x, &c->err);
     }
     if (o == s->hi) {
         const bool adv = s->mode & ND_MODE_ADV;
@@ -770,6 +772,53 @@ __device__ __noinline__ void after_dec_rest(const PeelView<CT>* Q, const PeelHot
 template <typename CT>
 __device__ __forceinline__ void after_dec(const RoundEnv<CT>& E, int32_t x, int64_t o) {
     if (o == E.k + 1 || o == E.hi || E.P.bcnt) after_dec_rest(E.Q, E.s, x, o, E.k);
+}
+
+// The same for up to four r-cliques of every lane at once (bit i of what: x_i falls to k; bit 4 + i: it
+// falls below the window's bound), with one counter update per list for all of them: four calls of
+// the above are four trips to L2, one after another, in the chain that a short round waits for.
+template <typename CT>
+__device__ __noinline__ void after_dec4(const PeelView<CT>* Q, const PeelHot* s, int4 x4, unsigned what, int64_t k) {
+    PeelCtl* c = Q->ctl;
+    const unsigned act = __activemask(), below = act & nd_lanemask_lt();
+    const int lane = threadIdx.x & 31, leader = __ffs(act) - 1;
+    const bool adv = s->mode & ND_MODE_ADV;
+    unsigned at[2] = {0, 0}, all[2] = {0, 0};
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const unsigned b = __ballot_sync(act, what >> i & 1u);
+        at[i >> 2] += __popc(b & below);
+        all[i >> 2] += __popc(b);
+    }
+    unsigned base0 = 0, base1 = 0;
+    if (lane == leader) {
+        if (all[0]) base0 = atomicAdd(&c->h.nNext[s->t & 1], all[0]);
+        if (all[1]) base1 = atomicAdd(adv ? &c->h.nN2 : &c->h.nN, all[1]);
+    }
+    at[0] += __shfl_sync(act, base0, leader);
+    at[1] += __shfl_sync(act, base1, leader);
+    int32_t* next = s->wa ? Q->A[0] : Q->A[1];
+    int32_t* win = s->wn ^ (adv ? 1 : 0) ? Q->N[1] : Q->N[0];
+    const int32_t x[4] = {x4.x, x4.y, x4.z, x4.w};
+    const uint32_t cap = Q->cap;
+    const int32_t t1 = s->t + 1;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (what >> i & 1u) {
+            Q->rnd[x[i]] = t1;
+            Q->core[x[i]] = (int32_t)k;
+            if (at[0] < cap)
+                next[at[0]++] = x[i];
+            else
+                atomicExch(&c->err, 1);
+        }
+        if (what >> (4 + i) & 1u) {
+            if (at[1] < cap)
+                win[at[1]++] = x[i];
+            else
+                atomicExch(&c->err, 1);
+        }
+    }
 }
 
 // Whether a member of a destroyed S with round tag r has its count decremented on the device: not
@@ -1459,11 +1508,16 @@ struct UpdInc {
 #pragma unroll
                 for (int m = 0; m < 4; ++m) o[m] = dec_live(r[m], E.t) ? nd_atomic_dec(&E.P.cnt[x[m]]) : E.k;
             }
+            unsigned what = 0;
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
                 k.decs += r[m] != E.t;
-                after_dec(E, x[m], o[m]);
+                if (E.P.bcnt)
+                    after_dec(E, x[m], o[m]);
+                else
+                    what |= (o[m] == E.k + 1 ? 1u : 0u) << m | (o[m] == E.hi ? 16u : 0u) << m;
             }
+            if (what) after_dec4(E.Q, E.s, w, what, E.k);
         }
     }
 };
@@ -1530,9 +1584,15 @@ __device__ __forceinline__ unsigned next_chunk(PeelCtl* c, unsigned nA, unsigned
 // Measured against one warp each: (2,3) on a Chung-Lu graph of 200,001 vertices and 2.4 M edges, Update
 // 5.2 + heavy phase 2.3 ms before, 4.8 + 0.1 ms after; (3,4) on R-MAT scale 18, 490 -> 430 ms.
 __device__ __forceinline__ unsigned split_shift(unsigned nA, const Team& T) {
-    if (nA == 0 || nA > T.nwarps / 2) return 0;
+    if (nA == 0 || nA > T.nwarps / 2) return 0;  // short_limit
     const unsigned shift = 31 - __clz(T.nwarps / nA);
     return shift < 7 ? shift : 7;
+}
+
+// The most r-cliques of a round whose warps (blocks for staged variants) need no counter to share them.
+template <typename U>
+__device__ __forceinline__ unsigned short_limit(const Team& T) {
+    return is_staged<U>::value ? 2 * T.nblocks : T.nwarps / 2;
 }
 
 // the heavy-phase threshold of this decomposition: a tuned value if given (capped by what a warp's
@@ -1601,7 +1661,7 @@ __device__ __forceinline__ void phase_update(const GraphView& g, const PeelView<
         constexpr int kOwn = is_staged<U>::value ? kI24 : 1;
         __shared__ int32_t s_w[kCap], s_x[kCap], s_y[kCap], s_b[kCap], s_p[kCap + kMaxWarpsPerBlock];
         if constexpr (is_staged<U>::value) {
-            if (nA <= 2 * T.nblocks) {
+            if (nA <= short_limit<U>(T)) {
                 Stage24 stg{s_w, s_x, s_y, s_b, s_p};
 #pragma unroll 1
                 for (unsigned i = T.block; i < nA; i += T.nblocks) {
@@ -1752,28 +1812,28 @@ __device__ __forceinline__ unsigned long long globaltimer() {
     return t;
 }
 
-__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p) {
-    unsigned long long v;
-    asm volatile("ld.acquire.gpu.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-
 __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
     unsigned long long v;
     asm volatile("ld.relaxed.gpu.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
 
-__device__ __forceinline__ int ld_relaxed_i32(const int* p) {
-    int v;
-    asm volatile("ld.relaxed.gpu.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+__device__ __forceinline__ unsigned ld_relaxed_u32(const unsigned* p) {
+    unsigned v;
+    asm volatile("ld.relaxed.gpu.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
 
+__device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
 
-__device__ __forceinline__ unsigned long long atom_add_acq_rel_u64(unsigned long long* p, unsigned long long v) {
+__device__ __forceinline__ void fence_acq_rel() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+
+
+__device__ __forceinline__ unsigned long long atom_add_release_u64(unsigned long long* p, unsigned long long v) {
     unsigned long long old;
-    asm volatile("atom.acq_rel.gpu.global.add.u64 %0, [%1], %2;" : "=l"(old) : "l"(p), "l"(v) : "memory");
+    asm volatile("atom.release.gpu.global.add.u64 %0, [%1], %2;" : "=l"(old) : "l"(p), "l"(v) : "memory");
     return old;
 }
 
@@ -1785,7 +1845,9 @@ __device__ __forceinline__ void st_release_u64(unsigned long long* p, unsigned l
 struct LoopState {
     PeelHot s;      // the round's state, copied from the control block after every barrier
     PeelCtl* c;
-    unsigned long long target;  // arrivals after which the next grid barrier opens
+    unsigned long long arrivals;  // after which the grid barrier opens
+    unsigned barrier;             // its number
+    unsigned short_a;             // |A| up to which a round is short: no dynamic chunks, no sort
     unsigned long long listed, decs;  // this block's counters
     unsigned long long last, in_round, ph_ns[7];  // block 0: time of the last barrier, of this round's Update, of each phase
     int ok;
@@ -1803,18 +1865,19 @@ struct LoopState {
 // The serial step that runs inside a barrier.
 enum Serial { kNothing, kRound, kAfterMin, kAfterSelect, kAfterUpdate, kContracted, kClearWindow, kRefilled, kHeavyScan };
 
-__device__ __forceinline__ void load_hot(LoopState* L) {
+// the hot state from 16-byte word `from` on, from the control block, by one warp
+__device__ __forceinline__ void load_hot(LoopState* L, unsigned from = 0) {
     const unsigned lane = threadIdx.x & 31;
-    if (lane < sizeof(PeelHot) / 16)
+    if (lane >= from && lane < sizeof(PeelHot) / 16)
         reinterpret_cast<int4*>(&L->s)[lane] = reinterpret_cast<const int4*>(&L->c->h)[lane];
 }
 
 // The serial step, run by one warp between a barrier's last arrival and its release: it sees every
 // write made before the barrier. Everything the next phases branch on is decided here, so that every
-// block reads the same values. The state passes through shared memory: one round trip to L2 for all
-// of it.
+// block reads the same values. The counters come from the control block with one round trip to L2, the
+// loop state is the block's own copy; both go back for the other blocks to load.
 __device__ __noinline__ void serial_step(LoopState* L, int what, int64_t arg) {
-    load_hot(L);
+    load_hot(L, 8);
     __syncwarp();
     if ((threadIdx.x & 31) == 0) {
         PeelHot& s = L->s;
@@ -1857,41 +1920,73 @@ __device__ __noinline__ void serial_step(LoopState* L, int what, int64_t arg) {
     __syncwarp();
 }
 
-// Grid barrier. The block that arrives last runs the serial step in its thread 0 and then releases
-// the others, so a control step costs no extra barrier. Arrival is an acquire-release RMW and the
-// release a release store; waiting blocks poll with relaxed loads and acquire once they are released,
-// so all writes before the barrier are visible after it (an acquire per poll empties the L1 cache
-// under the other block of the SM, which may still be working). Then the first warp copies the round's state into shared memory. The
-// wait is bounded by the global timer: after ctl->bar_timeout_ns (kBarrierTimeoutNs by default), or
-// once another block gave up (looked at every 64 polls), a block sets ctl->err bit 8 and the function
-// returns false. An empty barrier takes 1.75 us on 304 blocks (0.9 us on 8, 1.6 us on 16), the serial
-// step another 0.7: short rounds are bound by their own chains of accesses, at 0.35 us each, and not by
-// the barrier, and letting one block run them alone with block barriers gained nothing measurable.
+// The commonest serial step: a short same-level round ended, and the next one is short and of the same
+// level too (no heavy r-cliques, no contraction, no sort, no cap reached). Only |A| is then new; the
+// other changes every block makes for itself (short_next). Returns |A|, or 0 when the full step is due.
+// Run by one thread of the block that arrived last.
+__device__ __forceinline__ unsigned short_step(LoopState* L) {
+    const PeelHot& s = L->s;
+    PeelCtl* c = L->c;
+    if (s.mode & ND_MODE_ADV) return 0;
+    unsigned* slot = &c->h.nNext[s.t & 1];
+    const unsigned next = ld_relaxed_u32(slot), heavy = ld_relaxed_u32(&c->h.nH);
+    if (heavy || next == 0 || next > L->short_a || (int64_t)s.t + 1 >= s.max_rounds) return 0;
+    if (s.contract_every > 0 && s.peeled_since + s.nA >= s.contract_every) return 0;
+    if (s.t < L->round_cap) {
+        L->round_size[s.t] = s.nA;
+        L->round_level[s.t] = s.k;
+    }
+    *slot = 0;  // for the round after the next one; this block's next arrival makes it visible before that
+    return next;
+}
+
+__device__ __forceinline__ void short_next(PeelHot& s, unsigned nA) {
+    s.finished += s.nA;
+    s.peeled_since += s.nA;
+    s.t += 1;
+    s.wa ^= 1;
+    s.nA = nA;
+    s.sorta = 0;
+}
+
+// Grid barrier. The block that arrives last runs the serial step and then releases the others, so a
+// control step costs no extra barrier. Arrival is a release RMW, which the last block follows with a
+// fence; the release word holds the barrier's number and, after a short step, the next |A|. Waiting
+// blocks poll it with relaxed loads and fence once they are released, so all writes before the
+// barrier are visible after it (an acquire per poll empties the L1 cache under the other block of the
+// SM, which may still be working). After a full step they load the state, after a short one they
+// need not. The wait is bounded by the global timer: after ctl->bar_timeout_ns (kBarrierTimeoutNs by
+// default), or once another block gave up (looked at every 64 polls), a block sets ctl->err bit 8 and
+// the function returns false.
+//
+// An empty barrier takes 1.75 us on 304 blocks (0.9 us on 8, 1.6 us on 16; 2.07 GHz). Short rounds are
+// bound by what follows one another between two of them: the slowest r-clique's chain of accesses at
+// 0.35 us each, and the step at the barrier, which took 1.9 us of loads, state and fences before there
+// was a short form of it. Letting one block run the shortest rounds alone, with block barriers, gained
+// nothing measurable.
 __device__ __noinline__ bool grid_barrier(LoopState* L, int what, int64_t arg = 0) {
     __syncthreads();
     if (threadIdx.x < 32) {
         PeelCtl* c = L->c;
-        unsigned long long target = 0;
         int last = 0;
+        unsigned word = 0;  // what the release word says: the next |A| of a short step, 0 after a full one
         if (threadIdx.x == 0) {
-            target = L->target + gridDim.x;
-            L->target = target;
-            last = atom_add_acq_rel_u64(&c->bar_arrive, 1ull) + 1 == target;
-            L->ok = 1;
-        }
-        last = __shfl_sync(0xffffffffu, last, 0);
-        if (last) {
-            serial_step(L, what, arg);
-            if (threadIdx.x == 0) st_release_u64(&c->bar_gen, target);
-        } else {
-            if (threadIdx.x == 0) {
-                unsigned long long t0 = 0;
+            L->arrivals += gridDim.x;
+            L->barrier += 1;
+            last = atom_add_release_u64(&c->bar_arrive, 1ull) + 1 == L->arrivals;
+            if (last) {
+                fence_acq_rel();
+                if (what == kAfterUpdate) word = short_step(L);
+                if (word) st_relaxed_u64(&c->bar_gen, (unsigned long long)L->barrier << 32 | word);
+            } else {
+                unsigned long long t0 = 0, got;
 #pragma unroll 1
-                for (unsigned polls = 0; ld_relaxed_u64(&c->bar_gen) < target; ++polls) {
+                for (unsigned polls = 0; (int)((unsigned)((got = ld_relaxed_u64(&c->bar_gen)) >> 32) - L->barrier) < 0;
+                     ++polls) {
                     if ((polls & 63) == 63) {
                         const unsigned long long now = globaltimer();
                         if (!t0) t0 = now;
-                        if ((ld_relaxed_i32(&c->err) & 8) || now - t0 > c->bar_timeout_ns) {
+                        if ((ld_relaxed_u32((const unsigned*)&c->err) & 8) || now - t0 > c->bar_timeout_ns) {
                             atomicOr(&c->err, 8);
                             L->ok = 0;
                             break;
@@ -1899,10 +1994,20 @@ __device__ __noinline__ bool grid_barrier(LoopState* L, int what, int64_t arg = 
                     }
                     __nanosleep(20);
                 }
-                ld_acquire_u64(&c->bar_gen);
+                fence_acq_rel();
+                word = (unsigned)got;
             }
-            __syncwarp();
-            load_hot(L);
+            if (word) short_next(L->s, word);
+        }
+        last = __shfl_sync(0xffffffffu, last, 0);
+        word = __shfl_sync(0xffffffffu, word, 0);
+        if (!word) {
+            if (last) {
+                serial_step(L, what, arg);
+                if (threadIdx.x == 0) st_release_u64(&c->bar_gen, (unsigned long long)L->barrier << 32);
+            } else {
+                load_hot(L);
+            }
         }
     }
     __syncthreads();
@@ -1937,7 +2042,10 @@ __global__ void __launch_bounds__(512, 2) k_peel_loop(GraphView g, PeelView<CT> 
         Q = P;
         h = g;
         L.c = c;
-        L.target = 0;
+        L.s = c->h;
+        L.arrivals = 0;
+        L.barrier = 0;
+        L.ok = 1;
         L.listed = L.decs = 0;
         L.round_size = P.round_size;
         L.round_level = P.round_level;
@@ -1946,6 +2054,9 @@ __global__ void __launch_bounds__(512, 2) k_peel_loop(GraphView g, PeelView<CT> 
         L.sort_min = P.abits ? P.sort_min : 0xffffffffu;
         L.cap = P.cap;
         L.hslices = P.hslices;
+        L.short_a = short_limit<U>(grid_team());
+        if (L.short_a >= L.sort_min) L.short_a = L.sort_min - 1;
+        if (L.short_a > P.cap) L.short_a = P.cap;
         L.round_ns = P.round_ns;
         L.last = L.in_round = 0;
         for (int i = 0; i < 7; ++i) L.ph_ns[i] = 0;
