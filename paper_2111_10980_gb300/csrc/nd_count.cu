@@ -76,10 +76,10 @@ struct CountTri {
 };
 
 template <typename CT, int R_>
-__global__ void __launch_bounds__(kTriThreads) k_count_tri(GraphView g, CT* __restrict__ cnt) {
+__global__ void __launch_bounds__(kTriThreads) k_count_tri(GraphView g, int tile, CT* __restrict__ cnt) {
     __shared__ unsigned s_own[kTriThreads];
     CountTri<CT, R_> sink{cnt, g.dg_eid, s_own + (threadIdx.x & ~31u)};
-    tri_list(g, sink);
+    tri_list(g, tile, sink);
 }
 
 // count[t] = |L(ab) ∩ L(ac) ∩ L(bc)|. Any two of the lists already intersect to the common
@@ -176,16 +176,17 @@ template <typename CT>
 void nd_count_launch(const GraphView& g, int r, int s, CT* cnt, int64_t n_r, cudaStream_t st) {
     if (n_r <= 0) return;
     int blk = blocks_for_warps(n_r);
+    const int tile = tri_tile(g.m);
     if (r == 1 && s == 2) {
         ND_K(k_count12<CT><<<blk, kThreads, 0, st>>>(g, cnt));
     } else if (r == 2 && s == 3) {
         ND_K(k_zero<CT><<<blk, kThreads, 0, st>>>(cnt, n_r));
-        ND_K(k_count_tri<CT, 2><<<blocks_for_warps((g.m + 31) / 32), kTriThreads, 0, st>>>(g, cnt));
+        ND_K(k_count_tri<CT, 2><<<blocks_for_warps((g.m + tile - 1) / tile), kTriThreads, 0, st>>>(g, tile, cnt));
     } else if (r == 3 && s == 4) {
         ND_K(k_count34<CT><<<blk, kThreads, 0, st>>>(g, cnt));
     } else if (r == 1 && s == 3) {
         ND_K(k_zero<CT><<<blk, kThreads, 0, st>>>(cnt, n_r));
-        ND_K(k_count_tri<CT, 1><<<blocks_for_warps((g.m + 31) / 32), kTriThreads, 0, st>>>(g, cnt));
+        ND_K(k_count_tri<CT, 1><<<blocks_for_warps((g.m + tile - 1) / tile), kTriThreads, 0, st>>>(g, tile, cnt));
     } else if (r == 2 && s == 4) {
         ND_K(k_zero<CT><<<blk, kThreads, 0, st>>>(cnt, n_r));
         ND_K(k_count24_flat<CT><<<blocks_for_warps(g.m), kQuadThreads, 0, st>>>(g, cnt));

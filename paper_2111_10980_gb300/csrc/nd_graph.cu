@@ -175,11 +175,11 @@ struct SupportSink {
     }
 };
 
-__global__ void __launch_bounds__(kTriThreads) k_edge_support(GraphView g, int32_t* __restrict__ sigma,
+__global__ void __launch_bounds__(kTriThreads) k_edge_support(GraphView g, int tile, int32_t* __restrict__ sigma,
                                                               int32_t* __restrict__ up) {
     __shared__ unsigned s_own[2 * kTriThreads];
     SupportSink sink{sigma, up, g.dg_eid, s_own + 2 * (threadIdx.x & ~31u)};
-    tri_list(g, sink);
+    tri_list(g, tile, sink);
 }
 
 // Writes L(a,b) in ascending w with, per entry: the canonical triangle id when w > b, else
@@ -557,7 +557,8 @@ void nd_dg_fill(const GraphView& g, const int32_t* key_hi, int64_t* dg_rp, int32
 
 void nd_edge_support(const GraphView& g, int32_t* sigma, int32_t* up, cudaStream_t st) {
     if (g.m <= 0) return;
-    ND_K(k_edge_support<<<blocks_for_warps((g.m + 31) / 32), kTriThreads, 0, st>>>(g, sigma, up));
+    const int tile = tri_tile(g.m);
+    ND_K(k_edge_support<<<blocks_for_warps((g.m + tile - 1) / tile), kTriThreads, 0, st>>>(g, tile, sigma, up));
 }
 
 void nd_edge_fill(const GraphView& g, int64_t* et_rp, int64_t* tbase, int32_t* et_w, int32_t* et_t, int32_t* tri_e,

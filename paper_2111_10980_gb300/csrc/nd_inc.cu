@@ -119,9 +119,9 @@ struct PutTri {
 };
 
 template <int R_>
-__global__ void __launch_bounds__(kTriThreads) k_inc_tri(GraphView g, IncFill F) {
+__global__ void __launch_bounds__(kTriThreads) k_inc_tri(GraphView g, int tile, IncFill F) {
     PutTri<R_> sink{F, g.dg_eid, IncRun{}};
-    tri_list(g, sink);
+    tri_list(g, tile, sink);
     inc_done(F, sink.run);
 }
 
@@ -224,7 +224,8 @@ int nd_inc_stride(int r, int s) {
 
 // the work items of a fill kernel, one per warp at a time
 static int64_t inc_items(int r, int s, int64_t n_r, int64_t m) {
-    return s == 3 ? (m + 31) / 32 : r == 2 && s == 4 ? m : n_r;
+    const int tile = tri_tile(m);
+    return s == 3 ? (m + tile - 1) / tile : r == 2 && s == 4 ? m : n_r;
 }
 
 int64_t nd_inc_rows(int r, int s, int64_t n_r, int64_t m, int64_t n_s, unsigned* run) {
@@ -236,12 +237,12 @@ int64_t nd_inc_rows(int r, int s, int64_t n_r, int64_t m, int64_t n_s, unsigned*
 
 void nd_inc_fill(const GraphView& g, int r, int s, int64_t n_r, const IncFill& F, cudaStream_t st) {
     if (n_r <= 0) return;
-    const int blk = blocks_for_warps(inc_items(r, s, n_r, g.m));
+    const int blk = blocks_for_warps(inc_items(r, s, n_r, g.m)), tile = tri_tile(g.m);
     static_assert(kTriThreads == kThreads && kQuadThreads == kThreads, "nd_inc_rows counts the warps");
     if (r == 1 && s == 3) {
-        ND_K(k_inc_tri<1><<<blk, kTriThreads, 0, st>>>(g, F));
+        ND_K(k_inc_tri<1><<<blk, kTriThreads, 0, st>>>(g, tile, F));
     } else if (r == 2 && s == 3) {
-        ND_K(k_inc_tri<2><<<blk, kTriThreads, 0, st>>>(g, F));
+        ND_K(k_inc_tri<2><<<blk, kTriThreads, 0, st>>>(g, tile, F));
     } else if (r == 2 && s == 4) {
         ND_K(k_inc24<<<blk, kQuadThreads, 0, st>>>(g, F));
     } else if (r == 3 && s == 4) {

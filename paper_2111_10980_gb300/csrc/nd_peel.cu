@@ -301,6 +301,27 @@ __device__ __noinline__ void phase_adv_min(const PeelView<CT>& P, const PeelHot&
     if (threadIdx.x == 0 && mn != ULLONG_MAX) atomicMin(&P.ctl->h.minN, mn);
 }
 
+// The scans over long lists (window, alive list) take 256 entries per warp and step, so that a list they
+// append to costs one counter update per 256 entries looked at: with one per 32 the 83 M triangles of
+// R-MAT scale 18 took 2 ms per scan, all of it in line at one counter.
+constexpr int kScanItems = 8;
+
+// places in list for the entries that bit i of `take` marks in this lane (entry i of the step is entry
+// 32 i + lane); the whole warp calls it and gets the place of its first one
+__device__ __forceinline__ unsigned scan_places(unsigned* counter, unsigned take, unsigned (&at)[kScanItems]) {
+    const unsigned full = 0xffffffffu;
+    unsigned total = 0;
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) {
+        const unsigned b = __ballot_sync(full, take >> i & 1u);
+        at[i] = total + __popc(b & nd_lanemask_lt());
+        total += __popc(b);
+    }
+    unsigned base = 0;
+    if (total && (threadIdx.x & 31) == 0) base = atomicAdd(counter, total);
+    return __shfl_sync(full, base, 0);
+}
+
 // refill 1/4: compact L into L' (alive only), global minimum count, clear the histogram
 template <typename CT>
 __device__ __noinline__ void phase_refill_scan(const PeelView<CT>& P, const PeelHot& s, const Team& T) {
@@ -312,17 +333,31 @@ __device__ __noinline__ void phase_refill_scan(const PeelView<CT>& P, const Peel
     const int32_t lmat = s.lmat;
     int64_t n = lmat ? (int64_t)clampn(s.nL, P.cap) : s.n_r;
     unsigned long long mn = ULLONG_MAX;
-    // grid-stride in whole-warp steps so that appends aggregate per warp
-    for (int64_t base = T.thread() - (threadIdx.x & 31); base < n; base += T.nthreads()) {
-        int64_t i = base + (threadIdx.x & 31);
-        if (i < n) {
-            int32_t R = lmat ? L[i] : (int32_t)i;
-            if (P.rnd[R] == ND_UNPEELED) {
-                unsigned long long v = (unsigned long long)P.cnt[R];
-                mn = v < mn ? v : mn;
-                nd_append(&c->h.nL2, L2, P.cap, R, &c->err);
-            }
+    const int lane = threadIdx.x & 31;
+    for (int64_t base = (T.thread() - lane) * kScanItems; base < n; base += T.nthreads() * kScanItems) {
+        int32_t R[kScanItems];
+        unsigned take = 0, at[kScanItems];
+#pragma unroll
+        for (int i = 0; i < kScanItems; ++i) {
+            const int64_t p = base + 32 * i + lane;
+            R[i] = p < n ? (lmat ? L[p] : (int32_t)p) : -1;
         }
+#pragma unroll
+        for (int i = 0; i < kScanItems; ++i)
+            if (R[i] >= 0 && P.rnd[R[i]] == ND_UNPEELED) {
+                take |= 1u << i;
+                unsigned long long v = (unsigned long long)P.cnt[R[i]];
+                mn = v < mn ? v : mn;
+            }
+        const unsigned b = scan_places(&c->h.nL2, take, at);
+#pragma unroll
+        for (int i = 0; i < kScanItems; ++i)
+            if (take >> i & 1u) {
+                if (b + at[i] < P.cap)
+                    L2[b + at[i]] = R[i];
+                else
+                    atomicExch(&c->err, 1);
+            }
     }
     mn = block_min(mn);
     if (threadIdx.x == 0 && mn != ULLONG_MAX) atomicMin(&c->h.gmin, mn);
@@ -409,12 +444,27 @@ template <typename CT>
 __device__ __noinline__ void phase_refill_select(const PeelView<CT>& P, const int32_t* L, unsigned n, int32_t* N, int64_t hi,
                                     const Team& T) {
     PeelCtl* c = P.ctl;
-    for (int64_t base = T.thread() - (threadIdx.x & 31); base < n; base += T.nthreads()) {
-        int64_t i = base + (threadIdx.x & 31);
-        if (i < n) {
-            int32_t R = L[i];
-            if ((int64_t)P.cnt[R] < hi) nd_append(&c->h.nN, N, P.cap, R, &c->err);
+    const int lane = threadIdx.x & 31;
+    for (int64_t base = (T.thread() - lane) * kScanItems; base < n; base += T.nthreads() * kScanItems) {
+        int32_t R[kScanItems];
+        unsigned take = 0, at[kScanItems];
+#pragma unroll
+        for (int i = 0; i < kScanItems; ++i) {
+            const int64_t p = base + 32 * i + lane;
+            R[i] = p < n ? L[p] : -1;
         }
+#pragma unroll
+        for (int i = 0; i < kScanItems; ++i)
+            if (R[i] >= 0 && (int64_t)P.cnt[R[i]] < hi) take |= 1u << i;
+        const unsigned b = scan_places(&c->h.nN, take, at);
+#pragma unroll
+        for (int i = 0; i < kScanItems; ++i)
+            if (take >> i & 1u) {
+                if (b + at[i] < P.cap)
+                    N[b + at[i]] = R[i];
+                else
+                    atomicExch(&c->err, 1);
+            }
     }
 }
 
@@ -429,23 +479,48 @@ __device__ __noinline__ void phase_adv_select(const PeelView<CT>& P, const PeelH
     int32_t* A = pick(P.A, s.wa);
     unsigned n = clampn(s.nN, P.cap);
     int32_t t = s.t;
-    for (int64_t base = T.thread() - (threadIdx.x & 31); base < n; base += T.nthreads()) {
-        int64_t i = base + (threadIdx.x & 31);
-        if (i < n) {
-            int32_t R = N[i];
-            if (P.rnd[R] == ND_UNPEELED) {
-                if ((int64_t)P.cnt[R] <= kn) {
-                    if (P.bcnt) atomicSub(&P.bcnt[(int64_t)P.cnt[R]], 1u);
-                    P.rnd[R] = t;
-                    P.core[R] = (int32_t)kn;
-                    if (P.et_rnd) set_tri_round(P, R, t);
-                    mark_a(P, R);
-                    nd_append(&c->h.cntA, A, P.cap, R, &c->err);
-                } else {
-                    nd_append(&c->h.nN2, N2, P.cap, R, &c->err);
-                }
-            }
+    const int lane = threadIdx.x & 31;
+    // a short window: one entry per lane and step, so that every warp has some
+    const int items = (int64_t)n > T.nthreads() * kScanItems ? kScanItems : 1;
+    for (int64_t base = (T.thread() - lane) * items; base < n; base += T.nthreads() * items) {
+        int32_t R[kScanItems];
+        unsigned sel = 0, rest = 0, at[kScanItems];
+#pragma unroll
+        for (int i = 0; i < kScanItems; ++i) {
+            const int64_t p = base + 32 * i + lane;
+            R[i] = i < items && p < n ? N[p] : -1;
         }
+#pragma unroll
+        for (int i = 0; i < kScanItems; ++i)
+            if (R[i] >= 0 && P.rnd[R[i]] == ND_UNPEELED) {
+                if ((int64_t)P.cnt[R[i]] <= kn)
+                    sel |= 1u << i;
+                else
+                    rest |= 1u << i;
+            }
+        unsigned b = scan_places(&c->h.cntA, sel, at);
+#pragma unroll
+        for (int i = 0; i < kScanItems; ++i)
+            if (sel >> i & 1u) {
+                if (P.bcnt) atomicSub(&P.bcnt[(int64_t)P.cnt[R[i]]], 1u);
+                P.rnd[R[i]] = t;
+                P.core[R[i]] = (int32_t)kn;
+                if (P.et_rnd) set_tri_round(P, R[i], t);
+                mark_a(P, R[i]);
+                if (b + at[i] < P.cap)
+                    A[b + at[i]] = R[i];
+                else
+                    atomicExch(&c->err, 1);
+            }
+        b = scan_places(&c->h.nN2, rest, at);
+#pragma unroll
+        for (int i = 0; i < kScanItems; ++i)
+            if (rest >> i & 1u) {
+                if (b + at[i] < P.cap)
+                    N2[b + at[i]] = R[i];
+                else
+                    atomicExch(&c->err, 1);
+            }
     }
 }
 

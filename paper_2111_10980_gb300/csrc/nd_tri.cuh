@@ -6,11 +6,20 @@
 
 constexpr int kTriThreads = 256;
 
-// A warp takes 32 DG edges u -> v at a time. Each lane sets one up: the shorter of N_DG(u) and N_DG(v)
-// drives and the longer is searched. The warp numbers the candidates of all 32 edges by a prefix sum and
+// Edges per warp and step: 32, and fewer where the graph has too few edges to give every resident warp as
+// many (a graph of 534 vertices and 7,700 edges at 32: 240 warps, each with a thousand candidates in a row,
+// 36 us for a count that takes 8 us with one edge each).
+inline int tri_tile(int64_t m) {
+    const int64_t warps = (int64_t)nd_sm_count() * 64;
+    const int64_t t = (m + warps - 1) / warps;
+    return (int)(t < 1 ? 1 : t > 32 ? 32 : t);
+}
+
+// A warp takes `tile` DG edges u -> v at a time. Each lane sets one up: the shorter of N_DG(u) and N_DG(v)
+// drives and the longer is searched. The warp numbers the candidates of all its edges by a prefix sum and
 // takes 32 at a time, whatever edges they belong to, so that the many edges with two or three
 // candidates fill its lanes as well as the few with thousands. The whole warp calls sink.tri() with each
-// lane's candidate: whether it is a triangle, the slot of u -> v among the 32 edges, its edge, the DG
+// lane's candidate: whether it is a triangle, the slot of u -> v among the edges, its edge, the DG
 // positions of the other two edges (the first is u's if of_u), and the vertices. sink.end() is called once per edge by the lane
 // that set it up.
 //
@@ -18,12 +27,12 @@ constexpr int kTriThreads = 256;
 // merging the two undirected rows, which meets each triangle three times: (2,3) counts of R-MAT scale 20
 // 42 -> 16.5 ms, of a Chung-Lu graph with 2.4 M edges 1.10 -> 0.33 ms.
 template <typename Sink>
-__device__ __forceinline__ void tri_list(const GraphView& g, Sink& sink) {
+__device__ __forceinline__ void tri_list(const GraphView& g, int tile, Sink& sink) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t j0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; j0 < g.m; j0 += nwarps * 32) {
-        const int64_t j = j0 + lane;
+    for (int64_t j0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * tile; j0 < g.m; j0 += nwarps * tile) {
+        const int64_t j = lane < tile ? j0 + lane : g.m;
         int32_t u = 0, v = 0, e = 0, xb = 0, xn = 0, yb = 0, yn = 0;  // DG positions are below m < 2^31
         int32_t of_u = 0;
         if (j < g.m) {
