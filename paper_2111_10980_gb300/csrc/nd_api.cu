@@ -7,6 +7,7 @@
 #include <algorithm>
 #include <atomic>
 #include <climits>
+#include <cstddef>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -71,6 +72,42 @@ void nd_free(nd_ctx* ctx, DBuf& b) {
     ctx->in_use -= b.bytes;
     b.p = nullptr;
     b.bytes = 0;
+}
+
+int DGroup::alloc(nd_ctx* c) {
+    constexpr size_t kArena = (size_t)4 << 20;
+    size_t total = 0;
+    for (auto& w : want) total += (std::max<size_t>(w.second, 16) + 255) & ~(size_t)255;
+    if (total <= kArena) {
+        if (nd_alloc(c, arena, total) == ND_OK) {
+            size_t at = 0;
+            for (auto& w : want) {
+                const size_t bytes = (std::max<size_t>(w.second, 16) + 255) & ~(size_t)255;
+                w.first->p = (char*)arena.p + at;
+                w.first->bytes = bytes;
+                at += bytes;
+            }
+            return ND_OK;
+        }
+        // an allocator may have room for each and not for all in one piece
+    }
+    for (auto& w : want)
+        if (int rc = nd_alloc(c, *w.first, w.second)) {
+            free(c);
+            return rc;
+        }
+    return ND_OK;
+}
+
+void DGroup::free(nd_ctx* c) {
+    for (auto& w : want) {
+        if (arena.p)
+            *w.first = DBuf();
+        else
+            nd_free(c, *w.first);
+    }
+    nd_free(c, arena);
+    want.clear();
 }
 
 #define ND_TRY(x)                       \
@@ -151,12 +188,17 @@ extern "C" int nd_ctx_create(int device, void* stream, size_t mem_budget, nd_ctx
         cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
     }
     cudaGetLastError();
-    if (cudaMallocHost(&c->pinned, 4096) != cudaSuccess) {
+    if (cudaMallocHost(&c->pinned, nd_ctx::kPinned) != cudaSuccess) {
         cudaGetLastError();
         if (c->own_stream) cudaStreamDestroy(c->stream);
         delete c;
         return nd_set_error(ND_ECUDA, "cudaMallocHost failed");
     }
+    for (cudaEvent_t& e : c->ev)
+        if (cudaEventCreate(&e) != cudaSuccess) {
+            nd_ctx_destroy(c);
+            return nd_set_error(ND_ECUDA, "cudaEventCreate failed");
+        }
     *out = c;
     return ND_OK;
 }
@@ -203,6 +245,8 @@ extern "C" int nd_ctx_destroy(nd_ctx* ctx) {
     if (ctx->stage) cudaFreeHost(ctx->stage);
     for (cudaStream_t x : ctx->cap_st)
         if (x) cudaStreamDestroy(x);
+    for (cudaEvent_t e : ctx->ev)
+        if (e) cudaEventDestroy(e);
     if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
     cudaGetLastError();
     delete ctx;
@@ -376,23 +420,25 @@ static int ensure_base(nd_graph* g) {
     nd_build_split((const int64_t*)g->rp.p, (const int32_t*)g->col.p, g->n, (int64_t*)g->split.p,
                    (int64_t*)updeg.p, st);
     nd_scan_i64((const int64_t*)updeg.p, (int64_t*)g->ebase.p, g->n, tmp.p, st);
-    int64_t m_up = 0;
-    rc = nd_check_launch("edge index");
-    if (!rc) rc = read_back(g, (int64_t*)g->ebase.p + g->n, &m_up, "edge index");
+    // the edge ids are checked against m on the device, so everything is read back once at the end
+    GraphView v = nd_view(g);
+    rc = scalar_zero(g);
+    if (!rc) {
+        nd_build_pos2e(v, (int32_t*)g->pos2e.p, (int32_t*)g->eu.p, (int32_t*)g->ev.p, (int*)g->scal.p, st);
+        nd_max_deg((const int64_t*)g->rp.p, g->n, (unsigned long long*)g->scal.p + 1, st);
+        cudaMemcpyAsync((int64_t*)g->scal.p + 2, (int64_t*)g->ebase.p + g->n, 8, cudaMemcpyDeviceToDevice, st);
+        rc = nd_check_launch("edge index");
+    }
+    unsigned long long sc[3] = {0, 0, 0};
+    if (!rc) rc = read_back(g, g->scal.p, &sc, "edge index");
     nd_free(c, updeg);
     nd_free(c, tmp);
     if (rc) return rc;
+    const int64_t m_up = (int64_t)sc[2];
     if (m_up != g->m)
         return nd_set_error(ND_EINVAL, "the CSR is not symmetric (%lld upper entries for %lld edges); load it with "
                                        "ND_VALIDATE for details",
                             (long long)m_up, (long long)g->m);
-    GraphView v = nd_view(g);
-    ND_TRY(scalar_zero(g));
-    nd_build_pos2e(v, (int32_t*)g->pos2e.p, (int32_t*)g->eu.p, (int32_t*)g->ev.p, (int*)g->scal.p, st);
-    nd_max_deg((const int64_t*)g->rp.p, g->n, (unsigned long long*)g->scal.p + 1, st);
-    unsigned long long sc[2] = {0, 0};
-    ND_TRY(nd_check_launch("edge index"));
-    ND_TRY(read_back(g, g->scal.p, &sc, "edge index"));
     if (sc[0] & 1)
         return nd_set_error(ND_EINVAL, "the CSR is not symmetric or has a self-loop; load it with ND_VALIDATE "
                                        "for details");
@@ -430,16 +476,11 @@ static int build_dg(nd_graph* g, int mode) {
     nd_scan_i64((const int64_t*)outdeg.p, (int64_t*)g->dg_rp.p, g->n, tmp.p, st);
     v = nd_view(g);
     nd_dg_fill(v, key_hi, (int64_t*)g->dg_rp.p, (int32_t*)g->dg_col.p, (int32_t*)g->dg_eid.p, st);
-    scalar_zero(g);
-    nd_max_deg((const int64_t*)g->dg_rp.p, g->n, (unsigned long long*)g->scal.p, st);
-    unsigned long long mo = 0;
     rc = nd_check_launch("orientation");
-    if (!rc) rc = read_back(g, g->scal.p, &mo, "orientation");
     nd_free(c, key);
     nd_free(c, outdeg);
     nd_free(c, tmp);
     if (rc) return rc;
-    g->maxout = (int64_t)mo;
     g->orient = mode;
     return ND_OK;
 }
@@ -562,10 +603,7 @@ int nd_prepare(nd_graph* g, int r, int s, int64_t* n_r, double* t_orient, double
     if (!rs_supported(r, s)) return nd_set_error(ND_EINVAL, "(r,s) = (%d,%d) is not supported", r, s);
     nd_ctx* c = g->ctx;
     ND_CUDA(cudaSetDevice(c->device));
-    cudaEvent_t e0, e1, e2;
-    cudaEventCreate(&e0);
-    cudaEventCreate(&e1);
-    cudaEventCreate(&e2);
+    cudaEvent_t e0 = c->ev[0], e1 = c->ev[1], e2 = c->ev[2];
     cudaEventRecord(e0, c->stream);
     int rc = ensure_base(g);
     if (!rc && g->orient < 0) rc = build_dg(g, ND_ORIENT_DEGREE);
@@ -579,9 +617,6 @@ int nd_prepare(nd_graph* g, int r, int s, int64_t* n_r, double* t_orient, double
         cudaEventElapsedTime(&a, e0, e1);
         cudaEventElapsedTime(&b, e1, e2);
     }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    cudaEventDestroy(e2);
     if (rc) return rc;
     if (t_orient) *t_orient = a;
     if (t_index) *t_index = b;
@@ -718,7 +753,7 @@ static bool wants_inc(const nd_ctx* c, int r, int s, int flags, int64_t n_s) {
 }
 
 void nd_free_inc(nd_ctx* c, IncBufs& b) {
-    for (DBuf* x : {&b.off, &b.list, &b.row, &b.dead, &b.status}) nd_free(c, *x);
+    b.mem.free(c);
 }
 
 static int build_inc(nd_graph* g, int r, int s, const DBuf& cnt, int w, int64_t n_r, int64_t n_s, IncBufs& b) {
@@ -729,33 +764,33 @@ static int build_inc(nd_graph* g, int r, int s, const DBuf& cnt, int w, int64_t 
     const int64_t entries = n_s * binom64(s, r);
     IncFill F;
     F.rows = nd_inc_rows(r, s, n_r, g->m, n_s, &F.run);
-    DBuf cursor, tmp;
-    int rc = ND_OK;
-    if ((rc = nd_alloc(c, b.off, 8 * (n_r + 1))) || (rc = nd_alloc(c, cursor, 8 * (n_r + 1))) ||
-        (rc = nd_alloc(c, tmp, nd_scan_tmp_bytes(n_r))) || (rc = nd_alloc(c, b.list, 4 * std::max<int64_t>(entries, 1))) ||
-        (rc = nd_alloc(c, b.row, 4 * b.stride * F.rows)) ||
-        (rc = nd_alloc(c, b.dead, 4 * (F.rows / 32 + 1))) || (rc = nd_alloc(c, b.status, 16))) {
-        nd_free(c, cursor);
-        nd_free(c, tmp);
-        nd_free_inc(c, b);
-        return rc;
-    }
+    b.mem.add(b.off, 8 * (n_r + 1));
+    b.mem.add(b.cursor, 8 * (n_r + 1));
+    b.mem.add(b.tmp, nd_scan_tmp_bytes(n_r));
+    b.mem.add(b.list, 4 * std::max<int64_t>(entries, 1));
+    b.mem.add(b.row, 4 * b.stride * F.rows);
+    b.mem.add(b.dead, 4 * (F.rows / 32 + 1));
+    b.mem.add(b.status, 16);
+    int rc = b.mem.alloc(c);
+    if (rc) return rc;
     if (w == 8)
-        nd_scan_i64((const int64_t*)cnt.p, (int64_t*)b.off.p, n_r, tmp.p, st);
+        nd_scan_i64((const int64_t*)cnt.p, (int64_t*)b.off.p, n_r, b.tmp.p, st);
     else
-        nd_scan_i32((const int32_t*)cnt.p, (int64_t*)b.off.p, n_r, tmp.p, st);
-    cudaMemcpyAsync(cursor.p, b.off.p, 8 * (n_r + 1), cudaMemcpyDeviceToDevice, st);
+        nd_scan_i32((const int32_t*)cnt.p, (int64_t*)b.off.p, n_r, b.tmp.p, st);
+    cudaMemcpyAsync(b.cursor.p, b.off.p, 8 * (n_r + 1), cudaMemcpyDeviceToDevice, st);
     cudaMemsetAsync(b.dead.p, 0, b.dead.bytes, st);
     cudaMemsetAsync(b.status.p, 0, b.status.bytes, st);
-    F.cursor = (unsigned long long*)cursor.p;
+    F.cursor = (unsigned long long*)b.cursor.p;
     F.list = (uint32_t*)b.list.p;
     F.row = (int32_t*)b.row.p;
     F.status = (unsigned int*)b.status.p;
     F.entries = entries;
     nd_inc_fill(nd_view(g), r, s, n_r, F, st);
     rc = nd_check_launch("incidence lists");
-    nd_free(c, cursor);
-    nd_free(c, tmp);
+    if (!b.mem.arena.p) {
+        nd_free(c, b.cursor);
+        nd_free(c, b.tmp);
+    }
     if (rc) nd_free_inc(c, b);
     return rc;
 }
@@ -844,27 +879,34 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags
     DBuf ilen, iprev, ctl, A0, A1, N0, N1, L0, L1, H, rs, rl, rt, etr, hsc, abits, ccol, cpos, clen, cprev, bcnt, hcnt, hpre, lw, lt,
         ltp, llen, lprev;
     const int64_t nent = std::max<int64_t>(3 * g->n3, 1);
-    if ((rc = nd_alloc(c, ctl, sizeof(PeelCtl))) || (rc = nd_alloc(c, A0, 4 * cap)) || (rc = nd_alloc(c, A1, 4 * cap)) ||
-        (rc = nd_alloc(c, N0, 4 * cap)) || (rc = nd_alloc(c, N1, 4 * cap)) || (rc = nd_alloc(c, L0, 4 * cap)) ||
-        (rc = nd_alloc(c, L1, 4 * cap)) || (rc = nd_alloc(c, H, 4 * hcap)) || (rc = nd_alloc(c, rs, 8 * rcap)) ||
-        (rc = nd_alloc(c, rl, 8 * rcap)) || (rc = nd_alloc(c, rt, 8 * rcap)) || (lists34 && (rc = nd_alloc(c, etr, 4 * std::max<int64_t>(3 * g->n3, 1)))) ||
-        (staged && (rc = nd_alloc(c, hsc, 4 * 5 * (hstage + 1) * hslices))) ||
-        (rc = nd_alloc(c, abits, r == 3 && !inc ? 4 * ((cap + 31) / 32) : 4)) ||
-        (contract && ((rc = nd_alloc(c, ccol, 4 * std::max<int64_t>(g->nnz, 1))) ||
-                      (rc = nd_alloc(c, cpos, 4 * std::max<int64_t>(g->nnz, 1))) ||
-                      (rc = nd_alloc(c, clen, 4 * std::max<int64_t>(g->n, 1))) ||
-                      (rc = nd_alloc(c, cprev, 4 * std::max<int64_t>(g->n, 1))))) ||
-        (contract_inc && ((rc = nd_alloc(c, ilen, 4 * cap)) || (rc = nd_alloc(c, iprev, 4 * cap)))) ||
-        (dense && (rc = nd_alloc(c, bcnt, 4 * std::max<int64_t>(bmax, 1)))) ||
-        (staged && ((rc = nd_alloc(c, hcnt, 4 * (hslices + 1))) || (rc = nd_alloc(c, hpre, 8 * (hslices + 1))))) ||
-        (contract34 && ((rc = nd_alloc(c, lw, 4 * nent)) || (rc = nd_alloc(c, lt, 4 * nent)) ||
-                        (rc = nd_alloc(c, ltp, 4 * nent)) || (rc = nd_alloc(c, llen, 4 * std::max<int64_t>(g->m, 1))) ||
-                        (rc = nd_alloc(c, lprev, 4 * std::max<int64_t>(g->m, 1)))))) {
-        for (DBuf* b : {&ctl, &A0, &A1, &N0, &N1, &L0, &L1, &H, &rs, &rl, &rt, &etr, &hsc, &abits, &ccol, &cpos, &clen,
-                        &cprev, &bcnt, &hcnt, &hpre, &lw, &lt, &ltp, &llen, &lprev, &ilen, &iprev})
-            nd_free(c, *b);
-        return rc;
+    DGroup mem;
+    mem.add(ctl, sizeof(PeelCtl));
+    for (DBuf* b : {&A0, &A1, &N0, &N1, &L0, &L1}) mem.add(*b, 4 * cap);
+    mem.add(H, 4 * hcap);
+    for (DBuf* b : {&rs, &rl, &rt}) mem.add(*b, 8 * rcap);
+    mem.add(abits, r == 3 && !inc ? 4 * ((cap + 31) / 32) : 4);
+    if (lists34) mem.add(etr, 4 * nent);
+    if (staged) {
+        mem.add(hsc, 4 * 5 * (hstage + 1) * hslices);
+        mem.add(hcnt, 4 * (hslices + 1));
+        mem.add(hpre, 8 * (hslices + 1));
     }
+    if (contract) {
+        mem.add(ccol, 4 * g->nnz);
+        mem.add(cpos, 4 * g->nnz);
+        mem.add(clen, 4 * (int64_t)g->n);
+        mem.add(cprev, 4 * (int64_t)g->n);
+    }
+    if (contract_inc) {
+        mem.add(ilen, 4 * cap);
+        mem.add(iprev, 4 * cap);
+    }
+    if (dense) mem.add(bcnt, 4 * std::max<int64_t>(bmax, 1));
+    if (contract34) {
+        for (DBuf* b : {&lw, &lt, &ltp}) mem.add(*b, 4 * nent);
+        for (DBuf* b : {&llen, &lprev}) mem.add(*b, 4 * g->m);
+    }
+    if ((rc = mem.alloc(c))) return rc;
     PeelView<CT> P;
     P.cnt = (CT*)cnt.p;
     P.rnd = (int32_t*)po.rnd.p;
@@ -998,7 +1040,6 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags
         if (e == cudaSuccess) {
             looped = true;
             persistent_launches = 1;
-            rc = nd_sync(c, "peel (persistent)");
         } else {
             cudaGetLastError();
             if (flags & ND_PEEL_PERSISTENT)
@@ -1070,12 +1111,22 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags
     }
     if (exec) cudaGraphExecDestroy(exec);
     if (graph) cudaGraphDestroy(graph);
+    // one read-back of the statistics and, of most runs, of the whole record
+    constexpr int64_t kRec = 2048;
+    constexpr size_t kHead = offsetof(PeelCtl, hist), kRecAt = 4096;
+    static_assert(kHead <= kRecAt && kRecAt + 3 * 8 * kRec <= nd_ctx::kPinned, "the read-back fits");
+    const int64_t nfirst = std::min<int64_t>(kRec, rcap);
     if (!rc) {
         PeelCtl h;
-        cudaMemcpyAsync(c->pinned, P.ctl, std::min<size_t>(sizeof(PeelCtl), 4096), cudaMemcpyDeviceToHost, st);
-        rc = nd_sync(c, "peel stats");
+        char* pin = (char*)c->pinned;
+        cudaMemcpyAsync(pin, P.ctl, kHead, cudaMemcpyDeviceToHost, st);
+        const void* rec[3] = {rs.p, rl.p, rt.p};
+        for (int i = 0; i < 3; ++i)
+            cudaMemcpyAsync(pin + kRecAt + 8 * kRec * i, rec[i], 8 * nfirst, cudaMemcpyDeviceToHost, st);
+        cudaEventRecord(c->ev[7], st);
+        rc = nd_sync(c, "peel");
         if (!rc) {
-            memcpy(&h, c->pinned, std::min<size_t>(sizeof(PeelCtl), 4096));
+            memcpy(&h, pin, kHead);
             if (h.err & 8) rc = nd_set_error(ND_ETIMEOUT, "peel: a grid barrier of the persistent kernel timed out");
             else if (h.err & 1) rc = nd_set_error(ND_EINTERNAL, "peel: a work list overflowed");
             else if (h.err & 2) rc = nd_set_error(ND_ETIMEOUT, "peel: round cap reached");
@@ -1102,16 +1153,18 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags
         po.sizes.resize(nrec);
         po.levels.resize(nrec);
         po.round_ns.resize(nrec);
-        if (nrec) {
-            cudaMemcpyAsync(po.sizes.data(), rs.p, 8 * nrec, cudaMemcpyDeviceToHost, st);
-            cudaMemcpyAsync(po.levels.data(), rl.p, 8 * nrec, cudaMemcpyDeviceToHost, st);
-            cudaMemcpyAsync(po.round_ns.data(), rt.p, 8 * nrec, cudaMemcpyDeviceToHost, st);
-            rc = nd_sync(c, "peel record");
+        std::vector<int64_t>* out[3] = {&po.sizes, &po.levels, &po.round_ns};
+        const DBuf* rec[3] = {&rs, &rl, &rt};
+        const int64_t head = std::min<int64_t>(nrec, nfirst);
+        for (int i = 0; i < 3; ++i) {
+            memcpy(out[i]->data(), (char*)c->pinned + kRecAt + 8 * kRec * i, 8 * head);
+            if (nrec > head)
+                cudaMemcpyAsync(out[i]->data() + head, (int64_t*)rec[i]->p + head, 8 * (nrec - head),
+                                cudaMemcpyDeviceToHost, st);
         }
+        if (nrec > head) rc = nd_sync(c, "peel record");
     }
-    for (DBuf* b : {&ctl, &A0, &A1, &N0, &N1, &L0, &L1, &H, &rs, &rl, &rt, &etr, &hsc, &abits, &ccol, &cpos, &clen,
-                    &cprev, &bcnt, &hcnt, &hpre, &lw, &lt, &ltp, &llen, &lprev, &ilen, &iprev})
-        nd_free(c, *b);
+    mem.free(c);
     return rc;
 }
 
@@ -1125,12 +1178,7 @@ int nd_decompose_dev(nd_graph* g, int r, int s, int count_width, int flags, Peel
     ND_TRY(nd_prepare(g, r, s, &n_r, &t_or, &t_ix));
     int w = 0;
     ND_TRY(nd_pick_width(g, r, s, count_width, &w));
-    cudaEvent_t e0, e1, e2, e3, eh;
-    cudaEventCreate(&e0);
-    cudaEventCreate(&e1);
-    cudaEventCreate(&e2);
-    cudaEventCreate(&e3);
-    cudaEventCreate(&eh);
+    cudaEvent_t e0 = c->ev[3], e1 = c->ev[4], e3 = c->ev[5], eh = c->ev[6], e2 = c->ev[7];  // e2: recorded by run_peel
     DBuf cnt;
     int rc = nd_alloc(c, po.core, 4 * std::max<int64_t>(n_r, 1));
     if (!rc) rc = nd_alloc(c, po.rnd, 4 * std::max<int64_t>(n_r, 1));
@@ -1167,19 +1215,12 @@ int nd_decompose_dev(nd_graph* g, int r, int s, int count_width, int flags, Peel
         rc = (w == 8) ? run_peel<int64_t>(g, r, s, cnt, n_r, flags, po, use_inc ? &inc : nullptr)
                       : run_peel<int32_t>(g, r, s, cnt, n_r, flags, po, use_inc ? &inc : nullptr);
     nd_free_inc(c, inc);
-    cudaEventRecord(e2, c->stream);
-    if (!rc) rc = nd_sync(c, "nd_decompose");
     float tc = 0, tp = 0, th = 0;
     if (!rc) {
         cudaEventElapsedTime(&tc, e0, e1);
         cudaEventElapsedTime(&tp, e3, e2);
         cudaEventElapsedTime(&th, e0, eh);
     }
-    cudaEventDestroy(eh);
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    cudaEventDestroy(e2);
-    cudaEventDestroy(e3);
     nd_free(c, cnt);
     for (DBuf* b : {&g->hoff, &g->htab, &g->hpos}) nd_free(c, *b);
     if (rc) return rc;

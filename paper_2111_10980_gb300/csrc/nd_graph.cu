@@ -85,8 +85,13 @@ __global__ void k_pos2e(GraphView g, int32_t* __restrict__ pos2e, int32_t* __res
             int64_t id;
             if (v > u) {
                 id = g.ebase[u] + (p - g.split[u]);
-                eu[id] = (int32_t)u;
-                ev[id] = v;
+                if (id < g.m) {
+                    eu[id] = (int32_t)u;
+                    ev[id] = v;
+                } else {  // more upper than lower entries
+                    atomicOr(err, 1);
+                    id = 0;
+                }
             } else {
                 int64_t vb = g.rp[v], ve = g.rp[v + 1];
                 int64_t q = vb + nd_lower_bound(g.col + vb, ve - vb, (int32_t)u);

@@ -5,6 +5,7 @@
 
 #include <atomic>
 #include <cstdint>
+#include <utility>
 #include <vector>
 
 #include "nd.h"
@@ -25,7 +26,9 @@ struct nd_ctx {
     nd_alloc_fn af = nullptr;
     nd_free_fn ff = nullptr;
     void* user = nullptr;
-    void* pinned = nullptr;  // 4 KiB of pinned host memory for scalar read-backs
+    void* pinned = nullptr;  // kPinned bytes of pinned host memory for read-backs
+    static constexpr size_t kPinned = 64 << 10;
+    cudaEvent_t ev[8] = {nullptr};  // timing of the phases: [0..2] nd_prepare, [3..7] nd_decompose
     cudaStream_t cap_st[2] = {nullptr, nullptr};  // extra streams used only to capture graph bodies
     // nd_ctx_set_limits (0: default)
     int64_t max_rounds = 0;
@@ -54,7 +57,6 @@ struct nd_graph {
     // orientation
     int orient = -1;
     DBuf dg_rp, dg_col, dg_eid;
-    int64_t maxout = 0;
     // triangle index
     bool have_tri = false;
     int64_t n3 = 0;
@@ -79,8 +81,20 @@ struct PeelOut {
     std::vector<int64_t> sizes, levels, round_ns;
 };
 
+// Buffers that live and die together. Small ones come out of one allocation: the thirty of a short
+// decomposition cost it as much time as its rounds.
+struct DGroup {
+    std::vector<std::pair<DBuf*, size_t>> want;
+    DBuf arena;
+    void add(DBuf& b, size_t bytes) { want.emplace_back(&b, bytes); }
+    int alloc(nd_ctx* c);
+    void free(nd_ctx* c);
+};
+
 // Incidence lists of the s-cliques (nd_inc.cu).
 struct IncBufs {
+    DGroup mem;  // holds the others
+    DBuf cursor, tmp;  // only while they are filled
     DBuf off, list, row, dead, status;
     int32_t stride = 0;
     int64_t n_s = 0;
