@@ -311,9 +311,11 @@ typedef struct nd_server_cfg {
     int32_t workers;       /* batches running on the device at once, each on its own stream (>= 1) */
     int32_t max_batch;     /* most requests merged into one batch (>= 1) */
     int32_t queue_cap;     /* most requests waiting for admission; nd_submit returns ND_EBUSY beyond */
-    int32_t flags;         /* how a worker launches a batch's peeling loop: 0 or ND_PEEL_LOOP_GRAPH (a CUDA
-                              graph per batch; the workers' batches share the SMs), ND_PEEL_PERSISTENT
-                              (one cooperative kernel per batch, holding every SM; batches take turns) */
+    int32_t flags;         /* how a worker launches a batch's peeling loop: ND_PEEL_LOOP_GRAPH (a CUDA graph
+                              per batch; the workers' batches share the SMs), ND_PEEL_PERSISTENT (one
+                              cooperative kernel per batch, holding every SM; batches take turns), or 0
+                              (a cooperative kernel on 1 / workers of the SMs for batches of up to 2^20
+                              r-cliques, a CUDA graph for larger ones; the batches share the SMs) */
 } nd_server_cfg;
 
 typedef struct nd_result {

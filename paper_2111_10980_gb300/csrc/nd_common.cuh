@@ -390,6 +390,7 @@ struct PeelView {
     // (2,3) with contraction: the lists' current lengths and those after the previous contraction; else NULL
     int32_t* inc_len;
     int32_t* inc_prev;
+    int32_t grid_share;  // persistent kernel: it takes 1 / grid_share of the GPU's blocks
     // driving-list length above which Update defers an r-clique to the heavy phase (0: the
     // variant's built-in threshold)
     int64_t heavy_work;

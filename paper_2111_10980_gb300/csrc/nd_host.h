@@ -35,6 +35,7 @@ struct nd_ctx {
     int64_t barrier_ns = 0;
     int64_t count_limit = 0;
     int32_t limit_flags = 0;
+    int peel_share = 1;  // of a server's worker: the workers whose peel kernels share the GPU
     int64_t inc_bytes = (int64_t)16 << 30;  // most device bytes of a decomposition's incidence lists
     void* stage = nullptr;  // pinned staging of batches (grown on demand)
     size_t stage_bytes = 0;

@@ -2269,6 +2269,7 @@ cudaError_t launch_peel_loop(const GraphView& g, const PeelView<CT>& P, cudaStre
     }
     if (per_sm < 1) return cudaErrorCooperativeLaunchTooLarge;
     int blocks = nd_sm_count() * (per_sm < 2 ? per_sm : 2);
+    if (P.grid_share > 1) blocks = blocks / P.grid_share > 8 ? blocks / P.grid_share : 8;
     GraphView gv = g;
     PeelView<CT> pv = P;
     void* args[] = {&gv, &pv};

@@ -160,7 +160,7 @@ int host_threads() {
 // Runs one union decomposition for the requests in idx (all with the same (r,s)). A request whose
 // CSR fails a check gets ND_EINVAL and is left out; the others run. peel_flags chooses how the
 // peeling loop is launched: nd_batch_run takes the cooperative persistent kernel (one launch for
-// the whole loop), the server's workers the loop graph, so that their batches share the SMs.
+// the whole loop), the server's workers what their configuration says (a share of the SMs by default).
 int run_group(nd_ctx* ctx, nd_request* const* reqs, std::vector<int> idx, nd_batch_stats* st, int peel_flags) {
     int r = reqs[idx[0]]->r, s = reqs[idx[0]]->s;
     cudaStream_t stream = ctx->stream;
@@ -437,8 +437,7 @@ static void worker_loop(nd_server* sv, int w) {
         double t0 = now_ms();
         std::vector<nd_request*> reqs(batch.size());
         for (size_t i = 0; i < batch.size(); ++i) reqs[i] = &batch[i]->req;
-        batch_impl(ctx, reqs.data(), (int)reqs.size(), nullptr,
-                   sv->cfg.flags == ND_PEEL_PERSISTENT ? ND_PEEL_PERSISTENT : ND_PEEL_LOOP_GRAPH);
+        batch_impl(ctx, reqs.data(), (int)reqs.size(), nullptr, sv->cfg.flags);
         double t1 = now_ms();
         {
             std::lock_guard<std::mutex> lk(sv->mu);
@@ -479,6 +478,7 @@ extern "C" int nd_server_create(nd_ctx* ctx, const nd_server_cfg* cfg, nd_server
         c->max_rounds = ctx->max_rounds;
         c->barrier_ns = ctx->barrier_ns;
         c->count_limit = ctx->count_limit;
+        c->peel_share = cfg->workers;
         for (int i = 0; i < 64; ++i) {
             c->tune_heavy[i] = ctx->tune_heavy[i];
             c->tune_flags[i] = ctx->tune_flags[i];
