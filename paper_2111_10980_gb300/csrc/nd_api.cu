@@ -523,29 +523,46 @@ static int ensure_tri(nd_graph* g) {
     rc = nd_check_launch("triangle index");
     if (!rc) rc = read_back(g, (int64_t*)g->et_rp.p + m, &tot[0], "triangle index");
     if (!rc) rc = read_back(g, (int64_t*)g->tbase.p + m, &tot[1], "triangle index");
-    nd_free(c, sigma);
     nd_free(c, up);
     nd_free(c, tmp);
-    if (rc) return rc;
+    if (rc) {
+        nd_free(c, sigma);
+        return rc;
+    }
     int64_t n3 = tot[1];
-    if (tot[0] != 3 * n3) return nd_set_error(ND_EINTERNAL, "triangle index: %lld entries for %lld triangles",
-                                              (long long)tot[0], (long long)n3);
-    if (n3 > INT32_MAX) return nd_set_error(ND_EOVERFLOW, "%lld triangles: more than 2^31-1", (long long)n3);
-    if ((rc = nd_alloc(c, g->et_w, sizeof(int32_t) * std::max<int64_t>(3 * n3, 1))) ||
+    if (tot[0] != 3 * n3)
+        rc = nd_set_error(ND_EINTERNAL, "triangle index: %lld entries for %lld triangles", (long long)tot[0],
+                          (long long)n3);
+    else if (n3 > INT32_MAX)
+        rc = nd_set_error(ND_EOVERFLOW, "%lld triangles: more than 2^31-1", (long long)n3);
+    if (rc || (rc = nd_alloc(c, g->et_w, sizeof(int32_t) * std::max<int64_t>(3 * n3, 1))) ||
         (rc = nd_alloc(c, g->et_t, sizeof(int32_t) * std::max<int64_t>(3 * n3, 1))) ||
         (rc = nd_alloc(c, g->tri_e, sizeof(int32_t) * std::max<int64_t>(3 * n3, 1))) ||
-        (rc = nd_alloc(c, g->tri_pos, sizeof(int32_t) * std::max<int64_t>(3 * n3, 1))))
+        (rc = nd_alloc(c, g->tri_pos, sizeof(int32_t) * std::max<int64_t>(3 * n3, 1)))) {
+        nd_free(c, sigma);
         return rc;
+    }
+    // scratch of the short lists; without room for it every list is intersected out of the rows
+    DGroup scratch;
+    DBuf cursor, entries;
+    scratch.add(cursor, sizeof(int32_t) * m);
+    scratch.add(entries, sizeof(int32_t) * 9 * n3);
+    const bool gather = n3 > 0 && scratch.alloc(c) == ND_OK;
+    if (gather) cudaMemsetAsync(cursor.p, 0, sizeof(int32_t) * m, st);
     g->n3 = n3;
-    ND_TRY(scalar_zero(g));
+    scalar_zero(g);  // a failure surfaces at the launch check below
     v = nd_view(g);
     nd_edge_fill(v, (int64_t*)g->et_rp.p, (int64_t*)g->tbase.p, (int32_t*)g->et_w.p, (int32_t*)g->et_t.p,
-                 (int32_t*)g->tri_e.p, (int32_t*)g->tri_pos.p, (int*)g->scal.p, st);
+                 (int32_t*)g->tri_e.p, (int32_t*)g->tri_pos.p, (const int32_t*)sigma.p,
+                 gather ? (int32_t*)cursor.p : nullptr, gather ? (int32_t*)entries.p : nullptr, (int*)g->scal.p, st);
     v = nd_view(g);
     nd_edge_fill_tid(v, (int32_t*)g->et_t.p, (int32_t*)g->tri_pos.p, st);
     int err = 0;
-    ND_TRY(nd_check_launch("triangle index"));
-    ND_TRY(read_back(g, g->scal.p, &err, "triangle index"));
+    rc = nd_check_launch("triangle index");
+    if (!rc) rc = read_back(g, g->scal.p, &err, "triangle index");
+    scratch.free(c);
+    nd_free(c, sigma);
+    if (rc) return rc;
     if (err)
         return nd_set_error(ND_EINVAL, "the CSR is not a simple graph in ascending rows; load it with ND_VALIDATE for "
                                        "details");
