@@ -202,7 +202,7 @@ __device__ __forceinline__ bool nd_prefer_merge(int64_t n_short, int64_t n_long)
     return n_long <= 8 * n_short + 64;
 }
 
-__device__ __forceinline__ int64_t nd_atomic_dec(int32_t* p) { return (int64_t)atomicSub(p, 1); }
+__device__ __forceinline__ int32_t nd_atomic_dec(int32_t* p) { return atomicSub(p, 1); }
 __device__ __forceinline__ int64_t nd_atomic_dec(int64_t* p) {
     return (int64_t)atomicAdd(reinterpret_cast<unsigned long long*>(p), 0xffffffffffffffffull);
 }

@@ -826,12 +826,16 @@ struct RoundEnv {
     const PeelView<CT>* Q;
     const PeelHot* s;
     int32_t t;
-    int64_t k, hi;
+    // in the counts' own type: the count from which a decrement schedules an r-clique (k + 1), and the
+    // window's bound (a value no count has when the window is open above)
+    CT k1, hi;
 };
+
+__device__ __forceinline__ int64_t round_level(const PeelHot& s) { return (s.mode & ND_MODE_ADV) ? knew_of(s) : s.k; }
 
 template <typename CT>
 __device__ __forceinline__ RoundEnv<CT> round_env(const PeelView<CT>& P, const PeelView<CT>* Q, const PeelHot* s) {
-    return RoundEnv<CT>{P, Q, s, s->t, (s->mode & ND_MODE_ADV) ? knew_of(*s) : s->k, s->hi};
+    return RoundEnv<CT>{P, Q, s, s->t, (CT)(round_level(*s) + 1), (int64_t)(CT)s->hi == s->hi ? (CT)s->hi : (CT)-1};
 }
 
 // |A| and A of the round
@@ -851,8 +855,9 @@ struct UpdCounters {
 // bucket window's bound and joins N. Most decrements do neither, and so the rest is out of
 // line, with its pointers in shared memory, and costs the loops around it no registers.
 template <typename CT>
-__device__ __noinline__ void after_dec_rest(const PeelView<CT>* Q, const PeelHot* s, int32_t x, int64_t o, int64_t k) {
+__device__ __noinline__ void after_dec_rest(const PeelView<CT>* Q, const PeelHot* s, int32_t x, int64_t o) {
     PeelCtl* c = Q->ctl;
+    const int64_t k = round_level(*s);
     // dense buckets: a count above k + 1 moves down one bucket; at k + 1 the r-clique is scheduled
     // now and leaves the buckets; at or below k it was scheduled already
     if (Q->bcnt && o > k) {
@@ -874,15 +879,15 @@ __device__ __noinline__ void after_dec_rest(const PeelView<CT>* Q, const PeelHot
 }
 
 template <typename CT>
-__device__ __forceinline__ void after_dec(const RoundEnv<CT>& E, int32_t x, int64_t o) {
-    if (o == E.k + 1 || o == E.hi || E.P.bcnt) after_dec_rest(E.Q, E.s, x, o, E.k);
+__device__ __forceinline__ void after_dec(const RoundEnv<CT>& E, int32_t x, CT o) {
+    if (o == E.k1 || o == E.hi || E.P.bcnt) after_dec_rest(E.Q, E.s, x, (int64_t)o);
 }
 
 // The same for up to four r-cliques of every lane at once (bit i of what: x_i falls to k; bit 4 + i: it
 // falls below the window's bound), with one counter update per list for all of them: four calls of
 // the above are four trips to L2, one after another, in the chain that a short round waits for.
 template <typename CT>
-__device__ __noinline__ void after_dec4(const PeelView<CT>* Q, const PeelHot* s, int4 x4, unsigned what, int64_t k) {
+__device__ __noinline__ void after_dec4(const PeelView<CT>* Q, const PeelHot* s, int4 x4, unsigned what) {
     PeelCtl* c = Q->ctl;
     const unsigned act = __activemask(), below = act & nd_lanemask_lt();
     const int lane = threadIdx.x & 31, leader = __ffs(act) - 1;
@@ -905,12 +910,14 @@ __device__ __noinline__ void after_dec4(const PeelView<CT>* Q, const PeelHot* s,
     int32_t* win = s->wn ^ (adv ? 1 : 0) ? Q->N[1] : Q->N[0];
     const int32_t x[4] = {x4.x, x4.y, x4.z, x4.w};
     const uint32_t cap = Q->cap;
-    const int32_t t1 = s->t + 1;
+    const int32_t t1 = s->t + 1, k = (int32_t)round_level(*s);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         if (what >> i & 1u) {
             Q->rnd[x[i]] = t1;
-            Q->core[x[i]] = (int32_t)k;
+            Q->core[x[i]] = k;
+            if (Q->et_rnd) set_tri_round(*Q, x[i], t1);
+            mark_a(*Q, x[i]);
             if (at[0] < cap)
                 next[at[0]++] = x[i];
             else
@@ -923,6 +930,21 @@ __device__ __noinline__ void after_dec4(const PeelView<CT>* Q, const PeelHot* s,
                 atomicExch(&c->err, 1);
         }
     }
+}
+
+// The (3,4) form: the other three triangles of a destroyed 4-clique; a count that was not decremented
+// comes as k.
+template <typename CT>
+__device__ __forceinline__ void after_dec3(const RoundEnv<CT>& E, int32_t x0, int32_t x1, int32_t x2, CT o0, CT o1, CT o2) {
+    if (E.P.bcnt) {
+        after_dec(E, x0, o0);
+        after_dec(E, x1, o1);
+        after_dec(E, x2, o2);
+        return;
+    }
+    const unsigned what = (o0 == E.k1 ? 1u : 0u) | (o1 == E.k1 ? 2u : 0u) | (o2 == E.k1 ? 4u : 0u) |
+                          (o0 == E.hi ? 16u : 0u) | (o1 == E.hi ? 32u : 0u) | (o2 == E.hi ? 64u : 0u);
+    if (what) after_dec4(E.Q, E.s, make_int4(x0, x1, x2, -1), what);
 }
 
 // Whether a member of a destroyed S with round tag r has its count decremented on the device: not
@@ -946,7 +968,7 @@ __device__ __forceinline__ void update_func(const RoundEnv<CT>& E, int32_t R, co
     if (owner != R) return;
     k.listed++;
     // issue every decrement before looking at any result (the atomics overlap in flight)
-    int64_t old[M];
+    CT old[M];
 #pragma unroll
     for (int i = 0; i < M; ++i) old[i] = dec_live(ro[i], E.t) ? nd_atomic_dec(&E.P.cnt[o[i]]) : 0;
 #pragma unroll
@@ -1353,13 +1375,11 @@ struct Upd34 {
         if (r2 < E.t || (r2 == E.t && id2 < R)) return;
         k.listed++;
         // issue the decrements before looking at any result (the atomics overlap in flight)
-        int64_t o0 = dec_live(r0, E.t) ? nd_atomic_dec(&E.P.cnt[id0]) : 0;
-        int64_t o1 = dec_live(r1, E.t) ? nd_atomic_dec(&E.P.cnt[id1]) : 0;
-        int64_t o2 = dec_live(r2, E.t) ? nd_atomic_dec(&E.P.cnt[id2]) : 0;
+        CT o0 = dec_live(r0, E.t) ? nd_atomic_dec(&E.P.cnt[id0]) : (CT)(E.k1 - 1);
+        CT o1 = dec_live(r1, E.t) ? nd_atomic_dec(&E.P.cnt[id1]) : (CT)(E.k1 - 1);
+        CT o2 = dec_live(r2, E.t) ? nd_atomic_dec(&E.P.cnt[id2]) : (CT)(E.k1 - 1);
         k.decs += (r0 != E.t) + (r1 != E.t) + (r2 != E.t);
-        if (dec_live(r0, E.t)) after_dec(E, id0, o0);
-        if (dec_live(r1, E.t)) after_dec(E, id1, o1);
-        if (dec_live(r2, E.t)) after_dec(E, id2, o2);
+        after_dec3(E, id0, id1, id2, o0, o1, o2);
     }
 
     // Light Update over a group of at most 32 triangles of A, with a queue of candidates per warp.
@@ -1506,7 +1526,7 @@ struct Upd34 {
                 p2[x] = *reinterpret_cast<const int4*>(t2[x] + s2[x]);
             }
         }
-        int64_t o0[N], o1[N], o2[N];
+        CT o0[N], o1[N], o2[N];
 #pragma unroll
         for (int x = 0; x < N; ++x) {
             i1[x] = r1[x] = i2[x] = r2[x] = 0;
@@ -1518,18 +1538,16 @@ struct Upd34 {
         // the decrements of every 4-clique go out before any result is looked at
 #pragma unroll
         for (int x = 0; x < N; ++x) {
-            o0[x] = live[x] && (me[x] & 64) ? nd_atomic_dec(&E.P.cnt[id0[x]]) : 0;
-            o1[x] = live[x] && dec_live(r1[x], E.t) ? nd_atomic_dec(&E.P.cnt[i1[x]]) : 0;
-            o2[x] = live[x] && dec_live(r2[x], E.t) ? nd_atomic_dec(&E.P.cnt[i2[x]]) : 0;
+            o0[x] = live[x] && (me[x] & 64) ? nd_atomic_dec(&E.P.cnt[id0[x]]) : (CT)(E.k1 - 1);
+            o1[x] = live[x] && dec_live(r1[x], E.t) ? nd_atomic_dec(&E.P.cnt[i1[x]]) : (CT)(E.k1 - 1);
+            o2[x] = live[x] && dec_live(r2[x], E.t) ? nd_atomic_dec(&E.P.cnt[i2[x]]) : (CT)(E.k1 - 1);
         }
 #pragma unroll
         for (int x = 0; x < N; ++x) {
             if (!live[x]) continue;
             k.listed++;
             k.decs += !(me[x] & 32) + (r1[x] != E.t) + (r2[x] != E.t);
-            if (me[x] & 64) after_dec(E, id0[x], o0[x]);
-            if (dec_live(r1[x], E.t)) after_dec(E, i1[x], o1[x]);
-            if (dec_live(r2[x], E.t)) after_dec(E, i2[x], o2[x]);
+            after_dec3(E, id0[x], i1[x], i2[x], o0[x], o1[x], o2[x]);
         }
     }
 };
@@ -1602,15 +1620,15 @@ struct UpdInc {
             const int4 w = v[kVec ? i : 0];
             const int32_t x[4] = {w.x, w.y, w.z, w.w};
             int32_t r[4];
-            int64_t o[4];
+            CT o[4];
 #pragma unroll
             for (int m = 0; m < 4; ++m) r[m] = x[m] >= 0 && x[m] != R ? E.P.rnd[x[m]] : E.t;
             if (shared) {
 #pragma unroll
-                for (int m = 0; m < 4; ++m) o[m] = x[m] >= 0 && x[m] != R ? nd_atomic_dec(&E.P.cnt[x[m]]) : E.k;
+                for (int m = 0; m < 4; ++m) o[m] = x[m] >= 0 && x[m] != R ? nd_atomic_dec(&E.P.cnt[x[m]]) : (CT)(E.k1 - 1);
             } else {
 #pragma unroll
-                for (int m = 0; m < 4; ++m) o[m] = dec_live(r[m], E.t) ? nd_atomic_dec(&E.P.cnt[x[m]]) : E.k;
+                for (int m = 0; m < 4; ++m) o[m] = dec_live(r[m], E.t) ? nd_atomic_dec(&E.P.cnt[x[m]]) : (CT)(E.k1 - 1);
             }
             unsigned what = 0;
 #pragma unroll
@@ -1619,9 +1637,9 @@ struct UpdInc {
                 if (E.P.bcnt)
                     after_dec(E, x[m], o[m]);
                 else
-                    what |= (o[m] == E.k + 1 ? 1u : 0u) << m | (o[m] == E.hi ? 16u : 0u) << m;
+                    what |= (o[m] == E.k1 ? 1u : 0u) << m | (o[m] == E.hi ? 16u : 0u) << m;
             }
-            if (what) after_dec4(E.Q, E.s, w, what, E.k);
+            if (what) after_dec4(E.Q, E.s, w, what);
         }
     }
 };
@@ -1708,10 +1726,42 @@ __device__ __forceinline__ int64_t heavy_limit(const PeelView<CT>& P) {
     return h;
 }
 
+// A round with fewer r-cliques than half the warps: 2^shift warps share each one, 32 candidates each in turn.
 template <typename CT, typename U>
-__device__ __forceinline__ void phase_update(const GraphView& g, const PeelView<CT>& P, const PeelView<CT>* Q,
-                                             const PeelHot& s, const Team& T, unsigned long long* listed,
-                                             unsigned long long* decs) {
+__device__ __forceinline__ void shared_round(const GraphView& g, const PeelView<CT>& P, const PeelView<CT>* Q,
+                                             const PeelHot& s, const int32_t* A, unsigned nA, const Team& T,
+                                             UpdCounters& k) {
+    const RoundEnv<CT> E = round_env(P, Q, &s);
+    const unsigned shift = split_shift(nA, T), i = T.warp >> shift, part = T.warp & ((1u << shift) - 1u);
+    const int lane = threadIdx.x & 31;
+    if (i >= nA) return;
+    const int32_t R = A[i];
+    Prep q;
+    int64_t n0 = U::prep(g, P, R, q), j0 = part * 32 + lane, dj = (int64_t)32 << shift;
+    if constexpr (is_inc<U>::value) q.hk[0] = 1;
+    if (part == 0 && lane == 0) unmark_a(P, R);
+    if (n0 > heavy_limit<U>(P) << shift) {
+        // one of the warps hands it over; with no room there it lists all of it itself
+        if (part != 0 || defer_heavy(Q, R)) n0 = 0;
+        j0 = lane;
+        dj = 32;
+    }
+#pragma unroll 1
+    for (int64_t j = j0; j < n0; j += dj) U::cand(g, E, R, q, j, k);
+}
+
+// The same out of line, for a variant whose other rounds are short of registers (all pointers in shared
+// memory).
+template <typename CT, typename U>
+__device__ __noinline__ void shared_round_apart(const GraphView* H, const PeelView<CT>* Q, const PeelHot& s,
+                                                const int32_t* A, unsigned nA, const Team& T, UpdCounters& k) {
+    shared_round<CT, U>(*H, *Q, Q, s, A, nA, T, k);
+}
+
+template <typename CT, typename U>
+__device__ __forceinline__ void phase_update(const GraphView& g, const PeelView<CT>& P, const GraphView* H,
+                                             const PeelView<CT>* Q, const PeelHot& s, const Team& T,
+                                             unsigned long long* listed, unsigned long long* decs) {
     if (s.done) return;
     const RoundEnv<CT> E = round_env(P, Q, &s);
     const int32_t* A = pick(P.A, s.wa);
@@ -1719,25 +1769,11 @@ __device__ __forceinline__ void phase_update(const GraphView& g, const PeelView<
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     UpdCounters k;
     if constexpr (!is_staged<U>::value) {
-        const unsigned shift = split_shift(nA, T);
-        if (shift) {
-            // fewer r-cliques than half the warps: 2^shift warps share each one, 32 candidates each in turn
-            const unsigned i = T.warp >> shift, part = T.warp & ((1u << shift) - 1u);
-            if (i < nA) {
-                const int32_t R = A[i];
-                Prep q;
-                int64_t n0 = U::prep(g, P, R, q), j0 = part * 32 + lane, dj = (int64_t)32 << shift;
-                if constexpr (is_inc<U>::value) q.hk[0] = 1;
-                if (part == 0 && lane == 0) unmark_a(P, R);
-                if (n0 > heavy_limit<U>(P) << shift) {
-                    // one of the warps hands it over; with no room there it lists all of it itself
-                    if (part != 0 || defer_heavy(Q, R)) n0 = 0;
-                    j0 = lane;
-                    dj = 32;
-                }
-#pragma unroll 1
-                for (int64_t j = j0; j < n0; j += dj) U::cand(g, E, R, q, j, k);
-            }
+        if (split_shift(nA, T)) {
+            if constexpr (is_queued<U>::value)
+                shared_round_apart<CT, U>(H, Q, s, A, nA, T, k);
+            else
+                shared_round<CT, U>(g, P, Q, s, A, nA, T, k);
             add_counters(listed, decs, k);
             return;
         }
@@ -1889,9 +1925,13 @@ __device__ __forceinline__ void phase_heavy_pairs(const GraphView& g, const Peel
 template <typename CT, typename U>
 __global__ void k_update(GraphView g, PeelView<CT> P) {
     __shared__ PeelView<CT> Q;
-    if (threadIdx.x == 0) Q = P;
+    __shared__ GraphView h;
+    if (threadIdx.x == 0) {
+        Q = P;
+        h = g;
+    }
     __syncthreads();
-    phase_update<CT, U>(g, P, &Q, P.ctl->h, grid_team(), &P.ctl->listed, &P.ctl->decs);
+    phase_update<CT, U>(g, P, &h, &Q, P.ctl->h, grid_team(), &P.ctl->listed, &P.ctl->decs);
 }
 template <typename CT, typename U>
 __global__ void k_update_heavy(GraphView g, PeelView<CT> P) {
@@ -2227,7 +2267,7 @@ __global__ void __launch_bounds__(512, 2) k_peel_loop(GraphView g, PeelView<CT> 
                 if (!grid_barrier(&L, kNothing)) return;
                 book(3, tr);
             }
-            phase_update<CT, U>(g, P, &Q, s, T, &L.listed, &L.decs);
+            phase_update<CT, U>(g, P, &h, &Q, s, T, &L.listed, &L.decs);
             if (!grid_barrier(&L, kAfterUpdate)) return;
             book(4, tr);
             continue;

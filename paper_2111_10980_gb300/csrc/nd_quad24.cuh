@@ -65,6 +65,10 @@ __device__ __forceinline__ void quad24_list(const GraphView& g, Sink& sink) {
             }
             c += __popc(mk);
         }
+        if (c < 2) {  // a 4-clique needs two vertices of I
+            __syncwarp();
+            continue;
+        }
         if constexpr (Sink::kTally)
             for (int i = lane; i < c && i < kC24; i += 32) s_c[wid][i] = 0;
         __syncwarp();
