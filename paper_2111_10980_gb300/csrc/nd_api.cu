@@ -453,7 +453,7 @@ int nd_kcore_rounds(nd_graph* g, DBuf& rnd_out);  // degeneracy ranking (below)
 static int build_dg(nd_graph* g, int mode) {
     nd_ctx* c = g->ctx;
     cudaStream_t st = c->stream;
-    DBuf key, outdeg, tmp;
+    DBuf key, outdeg, tmp, tail;
     int rc = ND_OK;
     const int32_t* key_hi = nullptr;
     if (mode == ND_ORIENT_DEGENERACY) {
@@ -462,6 +462,7 @@ static int build_dg(nd_graph* g, int mode) {
     }
     for (DBuf* b : {&g->dg_rp, &g->dg_col, &g->dg_eid}) nd_free(c, *b);
     if ((rc = nd_alloc(c, outdeg, sizeof(int64_t) * std::max<int64_t>(g->n, 1))) ||
+        (rc = nd_alloc(c, tail, sizeof(int32_t) * std::max<int64_t>(nd_dg_segments(g->m), 1))) ||
         (rc = nd_alloc(c, tmp, nd_scan_tmp_bytes(g->n))) ||
         (rc = nd_alloc(c, g->dg_rp, sizeof(int64_t) * (g->n + 1))) ||
         (rc = nd_alloc(c, g->dg_col, sizeof(int32_t) * std::max<int64_t>(g->m, 1))) ||
@@ -469,17 +470,20 @@ static int build_dg(nd_graph* g, int mode) {
         nd_free(c, key);
         nd_free(c, outdeg);
         nd_free(c, tmp);
+        nd_free(c, tail);
         return rc;
     }
     GraphView v = nd_view(g);
-    nd_dg_count(v, key_hi, (int64_t*)outdeg.p, st);
+    cudaMemsetAsync(outdeg.p, 0, outdeg.bytes, st);  // a failure surfaces at the launch check below
+    nd_dg_count(v, key_hi, (int64_t*)outdeg.p, (int32_t*)tail.p, st);
     nd_scan_i64((const int64_t*)outdeg.p, (int64_t*)g->dg_rp.p, g->n, tmp.p, st);
     v = nd_view(g);
-    nd_dg_fill(v, key_hi, (int64_t*)g->dg_rp.p, (int32_t*)g->dg_col.p, (int32_t*)g->dg_eid.p, st);
+    nd_dg_fill(v, key_hi, (int64_t*)g->dg_rp.p, (const int32_t*)tail.p, (int32_t*)g->dg_col.p, (int32_t*)g->dg_eid.p, st);
     rc = nd_check_launch("orientation");
     nd_free(c, key);
     nd_free(c, outdeg);
     nd_free(c, tmp);
+    nd_free(c, tail);
     if (rc) return rc;
     g->orient = mode;
     return ND_OK;

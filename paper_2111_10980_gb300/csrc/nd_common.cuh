@@ -429,9 +429,11 @@ void nd_build_split(const int64_t* rp, const int32_t* col, int32_t n, int64_t* s
                     cudaStream_t st);
 void nd_build_pos2e(const GraphView& g, int32_t* pos2e, int32_t* eu, int32_t* ev, int* err, cudaStream_t st);
 // key(v) = (key_hi[v] or degree, v); key_hi NULL means degree
-void nd_dg_count(const GraphView& g, const int32_t* key_hi, int64_t* outdeg, cudaStream_t st);
-void nd_dg_fill(const GraphView& g, const int32_t* key_hi, int64_t* dg_rp_in, int32_t* dg_col, int32_t* dg_eid,
-                cudaStream_t st);
+// outdeg zeroed by the caller; tail: nd_dg_segments(m) int32, from the count to the fill
+int64_t nd_dg_segments(int64_t m);
+void nd_dg_count(const GraphView& g, const int32_t* key_hi, int64_t* outdeg, int32_t* tail, cudaStream_t st);
+void nd_dg_fill(const GraphView& g, const int32_t* key_hi, int64_t* dg_rp, const int32_t* tail, int32_t* dg_col,
+                int32_t* dg_eid, cudaStream_t st);
 // per canonical edge: sigma += |N(a) ∩ N(b)|, up += |{w in N(a) ∩ N(b) : w > b}| (zeroed by the caller)
 void nd_edge_support(const GraphView& g, int32_t* sigma, int32_t* up, cudaStream_t st);
 // cursor (m, zeroed) and entries (9 n3): scratch of the short lists, or NULL: every list out of the rows
