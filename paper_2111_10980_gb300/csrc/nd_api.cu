@@ -1243,10 +1243,14 @@ int nd_decompose_dev(nd_graph* g, int r, int s, int count_width, int flags, Peel
         if (use_inc)
             for (DBuf* b : {&g->hoff, &g->htab, &g->hpos}) nd_free(c, *b);  // the lists replace it
     }
-    if (!rc)
-        rc = (w == 8) ? run_peel<int64_t>(g, r, s, cnt, n_r, flags, po, use_inc ? &inc : nullptr)
-                      : run_peel<int32_t>(g, r, s, cnt, n_r, flags, po, use_inc ? &inc : nullptr);
+    auto peel = [&](const IncBufs* lists) {
+        return (w == 8) ? run_peel<int64_t>(g, r, s, cnt, n_r, flags, po, lists)
+                        : run_peel<int32_t>(g, r, s, cnt, n_r, flags, po, lists);
+    };
+    if (!rc) rc = peel(use_inc ? &inc : nullptr);
     nd_free_inc(c, inc);
+    // the lists may have taken the room of the peel's own buffers, which are allocated before it begins
+    if (use_inc && rc == ND_ENOMEM) rc = peel(nullptr);
     float tc = 0, tp = 0, th = 0;
     if (!rc) {
         cudaEventElapsedTime(&tc, e0, e1);

@@ -430,7 +430,13 @@ extern "C" int nd_hierarchy(nd_graph* g, int r, int s, const int32_t* core, int3
         return rc;
     }
     const int64_t nb = (int64_t)lo_hi[1] + 1;
-    if ((rc = nd_alloc(c, b[kHist], 4 * nb))) {
+    rc = nd_alloc(c, b[kHist], 4 * nb);
+    if (rc == ND_ENOMEM && lists) {  // the lists may have taken the room
+        nd_free_inc(c, inc);
+        lists = false;
+        rc = nd_alloc(c, b[kHist], 4 * nb);
+    }
+    if (rc) {
         release();
         return rc;
     }

@@ -65,3 +65,45 @@ def test_no_s_clique(nd, r, s):
         assert st["n_s"] == 0 and not np.any(core) and st["rho"] == (1 if st["n_r"] else 0)
     finally:
         nd.nd_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("r,s", [(2, 3), (2, 4), (3, 5)])
+def test_the_memory_of_a_run_without_lists_is_enough(nd, r, s):
+    """A decomposition succeeds in exactly the bytes it needs without lists, wherever a run that tries
+    them first runs out."""
+    import torch
+
+    g = gg.with_planted(gg.chung_lu(1200, 6.0, 2.3, seed=91), 30 if (r, s) == (2, 4) else 12, 14, 20, 0.85, seed=92)
+    want = orc.decompose(g, r, s)
+    rows = 4 * ((math.comb(s, r) + 3) // 4 * 4) * want.n_s
+    alloc, free = nd.torch_allocator_hooks(0)
+    held = {"now": 0, "peak": 0}
+
+    def run(refuse, cap):
+        held.update(now=0, peak=0)
+
+        def take(nbytes, stream):
+            if refuse and nbytes >= rows or held["now"] + nbytes > cap:
+                return 0
+            held["now"] += nbytes
+            held["peak"] = max(held["peak"], held["now"])
+            return alloc(nbytes, stream)
+
+        def give(p, nbytes, stream):
+            held["now"] -= nbytes
+            free(p, nbytes, stream)
+
+        ctx = nd.nd_ctx_create(0, stream=torch.cuda.Stream())
+        nd.nd_ctx_set_allocator(ctx, take, give)
+        try:
+            G = nd.nd_load_csr(ctx, g.rowptr, g.col)
+            core, rnd, st = nd.nd_decompose(G, r, s)
+            nd.nd_graph_free(G)
+        finally:
+            nd.nd_ctx_destroy(ctx)
+        assert np.array_equal(core, want.core) and np.array_equal(rnd, want.round) and st["listed"] == want.n_s
+        return held["peak"]
+
+    alone = run(True, 1 << 40)
+    for extra in (0, rows // 2, rows, 2 * rows):
+        run(False, alone + extra)
