@@ -855,24 +855,23 @@ struct UpdCounters {
 // bucket window's bound and joins N. Most decrements do neither, and so the rest is out of
 // line, with its pointers in shared memory, and costs the loops around it no registers.
 template <typename CT>
-__device__ __noinline__ void after_dec_rest(const PeelView<CT>* Q, const PeelHot* s, int32_t x, int64_t o) {
+__device__ __noinline__ void after_dec_rest(const PeelView<CT>* Q, const PeelHot* s, int32_t x, CT o, CT k1) {
     PeelCtl* c = Q->ctl;
-    const int64_t k = round_level(*s);
     // dense buckets: a count above k + 1 moves down one bucket; at k + 1 the r-clique is scheduled
     // now and leaves the buckets; at or below k it was scheduled already
-    if (Q->bcnt && o > k) {
+    if (Q->bcnt && (int64_t)o > round_level(*s)) {
         atomicSub(&Q->bcnt[o], 1u);
-        if (o > k + 1) atomicAdd(&Q->bcnt[o - 1], 1u);
+        if (o != k1) atomicAdd(&Q->bcnt[o - 1], 1u);
     }
-    if (o == k + 1) {
+    if (o == k1) {
         const int32_t t1 = s->t + 1;
         Q->rnd[x] = t1;
-        Q->core[x] = (int32_t)k;
+        Q->core[x] = (int32_t)(k1 - 1);
         if (Q->et_rnd) set_tri_round(*Q, x, t1);
         mark_a(*Q, x);
         nd_append(&c->h.nNext[s->t & 1], s->wa ? Q->A[0] : Q->A[1], Q->cap, x, &c->err);
     }
-    if (o == s->hi) {
+    if ((int64_t)o == s->hi) {
         const bool adv = s->mode & ND_MODE_ADV;
         nd_append(adv ? &c->h.nN2 : &c->h.nN, s->wn ^ (adv ? 1 : 0) ? Q->N[1] : Q->N[0], Q->cap, x, &c->err);
     }
@@ -880,14 +879,14 @@ __device__ __noinline__ void after_dec_rest(const PeelView<CT>* Q, const PeelHot
 
 template <typename CT>
 __device__ __forceinline__ void after_dec(const RoundEnv<CT>& E, int32_t x, CT o) {
-    if (o == E.k1 || o == E.hi || E.P.bcnt) after_dec_rest(E.Q, E.s, x, (int64_t)o);
+    if (o == E.k1 || o == E.hi || E.P.bcnt) after_dec_rest(E.Q, E.s, x, o, E.k1);
 }
 
 // The same for up to four r-cliques of every lane at once (bit i of what: x_i falls to k; bit 4 + i: it
 // falls below the window's bound), with one counter update per list for all of them: four calls of
 // the above are four trips to L2, one after another, in the chain that a short round waits for.
 template <typename CT>
-__device__ __noinline__ void after_dec4(const PeelView<CT>* Q, const PeelHot* s, int4 x4, unsigned what) {
+__device__ __noinline__ void after_dec4(const PeelView<CT>* Q, const PeelHot* s, int4 x4, unsigned what, CT k1) {
     PeelCtl* c = Q->ctl;
     const unsigned act = __activemask(), below = act & nd_lanemask_lt();
     const int lane = threadIdx.x & 31, leader = __ffs(act) - 1;
@@ -910,7 +909,7 @@ __device__ __noinline__ void after_dec4(const PeelView<CT>* Q, const PeelHot* s,
     int32_t* win = s->wn ^ (adv ? 1 : 0) ? Q->N[1] : Q->N[0];
     const int32_t x[4] = {x4.x, x4.y, x4.z, x4.w};
     const uint32_t cap = Q->cap;
-    const int32_t t1 = s->t + 1, k = (int32_t)round_level(*s);
+    const int32_t t1 = s->t + 1, k = (int32_t)(k1 - 1);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         if (what >> i & 1u) {
@@ -944,7 +943,7 @@ __device__ __forceinline__ void after_dec3(const RoundEnv<CT>& E, int32_t x0, in
     }
     const unsigned what = (o0 == E.k1 ? 1u : 0u) | (o1 == E.k1 ? 2u : 0u) | (o2 == E.k1 ? 4u : 0u) |
                           (o0 == E.hi ? 16u : 0u) | (o1 == E.hi ? 32u : 0u) | (o2 == E.hi ? 64u : 0u);
-    if (what) after_dec4(E.Q, E.s, make_int4(x0, x1, x2, -1), what);
+    if (what) after_dec4(E.Q, E.s, make_int4(x0, x1, x2, -1), what, E.k1);
 }
 
 // Whether a member of a destroyed S with round tag r has its count decremented on the device: not
@@ -1639,7 +1638,7 @@ struct UpdInc {
                 else
                     what |= (o[m] == E.k1 ? 1u : 0u) << m | (o[m] == E.hi ? 16u : 0u) << m;
             }
-            if (what) after_dec4(E.Q, E.s, w, what);
+            if (what) after_dec4(E.Q, E.s, w, what, E.k1);
         }
     }
 };
