@@ -1,0 +1,62 @@
+"""Sizes at which the kernels change their way: closed forms on cliques whose edges have 127, 128 and
+129 common neighbours (lists gathered and ordered up to 128, merged out of the rows beyond), next to a
+hub whose row runs over many segments of the edge index, long runs of empty rows before, between and
+after, and graphs too small to fill a warp."""
+import itertools
+
+import numpy as np
+import pytest
+
+import graphgen as gg
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def nd():
+    import paper_2111_10980_gb300 as nd
+
+    nd.lib()
+    return nd
+
+
+def _graph(cliques, leaves, gap):
+    """Cliques of these sizes, then a star with that many leaves, with `gap` isolated vertices around each."""
+    us, vs, first, at = [], [], [], gap
+    for n in cliques:
+        iu, ju = np.triu_indices(n, 1)
+        us.append(iu + at)
+        vs.append(ju + at)
+        first.append(at)
+        at += n + gap
+    us.append(np.full(leaves, at + leaves // 2))  # the hub in the middle of its leaves' ids
+    vs.append(at + np.delete(np.arange(leaves + 1), leaves // 2))
+    n = at + leaves + 1 + gap
+    return gg.csr_from_edges(n, np.concatenate(us).astype(np.int32), np.concatenate(vs).astype(np.int32)), first
+
+
+@pytest.mark.parametrize("cliques,leaves,gap", [((129, 130, 131), 5000, 300), ((2, 3, 4, 5), 1, 0), ((33, 34), 70, 40)])
+def test_cliques_and_a_hub(nd, cliques, leaves, gap):
+    g, first = _graph(cliques, leaves, gap)
+    ctx = nd.nd_ctx_create(0)
+    G = nd.nd_load_csr(ctx, g.rowptr, g.col, flags=nd.ND_VALIDATE)
+    try:
+        edges = nd.nd_rcliques(G, 2)
+        assert np.array_equal(edges, g.edges())
+        tri = nd.nd_rcliques(G, 3)
+        want = [np.array(list(itertools.combinations(range(n), 3)), np.int32).reshape(-1, 3) + a
+                for n, a in zip(cliques, first)]
+        assert np.array_equal(tri, np.concatenate(want))
+        for r, s, cl in ((2, 3, edges), (3, 4, tri)):
+            core, rnd, st = nd.nd_decompose(G, r, s)
+            counts, _, n_s = nd.nd_count(G, r, s)
+            # every r-clique of K_n lies in n - r of its s-cliques, and all of them go at once
+            expect = np.zeros(len(cl), np.int64)
+            for n, a in zip(cliques, first):
+                expect[(cl[:, 0] >= a) & (cl[:, -1] < a + n)] = n - r
+            assert np.array_equal(core, expect) and np.array_equal(counts, expect), (r, s)
+            assert st["rho"] == len(np.unique(expect)) and st["listed"] == n_s == st["n_s"]
+            assert np.array_equal(rnd, np.searchsorted(np.unique(expect), expect))
+    finally:
+        nd.nd_graph_free(G)
+        nd.nd_ctx_destroy(ctx)
