@@ -440,8 +440,8 @@ static int ensure_base(nd_graph* g) {
                                        "ND_VALIDATE for details",
                             (long long)m_up, (long long)g->m);
     if (sc[0] & 1)
-        return nd_set_error(ND_EINVAL, "the CSR is not symmetric or has a self-loop; load it with ND_VALIDATE "
-                                       "for details");
+        return nd_set_error(ND_EINVAL, "the CSR is not symmetric, has a self-loop or an id out of range; load it with "
+                                       "ND_VALIDATE for details");
     unsigned long long md = sc[1];
     g->maxdeg = (int64_t)md;
     g->have_base = true;

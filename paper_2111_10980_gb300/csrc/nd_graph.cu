@@ -101,8 +101,8 @@ __device__ __forceinline__ int64_t row_of(const int64_t* __restrict__ rp, int64_
     return lo;
 }
 
-// A CSR entry whose reverse entry is missing (or a self-loop) sets *err and gets edge id 0, so
-// that no later kernel indexes outside the edge arrays.
+// A CSR entry whose reverse entry is missing, a self-loop or an id that is no vertex sets *err and gets edge
+// id 0, so that no later kernel indexes outside the edge arrays; no row is looked up by such an id.
 __global__ void k_pos2e(GraphView g, int64_t nnz, int64_t seg, int32_t* __restrict__ pos2e, int32_t* __restrict__ eu,
                         int32_t* __restrict__ ev, int* err) {
     const int lane = threadIdx.x & 31;
@@ -116,7 +116,10 @@ __global__ void k_pos2e(GraphView g, int64_t nnz, int64_t seg, int32_t* __restri
                 u = row_of(g.rp, g.n, u0, p);
                 const int32_t v = g.col[p];
                 int64_t id;
-                if (v > u) {
+                if ((uint32_t)v >= (uint32_t)g.n) {
+                    atomicOr(err, 1);
+                    id = 0;
+                } else if (v > u) {
                     id = g.ebase[u] + (p - g.split[u]);
                     if (id >= 0 && id < g.m) {
                         eu[id] = (int32_t)u;

@@ -9,6 +9,7 @@
   matches the oracle.
 * Count overflow: with a width-4 count limit below the graph's largest count, width 4 gives
   ND_EOVERFLOW, while width 8 (and the automatic choice) give the oracle's result.
+* Malformed graphs loaded without ND_VALIDATE: refused before an entry is used as an index.
 """
 import time
 
@@ -122,5 +123,26 @@ def test_limits_reject_bad_arguments(nd):
         with pytest.raises(nd.NdError) as ei:
             nd.nd_ctx_set_limits(ctx, flags=0x100)
         assert ei.value.code == nd.ND_EINVAL
+    finally:
+        nd.nd_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("bad_id", [-1, -(1 << 31), 60, (1 << 31) - 1])
+@pytest.mark.parametrize("where", ["first", "last", "all"])
+def test_ids_out_of_range_are_refused_without_validate(nd, bad_id, where):
+    """A CSR with ids that are no vertices is refused with ND_EINVAL before any row is looked up by one of
+    them, whether or not its upper and lower entries still balance."""
+    g = gg.chung_lu(60, 6.0, 2.3, seed=62)
+    col = g.col.copy()
+    col[{"first": 0, "last": -1, "all": slice(None)}[where]] = bad_id
+    ctx = nd.nd_ctx_create(0)
+    try:
+        G = nd.nd_load_csr(ctx, g.rowptr, col)
+        with pytest.raises(nd.NdError) as ei:
+            nd.nd_decompose(G, 2, 3)
+        assert ei.value.code == nd.ND_EINVAL
+        nd.nd_graph_free(G)
+        core, rnd, _ = _decompose(nd, ctx, g, 2, 3)
+        assert np.array_equal(core, orc.decompose(g, 2, 3).core)
     finally:
         nd.nd_ctx_destroy(ctx)
