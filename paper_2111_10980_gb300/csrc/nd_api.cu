@@ -442,6 +442,7 @@ static int ensure_base(nd_graph* g) {
     if (sc[0] & 1)
         return nd_set_error(ND_EINVAL, "the CSR is not symmetric, has a self-loop or an id out of range; load it with "
                                        "ND_VALIDATE for details");
+    g->rows = (int)sc[0] & 6;
     unsigned long long md = sc[1];
     g->maxdeg = (int64_t)md;
     g->have_base = true;
@@ -477,6 +478,19 @@ static int build_dg(nd_graph* g, int mode) {
     cudaMemsetAsync(outdeg.p, 0, outdeg.bytes, st);  // a failure surfaces at the launch check below
     nd_dg_count(v, key_hi, (int64_t*)outdeg.p, (int32_t*)tail.p, st);
     nd_scan_i64((const int64_t*)outdeg.p, (int64_t*)g->dg_rp.p, g->n, tmp.p, st);
+    if (g->rows) {
+        // duplicates on one side of an edge only: DG has another number of edges than the CSR
+        int64_t edges = 0;
+        rc = nd_check_launch("orientation");
+        if (!rc) rc = read_back(g, (int64_t*)g->dg_rp.p + g->n, &edges, "orientation");
+        if (!rc && edges != g->m)
+            rc = nd_set_error(ND_EINVAL, "the CSR is not symmetric (an entry is there more often than its reverse); load "
+                                         "it with ND_VALIDATE for details");
+        if (rc) {
+            for (DBuf* b : {&key, &outdeg, &tmp, &tail}) nd_free(c, *b);
+            return rc;
+        }
+    }
     v = nd_view(g);
     nd_dg_fill(v, key_hi, (int64_t*)g->dg_rp.p, (const int32_t*)tail.p, (int32_t*)g->dg_col.p, (int32_t*)g->dg_eid.p, st);
     rc = nd_check_launch("orientation");
@@ -503,6 +517,8 @@ extern "C" int nd_orient(nd_graph* g, int mode) {
 // triangle index (r = 3)
 static int ensure_tri(nd_graph* g) {
     if (g->have_tri) return ND_OK;
+    const char* kNotSimple = "the CSR is not a simple graph in ascending rows; load it with ND_VALIDATE for details";
+    if (g->rows & 4) return nd_set_error(ND_EINVAL, "%s", kNotSimple);
     nd_ctx* c = g->ctx;
     cudaStream_t st = c->stream;
     DBuf sigma, up, tmp;
@@ -523,20 +539,24 @@ static int ensure_tri(nd_graph* g) {
     nd_edge_support(v, (int32_t*)sigma.p, (int32_t*)up.p, st);
     nd_scan_i32((const int32_t*)sigma.p, (int64_t*)g->et_rp.p, m, tmp.p, st);
     nd_scan_i32((const int32_t*)up.p, (int64_t*)g->tbase.p, m, tmp.p, st);
-    int64_t tot[2] = {0, 0};
+    int64_t n3 = 0;
+    int err = 0;
     rc = nd_check_launch("triangle index");
-    if (!rc) rc = read_back(g, (int64_t*)g->et_rp.p + m, &tot[0], "triangle index");
-    if (!rc) rc = read_back(g, (int64_t*)g->tbase.p + m, &tot[1], "triangle index");
+    if (!rc) rc = read_back(g, (int64_t*)g->tbase.p + m, &n3, "triangle index");
+    if (!rc && g->rows) {
+        rc = scalar_zero(g);
+        if (!rc) nd_dup_check(v, (const int32_t*)sigma.p, (int*)g->scal.p, st);
+        if (!rc) rc = nd_check_launch("triangle index");
+        if (!rc) rc = read_back(g, g->scal.p, &err, "triangle index");
+    }
     nd_free(c, up);
     nd_free(c, tmp);
     if (rc) {
         nd_free(c, sigma);
         return rc;
     }
-    int64_t n3 = tot[1];
-    if (tot[0] != 3 * n3)
-        rc = nd_set_error(ND_EINTERNAL, "triangle index: %lld entries for %lld triangles", (long long)tot[0],
-                          (long long)n3);
+    if (err)
+        rc = nd_set_error(ND_EINVAL, "%s", kNotSimple);
     else if (n3 > INT32_MAX)
         rc = nd_set_error(ND_EOVERFLOW, "%lld triangles: more than 2^31-1", (long long)n3);
     if (rc || (rc = nd_alloc(c, g->et_w, sizeof(int32_t) * std::max<int64_t>(3 * n3, 1))) ||
@@ -554,22 +574,16 @@ static int ensure_tri(nd_graph* g) {
     const bool gather = n3 > 0 && scratch.alloc(c) == ND_OK;
     if (gather) cudaMemsetAsync(cursor.p, 0, sizeof(int32_t) * m, st);
     g->n3 = n3;
-    scalar_zero(g);  // a failure surfaces at the launch check below
     v = nd_view(g);
     nd_edge_fill(v, (int64_t*)g->et_rp.p, (int64_t*)g->tbase.p, (int32_t*)g->et_w.p, (int32_t*)g->et_t.p,
                  (int32_t*)g->tri_e.p, (int32_t*)g->tri_pos.p, (const int32_t*)sigma.p,
-                 gather ? (int32_t*)cursor.p : nullptr, gather ? (int32_t*)entries.p : nullptr, (int*)g->scal.p, st);
+                 gather ? (int32_t*)cursor.p : nullptr, gather ? (int32_t*)entries.p : nullptr, st);
     v = nd_view(g);
     nd_edge_fill_tid(v, (int32_t*)g->et_t.p, (int32_t*)g->tri_pos.p, st);
-    int err = 0;
     rc = nd_check_launch("triangle index");
-    if (!rc) rc = read_back(g, g->scal.p, &err, "triangle index");
     scratch.free(c);
     nd_free(c, sigma);
     if (rc) return rc;
-    if (err)
-        return nd_set_error(ND_EINVAL, "the CSR is not a simple graph in ascending rows; load it with ND_VALIDATE for "
-                                       "details");
     g->have_tri = true;
     return ND_OK;
 }
@@ -768,9 +782,12 @@ static int build_tri_hash(nd_graph* g, DBuf& hoff, DBuf& htab, DBuf& hpos) {
 // is asked to contract before every round contracts its triangle lists. The lists are an accelerator and must leave room for others,
 // hence the bound (nd_ctx::inc_bytes); the (3,4) lists of R-MAT graphs from scale 17 on, for instance, are over it, and
 // their s-cliques are listed again by Update.
-static bool wants_inc(const nd_ctx* c, int r, int s, int flags, int64_t n_s) {
+static bool wants_inc(const nd_graph* g, int r, int s, int flags, int64_t n_s) {
     if ((r == 1 && s == 2) || (r == 3 && s == 4 && (flags & ND_CONTRACT_ALWAYS))) return false;
-    return n_s < INT32_MAX && n_s <= c->inc_bytes / (4 * (nd_inc_stride(r, s) + binom64(s, r)));
+    // (1,4) and (2,5) count from every r-clique and fill from the lowest of each s-clique: the places that the
+    // counts reserve are the ones that are filled only if no row holds an entry twice or out of order
+    if (g->rows && ((r == 1 && s == 4) || (r == 2 && s == 5))) return false;
+    return n_s < INT32_MAX && n_s <= g->ctx->inc_bytes / (4 * (nd_inc_stride(r, s) + binom64(s, r)));
 }
 
 void nd_free_inc(nd_ctx* c, IncBufs& b) {
@@ -837,7 +854,7 @@ int nd_build_inc(nd_graph* g, int r, int s, int64_t n_r, IncBufs& b, bool* built
     if (!rc) rc = nd_count_into(g, r, s, w, n_r, cnt);
     if (!rc) rc = sum_counts(g, cnt, w, n_r, &tot);
     const int64_t n_s = (int64_t)(tot / (unsigned long long)binom64(s, r));
-    if (!rc && wants_inc(c, r, s, 0, n_s)) {
+    if (!rc && wants_inc(g, r, s, 0, n_s)) {
         rc = build_inc(g, r, s, cnt, w, n_r, n_s, b);
         if (!rc) rc = read_back(g, b.status.p, &status, "incidence lists");
         if (!rc && (status[2] || status[1] != n_s))
@@ -1233,7 +1250,7 @@ int nd_decompose_dev(nd_graph* g, int r, int s, int count_width, int flags, Peel
     cudaEventRecord(e3, c->stream);
     const int64_t n_s = (int64_t)(tot / (unsigned long long)binom64(s, r));
     IncBufs inc;
-    bool use_inc = !rc && wants_inc(c, r, s, flags, n_s);
+    bool use_inc = !rc && wants_inc(g, r, s, flags, n_s);
     if (use_inc) {
         rc = build_inc(g, r, s, cnt, w, n_r, n_s, inc);
         if (rc == ND_ENOMEM) {

@@ -436,9 +436,11 @@ void nd_dg_fill(const GraphView& g, const int32_t* key_hi, int64_t* dg_rp, const
                 int32_t* dg_eid, cudaStream_t st);
 // per canonical edge: sigma += |N(a) ∩ N(b)|, up += |{w in N(a) ∩ N(b) : w > b}| (zeroed by the caller)
 void nd_edge_support(const GraphView& g, int32_t* sigma, int32_t* up, cudaStream_t st);
+// *err unless the triangle lists of a CSR with duplicate entries are those of a simple graph
+void nd_dup_check(const GraphView& g, const int32_t* sigma, int* err, cudaStream_t st);
 // cursor (m, zeroed) and entries (9 n3): scratch of the short lists, or NULL: every list out of the rows
 void nd_edge_fill(const GraphView& g, int64_t* et_rp, int64_t* tbase, int32_t* et_w, int32_t* et_t,
-                  int32_t* tri_e, int32_t* tri_pos, const int32_t* sigma, int32_t* cursor, int32_t* entries, int* err,
+                  int32_t* tri_e, int32_t* tri_pos, const int32_t* sigma, int32_t* cursor, int32_t* entries,
                   cudaStream_t st);
 void nd_edge_fill_tid(const GraphView& g, int32_t* et_t, int32_t* tri_pos, cudaStream_t st);
 void nd_tri_tuples(const GraphView& g, int32_t* out, cudaStream_t st);

@@ -101,8 +101,10 @@ __device__ __forceinline__ int64_t row_of(const int64_t* __restrict__ rp, int64_
     return lo;
 }
 
-// A CSR entry whose reverse entry is missing, a self-loop or an id that is no vertex sets *err and gets edge
-// id 0, so that no later kernel indexes outside the edge arrays; no row is looked up by such an id.
+// A CSR entry whose reverse entry is missing, a self-loop or an id that is no vertex sets bit 0 of *err and
+// gets edge id 0, so that no later kernel indexes outside the edge arrays; no row is looked up by such an id.
+// An entry equal to the one before it in its row sets bit 1, one below it bit 2 (without either, and with as many
+// upper as lower entries, the graph is simple); what depends on that is nd_api.cu's to refuse.
 __global__ void k_pos2e(GraphView g, int64_t nnz, int64_t seg, int32_t* __restrict__ pos2e, int32_t* __restrict__ eu,
                         int32_t* __restrict__ ev, int* err) {
     const int lane = threadIdx.x & 31;
@@ -115,6 +117,7 @@ __global__ void k_pos2e(GraphView g, int64_t nnz, int64_t seg, int32_t* __restri
             if (p < s1) {
                 u = row_of(g.rp, g.n, u0, p);
                 const int32_t v = g.col[p];
+                if (p > g.rp[u] && g.col[p - 1] >= v) atomicOr(err, g.col[p - 1] == v ? 2 : 4);
                 int64_t id;
                 if ((uint32_t)v >= (uint32_t)g.n) {
                     atomicOr(err, 1);
@@ -267,6 +270,23 @@ __global__ void __launch_bounds__(kTriThreads) k_edge_support(GraphView g, int t
     tri_list(g, tile, sink);
 }
 
+// Whether a CSR with duplicate entries has the triangle lists of a simple graph: *err is set if a duplicate's
+// edge lies in a triangle (two entries of a list would be equal, and k_edge_order would give both the same
+// place, leaving the next one unwritten), or if an upper entry has no reverse (the rows would hold triangles
+// that DG does not).
+__global__ void k_dup_check(GraphView g, int64_t nnz, int64_t seg, const int32_t* __restrict__ sigma, int* err) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t s0 = gwarp() * seg; s0 < nnz; s0 += nwarps() * seg) {
+        const int64_t s1 = s0 + seg < nnz ? s0 + seg : nnz;
+        for (int64_t p = s0 + lane; p < s1; p += 32) {
+            const int64_t u = row_of(g.rp, g.n, 0, p);
+            const int32_t v = g.col[p];
+            if (p > g.rp[u] && g.col[p - 1] == v && (sigma[g.pos2e[p - 1]] || sigma[g.pos2e[p]])) atomicOr(err, 1);
+            if (v > u && nd_find(g.col + g.rp[v], g.split[v] - g.rp[v], (int32_t)u) < 0) atomicOr(err, 1);
+        }
+    }
+}
+
 // Lists of up to kShortList entries are not intersected out of the two rows, which are far longer, but
 // gathered: a second listing of the triangles over DG appends every triangle to the short lists among
 // its three (k_edge_gather, in no order), and k_edge_order puts each list in order by counting for every
@@ -280,17 +300,10 @@ struct GatherSink {
     const int32_t* eid;
     int32_t* cursor;
     int32_t *w_in, *p_in, *q_in;  // per entry: the vertex; the edge to et_t (see k_edge_fill); of an upper entry, bc
-    int* err;
     __device__ void begin(int) const {}
     __device__ void put(int32_t e, int32_t w, int32_t p, int32_t q) const {
-        const int32_t n = sigma[e];
-        if (n > kShortList) return;
-        const int32_t k = atomicAdd(&cursor[e], 1);
-        if (k >= n) {
-            atomicOr(err, 1);
-            return;
-        }
-        const int64_t at = et_rp[e] + k;
+        if (sigma[e] > kShortList) return;
+        const int64_t at = et_rp[e] + atomicAdd(&cursor[e], 1);
         w_in[at] = w;
         p_in[at] = p;
         q_in[at] = q;
@@ -383,11 +396,10 @@ __global__ void k_edge_order(GraphView g, const int64_t* __restrict__ et_rp, con
 // (temporarily) the id of edge (a,w); and the edges of every triangle whose lowest edge is e. Lists of up to
 // `above` entries are left out (k_edge_gather and k_edge_order write them; 0 without room for that). Edges
 // without triangles, most of them in a sparse graph, cost a lane a look and not a warp an intersection
-// (Chung-Lu, a million vertices, 15 M edges: 13.2 ms here of 16.3 before). The rows of a CSR with duplicates do not give what DG
-// gave for sigma: nothing is written outside the edge's list then, and *err is set.
+// (Chung-Lu, a million vertices, 15 M edges: 13.2 ms here of 16.3 before).
 __global__ void k_edge_fill(GraphView g, const int64_t* __restrict__ et_rp, const int64_t* __restrict__ tbase,
                             int32_t* __restrict__ et_w, int32_t* __restrict__ et_t, int32_t* __restrict__ tri_e,
-                            int32_t* __restrict__ tri_pos, int64_t above, int* err) {
+                            int32_t* __restrict__ tri_pos, int64_t above) {
     const int lane = threadIdx.x & 31;
     const unsigned full = 0xffffffffu;
     for (int64_t e0 = gwarp() * 32; e0 < g.m; e0 += nwarps() * 32) {
@@ -419,7 +431,6 @@ __global__ void k_edge_fill(GraphView g, const int64_t* __restrict__ et_rp, cons
             // writes common element w, found at driver position p and other-list position q, as entry
             // `local` of L(a,b)
             auto put = [&](int64_t local, int64_t p, int64_t q, int32_t w) {
-                if (local >= sig || (w > b) != (local >= split_e)) return;  // no simple graph: reported below
                 int64_t pa = a_drives ? p : q;  // position of w in N(a)
                 int64_t pb = a_drives ? q : p;  // position of w in N(b)
                 int32_t e_aw = g.pos2e[pa], e_bw = g.pos2e[pb];
@@ -448,7 +459,6 @@ __global__ void k_edge_fill(GraphView g, const int64_t* __restrict__ et_rp, cons
                     int y = __shfl_up_sync(0xffffffffu, inc, o);
                     if (lane >= o) inc += y;
                 }
-                if (lane == 31 && inc != sig) atomicOr(err, 1);
                 int64_t local = inc - cnt;
                 nd_merge_walk(X, nx, Y, ny, run, [&](int i, int j, int32_t w) { put(local++, xb + i, yb + j, w); });
             } else {
@@ -461,7 +471,6 @@ __global__ void k_edge_fill(GraphView g, const int64_t* __restrict__ et_rp, cons
                     if (q >= 0) put(pos + __popc(m & nd_lanemask_lt()), p, yb + q, g.col[p]);
                     pos += __popc(m);
                 }
-                if (lane == 0 && pos != sig) atomicOr(err, 1);
             }
         }
     }
@@ -502,11 +511,9 @@ __global__ void k_edge_fill_tid(GraphView g, int32_t* __restrict__ et_t, int32_t
             const int32_t oa = __shfl_sync(full, a, own), ob = __shfl_sync(full, b, own);
             if (p >= total) continue;
             const int32_t e2 = et_t[j], w = g.et_w[j];
-            if ((uint32_t)e2 >= (uint64_t)g.m) continue;  // not filled (see k_edge_fill's err)
             const int64_t l2 = g.et_rp[e2], h2 = g.et_rp[e2 + 1], t2 = g.tbase[e2];
             const int64_t s2 = (h2 - l2) - (g.tbase[e2 + 1] - t2);
             const int64_t at = nd_lower_bound(g.et_w + l2 + s2, h2 - l2 - s2, ob), tid = t2 + at;
-            if (at >= h2 - l2 - s2) continue;
             et_t[j] = (int32_t)tid;
             tri_pos[3 * tid + (w > oa ? 1 : 2)] = (int32_t)k;
         }
@@ -767,19 +774,24 @@ void nd_edge_support(const GraphView& g, int32_t* sigma, int32_t* up, cudaStream
     ND_K(k_edge_support<<<blocks_for_warps((g.m + tile - 1) / tile), kTriThreads, 0, st>>>(g, tile, sigma, up));
 }
 
+void nd_dup_check(const GraphView& g, const int32_t* sigma, int* err, cudaStream_t st) {
+    if (g.m <= 0) return;
+    ND_K(k_dup_check<<<blocks_for_segments(2 * g.m), kThreads, 0, st>>>(g, 2 * g.m, seg_len(2 * g.m), sigma, err));
+}
+
 void nd_edge_fill(const GraphView& g, int64_t* et_rp, int64_t* tbase, int32_t* et_w, int32_t* et_t, int32_t* tri_e,
-                  int32_t* tri_pos, const int32_t* sigma, int32_t* cursor, int32_t* entries, int* err, cudaStream_t st) {
+                  int32_t* tri_pos, const int32_t* sigma, int32_t* cursor, int32_t* entries, cudaStream_t st) {
     if (g.m <= 0) return;
     const int64_t nent = 3 * g.n3;
     if (cursor) {
         const int tile = tri_tile(g.m);
-        GatherSink sink{et_rp, sigma, g.dg_eid, cursor, entries, entries + nent, entries + 2 * nent, err};
+        GatherSink sink{et_rp, sigma, g.dg_eid, cursor, entries, entries + nent, entries + 2 * nent};
         ND_K(k_edge_gather<<<blocks_for_warps((g.m + tile - 1) / tile), kTriThreads, 0, st>>>(g, tile, sink));
         ND_K(k_edge_order<<<blocks_for_warps((g.m + 31) / 32), kThreads, 0, st>>>(
             g, et_rp, tbase, entries, entries + nent, entries + 2 * nent, et_w, et_t, tri_e, tri_pos));
     }
     ND_K(k_edge_fill<<<blocks_for_warps((g.m + 31) / 32), kThreads, 0, st>>>(g, et_rp, tbase, et_w, et_t, tri_e, tri_pos,
-                                                                                 cursor ? kShortList : 0, err));
+                                                                                 cursor ? kShortList : 0));
 }
 
 void nd_edge_fill_tid(const GraphView& g, int32_t* et_t, int32_t* tri_pos, cudaStream_t st) {

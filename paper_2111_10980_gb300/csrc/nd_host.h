@@ -57,6 +57,7 @@ struct nd_graph {
     int64_t edge_mindeg = -1;  // max over edges of min(deg u, deg v); -1 until needed
     // orientation
     int orient = -1;
+    int rows = 0;  // of a CSR that was not validated: 2 a row holds an entry twice, 4 a row is out of order
     DBuf dg_rp, dg_col, dg_eid;
     // triangle index
     bool have_tri = false;

@@ -146,3 +146,81 @@ def test_ids_out_of_range_are_refused_without_validate(nd, bad_id, where):
         assert np.array_equal(core, orc.decompose(g, 2, 3).core)
     finally:
         nd.nd_ctx_destroy(ctx)
+
+
+def _csr(n, rows):
+    """CSR of these rows as they are: {vertex: entries}."""
+    rowptr = np.zeros(n + 1, np.int64)
+    for u, row in rows.items():
+        rowptr[u + 1] = len(row)
+    return np.cumsum(rowptr), np.concatenate([np.asarray(rows.get(u, ()), np.int32) for u in range(n)]).astype(np.int32)
+
+
+def _clique_rows(k):
+    return {u: [v for v in range(k) if v != u] for u in range(k)}
+
+
+def _refused(nd, ctx, n, rows, call):
+    G = nd.nd_load_csr(ctx, *_csr(n, rows))
+    try:
+        with pytest.raises(nd.NdError) as ei:
+            call(G)
+        assert ei.value.code == nd.ND_EINVAL
+    finally:
+        nd.nd_graph_free(G)
+
+
+@pytest.mark.parametrize("k", [4, 40, 130, 131])
+def test_a_duplicate_edge_of_a_triangle_is_refused_by_the_triangle_index(nd, k):
+    """An edge that its two rows hold twice, in cliques whose edges have up to 128 common neighbours (lists
+    ordered by counting) and more (lists merged out of the rows); so are rows out of order."""
+    ctx = nd.nd_ctx_create(0)
+    try:
+        for u, v in ((0, 1), (0, k - 1), (k - 2, k - 1)):
+            rows = _clique_rows(k)
+            rows[u] = sorted(rows[u] + [v])
+            rows[v] = sorted(rows[v] + [u])
+            _refused(nd, ctx, k, rows, lambda G: nd.nd_rcliques(G, 3))
+            for r, s in ((3, 4), (3, 5), (4, 5)):
+                _refused(nd, ctx, k, rows, lambda G: nd.nd_decompose(G, r, s))
+        rows = _clique_rows(k)
+        rows[0] = rows[0][:-2] + rows[0][:-3:-1]
+        _refused(nd, ctx, k, rows, lambda G: nd.nd_count(G, 3, 4))
+    finally:
+        nd.nd_ctx_destroy(ctx)
+
+
+def test_entries_without_or_with_too_many_reverses_are_refused(nd):
+    """As many upper as lower entries, and every lower entry has a reverse, but not every upper one: a
+    duplicate lower entry makes up the number."""
+    ctx = nd.nd_ctx_create(0)
+    try:
+        # 0-1 twice in row 0, once in row 1; 8-9 the other way round, so that the totals agree. Vertex 1 and vertex 8
+        # have the larger degree, so both sides of the orientation take the doubled row
+        rows = {0: [1, 1], 1: [0, 2, 3, 4], 2: [1], 3: [1], 4: [1], 5: [8], 6: [8], 7: [8], 8: [5, 6, 7, 9], 9: [8, 8]}
+        _refused(nd, ctx, 10, rows, lambda G: nd.nd_orient(G, nd.ND_ORIENT_DEGREE))
+        # vertex 0 lists 3, which does not list 0; 5 lists 4 twice and has the smaller degree of the two, so that
+        # the orientation takes as many edges as there should be
+        rows = {0: [1, 2, 3], 1: [0, 2, 3], 2: [0, 1, 3], 3: [1, 2], 4: [5, 6, 7], 5: [4, 4], 6: [4], 7: [4]}
+        _refused(nd, ctx, 8, rows, lambda G: nd.nd_rcliques(G, 3))
+    finally:
+        nd.nd_ctx_destroy(ctx)
+
+
+def test_a_duplicate_edge_outside_triangles_is_accepted(nd):
+    """The triangles and their cores are those of the graph without the duplicate."""
+    k, ctx = 6, nd.nd_ctx_create(0)
+    try:
+        got = []
+        for times in (1, 2):
+            rows = _clique_rows(k)
+            rows[k - 1] = rows[k - 1] + [k] * times
+            rows[k] = [k - 1] * times
+            G = nd.nd_load_csr(ctx, *_csr(k + 1, rows))
+            got.append([nd.nd_rcliques(G, 3)] + [nd.nd_decompose(G, 3, s)[0] for s in (4, 5)])
+            nd.nd_graph_free(G)
+        for a, b in zip(*got):
+            assert np.array_equal(a, b)
+        assert np.array_equal(got[0][1], np.full(20, k - 3))
+    finally:
+        nd.nd_ctx_destroy(ctx)
