@@ -462,6 +462,7 @@ static int build_dg(nd_graph* g, int mode) {
         key_hi = (const int32_t*)key.p;
     }
     for (DBuf* b : {&g->dg_rp, &g->dg_col, &g->dg_eid}) nd_free(c, *b);
+    g->orient = -1;  // until there is a new one
     if ((rc = nd_alloc(c, outdeg, sizeof(int64_t) * std::max<int64_t>(g->n, 1))) ||
         (rc = nd_alloc(c, tail, sizeof(int32_t) * std::max<int64_t>(nd_dg_segments(g->m), 1))) ||
         (rc = nd_alloc(c, tmp, nd_scan_tmp_bytes(g->n))) ||

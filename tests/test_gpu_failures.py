@@ -224,3 +224,44 @@ def test_a_duplicate_edge_outside_triangles_is_accepted(nd):
         assert np.array_equal(got[0][1], np.full(20, k - 3))
     finally:
         nd.nd_ctx_destroy(ctx)
+
+
+def test_another_orientation_without_memory_leaves_the_graph_usable(nd):
+    """nd_orient to another mode, refused each of its allocations in turn: ND_ENOMEM, and the next call on the
+    graph orients it again."""
+    import torch
+
+    g = gg.chung_lu(300, 10.0, 2.2, seed=63)
+    want = orc.decompose(g, 2, 3)
+    alloc, free = nd.torch_allocator_hooks(0)
+    left = [None]
+
+    def take(nbytes, stream):
+        if left[0] is not None:
+            left[0] -= 1
+            if left[0] < 0:
+                return 0
+        return alloc(nbytes, stream)
+
+    ctx = nd.nd_ctx_create(0, stream=torch.cuda.Stream())
+    nd.nd_ctx_set_allocator(ctx, take, free)
+    G = nd.nd_load_csr(ctx, g.rowptr, g.col)
+    refused = 0
+    try:
+        for i in range(200):
+            nd.nd_orient(G, nd.ND_ORIENT_DEGREE)
+            left[0] = i
+            try:
+                nd.nd_orient(G, nd.ND_ORIENT_DEGENERACY)
+                break
+            except nd.NdError as e:
+                assert e.code == nd.ND_ENOMEM
+                refused += 1
+            finally:
+                left[0] = None
+            core, rnd, st = nd.nd_decompose(G, 2, 3)
+            assert np.array_equal(core, want.core) and np.array_equal(rnd, want.round)
+        assert 5 < refused < 199
+    finally:
+        nd.nd_graph_free(G)
+        nd.nd_ctx_destroy(ctx)
