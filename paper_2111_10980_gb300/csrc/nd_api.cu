@@ -74,10 +74,15 @@ void nd_free(nd_ctx* ctx, DBuf& b) {
     b.bytes = 0;
 }
 
-int DGroup::alloc(nd_ctx* c) {
-    constexpr size_t kArena = (size_t)4 << 20;
+size_t DGroup::bytes() const {
     size_t total = 0;
     for (auto& w : want) total += (std::max<size_t>(w.second, 16) + 255) & ~(size_t)255;
+    return total;
+}
+
+int DGroup::alloc(nd_ctx* c) {
+    constexpr size_t kArena = (size_t)4 << 20;
+    const size_t total = bytes();
     if (total <= kArena) {
         if (nd_alloc(c, arena, total) == ND_OK) {
             size_t at = 0;
@@ -779,37 +784,41 @@ static int build_tri_hash(nd_graph* g, DBuf& hoff, DBuf& htab, DBuf& hpos) {
     return nd_check_launch("triangle hash");
 }
 
-// Which decompositions are peeled from incidence lists. (1,2) has them in the CSR itself; a (3,4) run that
+// Whether a decomposition is peeled from incidence lists, and b's buffers if so. (1,2) has them in the CSR itself; a (3,4) run that
 // is asked to contract before every round contracts its triangle lists. The lists are an accelerator and must leave room for others,
-// hence the bound (nd_ctx::inc_bytes); the (3,4) lists of R-MAT graphs from scale 17 on, for instance, are over it, and
-// their s-cliques are listed again by Update.
-static bool wants_inc(const nd_graph* g, int r, int s, int flags, int64_t n_s) {
+// hence the bound (nd_ctx::inc_bytes, on all the buffers together; a server's batch is charged that much); the (3,4)
+// lists of R-MAT graphs from scale 17 on, for instance, are over it, and their s-cliques are listed again by Update.
+static bool plan_inc(const nd_graph* g, int r, int s, int flags, int64_t n_r, int64_t n_s, IncBufs& b) {
     if ((r == 1 && s == 2) || (r == 3 && s == 4 && (flags & ND_CONTRACT_ALWAYS))) return false;
     // (1,4) and (2,5) count from every r-clique and fill from the lowest of each s-clique: the places that the
     // counts reserve are the ones that are filled only if no row holds an entry twice or out of order
     if (g->rows && ((r == 1 && s == 4) || (r == 2 && s == 5))) return false;
-    return n_s < INT32_MAX && n_s <= g->ctx->inc_bytes / (4 * (nd_inc_stride(r, s) + binom64(s, r)));
+    if (n_s >= INT32_MAX) return false;
+    b.stride = nd_inc_stride(r, s);
+    b.n_s = n_s;
+    for (bool tight : {false, true}) {
+        b.rows = nd_inc_rows(r, s, n_r, g->m, n_s, tight, &b.run);
+        b.mem.want.clear();
+        b.mem.add(b.off, 8 * (n_r + 1));
+        b.mem.add(b.cursor, 8 * (n_r + 1));
+        b.mem.add(b.tmp, nd_scan_tmp_bytes(n_r));
+        b.mem.add(b.list, 4 * n_s * binom64(s, r));
+        b.mem.add(b.row, 4 * b.stride * b.rows);
+        b.mem.add(b.dead, 4 * (b.rows / 32 + 1));
+        b.mem.add(b.status, 16);
+        if (b.mem.bytes() <= (size_t)g->ctx->inc_bytes) return true;
+    }
+    return false;
 }
 
 void nd_free_inc(nd_ctx* c, IncBufs& b) {
     b.mem.free(c);
 }
 
-static int build_inc(nd_graph* g, int r, int s, const DBuf& cnt, int w, int64_t n_r, int64_t n_s, IncBufs& b) {
+// allocates and fills what plan_inc found
+static int build_inc(nd_graph* g, int r, int s, const DBuf& cnt, int w, int64_t n_r, IncBufs& b) {
     nd_ctx* c = g->ctx;
     cudaStream_t st = c->stream;
-    b.stride = nd_inc_stride(r, s);
-    b.n_s = n_s;
-    const int64_t entries = n_s * binom64(s, r);
-    IncFill F;
-    F.rows = nd_inc_rows(r, s, n_r, g->m, n_s, &F.run);
-    b.mem.add(b.off, 8 * (n_r + 1));
-    b.mem.add(b.cursor, 8 * (n_r + 1));
-    b.mem.add(b.tmp, nd_scan_tmp_bytes(n_r));
-    b.mem.add(b.list, 4 * std::max<int64_t>(entries, 1));
-    b.mem.add(b.row, 4 * b.stride * F.rows);
-    b.mem.add(b.dead, 4 * (F.rows / 32 + 1));
-    b.mem.add(b.status, 16);
     int rc = b.mem.alloc(c);
     if (rc) return rc;
     if (w == 8)
@@ -819,11 +828,14 @@ static int build_inc(nd_graph* g, int r, int s, const DBuf& cnt, int w, int64_t 
     cudaMemcpyAsync(b.cursor.p, b.off.p, 8 * (n_r + 1), cudaMemcpyDeviceToDevice, st);
     cudaMemsetAsync(b.dead.p, 0, b.dead.bytes, st);
     cudaMemsetAsync(b.status.p, 0, b.status.bytes, st);
+    IncFill F;
     F.cursor = (unsigned long long*)b.cursor.p;
     F.list = (uint32_t*)b.list.p;
     F.row = (int32_t*)b.row.p;
     F.status = (unsigned int*)b.status.p;
-    F.entries = entries;
+    F.rows = b.rows;
+    F.entries = b.n_s * binom64(s, r);
+    F.run = b.run;
     nd_inc_fill(nd_view(g), r, s, n_r, F, st);
     rc = nd_check_launch("incidence lists");
     if (!b.mem.arena.p) {
@@ -855,8 +867,8 @@ int nd_build_inc(nd_graph* g, int r, int s, int64_t n_r, IncBufs& b, bool* built
     if (!rc) rc = nd_count_into(g, r, s, w, n_r, cnt);
     if (!rc) rc = sum_counts(g, cnt, w, n_r, &tot);
     const int64_t n_s = (int64_t)(tot / (unsigned long long)binom64(s, r));
-    if (!rc && wants_inc(g, r, s, 0, n_s)) {
-        rc = build_inc(g, r, s, cnt, w, n_r, n_s, b);
+    if (!rc && plan_inc(g, r, s, 0, n_r, n_s, b)) {
+        rc = build_inc(g, r, s, cnt, w, n_r, b);
         if (!rc) rc = read_back(g, b.status.p, &status, "incidence lists");
         if (!rc && (status[2] || status[1] != n_s))
             rc = nd_set_error(ND_EINTERNAL, "incidence lists: %u of %lld s-cliques", status[1], (long long)n_s);
@@ -1251,9 +1263,9 @@ int nd_decompose_dev(nd_graph* g, int r, int s, int count_width, int flags, Peel
     cudaEventRecord(e3, c->stream);
     const int64_t n_s = (int64_t)(tot / (unsigned long long)binom64(s, r));
     IncBufs inc;
-    bool use_inc = !rc && wants_inc(g, r, s, flags, n_s);
+    bool use_inc = !rc && plan_inc(g, r, s, flags, n_r, n_s, inc);
     if (use_inc) {
-        rc = build_inc(g, r, s, cnt, w, n_r, n_s, inc);
+        rc = build_inc(g, r, s, cnt, w, n_r, inc);
         if (rc == ND_ENOMEM) {
             use_inc = false;
             rc = ND_OK;

@@ -458,7 +458,7 @@ int nd_peel_heavy_slices();
 
 // Incidence lists of the s-cliques (nd_inc.cu), what filling them writes: cursor[R] starts at the first
 // place of R's list; status[0] counts the rows handed out, status[1] the s-cliques that got one, status[2]
-// is set when one has no room. Warps take rows in runs of `run`, so a few stay unused.
+// is set when one has no room. Warps take rows in runs of `run` or more, so a few stay unused.
 struct IncFill {
     unsigned long long* cursor;
     uint32_t* list;
@@ -468,8 +468,8 @@ struct IncFill {
     unsigned run;
 };
 int nd_inc_stride(int r, int s);
-// the rows to allocate for n_s s-cliques, and the length of a run
-int64_t nd_inc_rows(int r, int s, int64_t n_r, int64_t m, int64_t n_s, unsigned* run);
+// the rows to allocate for n_s s-cliques, and the length of a run (tight: no row more than n_s)
+int64_t nd_inc_rows(int r, int s, int64_t n_r, int64_t m, int64_t n_s, bool tight, unsigned* run);
 void nd_inc_fill(const GraphView& g, int r, int s, int64_t n_r, const IncFill& F, cudaStream_t st);
 
 // counting (nd_count.cu): counts into cnt (CT = int32_t or int64_t), zero-initialised

@@ -36,7 +36,7 @@ struct nd_ctx {
     int64_t count_limit = 0;
     int32_t limit_flags = 0;
     int peel_share = 1;  // of a server's worker: the workers whose peel kernels share the GPU
-    int64_t inc_bytes = (int64_t)16 << 30;  // most device bytes of a decomposition's incidence lists
+    int64_t inc_bytes = (int64_t)16 << 30;  // most device bytes of a decomposition's incidence lists, all their buffers together
     void* stage = nullptr;  // pinned staging of batches (grown on demand)
     size_t stage_bytes = 0;
     // nd_ctx_set_tuning, indexed by r * 8 + s
@@ -89,6 +89,7 @@ struct DGroup {
     std::vector<std::pair<DBuf*, size_t>> want;
     DBuf arena;
     void add(DBuf& b, size_t bytes) { want.emplace_back(&b, bytes); }
+    size_t bytes() const;  // that alloc takes
     int alloc(nd_ctx* c);
     void free(nd_ctx* c);
 };
@@ -99,7 +100,8 @@ struct IncBufs {
     DBuf cursor, tmp;  // only while they are filled
     DBuf off, list, row, dead, status;
     int32_t stride = 0;
-    int64_t n_s = 0;
+    int64_t n_s = 0, rows = 0;
+    unsigned run = 0;
 };
 
 int nd_set_error(int code, const char* fmt, ...);

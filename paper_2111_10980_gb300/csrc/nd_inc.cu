@@ -3,7 +3,8 @@
 // listing the s-cliques of each peeled r-clique again (Algorithm 2, Update), which for one r-clique is
 // a chain of up to twenty-five dependent accesses and for all of them C(s,r) listings of each s-clique.
 //
-// The lists take (stride + C(s,r)) * 4 bytes for each s-clique and are built from the counts (their
+// The lists take (stride + C(s,r)) * 4 bytes for each s-clique, 16 for each r-clique (offsets, and cursors while
+// they are filled) and a few spare rows (nd_inc_rows); they are built from the counts (their
 // lengths) in one more listing. Rows come in listing order, so the members of neighbouring rows
 // lie close together; the order inside an r-clique's list is that of the atomics and has no meaning.
 //
@@ -30,8 +31,9 @@ int blocks_for_warps(int64_t items) {
     return (int)(want < cap ? want : cap);
 }
 
-// A warp's run of rows: F.run at a time from one counter (a counter update for every handful of matches is
-// what the first form of k_inc_tri waited for: 130 ms for the 374 M triangles of R-MAT scale 20).
+// A warp's run of rows: F.run at a time, or what it needs if that is more, from one counter (a counter update for
+// every handful of matches is what the first form of k_inc_tri waited for: 130 ms for the 374 M triangles of
+// R-MAT scale 20).
 struct IncRun {
     unsigned at = 0, left = 0, used = 0;
 };
@@ -60,20 +62,21 @@ __device__ __forceinline__ void inc_write(const IncFill& F, unsigned S, const in
     }
 }
 
-// The s-cliques of the lanes with hit set, members id[0..C). The whole warp calls it. F.run >= 32.
+// The s-cliques of the lanes with hit set, members id[0..C). The whole warp calls it.
 template <int C>
 __device__ __forceinline__ void inc_put(const IncFill& F, IncRun& run, bool hit, const int32_t* id) {
     const unsigned full = 0xffffffffu, mask = __ballot_sync(full, hit);
     const unsigned n = __popc(mask), rank = __popc(mask & nd_lanemask_lt());
     unsigned next = 0;
-    if (n > run.left) {
-        if ((threadIdx.x & 31) == 0) next = atomicAdd(&F.status[0], F.run);
+    const unsigned more = n > run.left ? n - run.left : 0, take = more > F.run ? more : F.run;
+    if (more) {
+        if ((threadIdx.x & 31) == 0) next = atomicAdd(&F.status[0], take);
         next = __shfl_sync(full, next, 0);
     }
     const unsigned S = rank < run.left ? run.at + rank : next + (rank - run.left);
-    if (n > run.left) {
-        run.at = next + (n - run.left);
-        run.left = F.run - (n - run.left);
+    if (more) {
+        run.at = next + more;
+        run.left = take - more;
     } else {
         run.at += n;
         run.left -= n;
@@ -228,11 +231,14 @@ static int64_t inc_items(int r, int s, int64_t n_r, int64_t m) {
     return s == 3 ? (m + tile - 1) / tile : r == 2 && s == 4 ? m : n_r;
 }
 
-int64_t nd_inc_rows(int r, int s, int64_t n_r, int64_t m, int64_t n_s, unsigned* run) {
+// A run is an eighth of a warp's share of the s-cliques, and at least 32 where there is room for that. Every warp
+// that finds an s-clique leaves less than a run unused: at most an eighth more rows, or 31 per warp. In runs
+// of 1 (`tight`) no row is left.
+int64_t nd_inc_rows(int r, int s, int64_t n_r, int64_t m, int64_t n_s, bool tight, unsigned* run) {
     const int64_t warps = (int64_t)blocks_for_warps(inc_items(r, s, n_r, m)) * (kThreads / 32);
-    const int64_t share = n_s / (8 * warps);  // an eighth of a warp's share, so at most an eighth more rows
-    *run = (unsigned)(share < 32 ? 32 : share > 1024 ? 1024 : share);
-    return n_s + warps * *run;
+    const int64_t share = n_s / (8 * warps);
+    *run = (unsigned)(tight ? 1 : share < 32 ? 32 : share > 1024 ? 1024 : share);
+    return n_s + (warps < n_s ? warps : n_s) * (*run - 1);
 }
 
 void nd_inc_fill(const GraphView& g, int r, int s, int64_t n_r, const IncFill& F, cudaStream_t st) {

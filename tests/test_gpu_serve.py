@@ -279,3 +279,68 @@ def test_malformed_requests_fail_alone(nd, ctx):
         assert ei.value.code == nd.ND_EINVAL
     finally:
         sv.close()
+
+
+class _Counted:
+    """Allocator hooks that count the bytes held and note every size."""
+
+    def __init__(self, nd):
+        import threading
+
+        self.alloc, self.free = nd.torch_allocator_hooks(0)
+        self.lock, self.now, self.peak, self.sizes = threading.Lock(), 0, 0, []
+
+    def take(self, nbytes, stream):
+        with self.lock:
+            self.now += nbytes
+            self.peak = max(self.peak, self.now)
+            self.sizes.append(nbytes)
+        return self.alloc(nbytes, stream)
+
+    def give(self, p, nbytes, stream):
+        with self.lock:
+            self.now -= nbytes
+        self.free(p, nbytes, stream)
+
+
+def _serve_one(nd, g, r, s, want, **cfg):
+    import torch
+
+    c = nd.nd_ctx_create(0, stream=torch.cuda.Stream())
+    hooks = _Counted(nd)
+    nd.nd_ctx_set_allocator(c, hooks.take, hooks.give)
+    sv = nd.nd_server_create(c, workers=1, max_batch=1, **cfg)
+    try:
+        out = np.full(want.size, -1, np.int32)
+        t = sv.submit(g.rowptr, g.col, r, s, out)
+        sv.drain()
+        assert sv.poll(t)[0] == nd.ND_OK
+        assert np.array_equal(out, want)
+    finally:
+        sv.close()
+        nd.nd_ctx_destroy(c)
+    assert hooks.now == 0
+    return hooks
+
+
+@pytest.mark.parametrize("r,s", [(2, 3), (2, 4)])
+def test_server_memory_budget_holds_the_lists(nd, r, s):
+    """A graph without triangles needs no room for s-cliques: its batch stays within a budget of three times
+    the bytes of its edges' state."""
+    g = gg.path(20_001)
+    hooks = _serve_one(nd, g, r, s, np.zeros(g.m, np.int32), mem_budget=8 << 20)
+    assert hooks.peak <= 8 << 20
+
+
+def test_server_lists_in_the_room_there_is(nd):
+    """K_150 as (2,3), 551,300 triangles: with room for the lists and their spare rows, for the lists alone,
+    and for neither. The bytes of the lists never exceed the half of what the budget leaves."""
+    g = gg.complete(150)
+    want, rows = np.full(g.m, 148, np.int32), 4 * 4 * 551_300
+    seen = []
+    for budget in (16 << 20, 35 << 20, 64 << 20):
+        hooks = _serve_one(nd, g, 2, 3, want, mem_budget=budget)
+        most = max(hooks.sizes)
+        seen.append("none" if most < rows else "tight" if most < rows + 256 else "spare")
+        assert hooks.peak <= budget
+    assert seen == ["none", "tight", "spare"]
