@@ -263,8 +263,9 @@ ND_API int nd_nuclei(nd_graph *g, int r, int s, const int32_t *core, int32_t lev
  * the smallest r-clique id of the component of R's node; parent_level_out[R] and
  * parent_comp_out[R] = the level and smallest id of the parent node of R's node, -1 and -1 for a
  * root. With host pointers any output may be NULL; with ND_PTR_DEVICE all three are required.
- * *n_nodes_out (host, nullable): the number of nodes. Cost: every s-clique is listed once over all
- * levels (one union-find over the r-cliques, levels taken in decreasing order). Errors:
+ * *n_nodes_out (host, nullable): the number of nodes. Cost: every r-clique's s-cliques are visited
+ * once over all levels (one union-find over the r-cliques, levels taken in decreasing order), read from
+ * incidence lists where a count and one more listing of the graph to build them pay. Errors:
  * ND_EINVAL (NULL graph or core, unsupported (r,s), a core value outside [0, 2^26)),
  * ND_ENOMEM, ND_EOVERFLOW (more than INT32_MAX r-cliques), ND_EINTERNAL (as for nd_nuclei). */
 ND_API int nd_hierarchy(nd_graph *g, int r, int s, const int32_t *core, int32_t *comp_out, int32_t *parent_level_out,

@@ -4,9 +4,10 @@
 // in X_c; the connected nuclei at level c are the components of that relation. Components at a
 // higher level nest inside those of a lower one, so the levels together form the nucleus hierarchy.
 //
-// One warp per r-clique R of X_c reads the s-cliques containing R from their incidence lists (nd_inc.cu),
-// or, without memory for those, lists them with nd_gen.cuh; an s-clique whose r-subsets all lie in X_c is handled by its owner, the smallest id
-// among them, which unites the others with itself in a union-find over r-clique ids. Unions hook
+// One warp per r-clique R of X_c lists the s-cliques containing R with nd_gen.cuh or, where building them pays
+// (level_lists, hierarchy_lists), reads them from incidence lists (nd_inc.cu); an s-clique whose r-subsets all
+// lie in X_c is handled by its owner, the smallest id among them, which unites the others with itself in a
+// union-find over r-clique ids. Unions hook
 // the larger root under the smaller with a compare-and-swap, so every link points to a smaller id,
 // roots end as the smallest id of their component, and finds halve paths without conflicting with
 // the hooks (only roots are hooked, only non-roots are shortened). Every retry loop is bounded; a
@@ -106,7 +107,8 @@ __global__ void k_nuclei_union(GraphView g, const int32_t* __restrict__ core, in
 }
 
 // The same from the incidence lists: R's s-cliques and their members are read, not listed and looked up
-// ((2,3) hierarchy of R-MAT scale 16, 16 M triangles, 83 levels: 22.9 -> 7.4 ms, and 2.8 ms for counting and the lists).
+// ((2,3) hierarchy of R-MAT 2^16, 16.9 M triangles, 82 levels: the call 22.7 -> 11.4 ms, this kernel 7.4 of it and
+// counting and the lists 1.4).
 template <bool kBucket>
 __global__ void k_nuclei_union_inc(const int64_t* __restrict__ off, const uint32_t* __restrict__ list,
                                    const int32_t* __restrict__ row, int stride, const int32_t* __restrict__ core,
@@ -301,6 +303,81 @@ int thread_blocks(int64_t items) {
     return (int)std::max<int64_t>(1, std::min(want, cap));
 }
 
+// ---- whether to build incidence lists -------------------------------------------------------
+// The lists take a count and a fill of the whole graph. A hierarchy visits every s-clique from all of its
+// r-subsets and mostly gains; the pass over one level lists those of X alone, so few r-cliques are listed sooner.
+
+// out[0] += the work of listing every r-clique's s-cliques, out[1] += that of X's: the entries of the driving
+// lists (r = 2, where they differ most: one of a hub is as much as thousands of others), else the r-cliques
+__global__ void k_level_work(GraphView g, int r, const int32_t* __restrict__ core, int32_t level, int64_t n_r,
+                             unsigned long long* out) {
+    unsigned long long all = 0, in = 0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_r; i += (int64_t)gridDim.x * blockDim.x) {
+        int64_t w = 1;
+        if (r == 2) {
+            const int32_t u = g.eu[i], v = g.ev[i];
+            const int64_t du = g.rp[u + 1] - g.rp[u], dv = g.rp[v + 1] - g.rp[v];
+            w = du < dv ? du : dv;
+        }
+        all += w;
+        if (core[i] >= level) in += w;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        all += __shfl_down_sync(0xffffffffu, all, o);
+        in += __shfl_down_sync(0xffffffffu, in, o);
+    }
+    if ((threadIdx.x & 31) == 0 && all) {
+        atomicAdd(out, all);
+        if (in) atomicAdd(out + 1, in);
+    }
+}
+
+// nd_nuclei: from `least` r-cliques on, when X has at least share / 512 of the work. Measured, listing / lists in ms,
+// at level 0 and around the crossing: (1,3) R-MAT 2^17 472 / 125, its top level 373 / 109: always. (2,3) R-MAT 2^20
+// 514 / 148, its top level, with 29% of the work, 184 / 74; a flat R-MAT of 40,000 vertices 3.1 / 1.8, at 27% 1.36 /
+// 1.14, at 10% 0.67 / 0.91. (2,4) 500,009 vertices with communities 198 / 14, at 3% 37 / 11, at 0.01% 1.4 / 10.
+// (3,4) a million vertices 34 / 19, at 26% of the triangles 15.5 / 15.4, at 9% 7.4 / 14; 78,511 triangles 0.45 / 0.68.
+// (3,5), (3,6), (4,6) 50,000 vertices with communities 23 / 13, 169 / 87, 79 / 32; the flat graph 31 / 31, 84 / 81,
+// 32 / 27, at a third of the triangles 26 / 32. (1,4) and (2,5) count by listing from every r-clique, which is
+// the pass itself (122 / 163, 99 / 123), and (4,5) has its s-cliques at hand in the index (4.2 / 5.0): never.
+struct LevelRule {
+    int64_t least;
+    int share;
+};
+LevelRule level_rule(int r, int s) {
+    if (s == 3) return r == 1 ? LevelRule{0, 0} : LevelRule{1 << 16, 64};
+    if (r == 2 && s == 4) return LevelRule{1 << 12, 1};
+    if (r == 3 && s == 4) return LevelRule{1 << 21, 128};
+    if (r >= 3 && s >= r + 2) return LevelRule{1 << 12, 256};
+    return LevelRule{INT64_MAX, 0};
+}
+
+// sums: two zeroed device words
+int level_lists(nd_graph* g, int r, int s, const int32_t* core, int32_t level, int64_t n_r, unsigned long long* sums,
+                bool* want) {
+    const LevelRule rule = level_rule(r, s);
+    *want = n_r >= rule.least;
+    if (!*want || !rule.share) return ND_OK;
+    nd_ctx* c = g->ctx;
+    ND_K(k_level_work<<<thread_blocks(n_r), 256, 0, c->stream>>>(nd_view(g), r, core, level, n_r, sums));
+    int rc = nd_check_launch("nd_nuclei");
+    if (rc) return rc;
+    unsigned long long h[2];
+    cudaMemcpyAsync(c->pinned, sums, sizeof(h), cudaMemcpyDeviceToHost, c->stream);
+    if ((rc = nd_sync(c, "nd_nuclei"))) return rc;
+    memcpy(h, c->pinned, sizeof(h));
+    *want = (double)h[1] * 512 >= (double)h[0] * rule.share;
+    return ND_OK;
+}
+
+// nd_hierarchy, listing against lists: (2,3) R-MAT 2^16 22.7 / 11.4 ms, 20,000 edges 0.43 / 0.45; (3,4) a million
+// vertices 45 / 34, 118,000 triangles 0.74 / 0.84; (4,5) 5.8 / 6.4 and 4.9 / 5.8; larger s - r from 512 vertices on 1.2
+// ((4,6)) to 16 times ((2,4)) as fast.
+bool hierarchy_lists(const nd_graph* g, int r, int s, int64_t n_r) {
+    if (s >= r + 2) return g->m >= 1 << 11;
+    return r == 2 ? n_r >= 1 << 15 : r == 3 && n_r >= 1 << 17;
+}
+
 }  // namespace
 
 extern "C" int nd_nuclei(nd_graph* g, int r, int s, const int32_t* core, int32_t level, int32_t* comp_out, int flags,
@@ -329,7 +406,8 @@ extern "C" int nd_nuclei(nd_graph* g, int r, int s, const int32_t* core, int32_t
     GraphView v = nd_view(g);
     IncBufs inc;
     bool lists = false;
-    if (n_r) rc = nd_build_inc(g, r, s, n_r, inc, &lists);
+    if (n_r) rc = level_lists(g, r, s, cd, level, n_r, (unsigned long long*)((char*)scal.p + 16), &lists);
+    if (!rc && lists) rc = nd_build_inc(g, r, s, n_r, inc, &lists);
     if (!rc && lists)
         launch_union_inc<false>(inc, cd, level, nullptr, n_r, (int32_t*)parent.p, (int*)scal.p, st);
     else if (!rc && n_r && !dispatch_union(r, s, false, v, cd, level, nullptr, n_r, (int32_t*)parent.p, (int*)scal.p, st))
@@ -425,7 +503,7 @@ extern "C" int nd_hierarchy(nd_graph* g, int r, int s, const int32_t* core, int3
         release();
         return nd_set_error(ND_EINVAL, "nd_hierarchy: core numbers must lie in [0, 2^26) (got %d .. %d)", lo_hi[0], lo_hi[1]);
     }
-    if ((rc = nd_build_inc(g, r, s, n_r, inc, &lists))) {
+    if (hierarchy_lists(g, r, s, n_r) && (rc = nd_build_inc(g, r, s, n_r, inc, &lists))) {
         release();
         return rc;
     }

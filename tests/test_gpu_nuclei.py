@@ -4,6 +4,8 @@ component, -1 outside) and component counts are compared with the oracle's seque
 element by element, at every level of each decomposition, for every supported (r,s), on host and
 device pointers, including disjoint unions (components that must stay apart) and graphs with hubs.
 The core arrays given to both sides are the oracle's."""
+import math
+
 import numpy as np
 import pytest
 
@@ -152,3 +154,83 @@ def test_hierarchy_empty_and_bad_core(nd, ctx):
             nd.nd_hierarchy(G, 4, 7, np.zeros(g.n, np.int32))
     finally:
         nd.nd_graph_free(G)
+
+
+class _Hooks:
+    """Allocator hooks that note every size and refuse those of `refuse` bytes and more."""
+
+    def __init__(self, nd):
+        self.alloc, self.free = nd.torch_allocator_hooks(0)
+        self.refuse, self.sizes = 1 << 60, []
+
+    def take(self, nbytes, stream):
+        self.sizes.append(nbytes)
+        return 0 if nbytes >= self.refuse else self.alloc(nbytes, stream)
+
+    def largest(self, refuse, call):
+        """(result of call, the largest size it asked for) with this limit."""
+        self.refuse, self.sizes = refuse, []
+        try:
+            return call(), max(self.sizes, default=0)
+        finally:
+            self.refuse = 1 << 60
+
+
+def _lists(r, s, n_s):
+    """Bytes of the rows of the incidence lists."""
+    return 4 * ((math.comb(s, r) + 3) // 4 * 4) * n_s
+
+
+@pytest.mark.parametrize("r,s,scale,ef", [(1, 3, 13, 16), (2, 3, 14, 16), (2, 4, 12, 8), (3, 4, 14, 16), (3, 5, 11, 8), (3, 6, 9, 8), (4, 6, 9, 8)])
+def test_with_lists_and_by_listing(nd, r, s, scale, ef):
+    """Large enough for the incidence lists to be built, and without the memory for them: the same nuclei at
+    the lowest, a middle and the top level, and the same hierarchy."""
+    import torch
+
+    g = gg.rmat(scale, ef, seed=9601)
+    ctx = nd.nd_ctx_create(0, stream=torch.cuda.Stream())
+    hooks = _Hooks(nd)
+    nd.nd_ctx_set_allocator(ctx, hooks.take, hooks.free)
+    G = nd.nd_load_csr(ctx, g.rowptr, g.col)
+    try:
+        core, _, st = nd.nd_decompose(G, r, s, want_round=False)
+        rows = _lists(r, s, st["n_s"])
+        assert rows > 4 * core.size
+        dcore = torch.from_numpy(core).cuda()
+        for level in (0, int(np.median(core)), int(core.max())):
+            (want, n), most = hooks.largest(1 << 60, lambda: nd.nd_nuclei(G, r, s, dcore, level))
+            assert level or most >= rows
+            (got, k), most = hooks.largest(rows, lambda: nd.nd_nuclei(G, r, s, dcore, level))
+            assert level or most >= rows
+            assert k == n and torch.equal(got, want)
+        want, most = hooks.largest(1 << 60, lambda: nd.nd_hierarchy(G, r, s, dcore))
+        assert most >= rows
+        got, _ = hooks.largest(rows, lambda: nd.nd_hierarchy(G, r, s, dcore))
+        assert got[3] == want[3] and all(torch.equal(a, b) for a, b in zip(got[:3], want[:3]))
+    finally:
+        nd.nd_graph_free(G)
+        nd.nd_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("r,s", [(1, 4), (2, 3), (2, 4), (2, 5), (3, 4), (3, 5), (4, 5)])
+def test_a_level_of_few_r_cliques_is_listed(nd, r, s):
+    """The nuclei of a level that only one K_25 of a larger graph reaches take no room for the lists of the
+    whole graph."""
+    import torch
+
+    g = gg.with_planted(gg.chung_lu(40_000, 12.0, 2.3, seed=9701), 1, 25, 25, 1.0, seed=9702)
+    ctx = nd.nd_ctx_create(0, stream=torch.cuda.Stream())
+    hooks = _Hooks(nd)
+    nd.nd_ctx_set_allocator(ctx, hooks.take, hooks.free)
+    G = nd.nd_load_csr(ctx, g.rowptr, g.col)
+    try:
+        core, _, st = nd.nd_decompose(G, r, s, want_round=False)
+        top = int(core.max())
+        assert np.count_nonzero(core == top) == math.comb(25, r)
+        got, most = hooks.largest(1 << 60, lambda: nd.nd_nuclei(G, r, s, core, top))
+        want = orc.nuclei(g, r, s, core, top)
+        assert got[1] == want[1] == 1 and np.array_equal(got[0], want[0])
+        assert most <= 4 * core.size + 256
+    finally:
+        nd.nd_graph_free(G)
+        nd.nd_ctx_destroy(ctx)
