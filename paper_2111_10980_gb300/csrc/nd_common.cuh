@@ -472,6 +472,10 @@ int nd_inc_stride(int r, int s);
 int64_t nd_inc_rows(int r, int s, int64_t n_r, int64_t m, int64_t n_s, bool tight, unsigned* run);
 void nd_inc_fill(const GraphView& g, int r, int s, int64_t n_r, const IncFill& F, cudaStream_t st);
 
+// adds the s-cliques of a part of the graph to *out (zeroed) and returns which part: one in that many; for
+// s >= 5 each counts C(s,r) times
+int64_t nd_sample_cliques(const GraphView& g, int r, int s, int64_t n_r, unsigned long long* out, cudaStream_t st);
+
 // counting (nd_count.cu): counts into cnt (CT = int32_t or int64_t), zero-initialised
 template <typename CT>
 void nd_count_launch(const GraphView& g, int r, int s, CT* cnt, int64_t n_r, cudaStream_t st);

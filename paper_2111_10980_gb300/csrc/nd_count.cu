@@ -164,6 +164,54 @@ __global__ void k_count_gen(GraphView g, CT* __restrict__ cnt, int64_t n_r) {
     }
 }
 
+// Estimates of the number of s-cliques, from a part of the graph: *out += those of one tile of DG edges in
+// `every` (triangles), of one DG edge in `every` (4-cliques), of one r-clique in `every` (any (r,s), each s-clique
+// from C(s,r) of them)
+__device__ __forceinline__ void add_total(unsigned long long c, unsigned long long* out) {
+    for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
+    if ((threadIdx.x & 31) == 0 && c) atomicAdd(out, c);
+}
+
+struct TotalTri {
+    unsigned long long n = 0;
+    __device__ void begin(int) const {}
+    __device__ void tri(bool hit, int, int32_t, int32_t, int32_t, bool, int32_t, int32_t, int32_t) { n += hit; }
+    __device__ void end(int, int32_t, int32_t, int32_t) const {}
+};
+
+__global__ void __launch_bounds__(kTriThreads) k_sample_tri(GraphView g, int tile, int64_t every, unsigned long long* out) {
+    TotalTri sink;
+    tri_list(g, tile, sink, every);
+    add_total(sink.n, out);
+}
+
+struct Total24 {
+    unsigned long long n = 0;
+    static constexpr bool kTally = false;
+    __device__ void clique(bool hit, const int32_t (&)[6]) { n += hit; }
+};
+
+__global__ void __launch_bounds__(kQuadThreads) k_sample24(GraphView g, int64_t every, unsigned long long* out) {
+    Total24 sink;
+    quad24_list(g, sink, every);
+    add_total(sink.n, out);
+}
+
+template <int R_, int S_>
+__global__ void k_sample_gen(GraphView g, int64_t n_r, int64_t every, unsigned long long* out) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long c = 0;
+    for (int64_t id = gwarp() * every; id < n_r; id += nwarps() * every) {
+        int32_t v[4];
+        gen_verts<R_>(g, id, v);
+        const int32_t* list = nullptr;
+        int64_t len = 0;
+        gen_drive<R_>(g, id, v, list, len);
+        for (int64_t j = lane; j < len; j += 32) gen_cand<R_, S_>(g, v, list[j], [&](const int32_t*) { ++c; });
+    }
+    add_total(c, out);
+}
+
 template <typename CT>
 __global__ void k_zero(CT* p, int64_t n) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
@@ -203,6 +251,29 @@ void nd_count_launch(const GraphView& g, int r, int s, CT* cnt, int64_t n_r, cud
     } else if (r == 4 && s == 6) {
         ND_K(k_count_gen<CT, 4, 6><<<blk, kThreads, 0, st>>>(g, cnt, n_r));
     }
+}
+
+// at least 16,384 samples, a sixty-fourth of a large graph
+int64_t nd_sample_cliques(const GraphView& g, int r, int s, int64_t n_r, unsigned long long* out, cudaStream_t st) {
+    const int tile = tri_tile(g.m);
+    const int64_t items = s == 3 ? (g.m + tile - 1) / tile : s == 4 ? g.m : n_r;
+    const int64_t part = items >> 14, every = part < 1 ? 1 : part > 64 ? 64 : part;
+    const int blk = blocks_for_warps((items + every - 1) / every);
+    if (s == 3)
+        ND_K(k_sample_tri<<<blk, kTriThreads, 0, st>>>(g, tile, every, out));
+    else if (s == 4)
+        ND_K(k_sample24<<<blk, kQuadThreads, 0, st>>>(g, every, out));
+    else if (r == 2)
+        ND_K(k_sample_gen<2, 5><<<blk, kThreads, 0, st>>>(g, n_r, every, out));
+    else if (r == 3 && s == 5)
+        ND_K(k_sample_gen<3, 5><<<blk, kThreads, 0, st>>>(g, n_r, every, out));
+    else if (r == 3)
+        ND_K(k_sample_gen<3, 6><<<blk, kThreads, 0, st>>>(g, n_r, every, out));
+    else if (s == 5)
+        ND_K(k_sample_gen<4, 5><<<blk, kThreads, 0, st>>>(g, n_r, every, out));
+    else
+        ND_K(k_sample_gen<4, 6><<<blk, kThreads, 0, st>>>(g, n_r, every, out));
+    return every;
 }
 
 template void nd_count_launch<int32_t>(const GraphView&, int, int, int32_t*, int64_t, cudaStream_t);

@@ -32,8 +32,9 @@ __device__ __forceinline__ int stage_find24(const int32_t* a, int n, int32_t x) 
     return (lo < n && a[lo] == x) ? lo : -1;
 }
 
+// With `every` > 1 only one DG edge in that many is taken, for an estimate.
 template <typename Sink>
-__device__ __forceinline__ void quad24_list(const GraphView& g, Sink& sink) {
+__device__ __forceinline__ void quad24_list(const GraphView& g, Sink& sink, int64_t every = 1) {
     constexpr int kWarpsPerBlock = kQuadThreads / 32;
     __shared__ int32_t s_w[kWarpsPerBlock][kC24], s_eu[kWarpsPerBlock][kC24], s_ev[kWarpsPerBlock][kC24],
         s_b[kWarpsPerBlock][kC24], s_p[kWarpsPerBlock][kC24 + 1];
@@ -42,7 +43,7 @@ __device__ __forceinline__ void quad24_list(const GraphView& g, Sink& sink) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int32_t *sw = s_w[wid], *seu = s_eu[wid], *sev = s_ev[wid], *sb = s_b[wid], *sp = s_p[wid];
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; j < g.m; j += nwarps) {
+    for (int64_t j = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * every; j < g.m; j += nwarps * every) {
         const int32_t v = g.dg_col[j], e_uv = g.dg_eid[j];
         const int32_t u = g.eu[e_uv] == v ? g.ev[e_uv] : g.eu[e_uv];
         const int64_t ub = g.dg_rp[u], ue = g.dg_rp[u + 1], vb = g.dg_rp[v], vn = g.dg_rp[v + 1] - vb;

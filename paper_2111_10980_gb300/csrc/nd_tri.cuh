@@ -26,12 +26,13 @@ inline int tri_tile(int64_t m) {
 // Bound by the bisections' loads (L1 and L2) and, past them, by the sinks' atomics. Against one warp per edge
 // merging the two undirected rows, which meets each triangle three times: (2,3) counts of R-MAT scale 20
 // 42 -> 16.5 ms, of a Chung-Lu graph with 2.4 M edges 1.10 -> 0.33 ms.
+// With `every` > 1 only one tile of edges in that many is taken, for an estimate.
 template <typename Sink>
-__device__ __forceinline__ void tri_list(const GraphView& g, int tile, Sink& sink) {
+__device__ __forceinline__ void tri_list(const GraphView& g, int tile, Sink& sink, int64_t every = 1) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t j0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * tile; j0 < g.m; j0 += nwarps * tile) {
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5, apart = tile * every;
+    for (int64_t j0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * apart; j0 < g.m; j0 += nwarps * apart) {
         const int64_t j = lane < tile ? j0 + lane : g.m;
         int32_t u = 0, v = 0, e = 0, xb = 0, xn = 0, yb = 0, yn = 0;  // DG positions are below m < 2^31
         int32_t of_u = 0;

@@ -234,3 +234,60 @@ def test_a_level_of_few_r_cliques_is_listed(nd, r, s):
     finally:
         nd.nd_graph_free(G)
         nd.nd_ctx_destroy(ctx)
+
+
+def test_lists_that_cannot_fit_are_not_counted_for(nd):
+    """K_100 as (3,4), whose lists (125 MB) are over the context's budget: the hierarchy allocates neither counts'
+    directory nor anything else as large."""
+    import torch
+
+    g = gg.complete(100)
+    ctx = nd.nd_ctx_create(0, stream=torch.cuda.Stream(), mem_budget=100 << 20)
+    hooks = _Hooks(nd)
+    nd.nd_ctx_set_allocator(ctx, hooks.take, hooks.free)
+    G = nd.nd_load_csr(ctx, g.rowptr, g.col)
+    try:
+        core = np.full(len(nd.nd_rcliques(G, 3)), 97, np.int32)
+        got, most = hooks.largest(1 << 60, lambda: nd.nd_hierarchy(G, 3, 4, core))
+        assert got[3] == 1 and not got[0].any() and np.all(got[1] == -1) and np.all(got[2] == -1)
+        assert most <= 4 * core.size + 256
+    finally:
+        nd.nd_graph_free(G)
+        nd.nd_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("r,s", [(1, 3), (2, 3), (1, 4), (2, 4), (2, 5), (3, 4), (3, 5), (3, 6), (4, 6)])
+def test_a_budget_on_either_side_of_the_lists(nd, r, s):
+    """The hierarchy under budgets that leave half and twice the bytes of the lists, on a graph where the bound on the
+    counts does not settle which: read from the lists in one case, listed in the other, and the same."""
+    import torch
+
+    g = gg.rmat(13 if s < 5 else 10, 8, seed=9801)
+
+    def run(budget, core):
+        """The hierarchy (and the cores, if there are none yet), whether lists were built, bytes held by graph and index."""
+        ctx = nd.nd_ctx_create(0, stream=torch.cuda.Stream(), mem_budget=budget)
+        hooks = _Hooks(nd)
+        nd.nd_ctx_set_allocator(ctx, hooks.take, hooks.free)
+        G = nd.nd_load_csr(ctx, g.rowptr, g.col)
+        try:
+            n_s = nd.nd_count(G, r, s)[2]
+            if core is None:
+                core = torch.from_numpy(nd.nd_decompose(G, r, s, want_round=False)[0]).cuda()
+            held = nd.nd_ctx_bytes_in_use(ctx)
+            got, most = hooks.largest(1 << 60, lambda: nd.nd_hierarchy(G, r, s, core))
+            return core, n_s, held, most >= _lists(r, s, n_s), got
+        finally:
+            nd.nd_graph_free(G)
+            nd.nd_ctx_destroy(ctx)
+
+    core, n_s, held, built, want = run(0, None)
+    assert built
+    n_r = core.numel()
+    lists = _lists(r, s, n_s) + 4 * math.comb(s, r) * n_s + 16 * n_r
+    others = held + 14 * 4 * n_r + (1 << 16)  # the hierarchy's arrays of one int32 for each r-clique, and the counts
+    for budget, expect in ((others + lists // 2, False), (others + 2 * lists, True)):
+        *_, built, got = run(budget, core)
+        assert got[3] == want[3] and all(torch.equal(a, b) for a, b in zip(got[:3], want[:3]))
+        # the (3,4) count's directory is larger than its lists here and may take the room of twice them
+        assert built == expect or (r, s) == (3, 4)
