@@ -1268,14 +1268,17 @@ int nd_decompose_dev(nd_graph* g, int r, int s, int count_width, int flags, Peel
     cudaEventRecord(e0, c->stream);
     // (3,4): the hash directory of the long triangle lists serves the count's searches and the
     // peel's lookups; it is built inside the counting interval and freed with the decomposition
-    if (!rc && r == 3 && s == 4) {
-        rc = build_tri_hash(g, g->hoff, g->htab, g->hpos);
-        if (rc == ND_ENOMEM) {
-            // the directory is an accelerator: without room for it the lists are bisected
-            for (DBuf* b : {&g->hoff, &g->htab, &g->hpos}) nd_free(c, *b);
-            rc = ND_OK;
-        }
-    }
+    auto free_directory = [&]() {
+        for (DBuf* b : {&g->hoff, &g->htab, &g->hpos}) nd_free(c, *b);
+    };
+    auto directory = [&]() {
+        if (r != 3 || s != 4) return (int)ND_OK;
+        const int e = build_tri_hash(g, g->hoff, g->htab, g->hpos);
+        if (e != ND_ENOMEM) return e;
+        free_directory();  // it is an accelerator: without room for it the lists are bisected
+        return (int)ND_OK;
+    };
+    if (!rc) rc = directory();
     cudaEventRecord(eh, c->stream);
     if (!rc) rc = nd_count_into(g, r, s, w, n_r, cnt);
     cudaEventRecord(e1, c->stream);
@@ -1291,8 +1294,7 @@ int nd_decompose_dev(nd_graph* g, int r, int s, int count_width, int flags, Peel
             use_inc = false;
             rc = ND_OK;
         }
-        if (use_inc)
-            for (DBuf* b : {&g->hoff, &g->htab, &g->hpos}) nd_free(c, *b);  // the lists replace it
+        if (use_inc) free_directory();  // the lists replace it
     }
     auto peel = [&](const IncBufs* lists) {
         return (w == 8) ? run_peel<int64_t>(g, r, s, cnt, n_r, flags, po, lists)
@@ -1300,8 +1302,16 @@ int nd_decompose_dev(nd_graph* g, int r, int s, int count_width, int flags, Peel
     };
     if (!rc) rc = peel(use_inc ? &inc : nullptr);
     nd_free_inc(c, inc);
-    // the lists may have taken the room of the peel's own buffers, which are allocated before it begins
-    if (use_inc && rc == ND_ENOMEM) rc = peel(nullptr);
+    // the lists may have taken the room of the peel's own buffers, which are allocated before it begins; and so may
+    // the directory that a peel without them looks up
+    if (use_inc && rc == ND_ENOMEM) {
+        rc = directory();
+        if (!rc) rc = peel(nullptr);
+        if (rc == ND_ENOMEM && g->htab.p) {
+            free_directory();
+            rc = peel(nullptr);
+        }
+    }
     float tc = 0, tp = 0, th = 0;
     if (!rc) {
         cudaEventElapsedTime(&tc, e0, e1);
@@ -1309,7 +1319,7 @@ int nd_decompose_dev(nd_graph* g, int r, int s, int count_width, int flags, Peel
         cudaEventElapsedTime(&th, e0, eh);
     }
     nd_free(c, cnt);
-    for (DBuf* b : {&g->hoff, &g->htab, &g->hpos}) nd_free(c, *b);
+    free_directory();
     if (rc) return rc;
     S.n_r = n_r;
     S.n_s = n_s;

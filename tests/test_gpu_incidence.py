@@ -107,3 +107,42 @@ def test_the_memory_of_a_run_without_lists_is_enough(nd, r, s):
     alone = run(True, 1 << 40)
     for extra in (0, rows // 2, rows, 2 * rows):
         run(False, alone + extra)
+
+
+def test_a_peel_without_room_next_to_its_lists_has_its_directory(nd):
+    """K_60 as (3,4): when the peel's buffers are refused next to the incidence lists, the peel without them finds
+    the hash directory that it looks up, which had made room for the lists."""
+    import torch
+
+    g = gg.complete(60)
+    n_r, n_s = math.comb(60, 3), math.comb(60, 4)
+    table = 16 * g.m << 7  # 58 entries in 128 slots for every edge
+    alloc, free = nd.torch_allocator_hooks(0)
+    sizes, full, refused, arm = [], [False], [], False
+
+    def take(nbytes, stream):
+        if full[0]:
+            refused.append(nbytes)
+            return 0
+        sizes.append(nbytes)
+        return alloc(nbytes, stream)
+
+    def give(p, nbytes, stream):
+        if arm:
+            full[0] = (full[0] or nbytes == table) and not refused  # from when the directory goes until the lists do
+        free(p, nbytes, stream)
+
+    ctx = nd.nd_ctx_create(0, stream=torch.cuda.Stream())
+    nd.nd_ctx_set_allocator(ctx, take, give)
+    G = nd.nd_load_csr(ctx, g.rowptr, g.col)
+    try:
+        nd.nd_rcliques(G, 3)
+        for arm, tables in ((False, 1), (True, 2)):
+            sizes.clear()
+            core, rnd, st = nd.nd_decompose(G, 3, 4)
+            assert core.size == n_r and np.all(core == 57) and not rnd.any() and st["rho"] == 1 and st["listed"] == n_s
+            assert max(sizes) >= 4 * 4 * n_s and sizes.count(table) == tables and bool(refused) == arm
+    finally:
+        arm = False
+        nd.nd_graph_free(G)
+        nd.nd_ctx_destroy(ctx)
