@@ -315,8 +315,10 @@ typedef struct nd_server_cfg {
     int32_t flags;         /* how a worker launches a batch's peeling loop: ND_PEEL_LOOP_GRAPH (a CUDA graph
                               per batch; the workers' batches share the SMs), ND_PEEL_PERSISTENT (one
                               cooperative kernel per batch, holding every SM; batches take turns), or 0
-                              (a cooperative kernel on 1 / workers of the SMs for batches of up to 2^20
-                              r-cliques, a CUDA graph for larger ones; the batches share the SMs) */
+                              (with one worker ND_PEEL_PERSISTENT; with more a cooperative kernel on
+                              1 / workers of the SMs, at least 8 blocks, for batches of up to 2^20 r-cliques
+                              whose s-cliques are few for the rounds that their counts suggest, a CUDA graph
+                              for the others; the batches share the SMs) */
 } nd_server_cfg;
 
 typedef struct nd_result {

@@ -902,8 +902,39 @@ int nd_build_inc(nd_graph* g, int r, int s, int64_t n_r, IncBufs& b, bool* built
     return rc;
 }
 
+// Whether a server's worker that was not told how to peel runs its batch as a cooperative kernel on its share of
+// the SMs, where the workers' kernels fit side by side, or as a loop graph, whose kernels spread over all SMs.
+// A round costs about 7 us in the kernel and 20 in the graph, and nothing is captured; the work, one visit for each
+// r-clique of each s-clique at about 1e11 a second on the whole GPU, takes as many times as long as there are
+// workers. So the share wins when rounds * 13 us > work * (workers - 1) / 1e11 per s. The rounds are not known, but
+// equal counts go in few of them and skewed ones in many; the guess is 90 times what the largest count is above
+// the mean, over the mean, and 40 at least: (2,4) of R-MAT 2^10 to 2^16 and of planted communities go in 60 to 350
+// times the quotient, cliques and G(n, p) in 1 to 112 rounds. Measured with 8 workers, a request alone and 8 at
+// once, share / graph in ms: (2,4) R-MAT 2^14 (48 M 4-cliques, 7,212 rounds) 110 / 171 and 165 / 492, R-MAT 2^16 (270 M)
+// 363 / 366 and 659 / 1,250; (2,3) R-MAT 2^16 26 / 30 and 40 / 79; K_1000 as (2,3) (166 M triangles, one round) 47 / 16
+// and 137 / 106, K_250 as (2,4) 103 / 28 and 368 / 189. Beyond 2^20 r-cliques their scans weigh as much as the
+// rounds: 1.9 M edges of R-MAT 2^17 48 / 47 and 143 / 133, 3.8 M 92 / 74.
 template <typename CT>
-static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags, PeelOut& po,
+static int peel_shared(nd_graph* g, int r, int s, const DBuf& cnt, int64_t n_r, int64_t n_s, bool* shared) {
+    constexpr int64_t kShareMax = (int64_t)1 << 20;
+    constexpr double kLeastRounds = 40, kSkewRounds = 90, kVisitsPerRound = 1.3e6;
+    const double visits = (double)n_s * (double)binom64(s, r), work = visits * (g->ctx->peel_share - 1);
+    *shared = n_r <= kShareMax;
+    if (!*shared || work <= kLeastRounds * kVisitsPerRound) return ND_OK;
+    unsigned long long most = 0;
+    ND_TRY(scalar_zero(g));
+    if (sizeof(CT) == 8)
+        nd_max_i64((const int64_t*)cnt.p, n_r, (unsigned long long*)g->scal.p, g->ctx->stream);
+    else
+        nd_max_i32((const int32_t*)cnt.p, n_r, (unsigned long long*)g->scal.p, g->ctx->stream);
+    ND_TRY(nd_check_launch("peel setup"));
+    ND_TRY(read_back(g, g->scal.p, &most, "peel setup"));
+    *shared = work <= kSkewRounds * kVisitsPerRound * ((double)most * (double)n_r / visits - 1);
+    return ND_OK;
+}
+
+template <typename CT>
+static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int64_t n_s, int flags, PeelOut& po,
                     const IncBufs* inc = nullptr) {
     nd_ctx* c = g->ctx;
     cudaStream_t st = c->stream;
@@ -1106,18 +1137,12 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int flags
                  contract_every, contract_shift, inc ? (const unsigned int*)inc->status.p : nullptr, inc ? inc->n_s : 0);
     bool looped = false;
     int persistent_launches = 0;
-    // A server's workers that were not told how to peel run short decompositions as cooperative kernels on
-    // their share of the SMs, where they all fit side by side: a round costs 7 us against 20 in the loop
-    // graph, and nothing is captured (64 graphs of 30 to 10,000 vertices in a burst,
-    // four workers: 17.1 -> 8.1 ms). Beyond kShareMax r-cliques a round
-    // has work for the whole GPU, which the loop graph's kernels can spread over.
-    constexpr int64_t kShareMax = (int64_t)1 << 20;
     bool want_persistent = (flags & ND_PEEL_PERSISTENT) || !(flags & (ND_NO_GRAPH | ND_PEEL_LOOP_GRAPH));
     if (flags & ND_PEEL_PERSISTENT)
         P.grid_share = 1;
-    else if (c->peel_share > 1 && n_r > kShareMax)
-        want_persistent = false;
-    if (want_persistent) {
+    else if (want_persistent && c->peel_share > 1)
+        rc = peel_shared<CT>(g, r, s, cnt, n_r, n_s, &want_persistent);
+    if (want_persistent && !rc) {
         // preferred: the whole loop in one cooperative kernel
         cudaError_t e = nd_peel_persistent<CT>(v, r, s, P, st);
         if (e == cudaSuccess) {
@@ -1297,8 +1322,8 @@ int nd_decompose_dev(nd_graph* g, int r, int s, int count_width, int flags, Peel
         if (use_inc) free_directory();  // the lists replace it
     }
     auto peel = [&](const IncBufs* lists) {
-        return (w == 8) ? run_peel<int64_t>(g, r, s, cnt, n_r, flags, po, lists)
-                        : run_peel<int32_t>(g, r, s, cnt, n_r, flags, po, lists);
+        return (w == 8) ? run_peel<int64_t>(g, r, s, cnt, n_r, n_s, flags, po, lists)
+                        : run_peel<int32_t>(g, r, s, cnt, n_r, n_s, flags, po, lists);
     };
     if (!rc) rc = peel(use_inc ? &inc : nullptr);
     nd_free_inc(c, inc);
@@ -1437,7 +1462,7 @@ int nd_kcore_rounds(nd_graph* g, DBuf& rnd_out) {
     int rc = nd_alloc(c, po.core, 4 * std::max<int64_t>(n, 1));
     if (!rc) rc = nd_alloc(c, po.rnd, 4 * std::max<int64_t>(n, 1));
     if (!rc) rc = nd_count_into(g, 1, 2, 4, n, cnt);
-    if (!rc) rc = run_peel<int32_t>(g, 1, 2, cnt, n, 0, po);
+    if (!rc) rc = run_peel<int32_t>(g, 1, 2, cnt, n, g->m, 0, po);
     nd_free(c, cnt);
     nd_free(c, po.core);
     if (rc) {

@@ -1,6 +1,7 @@
 """Batches and the continuous-batching server: every graph's result in a batch, or served in a
 mix of concurrent requests, is the same as the graph decomposed alone and as the oracle's.
 The work is integer, so "the same" means bit for bit."""
+import math
 import time
 
 import numpy as np
@@ -344,3 +345,44 @@ def test_server_lists_in_the_room_there_is(nd):
         seen.append("none" if most < rows else "tight" if most < rows + 256 else "spare")
         assert hooks.peak <= budget
     assert seen == ["none", "tight", "spare"]
+
+
+@pytest.mark.parametrize("workers", [1, 3])
+@pytest.mark.parametrize("flags", ["0", "ND_PEEL_LOOP_GRAPH", "ND_PEEL_PERSISTENT"])
+def test_server_in_every_launch_mode(nd, ctx, flags, workers):
+    """Mixed requests, and with the default flags a batch of more than 2^20 r-cliques among them."""
+    items = mixed_graphs(24, 19)
+    want = [orc.decompose(g, r, s).core for g, r, s in items]
+    if flags == "0":
+        big = gg.chung_lu(120_000, 20.0, 2.4, seed=20)
+        assert big.m > 1 << 20
+        items.append((big, 2, 3))
+        want.append(alone(nd, ctx, big, 2, 3))
+    tickets, outs, results = _serve(nd, ctx, items, workers=workers, max_batch=4, flags=0 if flags == "0" else getattr(nd, flags))
+    for (g, r, s), t, (out, k), w in zip(items, tickets, outs, want):
+        assert results[t][0] == nd.ND_OK
+        assert np.array_equal(out[:k], w), (g.name, r, s)
+
+
+@pytest.mark.parametrize("name,r,s,shared", [("K400", 2, 3, False), ("K120", 2, 4, False), ("K30", 2, 3, True), ("rmat", 2, 4, True)])
+def test_server_shares_the_gpu_where_the_rounds_outweigh_the_work(nd, ctx, name, r, s, shared):
+    """By default a batch of equal counts with much work, which goes in one round, takes the loop graph, as the
+    launches show (one kernel for the whole loop against several for each round); a small one, and one with
+    skewed counts, a share of the SMs."""
+    g = gg.rmat(11, 16, 0.57, 0.19, 0.19, seed=21) if name == "rmat" else gg.complete(int(name[1:]))
+    want = orc.decompose(g, r, s).core if name == "rmat" else np.full(g.m, math.comb(g.n - 2, s - 2))
+    launches = []
+    for flags in (0, nd.ND_PEEL_LOOP_GRAPH):
+        sv = nd.nd_server_create(ctx, workers=8, max_batch=1, flags=flags)
+        try:
+            out = np.full(g.m, -1, np.int32)
+            before = nd.nd_kernel_launches()
+            t = sv.submit(g.rowptr, g.col, r, s, out)
+            sv.drain()
+            launches.append(nd.nd_kernel_launches() - before)
+            assert sv.poll(t)[0] == nd.ND_OK
+            assert np.array_equal(out, want)
+        finally:
+            sv.close()
+    # with the graph the two differ by the maximum of the counts, which the default looks at
+    assert (launches[0] < launches[1]) == shared, launches
