@@ -792,8 +792,8 @@ static int build_tri_hash(nd_graph* g, DBuf& hoff, DBuf& htab, DBuf& hpos) {
 
 // Whether a decomposition is peeled from incidence lists, and b's buffers if so. (1,2) has them in the CSR itself; a (3,4) run that
 // is asked to contract before every round contracts its triangle lists. The lists are an accelerator and must leave room for others,
-// hence the bound (nd_ctx::inc_bytes, on all the buffers together; a server's batch is charged that much; and what
-// the context's budget has left); the (3,4) lists of R-MAT graphs from scale 17 on, for instance, are over it, and their s-cliques are listed again by Update.
+// hence the bound (nd_ctx::inc_bytes on all the buffers together, what the context's budget has left, and what a
+// server's budget grants); the (3,4) lists of R-MAT graphs from scale 17 on, for instance, are over it, and their s-cliques are listed again by Update.
 static bool plan_inc(const nd_graph* g, int r, int s, int flags, int64_t n_r, int64_t n_s, IncBufs& b) {
     if ((r == 1 && s == 2) || (r == 3 && s == 4 && (flags & ND_CONTRACT_ALWAYS))) return false;
     // (1,4) and (2,5) count from every r-clique and fill from the lowest of each s-clique: the places that the
@@ -812,7 +812,10 @@ static bool plan_inc(const nd_graph* g, int r, int s, int flags, int64_t n_r, in
         b.mem.add(b.row, 4 * b.stride * b.rows);
         b.mem.add(b.dead, 4 * (b.rows / 32 + 1));
         b.mem.add(b.status, 16);
-        if (b.mem.bytes() <= (size_t)std::min(g->ctx->inc_bytes, budget_room(g->ctx))) return true;
+        const nd_ctx* c = g->ctx;
+        if (b.mem.bytes() <= (size_t)std::min(c->inc_bytes, budget_room(c)) &&
+            (!c->grant || c->grant(c->grant_arg, b.mem.bytes())))
+            return true;
     }
     b.mem.want.clear();
     return false;

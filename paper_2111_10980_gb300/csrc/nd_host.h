@@ -37,6 +37,8 @@ struct nd_ctx {
     int32_t limit_flags = 0;
     int peel_share = 1;  // of a server's worker: the workers whose peel kernels share the GPU
     int64_t inc_bytes = (int64_t)16 << 30;  // most device bytes of a decomposition's incidence lists, all their buffers together
+    bool (*grant)(void* arg, size_t bytes) = nullptr;  // of a server's worker: asks the budget for the lists' bytes
+    void* grant_arg = nullptr;
     void* stage = nullptr;  // pinned staging of batches (grown on demand)
     size_t stage_bytes = 0;
     // nd_ctx_set_tuning, indexed by r * 8 + s

@@ -393,9 +393,37 @@ struct nd_server {
     std::vector<nd_ctx*> wctx;
 };
 
+// A worker's claims on the budget for its batch's incidence lists, whose size is known only after counting. They
+// count as used while the batch runs.
+struct Grants {
+    nd_server* sv;
+    size_t taken = 0;
+};
+
+// The lists may take a share of what is left, and nothing that the oldest waiting request could be admitted with.
+static bool grant_lists(void* arg, size_t bytes) {
+    Grants* gr = (Grants*)arg;
+    nd_server* sv = gr->sv;
+    std::lock_guard<std::mutex> lk(sv->mu);
+    const size_t budget = sv->cfg.mem_budget, left = sv->used < budget ? budget - sv->used : 0;
+    if (bytes > left / (2 * (size_t)sv->cfg.workers)) return false;
+    if (!sv->queue.empty()) {
+        const size_t need = sv->queue.front()->est;
+        if (need <= left && need + bytes > left) return false;
+    }
+    sv->used += bytes;
+    gr->taken += bytes;
+    return true;
+}
+
 static void worker_loop(nd_server* sv, int w) {
     cudaSetDevice(sv->ctx->device);
     nd_ctx* ctx = sv->wctx[w];
+    Grants grants{sv};
+    if (sv->cfg.mem_budget) {
+        ctx->grant = grant_lists;
+        ctx->grant_arg = &grants;
+    }
     for (;;) {
         std::vector<Ticket*> batch;
         size_t est = 0;
@@ -424,13 +452,6 @@ static void worker_loop(nd_server* sv, int w) {
                     ++it;
                 }
             }
-            // incidence lists, whose size is known only after counting, may take a part of what the
-            // budget leaves; it counts as used while the batch runs
-            if (sv->cfg.mem_budget) {
-                const size_t held = sv->used + est, spare = held < sv->cfg.mem_budget ? sv->cfg.mem_budget - held : 0;
-                ctx->inc_bytes = (int64_t)std::min<size_t>(spare / (2 * (size_t)sv->cfg.workers), (size_t)16 << 30);
-                est += (size_t)ctx->inc_bytes;
-            }
             sv->used += est;
             sv->running++;
         }
@@ -448,7 +469,8 @@ static void worker_loop(nd_server* sv, int w) {
                 t->status = t->req.status;
                 sv->unfinished--;
             }
-            sv->used -= est;
+            sv->used -= est + grants.taken;
+            grants.taken = 0;
             sv->running--;
         }
         sv->cv_done.notify_all();

@@ -386,3 +386,29 @@ def test_server_shares_the_gpu_where_the_rounds_outweigh_the_work(nd, ctx, name,
             sv.close()
     # with the graph the two differ by the maximum of the counts, which the default looks at
     assert (launches[0] < launches[1]) == shared, launches
+
+
+def test_server_admits_what_fits_next_to_a_running_batch(nd, ctx):
+    """Two requests whose estimates fit the budget together run side by side: the first holds no room for lists
+    that it does not build (2.7 GB of them here)."""
+    g = gg.rmat(14, 16, 0.57, 0.19, 0.19, seed=22)
+    # what admission charges a request with r = 2: CSR, edge index, orientation and the state of the edges
+    est = 40 * (g.n + 1) + 80 * g.m + (1 << 16)
+    sv = nd.nd_server_create(ctx, workers=2, max_batch=1, mem_budget=2 * est + (1 << 20), flags=nd.ND_PEEL_LOOP_GRAPH)
+    outs = [np.full(g.m, -1, np.int32) for _ in range(2)]
+    try:
+        with pytest.raises(nd.NdError):  # the estimate is no smaller
+            small = nd.nd_server_create(ctx, workers=1, mem_budget=est - 64 * g.n)
+            try:
+                small.submit(g.rowptr, g.col, 2, 4, outs[0])
+            finally:
+                small.close()
+        first = sv.submit(g.rowptr, g.col, 2, 4, outs[0])
+        time.sleep(0.03)
+        second = sv.submit(g.rowptr, g.col, 2, 4, outs[1])
+        sv.drain()
+        (a, one), (b, two) = sv.poll(first), sv.poll(second)
+        assert a == b == nd.ND_OK and np.array_equal(*outs)
+        assert one["run_ms"] > 100 and two["queue_ms"] < one["run_ms"] / 2, (one, two)
+    finally:
+        sv.close()
