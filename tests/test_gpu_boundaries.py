@@ -1,8 +1,10 @@
 """Sizes at which the kernels change their way: closed forms on cliques whose edges have 127, 128 and
-129 common neighbours (lists gathered and ordered up to 128, merged out of the rows beyond), next to a
-hub whose row runs over many segments of the edge index, long runs of empty rows before, between and
-after, and graphs too small to fill a warp."""
+129 common neighbours (lists gathered and ordered up to 128, merged out of the rows beyond; the 4-cliques of
+an edge staged up to 128 common out-neighbours, walked beyond), next to a hub whose row runs over many
+segments of the edge index, long runs of empty rows before, between and after, and graphs too small to fill
+a warp."""
 import itertools
+import math
 
 import numpy as np
 import pytest
@@ -35,10 +37,24 @@ def _graph(cliques, leaves, gap):
     return gg.csr_from_edges(n, np.concatenate(us).astype(np.int32), np.concatenate(vs).astype(np.int32)), first
 
 
-@pytest.mark.parametrize("cliques,leaves,gap", [((129, 130, 131), 5000, 300), ((2, 3, 4, 5), 1, 0), ((33, 34), 70, 40)])
-def test_cliques_and_a_hub(nd, cliques, leaves, gap):
+@pytest.mark.parametrize("cliques,leaves,gap,limit", [((129, 130, 131), 5000, 300, None), ((129, 130, 131), 5000, 300, 14 << 20),
+                                                      ((2, 3, 4, 5), 1, 0, None), ((33, 34), 70, 40, None)])
+def test_cliques_and_a_hub(nd, cliques, leaves, gap, limit):
+    """With incidence lists, and where an allocator refuses their large buffers without."""
+    import torch
+
     g, first = _graph(cliques, leaves, gap)
-    ctx = nd.nd_ctx_create(0)
+    alloc, free = nd.torch_allocator_hooks(0)
+    refused = []
+
+    def hook(nbytes, stream):
+        if limit is not None and nbytes >= limit:
+            refused.append(nbytes)
+            return 0
+        return alloc(nbytes, stream)
+
+    ctx = nd.nd_ctx_create(0, stream=torch.cuda.Stream())
+    nd.nd_ctx_set_allocator(ctx, hook, free)
     G = nd.nd_load_csr(ctx, g.rowptr, g.col, flags=nd.ND_VALIDATE)
     try:
         edges = nd.nd_rcliques(G, 2)
@@ -47,16 +63,19 @@ def test_cliques_and_a_hub(nd, cliques, leaves, gap):
         want = [np.array(list(itertools.combinations(range(n), 3)), np.int32).reshape(-1, 3) + a
                 for n, a in zip(cliques, first)]
         assert np.array_equal(tri, np.concatenate(want))
-        for r, s, cl in ((2, 3, edges), (3, 4, tri)):
+        for r, s, cl in ((2, 3, edges), (2, 4, edges), (3, 4, tri)):
             core, rnd, st = nd.nd_decompose(G, r, s)
             counts, _, n_s = nd.nd_count(G, r, s)
-            # every r-clique of K_n lies in n - r of its s-cliques, and all of them go at once
+            # every r-clique of K_n lies in C(n - r, s - r) of its s-cliques, and all of them go at once
             expect = np.zeros(len(cl), np.int64)
             for n, a in zip(cliques, first):
-                expect[(cl[:, 0] >= a) & (cl[:, -1] < a + n)] = n - r
+                expect[(cl[:, 0] >= a) & (cl[:, -1] < a + n)] = math.comb(max(n - r, 0), s - r)
             assert np.array_equal(core, expect) and np.array_equal(counts, expect), (r, s)
             assert st["rho"] == len(np.unique(expect)) and st["listed"] == n_s == st["n_s"]
             assert np.array_equal(rnd, np.searchsorted(np.unique(expect), expect))
+            if limit is not None and n_s:
+                assert refused
+                refused.clear()
     finally:
         nd.nd_graph_free(G)
         nd.nd_ctx_destroy(ctx)
