@@ -95,8 +95,8 @@ typedef struct nd_stats {
     int64_t rho;        /* peeling rounds: each round peels every unpeeled r-clique whose count
                            is <= k, after k = max(k, minimum unpeeled count) */
     int64_t max_core;   /* largest core number */
-    int64_t listed;     /* s-cliques destroyed by Update over the run (each exactly once, by the
-                           smallest member of A it contains): equals n_s */
+    int64_t listed;     /* s-cliques destroyed by Update over the run (each exactly once, by one of
+                           the members of A it contains): equals n_s */
     int64_t advances;   /* rounds that moved to a new level k */
     int64_t refills;    /* bucket-window rebuilds */
     int32_t count_width;/* 4 or 8: bytes per count used on the device */
@@ -114,8 +114,9 @@ typedef struct nd_stats {
     double t_contract_ms;/* persistent peel kernel only: wall time of the graph contractions (block 0) */
     int64_t contractions;/* contractions run: (2,3) graph contraction (Section 5.6), by default one
                             whenever at least 2n edges were peeled since the previous one, compacting
-                            the adjacency rows that lost at least a quarter of their entries since
-                            then; (3,4) the same for the triangle lists, once 2m triangles were peeled */
+                            the adjacency rows (peeling from incidence lists: the edges' lists) that
+                            lost at least a quarter of their entries since then; (3,4) without incidence
+                            lists the same for the triangle lists, once 2m triangles were peeled */
     double t_hash_ms;   /* (3,4): the part of t_count_ms spent building the hash directory of the
                            triangle lists (0 otherwise); the counting kernel itself took
                            t_count_ms - t_hash_ms */
@@ -155,9 +156,9 @@ ND_API int nd_ctx_set_limits(nd_ctx *ctx, int64_t max_rounds, int64_t barrier_ti
 /* Per-(r,s) tuning of a context's decompositions (no counterpart in the paper), as chosen for
  * a device and a workload by an autotuner:
  *   heavy_work  length of an r-clique's driving list above which its Update runs on a whole block
- *               in the heavy phase instead of one warp (0: the built-in threshold: 4096 for most
- *               (r,s), 256 for (2,3), 96 for (2,4); (2,4) stages the common neighbourhood of a
- *               warp's edge in shared memory and takes at most 96)
+ *               in the heavy phase instead of one warp (0: the built-in threshold: 4096, but without
+ *               incidence lists 256 for (2,3) and 96 for (2,4), which stages the common
+ *               neighbourhood of a warp's edge in shared memory and takes at most 96)
  *   flags       ND_DENSE_BUCKETS and/or ND_CONTRACT_OFF, added to every nd_decompose of this (r,s)
  *               on the context (also inside batches and the server)
  * Errors: ND_EINVAL (NULL context, unsupported (r,s), negative threshold, other flags). */
@@ -216,7 +217,9 @@ ND_API int nd_count(nd_graph *g, int r, int s, int count_width, void *counts_out
  * r-clique (int32[n_r], canonical order); round_out (nullable) the peeling round in which
  * each r-clique was removed (int32[n_r], rounds numbered from 0); st (nullable, host) the
  * statistics. Pointers are host memory unless flags has ND_PTR_DEVICE. core_out may be NULL
- * (only the statistics are produced). count_width as in nd_count.
+ * (only the statistics are produced). count_width as in nd_count. A run takes up to 16 GiB more than it
+ * needs (incidence lists of its s-cliques), as far as the device, the context's budget and the
+ * allocator give them.
  * Errors: ND_EINVAL, ND_ENOMEM, ND_EOVERFLOW, ND_ETIMEOUT (round cap), ND_EINTERNAL. */
 ND_API int nd_decompose(nd_graph *g, int r, int s, int count_width, int32_t *core_out, int32_t *round_out, int flags,
                  nd_stats *st);
@@ -364,7 +367,8 @@ ND_API int nd_server_destroy(nd_server *sv);
  * pool has room), or a latency-critical loop where cudaMalloc/cudaFree may synchronise the
  * device. It runs the same counting and peeling kernels as nd_decompose(g, 1, 2, ...), with all
  * scratch in one fixed static device array (about 8.4 MB, held by every GPU that loads the
- * library until the process exits).
+ * library until the process exits). Its loop is one cooperative kernel, which starts once kernels of
+ * other streams leave all its blocks room.
  *   n        number of vertices, 0 <= n <= ND_NOALLOC_MAX_VERTICES (ND_EINVAL otherwise)
  *   rowptr   device int64[n+1], col device int32[rowptr[n]]: a symmetric CSR as in nd_load_csr
  *            (sorted rows, no loops, no duplicates; not validated here)
