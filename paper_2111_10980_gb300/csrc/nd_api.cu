@@ -7,6 +7,7 @@
 #include <algorithm>
 #include <atomic>
 #include <climits>
+#include <cmath>
 #include <cstddef>
 #include <cstdarg>
 #include <cstdio>
@@ -718,14 +719,23 @@ int nd_pick_width(const nd_graph* g, int r, int s, int count_width, int* w) {
     return ND_OK;
 }
 
-static int sum_counts(nd_graph* g, const DBuf& cnt, int w, int64_t n_r, unsigned long long* out) {
+// their sum and, if asked for, the largest
+static int sum_counts(nd_graph* g, const DBuf& cnt, int w, int64_t n_r, unsigned long long* out,
+                      unsigned long long* most = nullptr) {
     ND_TRY(scalar_zero(g));
-    if (w == 8)
-        nd_sum_i64((const int64_t*)cnt.p, n_r, (unsigned long long*)g->scal.p, g->ctx->stream);
-    else
-        nd_sum_i32((const int32_t*)cnt.p, n_r, (unsigned long long*)g->scal.p, g->ctx->stream);
+    unsigned long long *d = (unsigned long long*)g->scal.p, h[2] = {0, 0};
+    if (w == 8) {
+        nd_sum_i64((const int64_t*)cnt.p, n_r, d, g->ctx->stream);
+        if (most) nd_max_i64((const int64_t*)cnt.p, n_r, d + 1, g->ctx->stream);
+    } else {
+        nd_sum_i32((const int32_t*)cnt.p, n_r, d, g->ctx->stream);
+        if (most) nd_max_i32((const int32_t*)cnt.p, n_r, d + 1, g->ctx->stream);
+    }
     ND_TRY(nd_check_launch("sum"));
-    return read_back(g, g->scal.p, out, "sum");
+    ND_TRY(read_back(g, d, &h, "sum"));
+    *out = h[0];
+    if (most) *most = h[1];
+    return ND_OK;
 }
 
 extern "C" int nd_count(nd_graph* g, int r, int s, int count_width, void* counts_out, int flags, int64_t* n_r_out,
@@ -858,7 +868,7 @@ static int build_inc(nd_graph* g, int r, int s, const DBuf& cnt, int w, int64_t 
 
 // Counts the s-cliques of a prepared graph and builds their lists, for callers that read them without
 // peeling; *built stays false where nd_decompose would do without lists. R-MAT 2^17 (3,4), whose lists do not
-// fit: the sample takes 0.4 ms, the directory and the count that it saves 27 ms of a hierarchy of 1.1 s.
+// fit: the sample saves the directory and the count, 27 ms of a hierarchy of 1.1 s.
 int nd_build_inc(nd_graph* g, int r, int s, int64_t n_r, IncBufs& b, bool* built) {
     nd_ctx* c = g->ctx;
     *built = false;
@@ -868,9 +878,12 @@ int nd_build_inc(nd_graph* g, int r, int s, int64_t n_r, IncBufs& b, bool* built
     unsigned long long tot = 0;
     unsigned int status[3] = {0, 0, 0};
     int rc = nd_pick_width(g, r, s, 0, &w);
-    // A graph whose lists would not fit is not counted for them. No count exceeds count_bound(); where that does
-    // not settle it, a sample does, unless it comes within a tenth of the line.
-    const double most = (double)n_r * (double)count_bound(g, r, s) / (double)binom64(s, r);
+    // A graph whose lists would not fit is not counted for them. No count exceeds count_bound(), and m edges make at
+    // most (2m)^(s/2) / s! s-cliques; where these do not settle it, a sample does, unless it comes within a tenth
+    // of the line.
+    double most = 1;
+    for (int i = 1; i <= s; ++i) most *= std::sqrt(2.0 * (double)g->m) / i;
+    most = std::min(most, (double)n_r * (double)count_bound(g, r, s) / (double)binom64(s, r));
     if (!rc && !(most < INT32_MAX && plan_inc(g, r, s, 0, n_r, (int64_t)most, b))) {
         rc = scalar_zero(g);
         if (rc) return rc;
@@ -917,27 +930,18 @@ int nd_build_inc(nd_graph* g, int r, int s, int64_t n_r, IncBufs& b, bool* built
 // 363 / 366 and 659 / 1,250; (2,3) R-MAT 2^16 26 / 30 and 40 / 79; K_1000 as (2,3) (166 M triangles, one round) 47 / 16
 // and 137 / 106, K_250 as (2,4) 103 / 28 and 368 / 189. Beyond 2^20 r-cliques their scans weigh as much as the
 // rounds: 1.9 M edges of R-MAT 2^17 48 / 47 and 143 / 133, 3.8 M 92 / 74.
-template <typename CT>
-static int peel_shared(nd_graph* g, int r, int s, const DBuf& cnt, int64_t n_r, int64_t n_s, bool* shared) {
+// visits: all the counts together; most: the largest.
+static bool peel_shared(const nd_ctx* c, int64_t n_r, unsigned long long visits, unsigned long long most) {
     constexpr int64_t kShareMax = (int64_t)1 << 20;
     constexpr double kLeastRounds = 40, kSkewRounds = 90, kVisitsPerRound = 1.3e6;
-    const double visits = (double)n_s * (double)binom64(s, r), work = visits * (g->ctx->peel_share - 1);
-    *shared = n_r <= kShareMax;
-    if (!*shared || work <= kLeastRounds * kVisitsPerRound) return ND_OK;
-    unsigned long long most = 0;
-    ND_TRY(scalar_zero(g));
-    if (sizeof(CT) == 8)
-        nd_max_i64((const int64_t*)cnt.p, n_r, (unsigned long long*)g->scal.p, g->ctx->stream);
-    else
-        nd_max_i32((const int32_t*)cnt.p, n_r, (unsigned long long*)g->scal.p, g->ctx->stream);
-    ND_TRY(nd_check_launch("peel setup"));
-    ND_TRY(read_back(g, g->scal.p, &most, "peel setup"));
-    *shared = work <= kSkewRounds * kVisitsPerRound * ((double)most * (double)n_r / visits - 1);
-    return ND_OK;
+    if (n_r > kShareMax) return false;
+    const double skew = visits ? (double)most * (double)n_r / (double)visits - 1 : 0;
+    return (double)visits * (c->peel_share - 1) <= kVisitsPerRound * std::max(kLeastRounds, kSkewRounds * skew);
 }
 
+// shared: whether a server's worker that was not told how to peel takes its share of the SMs
 template <typename CT>
-static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int64_t n_s, int flags, PeelOut& po,
+static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, bool shared, int flags, PeelOut& po,
                     const IncBufs* inc = nullptr) {
     nd_ctx* c = g->ctx;
     cudaStream_t st = c->stream;
@@ -1143,9 +1147,9 @@ static int run_peel(nd_graph* g, int r, int s, DBuf& cnt, int64_t n_r, int64_t n
     bool want_persistent = (flags & ND_PEEL_PERSISTENT) || !(flags & (ND_NO_GRAPH | ND_PEEL_LOOP_GRAPH));
     if (flags & ND_PEEL_PERSISTENT)
         P.grid_share = 1;
-    else if (want_persistent && c->peel_share > 1)
-        rc = peel_shared<CT>(g, r, s, cnt, n_r, n_s, &want_persistent);
-    if (want_persistent && !rc) {
+    else if (c->peel_share > 1 && !shared)
+        want_persistent = false;
+    if (want_persistent) {
         // preferred: the whole loop in one cooperative kernel
         cudaError_t e = nd_peel_persistent<CT>(v, r, s, P, st);
         if (e == cudaSuccess) {
@@ -1310,8 +1314,9 @@ int nd_decompose_dev(nd_graph* g, int r, int s, int count_width, int flags, Peel
     cudaEventRecord(eh, c->stream);
     if (!rc) rc = nd_count_into(g, r, s, w, n_r, cnt);
     cudaEventRecord(e1, c->stream);
-    unsigned long long tot = 0;
-    if (!rc) rc = sum_counts(g, cnt, w, n_r, &tot);
+    unsigned long long tot = 0, most = 0;
+    if (!rc) rc = sum_counts(g, cnt, w, n_r, &tot, c->peel_share > 1 ? &most : nullptr);
+    const bool shared = c->peel_share > 1 && peel_shared(c, n_r, tot, most);
     cudaEventRecord(e3, c->stream);
     const int64_t n_s = (int64_t)(tot / (unsigned long long)binom64(s, r));
     IncBufs inc;
@@ -1325,8 +1330,8 @@ int nd_decompose_dev(nd_graph* g, int r, int s, int count_width, int flags, Peel
         if (use_inc) free_directory();  // the lists replace it
     }
     auto peel = [&](const IncBufs* lists) {
-        return (w == 8) ? run_peel<int64_t>(g, r, s, cnt, n_r, n_s, flags, po, lists)
-                        : run_peel<int32_t>(g, r, s, cnt, n_r, n_s, flags, po, lists);
+        return (w == 8) ? run_peel<int64_t>(g, r, s, cnt, n_r, shared, flags, po, lists)
+                        : run_peel<int32_t>(g, r, s, cnt, n_r, shared, flags, po, lists);
     };
     if (!rc) rc = peel(use_inc ? &inc : nullptr);
     nd_free_inc(c, inc);
@@ -1465,7 +1470,7 @@ int nd_kcore_rounds(nd_graph* g, DBuf& rnd_out) {
     int rc = nd_alloc(c, po.core, 4 * std::max<int64_t>(n, 1));
     if (!rc) rc = nd_alloc(c, po.rnd, 4 * std::max<int64_t>(n, 1));
     if (!rc) rc = nd_count_into(g, 1, 2, 4, n, cnt);
-    if (!rc) rc = run_peel<int32_t>(g, 1, 2, cnt, n, g->m, 0, po);
+    if (!rc) rc = run_peel<int32_t>(g, 1, 2, cnt, n, true, 0, po);
     nd_free(c, cnt);
     nd_free(c, po.core);
     if (rc) {

@@ -253,11 +253,11 @@ void nd_count_launch(const GraphView& g, int r, int s, CT* cnt, int64_t n_r, cud
     }
 }
 
-// at least 16,384 samples, a sixty-fourth of a large graph
+// a sixty-fourth of a large graph, and at least 16,384 DG edges or r-cliques (1,024 tiles of 32 edges)
 int64_t nd_sample_cliques(const GraphView& g, int r, int s, int64_t n_r, unsigned long long* out, cudaStream_t st) {
     const int tile = tri_tile(g.m);
     const int64_t items = s == 3 ? (g.m + tile - 1) / tile : s == 4 ? g.m : n_r;
-    const int64_t part = items >> 14, every = part < 1 ? 1 : part > 64 ? 64 : part;
+    const int64_t part = items >> (s == 3 ? 10 : 14), every = part < 1 ? 1 : part > 64 ? 64 : part;
     const int blk = blocks_for_warps((items + every - 1) / every);
     if (s == 3)
         ND_K(k_sample_tri<<<blk, kTriThreads, 0, st>>>(g, tile, every, out));
