@@ -719,18 +719,15 @@ int nd_pick_width(const nd_graph* g, int r, int s, int count_width, int* w) {
     return ND_OK;
 }
 
-// their sum and, if asked for, the largest
+// their sum and the largest
 static int sum_counts(nd_graph* g, const DBuf& cnt, int w, int64_t n_r, unsigned long long* out,
                       unsigned long long* most = nullptr) {
     ND_TRY(scalar_zero(g));
     unsigned long long *d = (unsigned long long*)g->scal.p, h[2] = {0, 0};
-    if (w == 8) {
-        nd_sum_i64((const int64_t*)cnt.p, n_r, d, g->ctx->stream);
-        if (most) nd_max_i64((const int64_t*)cnt.p, n_r, d + 1, g->ctx->stream);
-    } else {
-        nd_sum_i32((const int32_t*)cnt.p, n_r, d, g->ctx->stream);
-        if (most) nd_max_i32((const int32_t*)cnt.p, n_r, d + 1, g->ctx->stream);
-    }
+    if (w == 8)
+        nd_sum_max_i64((const int64_t*)cnt.p, n_r, d, g->ctx->stream);
+    else
+        nd_sum_max_i32((const int32_t*)cnt.p, n_r, d, g->ctx->stream);
     ND_TRY(nd_check_launch("sum"));
     ND_TRY(read_back(g, d, &h, "sum"));
     *out = h[0];
@@ -800,7 +797,7 @@ static int build_tri_hash(nd_graph* g, DBuf& hoff, DBuf& htab, DBuf& hpos) {
     return nd_check_launch("triangle hash");
 }
 
-// Whether a decomposition is peeled from incidence lists, and b's buffers if so. (1,2) has them in the CSR itself; a (3,4) run that
+// Whether incidence lists can be built, and b's buffers if so. (1,2) has them in the CSR itself; a (3,4) run that
 // is asked to contract before every round contracts its triangle lists. The lists are an accelerator and must leave room for others,
 // hence the bound (nd_ctx::inc_bytes on all the buffers together, what the context's budget has left, and what a
 // server's budget grants); the (3,4) lists of R-MAT graphs from scale 17 on, for instance, are over it, and their s-cliques are listed again by Update.
@@ -829,6 +826,32 @@ static bool plan_inc(const nd_graph* g, int r, int s, int flags, int64_t n_r, in
     }
     b.mem.want.clear();
     return false;
+}
+
+// A guess at the rounds of a peel, from how far the largest count is above the mean, over the mean (`skew`): equal
+// counts go in few rounds, skewed ones in many. Rounds over skew, measured: (2,4) of R-MAT 2^10 to 2^16 60 to 120,
+// (2,3) 18, (3,4) 35 to 60, (3,4) and (2,4) of planted communities 340 and 430; cliques and G(n, p), of skew 0 to 1.9,
+// go in 1 to 449 rounds.
+static double rounds_guess(int r, double skew) { return std::max(40.0, (r >= 3 ? 45.0 : 90.0) * skew); }
+
+static double count_skew(int64_t n_r, unsigned long long visits, unsigned long long most) {
+    return visits ? (double)most * (double)n_r / (double)visits - 1 : 0;
+}
+
+// Whether peeling from lists pays for building them. They save part of every round's chain of accesses (10 us and
+// more) and cost a listing, and Update scattered reads of lists and rows that outgrow the L2 cache. For the (r,s)
+// whose Update has a kernel of its own (the others look up every r-subset when they list: lists always pay)
+// that is, lists / none in ms: (3,4) R-MAT 2^12 (7 M 4-cliques) 7.3 / 12.0, 2^14 (48 M) 25.7 / 30.1, 2^15 (125 M) 62 / 58,
+// 2^16 (327 M) 167 / 118, G(400, 0.7) (125 M, 239 rounds) 34 / 23; (2,4) R-MAT 2^15 (125 M, 10,066 rounds) 132 / 266,
+// G(1500, 0.2) (13 M, 449 rounds) 14 / 31, G(400, 0.7) (125 M, 87 rounds) 42 / 33; (2,3) R-MAT 2^20 (375 M) 124 / 161,
+// G(1500, 0.5) (70 M, 113 rounds) 9.1 / 13.0. Equal counts go in one round, where lists lose: (2,3) K_1000 12.6 /
+// 11.5, (2,4) K_250 25 / 16, (3,4) K_150 3.6 / 2.2, (1,3) K_1000 37 / 11.
+// visits: all the counts together; most: the largest.
+static bool inc_pays(int r, int s, int64_t n_r, int64_t n_s, unsigned long long visits, unsigned long long most) {
+    const double per_round = s == 3 ? 2.5e6 : s == 4 && r == 2 ? 2e5 : s == 4 && r == 3 ? 1.1e5 : 0;
+    if (!per_round || !visits) return true;
+    if ((unsigned long long)n_r * most == visits) return false;
+    return r == 1 || (double)n_s <= per_round * rounds_guess(r, count_skew(n_r, visits, most));
 }
 
 void nd_free_inc(nd_ctx* c, IncBufs& b) {
@@ -922,21 +945,17 @@ int nd_build_inc(nd_graph* g, int r, int s, int64_t n_r, IncBufs& b, bool* built
 // the SMs, where the workers' kernels fit side by side, or as a loop graph, whose kernels spread over all SMs.
 // A round costs about 7 us in the kernel and 20 in the graph, and nothing is captured; the work, one visit for each
 // r-clique of each s-clique at about 1e11 a second on the whole GPU, takes as many times as long as there are
-// workers. So the share wins when rounds * 13 us > work * (workers - 1) / 1e11 per s. The rounds are not known, but
-// equal counts go in few of them and skewed ones in many; the guess is 90 times what the largest count is above
-// the mean, over the mean, and 40 at least: (2,4) of R-MAT 2^10 to 2^16 and of planted communities go in 60 to 350
-// times the quotient, cliques and G(n, p) in 1 to 112 rounds. Measured with 8 workers, a request alone and 8 at
-// once, share / graph in ms: (2,4) R-MAT 2^14 (48 M 4-cliques, 7,212 rounds) 110 / 171 and 165 / 492, R-MAT 2^16 (270 M)
+// workers. So the share wins when rounds * 13 us > work * (workers - 1) / 1e11 per s. Measured with 8 workers, a request
+// alone and 8 at once, share / graph in ms: (2,4) R-MAT 2^14 (48 M 4-cliques, 7,212 rounds) 110 / 171 and 165 / 492, R-MAT 2^16 (270 M)
 // 363 / 366 and 659 / 1,250; (2,3) R-MAT 2^16 26 / 30 and 40 / 79; K_1000 as (2,3) (166 M triangles, one round) 47 / 16
 // and 137 / 106, K_250 as (2,4) 103 / 28 and 368 / 189. Beyond 2^20 r-cliques their scans weigh as much as the
 // rounds: 1.9 M edges of R-MAT 2^17 48 / 47 and 143 / 133, 3.8 M 92 / 74.
 // visits: all the counts together; most: the largest.
-static bool peel_shared(const nd_ctx* c, int64_t n_r, unsigned long long visits, unsigned long long most) {
+static bool peel_shared(const nd_ctx* c, int r, int64_t n_r, unsigned long long visits, unsigned long long most) {
     constexpr int64_t kShareMax = (int64_t)1 << 20;
-    constexpr double kLeastRounds = 40, kSkewRounds = 90, kVisitsPerRound = 1.3e6;
-    if (n_r > kShareMax) return false;
-    const double skew = visits ? (double)most * (double)n_r / (double)visits - 1 : 0;
-    return (double)visits * (c->peel_share - 1) <= kVisitsPerRound * std::max(kLeastRounds, kSkewRounds * skew);
+    constexpr double kVisitsPerRound = 1.3e6;
+    return n_r <= kShareMax &&
+           (double)visits * (c->peel_share - 1) <= kVisitsPerRound * rounds_guess(r, count_skew(n_r, visits, most));
 }
 
 // shared: whether a server's worker that was not told how to peel takes its share of the SMs
@@ -1315,12 +1334,12 @@ int nd_decompose_dev(nd_graph* g, int r, int s, int count_width, int flags, Peel
     if (!rc) rc = nd_count_into(g, r, s, w, n_r, cnt);
     cudaEventRecord(e1, c->stream);
     unsigned long long tot = 0, most = 0;
-    if (!rc) rc = sum_counts(g, cnt, w, n_r, &tot, c->peel_share > 1 ? &most : nullptr);
-    const bool shared = c->peel_share > 1 && peel_shared(c, n_r, tot, most);
+    if (!rc) rc = sum_counts(g, cnt, w, n_r, &tot, &most);
+    const bool shared = c->peel_share > 1 && peel_shared(c, r, n_r, tot, most);
     cudaEventRecord(e3, c->stream);
     const int64_t n_s = (int64_t)(tot / (unsigned long long)binom64(s, r));
     IncBufs inc;
-    bool use_inc = !rc && plan_inc(g, r, s, flags, n_r, n_s, inc);
+    bool use_inc = !rc && inc_pays(r, s, n_r, n_s, tot, most) && plan_inc(g, r, s, flags, n_r, n_s, inc);
     if (use_inc) {
         rc = build_inc(g, r, s, cnt, w, n_r, inc);
         if (rc == ND_ENOMEM) {

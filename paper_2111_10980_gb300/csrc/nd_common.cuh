@@ -417,8 +417,9 @@ void nd_iota_i32(int32_t* p, int64_t n, cudaStream_t st);
 // *out = max over a[0..n) (int64 device scalar, must be pre-set to 0)
 void nd_max_i64(const int64_t* a, int64_t n, unsigned long long* out, cudaStream_t st);
 void nd_max_deg(const int64_t* rp, int32_t n, unsigned long long* out, cudaStream_t st);
-void nd_sum_i64(const int64_t* a, int64_t n, unsigned long long* out, cudaStream_t st);
-void nd_sum_i32(const int32_t* a, int64_t n, unsigned long long* out, cudaStream_t st);
+// out[0] += sum over a[0..n), out[1] = max (two int64 device scalars, pre-set to 0)
+void nd_sum_max_i64(const int64_t* a, int64_t n, unsigned long long* out, cudaStream_t st);
+void nd_sum_max_i32(const int32_t* a, int64_t n, unsigned long long* out, cudaStream_t st);
 void nd_max_i32(const int32_t* a, int64_t n, unsigned long long* out, cudaStream_t st);
 // narrow int64 counts to int32; *err set to 1 if a value exceeds limit (<= INT32_MAX)
 void nd_narrow_i64(const int64_t* in, int32_t* out, int64_t n, int64_t limit, int* err, cudaStream_t st);

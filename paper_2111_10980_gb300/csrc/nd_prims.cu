@@ -102,24 +102,40 @@ __global__ void k_iota_i32(int32_t* p, int64_t n) {
         p[i] = (int32_t)i;
 }
 
-template <typename T, bool kMax, bool kDiff>
-__global__ void k_reduce(const T* __restrict__ a, int64_t n, unsigned long long* out) {
+// out[0] += sum of a, out[1] = its maximum (both pre-set to 0; negative values count as 0)
+template <typename T>
+__global__ void k_sum_max(const T* __restrict__ a, int64_t n, unsigned long long* out) {
+    unsigned long long sum = 0, top = 0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const unsigned long long u = a[i] < 0 ? 0ull : (unsigned long long)a[i];
+        sum += u;
+        top = u > top ? u : top;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        sum += __shfl_down_sync(0xffffffffu, sum, o);
+        const unsigned long long y = __shfl_down_sync(0xffffffffu, top, o);
+        top = y > top ? y : top;
+    }
+    if ((threadIdx.x & 31) == 0 && top) {
+        atomicAdd(out, sum);
+        atomicMax(out + 1, top);
+    }
+}
+
+// the maximum of a, or of the differences of neighbours
+template <typename T, bool kDiff>
+__global__ void k_max(const T* __restrict__ a, int64_t n, unsigned long long* out) {
     unsigned long long acc = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         long long v = kDiff ? (long long)(a[i + 1] - a[i]) : (long long)a[i];
         unsigned long long u = v < 0 ? 0ull : (unsigned long long)v;
-        acc = kMax ? (u > acc ? u : acc) : acc + u;
+        acc = u > acc ? u : acc;
     }
     for (int o = 16; o > 0; o >>= 1) {
         unsigned long long y = __shfl_down_sync(0xffffffffu, acc, o);
-        acc = kMax ? (y > acc ? y : acc) : acc + y;
+        acc = y > acc ? y : acc;
     }
-    if ((threadIdx.x & 31) == 0) {
-        if (kMax)
-            atomicMax(out, acc);
-        else
-            atomicAdd(out, acc);
-    }
+    if ((threadIdx.x & 31) == 0) atomicMax(out, acc);
 }
 
 __global__ void k_narrow(const int64_t* __restrict__ in, int32_t* __restrict__ out, int64_t n, int64_t limit,
@@ -194,27 +210,27 @@ void nd_iota_i32(int32_t* p, int64_t n, cudaStream_t st) {
 
 void nd_max_i64(const int64_t* a, int64_t n, unsigned long long* out, cudaStream_t st) {
     if (n <= 0) return;
-    ND_K(k_reduce<int64_t, true, false><<<grid_for(n, 256), 256, 0, st>>>(a, n, out));
+    ND_K(k_max<int64_t, false><<<grid_for(n, 256), 256, 0, st>>>(a, n, out));
 }
 
 void nd_max_deg(const int64_t* rp, int32_t n, unsigned long long* out, cudaStream_t st) {
     if (n <= 0) return;
-    ND_K(k_reduce<int64_t, true, true><<<grid_for(n, 256), 256, 0, st>>>(rp, n, out));
+    ND_K(k_max<int64_t, true><<<grid_for(n, 256), 256, 0, st>>>(rp, n, out));
 }
 
-void nd_sum_i64(const int64_t* a, int64_t n, unsigned long long* out, cudaStream_t st) {
+void nd_sum_max_i64(const int64_t* a, int64_t n, unsigned long long* out, cudaStream_t st) {
     if (n <= 0) return;
-    ND_K(k_reduce<int64_t, false, false><<<grid_for(n, 256), 256, 0, st>>>(a, n, out));
+    ND_K(k_sum_max<int64_t><<<grid_for(n, 256), 256, 0, st>>>(a, n, out));
 }
 
-void nd_sum_i32(const int32_t* a, int64_t n, unsigned long long* out, cudaStream_t st) {
+void nd_sum_max_i32(const int32_t* a, int64_t n, unsigned long long* out, cudaStream_t st) {
     if (n <= 0) return;
-    ND_K(k_reduce<int32_t, false, false><<<grid_for(n, 256), 256, 0, st>>>(a, n, out));
+    ND_K(k_sum_max<int32_t><<<grid_for(n, 256), 256, 0, st>>>(a, n, out));
 }
 
 void nd_max_i32(const int32_t* a, int64_t n, unsigned long long* out, cudaStream_t st) {
     if (n <= 0) return;
-    ND_K(k_reduce<int32_t, true, false><<<grid_for(n, 256), 256, 0, st>>>(a, n, out));
+    ND_K(k_max<int32_t, false><<<grid_for(n, 256), 256, 0, st>>>(a, n, out));
 }
 
 void nd_narrow_i64(const int64_t* in, int32_t* out, int64_t n, int64_t limit, int* err, cudaStream_t st) {

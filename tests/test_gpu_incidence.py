@@ -110,13 +110,14 @@ def test_the_memory_of_a_run_without_lists_is_enough(nd, r, s):
 
 
 def test_a_peel_without_room_next_to_its_lists_has_its_directory(nd):
-    """K_60 as (3,4): when the peel's buffers are refused next to the incidence lists, the peel without them finds
-    the hash directory that it looks up, which had made room for the lists."""
+    """K_60 and K_5 as (3,4): when the peel's buffers are refused next to the incidence lists, the peel without them
+    finds the hash directory that it looks up, which had made room for the lists."""
     import torch
 
-    g = gg.complete(60)
-    n_r, n_s = math.comb(60, 3), math.comb(60, 4)
-    table = 16 * g.m << 7  # 58 entries in 128 slots for every edge
+    g = gg.disjoint_union(gg.complete(60), gg.complete(5))
+    n_s = math.comb(60, 4) + 5
+    want = np.repeat([57, 2], [math.comb(60, 3), 10])
+    table = 16 * math.comb(60, 2) << 7  # 58 entries in 128 slots for every edge of K_60
     alloc, free = nd.torch_allocator_hooks(0)
     sizes, full, refused, arm = [], [False], [], False
 
@@ -140,9 +141,43 @@ def test_a_peel_without_room_next_to_its_lists_has_its_directory(nd):
         for arm, tables in ((False, 1), (True, 2)):
             sizes.clear()
             core, rnd, st = nd.nd_decompose(G, 3, 4)
-            assert core.size == n_r and np.all(core == 57) and not rnd.any() and st["rho"] == 1 and st["listed"] == n_s
+            assert np.array_equal(core, want) and np.array_equal(rnd, want > 2) and st["rho"] == 2 and st["listed"] == n_s
             assert max(sizes) >= 4 * 4 * n_s and sizes.count(table) == tables and bool(refused) == arm
     finally:
         arm = False
         nd.nd_graph_free(G)
         nd.nd_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("r,s,n,other,lists", [(1, 3, 100, 0, False), (2, 3, 60, 0, False), (2, 4, 60, 0, False), (3, 4, 60, 0, False),
+                                               (2, 5, 20, 0, True), (1, 3, 100, 5, True), (2, 3, 60, 5, True), (2, 4, 60, 5, True),
+                                               (3, 4, 60, 5, True), (2, 4, 125, 5, False), (3, 4, 110, 5, False)])
+def test_lists_only_where_the_rounds_outweigh_them(nd, r, s, n, other, lists):
+    """Cliques, alone (equal counts: one round) and next to a smaller one (two rounds, however many s-cliques):
+    no lists where every (r,s) with an Update of its own is sooner without, and the closed form either way."""
+    import torch
+
+    g = gg.disjoint_union(gg.complete(n), gg.complete(other)) if other else gg.complete(n)
+    want = np.repeat([math.comb(n - r, s - r), math.comb(max(other - r, 0), s - r)], [math.comb(n, r), math.comb(other, r)])
+    n_s = math.comb(n, s) + math.comb(other, s)
+    alloc, free = nd.torch_allocator_hooks(0)
+    sizes = []
+
+    def take(nbytes, stream):
+        sizes.append(nbytes)
+        return alloc(nbytes, stream)
+
+    ctx = nd.nd_ctx_create(0, stream=torch.cuda.Stream())
+    nd.nd_ctx_set_allocator(ctx, take, free)
+    try:
+        G = nd.nd_load_csr(ctx, g.rowptr, g.col)
+        nd.nd_count(G, r, s)
+        sizes.clear()
+        core, rnd, st = nd.nd_decompose(G, r, s)
+        nd.nd_graph_free(G)
+    finally:
+        nd.nd_ctx_destroy(ctx)
+    assert np.array_equal(core, want) and np.array_equal(rnd, want == want[0] if other else 0 * want)
+    assert st["n_s"] == st["listed"] == n_s and st["rho"] == (2 if other else 1)
+    rows = 4 * ((math.comb(s, r) + 3) // 4 * 4) * n_s
+    assert (max(sizes) >= rows) == lists, sizes

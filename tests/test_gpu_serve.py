@@ -334,10 +334,10 @@ def test_server_memory_budget_holds_the_lists(nd, r, s):
 
 
 def test_server_lists_in_the_room_there_is(nd):
-    """K_150 as (2,3), 551,300 triangles: with room for the lists and their spare rows, for the lists alone,
-    and for neither. The bytes of the lists never exceed the half of what the budget leaves."""
-    g = gg.complete(150)
-    want, rows = np.full(g.m, 148, np.int32), 4 * 4 * 551_300
+    """K_150 and K_5 as (2,3), 551,310 triangles: with room for the lists and their spare rows, for the lists
+    alone, and for neither. The bytes of the lists never exceed the half of what the budget leaves."""
+    g = gg.disjoint_union(gg.complete(150), gg.complete(5))
+    want, rows = np.repeat(np.array([148, 3], np.int32), [11_175, 10]), 4 * 4 * 551_310
     seen = []
     for budget in (16 << 20, 35 << 20, 64 << 20):
         hooks = _serve_one(nd, g, 2, 3, want, mem_budget=budget)
