@@ -287,6 +287,15 @@ __global__ void k_dup_check(GraphView g, int64_t nnz, int64_t seg, const int32_t
     }
 }
 
+// The three kernels that write the lists give every warp a tile of up to 32 edges at a time, fewer where there would
+// not be four tiles for every resident warp. A tile is edge k0 of every m / tile, because the edges of a hub, whose
+// rows and lists are the longest, are neighbours, and a warp takes long lists one after another: with 32
+// consecutive edges the index of R-MAT 2^12 took 0.94 ms and of R-MAT 2^18 with 0.9 M edges 4.0, now 0.30 and 1.7
+// (one edge per warp 0.28 and 2.4); of a Chung-Lu graph with 15 M edges 12.7, now 9.4 (27.9).
+__device__ __forceinline__ int64_t tile_edge(const GraphView& g, int64_t k0, int64_t apart, int lane, int tile) {
+    return lane < tile ? lane * apart + k0 : g.m;
+}
+
 // Lists of up to kShortList entries are not intersected out of the two rows, which are far longer, but
 // gathered: a second listing of the triangles over DG appends every triangle to the short lists among
 // its three (k_edge_gather, in no order), and k_edge_order puts each list in order by counting for every
@@ -336,16 +345,17 @@ __global__ void __launch_bounds__(kTriThreads) k_edge_gather(GraphView g, int ti
     tri_list(g, tile, sink);
 }
 
-// One lane per entry of the short lists of 32 edges at a time; the place of an entry is the number of
+// One lane per entry of the short lists of a tile of edges at a time; the place of an entry is the number of
 // smaller ones in its list (no two are alike). Writes what k_edge_fill writes.
 __global__ void k_edge_order(GraphView g, const int64_t* __restrict__ et_rp, const int64_t* __restrict__ tbase,
                              const int32_t* __restrict__ w_in, const int32_t* __restrict__ p_in,
                              const int32_t* __restrict__ q_in, int32_t* __restrict__ et_w, int32_t* __restrict__ et_t,
-                             int32_t* __restrict__ tri_e, int32_t* __restrict__ tri_pos) {
+                             int32_t* __restrict__ tri_e, int32_t* __restrict__ tri_pos, int tile) {
     const int lane = threadIdx.x & 31;
     const unsigned full = 0xffffffffu;
-    for (int64_t e0 = gwarp() * 32; e0 < g.m; e0 += nwarps() * 32) {
-        const int64_t e = e0 + lane;
+    const int64_t apart = (g.m + tile - 1) / tile;
+    for (int64_t k0 = gwarp(); k0 < apart; k0 += nwarps()) {
+        const int64_t e = tile_edge(g, k0, apart, lane, tile);
         int64_t lo = 0, tb = 0;
         int32_t n = 0, low = 0;
         if (e < g.m) {
@@ -381,7 +391,7 @@ __global__ void k_edge_order(GraphView g, const int64_t* __restrict__ et_rp, con
             if (at >= olow) {
                 const int64_t tid = otb + (at - olow);
                 et_t[b + at] = (int32_t)tid;
-                tri_e[3 * tid + 0] = (int32_t)(e0 + own);
+                tri_e[3 * tid + 0] = (int32_t)(own * apart + k0);
                 tri_e[3 * tid + 1] = p_in[b + k];
                 tri_e[3 * tid + 2] = q_in[b + k];
                 tri_pos[3 * tid + 0] = at;
@@ -399,12 +409,13 @@ __global__ void k_edge_order(GraphView g, const int64_t* __restrict__ et_rp, con
 // (Chung-Lu, a million vertices, 15 M edges: 13.2 ms here of 16.3 before).
 __global__ void k_edge_fill(GraphView g, const int64_t* __restrict__ et_rp, const int64_t* __restrict__ tbase,
                             int32_t* __restrict__ et_w, int32_t* __restrict__ et_t, int32_t* __restrict__ tri_e,
-                            int32_t* __restrict__ tri_pos, int64_t above) {
+                            int32_t* __restrict__ tri_pos, int64_t above, int tile) {
     const int lane = threadIdx.x & 31;
     const unsigned full = 0xffffffffu;
-    for (int64_t e0 = gwarp() * 32; e0 < g.m; e0 += nwarps() * 32) {
+    const int64_t apart = (g.m + tile - 1) / tile;
+    for (int64_t k0 = gwarp(); k0 < apart; k0 += nwarps()) {
         // each lane looks one edge over and sets it up; those with triangles are then taken one after another
-        const int64_t el = e0 + lane;
+        const int64_t el = tile_edge(g, k0, apart, lane, tile);
         int32_t la = 0, lb = 0;
         int64_t lab = 0, lae = 0, lbb = 0, lbe = 0, lout = 0, lsig = 0, ltb = 0, lup = 0;
         if (el < g.m) {
@@ -419,7 +430,7 @@ __global__ void k_edge_fill(GraphView g, const int64_t* __restrict__ et_rp, cons
         }
         for (unsigned todo = __ballot_sync(full, lsig != 0); todo; todo &= todo - 1) {
             const int src = __ffs(todo) - 1;
-            const int64_t e = e0 + src;
+            const int64_t e = src * apart + k0;
             const int32_t b = __shfl_sync(full, lb, src);
             const int64_t ab = __shfl_sync(full, lab, src), ae = __shfl_sync(full, lae, src);
             const int64_t bb = __shfl_sync(full, lbb, src), be = __shfl_sync(full, lbe, src);
@@ -479,12 +490,13 @@ __global__ void k_edge_fill(GraphView g, const int64_t* __restrict__ et_rp, cons
 // For entries of L(a,b) with w < b, the triangle {a,w,b} has b as its largest vertex, so its
 // lowest edge is (a,w) (or (w,a)); its id is tbase[e'] + rank of b among the upper entries of L(e').
 // The entry is the triangle's (a,c) entry when a < w, its (b,c) entry when w < a (slots 1, 2).
-// A warp takes the lower entries of 32 edges together, 32 at a time.
-__global__ void k_edge_fill_tid(GraphView g, int32_t* __restrict__ et_t, int32_t* __restrict__ tri_pos) {
+// A warp takes the lower entries of a tile of edges together, 32 at a time.
+__global__ void k_edge_fill_tid(GraphView g, int32_t* __restrict__ et_t, int32_t* __restrict__ tri_pos, int tile) {
     const int lane = threadIdx.x & 31;
     const unsigned full = 0xffffffffu;
-    for (int64_t e0 = gwarp() * 32; e0 < g.m; e0 += nwarps() * 32) {
-        const int64_t e = e0 + lane;
+    const int64_t apart = (g.m + tile - 1) / tile;
+    for (int64_t k0 = gwarp(); k0 < apart; k0 += nwarps()) {
+        const int64_t e = tile_edge(g, k0, apart, lane, tile);
         int64_t lo = 0, low = 0;
         int32_t a = 0, b = 0;
         if (e < g.m) {
@@ -779,24 +791,30 @@ void nd_dup_check(const GraphView& g, const int32_t* sigma, int* err, cudaStream
     ND_K(k_dup_check<<<blocks_for_segments(2 * g.m), kThreads, 0, st>>>(g, 2 * g.m, seg_len(2 * g.m), sigma, err));
 }
 
+static int index_tile(int64_t m) {
+    const int64_t t = m / ((int64_t)nd_sm_count() * 256);
+    return (int)(t < 1 ? 1 : t > 32 ? 32 : t);
+}
+
 void nd_edge_fill(const GraphView& g, int64_t* et_rp, int64_t* tbase, int32_t* et_w, int32_t* et_t, int32_t* tri_e,
                   int32_t* tri_pos, const int32_t* sigma, int32_t* cursor, int32_t* entries, cudaStream_t st) {
     if (g.m <= 0) return;
     const int64_t nent = 3 * g.n3;
+    const int edges = index_tile(g.m), blk = blocks_for_warps((g.m + edges - 1) / edges);
     if (cursor) {
         const int tile = tri_tile(g.m);
         GatherSink sink{et_rp, sigma, g.dg_eid, cursor, entries, entries + nent, entries + 2 * nent};
         ND_K(k_edge_gather<<<blocks_for_warps((g.m + tile - 1) / tile), kTriThreads, 0, st>>>(g, tile, sink));
-        ND_K(k_edge_order<<<blocks_for_warps((g.m + 31) / 32), kThreads, 0, st>>>(
-            g, et_rp, tbase, entries, entries + nent, entries + 2 * nent, et_w, et_t, tri_e, tri_pos));
+        ND_K(k_edge_order<<<blk, kThreads, 0, st>>>(g, et_rp, tbase, entries, entries + nent, entries + 2 * nent, et_w, et_t,
+                                                    tri_e, tri_pos, edges));
     }
-    ND_K(k_edge_fill<<<blocks_for_warps((g.m + 31) / 32), kThreads, 0, st>>>(g, et_rp, tbase, et_w, et_t, tri_e, tri_pos,
-                                                                                 cursor ? kShortList : 0));
+    ND_K(k_edge_fill<<<blk, kThreads, 0, st>>>(g, et_rp, tbase, et_w, et_t, tri_e, tri_pos, cursor ? kShortList : 0, edges));
 }
 
 void nd_edge_fill_tid(const GraphView& g, int32_t* et_t, int32_t* tri_pos, cudaStream_t st) {
     if (g.m <= 0) return;
-    ND_K(k_edge_fill_tid<<<blocks_for_warps((g.m + 31) / 32), kThreads, 0, st>>>(g, et_t, tri_pos));
+    const int edges = index_tile(g.m);
+    ND_K(k_edge_fill_tid<<<blocks_for_warps((g.m + edges - 1) / edges), kThreads, 0, st>>>(g, et_t, tri_pos, edges));
 }
 
 

@@ -80,3 +80,46 @@ def test_cliques_and_a_hub(nd, cliques, leaves, gap, limit):
     finally:
         nd.nd_graph_free(G)
         nd.nd_ctx_destroy(ctx)
+
+
+def _hooked(nd, refuse):
+    """A context whose allocations are noted in a list, and refused where refuse(nbytes)."""
+    import torch
+
+    alloc, free = nd.torch_allocator_hooks(0)
+    sizes = []
+
+    def take(nbytes, stream):
+        sizes.append(nbytes)
+        return 0 if refuse(nbytes) else alloc(nbytes, stream)
+
+    ctx = nd.nd_ctx_create(0, stream=torch.cuda.Stream())
+    nd.nd_ctx_set_allocator(ctx, take, free)
+    return ctx, sizes
+
+
+def _scratch(n3):
+    """Bytes that gathering the short lists of n3 triangles takes."""
+    return (36 * n3 + 255) // 256 * 256
+
+
+@pytest.mark.parametrize("n", [1, 31, 4097, 60_000, 400_000])
+def test_the_triangle_index_gathered_and_merged(nd, n):
+    """The same index, seen through the triangles, the 4-cliques' counts and the (3,4) and (4,5) results, whether
+    the short lists are gathered or, refused the scratch, merged out of the rows; from one edge per warp and step of
+    the list kernels to 32."""
+    g = gg.chung_lu(n, min(24.0, n / 4), 2.2, seed=9901)
+    got, scratch = [], None
+    for refused in (False, True):
+        ctx, sizes = _hooked(nd, lambda nbytes: refused and nbytes == scratch)
+        G = nd.nd_load_csr(ctx, g.rowptr, g.col, flags=nd.ND_VALIDATE)
+        try:
+            tri = nd.nd_rcliques(G, 3)
+            scratch = _scratch(len(tri)) if len(tri) >= 1 << 16 else None  # fewer triangles are not gathered
+            assert scratch is None or scratch in sizes
+            got.append([tri, nd.nd_count(G, 3, 4)[0], *nd.nd_decompose(G, 3, 4)[:2], nd.nd_decompose(G, 4, 5)[0]])
+        finally:
+            nd.nd_graph_free(G)
+            nd.nd_ctx_destroy(ctx)
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
