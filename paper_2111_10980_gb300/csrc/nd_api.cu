@@ -546,10 +546,16 @@ static int ensure_tri(nd_graph* g) {
     nd_edge_support(v, (int32_t*)sigma.p, (int32_t*)up.p, st);
     nd_scan_i32((const int32_t*)sigma.p, (int64_t*)g->et_rp.p, m, tmp.p, st);
     nd_scan_i32((const int32_t*)up.p, (int64_t*)g->tbase.p, m, tmp.p, st);
-    int64_t n3 = 0;
     int err = 0;
-    rc = nd_check_launch("triangle index");
-    if (!rc) rc = read_back(g, (int64_t*)g->tbase.p + m, &n3, "triangle index");
+    unsigned long long h[2] = {0, 0};  // row entries that the short lists' edges would merge; triangles
+    rc = scalar_zero(g);
+    if (!rc) {
+        if (nd_gather_asks(m)) nd_row_work(v, (const int32_t*)sigma.p, (unsigned long long*)g->scal.p, st);
+        cudaMemcpyAsync((int64_t*)g->scal.p + 1, (int64_t*)g->tbase.p + m, 8, cudaMemcpyDeviceToDevice, st);
+        rc = nd_check_launch("triangle index");
+    }
+    if (!rc) rc = read_back(g, g->scal.p, &h, "triangle index");
+    const int64_t n3 = (int64_t)h[1];
     if (!rc && g->rows) {
         rc = scalar_zero(g);
         if (!rc) nd_dup_check(v, (const int32_t*)sigma.p, (int*)g->scal.p, st);
@@ -573,12 +579,12 @@ static int ensure_tri(nd_graph* g) {
         nd_free(c, sigma);
         return rc;
     }
-    // scratch of the short lists; without room for it every list is intersected out of the rows
+    // scratch of the short lists, where they are gathered; without it every list is intersected out of the rows
     DGroup scratch;
     DBuf cursor, entries;
     scratch.add(cursor, sizeof(int32_t) * m);
     scratch.add(entries, sizeof(int32_t) * 9 * n3);
-    const bool gather = n3 > 0 && scratch.alloc(c) == ND_OK;
+    const bool gather = nd_gather_pays(n3, h[0]) && scratch.alloc(c) == ND_OK;
     if (gather) cudaMemsetAsync(cursor.p, 0, sizeof(int32_t) * m, st);
     g->n3 = n3;
     v = nd_view(g);

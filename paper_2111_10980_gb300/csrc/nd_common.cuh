@@ -437,6 +437,11 @@ void nd_dg_fill(const GraphView& g, const int32_t* key_hi, int64_t* dg_rp, const
                 int32_t* dg_eid, cudaStream_t st);
 // per canonical edge: sigma += |N(a) ∩ N(b)|, up += |{w in N(a) ∩ N(b) : w > b}| (zeroed by the caller)
 void nd_edge_support(const GraphView& g, int32_t* sigma, int32_t* up, cudaStream_t st);
+// whether a graph of m edges may have its short lists gathered: then *rows (zeroed) from sigma, and whether n3 triangles
+// are worth that, instead of merging so many row entries
+inline bool nd_gather_asks(int64_t m) { return m >= 1 << 15; }
+void nd_row_work(const GraphView& g, const int32_t* sigma, unsigned long long* rows, cudaStream_t st);
+bool nd_gather_pays(int64_t n3, unsigned long long rows);
 // *err unless the triangle lists of a CSR with duplicate entries are those of a simple graph
 void nd_dup_check(const GraphView& g, const int32_t* sigma, int* err, cudaStream_t st);
 // cursor (m, zeroed) and entries (9 n3): scratch of the short lists, or NULL: every list out of the rows

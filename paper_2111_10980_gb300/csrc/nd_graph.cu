@@ -299,9 +299,27 @@ __device__ __forceinline__ int64_t tile_edge(const GraphView& g, int64_t k0, int
 // Lists of up to kShortList entries are not intersected out of the two rows, which are far longer, but
 // gathered: a second listing of the triangles over DG appends every triangle to the short lists among
 // its three (k_edge_gather, in no order), and k_edge_order puts each list in order by counting for every
-// entry the smaller ones. Chung-Lu, a million vertices, 15 M edges, 9 M triangles: the fill 13.2 ms out of the
-// rows alone, 4.3 + 0.8 ms here and 4.0 ms there with both, the index 18 -> 12.7 ms.
+// entry the smaller ones. That pays where the rows of these edges hold more than some 40 entries for each
+// triangle (nd_gather_pays). Index with / without, in ms: Chung-Lu, a million vertices (518 entries) 9.4 / 16.7, 200,001
+// vertices (343) 1.3 / 2.0; flat R-MAT of 40,000 vertices (131) 0.95 / 1.21; R-MAT 2^20 (49) 230 / 243, 2^15 (33) 2.41 /
+// 2.33, 2^12 (27) 0.34 / 0.29; G(3000, 0.1) (60) 1.77 / 1.75, G(1500, 0.2) (30) 1.37 / 1.11; under 65,536 triangles or
+// 32,768 edges launches are all that counts: 2,000 vertices 0.135 / 0.124.
 constexpr int kShortList = 128;
+
+// *rows += the row entries that merging (or, 16 for each that is bisected, searching) the rows of the edges with short
+// lists would look at
+__global__ void k_row_work(GraphView g, const int32_t* __restrict__ sigma, unsigned long long* rows) {
+    unsigned long long c = 0;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < g.m; e += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t n = sigma[e];
+        if (n == 0 || n > kShortList) continue;
+        const int32_t a = g.eu[e], b = g.ev[e];
+        const int64_t da = g.rp[a + 1] - g.rp[a], db = g.rp[b + 1] - g.rp[b], lo = da < db ? da : db, hi = da < db ? db : da;
+        c += nd_prefer_merge(lo, hi) ? lo + hi : 16 * lo;
+    }
+    for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
+    if ((threadIdx.x & 31) == 0 && c) atomicAdd(rows, c);
+}
 
 struct GatherSink {
     const int64_t* et_rp;
@@ -790,6 +808,13 @@ void nd_dup_check(const GraphView& g, const int32_t* sigma, int* err, cudaStream
     if (g.m <= 0) return;
     ND_K(k_dup_check<<<blocks_for_segments(2 * g.m), kThreads, 0, st>>>(g, 2 * g.m, seg_len(2 * g.m), sigma, err));
 }
+
+void nd_row_work(const GraphView& g, const int32_t* sigma, unsigned long long* rows, cudaStream_t st) {
+    if (g.m <= 0) return;
+    ND_K(k_row_work<<<blocks_for_threads(g.m), kThreads, 0, st>>>(g, sigma, rows));
+}
+
+bool nd_gather_pays(int64_t n3, unsigned long long rows) { return n3 >= 1 << 16 && rows > 40 * (unsigned long long)n3; }
 
 static int index_tile(int64_t m) {
     const int64_t t = m / ((int64_t)nd_sm_count() * 256);

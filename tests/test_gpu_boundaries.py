@@ -103,6 +103,37 @@ def _scratch(n3):
     return (36 * n3 + 255) // 256 * 256
 
 
+@pytest.mark.parametrize("leaves", [0, 1200])
+def test_short_lists_of_long_rows_are_gathered(nd, leaves):
+    """K_129, K_130 and K_131 (lists of 127, 128 and 129), alone and with so many leaves at every vertex of the first
+    two that their rows are not worth merging."""
+    cliques, us, vs, first, at = (129, 130, 131), [], [], [], 0
+    for n in cliques:
+        iu, ju = np.triu_indices(n, 1)
+        us.append(iu + at)
+        vs.append(ju + at)
+        first.append(at)
+        at += n
+    hung = at + np.arange(259 * leaves)
+    us.append(np.repeat(np.arange(259), leaves))
+    vs.append(hung)
+    g = gg.csr_from_edges(at + hung.size, np.concatenate(us).astype(np.int32), np.concatenate(vs).astype(np.int32))
+    n3 = sum(math.comb(n, 3) for n in cliques)
+    ctx, sizes = _hooked(nd, lambda nbytes: False)
+    G = nd.nd_load_csr(ctx, g.rowptr, g.col, flags=nd.ND_VALIDATE)
+    try:
+        tri = nd.nd_rcliques(G, 3)
+        assert (_scratch(n3) in sizes) == (leaves > 0)
+        want = [np.array(list(itertools.combinations(range(n), 3)), np.int32) + a for n, a in zip(cliques, first)]
+        assert np.array_equal(tri, np.concatenate(want))
+        core, rnd, st = nd.nd_decompose(G, 3, 4)
+        assert np.array_equal(core, np.repeat([n - 3 for n in cliques], [math.comb(n, 3) for n in cliques]))
+        assert np.array_equal(rnd, core - 126) and st["listed"] == sum(math.comb(n, 4) for n in cliques)
+    finally:
+        nd.nd_graph_free(G)
+        nd.nd_ctx_destroy(ctx)
+
+
 @pytest.mark.parametrize("n", [1, 31, 4097, 60_000, 400_000])
 def test_the_triangle_index_gathered_and_merged(nd, n):
     """The same index, seen through the triangles, the 4-cliques' counts and the (3,4) and (4,5) results, whether
