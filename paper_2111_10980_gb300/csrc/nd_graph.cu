@@ -115,9 +115,9 @@ __global__ void k_pos2e(GraphView g, int64_t nnz, int64_t seg, int32_t* __restri
             const int64_t p = p0 + lane;
             int64_t u = u0;
             if (p < s1) {
+                const int32_t v = g.col[p], prev = p > 0 ? g.col[p - 1] : -1;
                 u = row_of(g.rp, g.n, u0, p);
-                const int32_t v = g.col[p];
-                if (p > g.rp[u] && g.col[p - 1] >= v) atomicOr(err, g.col[p - 1] == v ? 2 : 4);
+                if (prev >= v && p > g.rp[u]) atomicOr(err, prev == v ? 2 : 4);
                 int64_t id;
                 if ((uint32_t)v >= (uint32_t)g.n) {
                     atomicOr(err, 1);
