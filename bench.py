@@ -406,12 +406,12 @@ def per_rs_summary(stats, rs):
 # scale 17): the traffic of these kernels grows with the s-cliques listed. Keyed by the fingerprint
 # of the library sources the captures were taken on; reported only while the sources still match.
 NCU_TRAFFIC = {
-    # R-MAT scale 17 (n_4 = 819,091,962): k_peel_loop (3,4) 247.50 GB read + 39.52 GB written, k_count34
-    # 54.53 GB + 0.56 GB; scaled by 16,996,482,431 / 819,091,962 = 20.750. The (2,3) kernels are not
+    # R-MAT scale 17 (n_4 = 819,091,962): k_peel_loop (3,4) 268.87 GB read + 63.06 GB written, k_count34
+    # 54.43 GB + 0.56 GB; scaled by 16,996,482,431 / 819,091,962 = 20.750. The (2,3) kernels are not
     # listed: at scale 17 their arrays fit in L2, so their DRAM bytes do not scale.
-    "37514f67ef4c48be": {
-        ("rmat20", "k_peel_loop(3,4)"): 5.9558e+12,
-        ("rmat20", "k_count34"): 1.1432e+12,
+    "64cc766f27c15912": {
+        ("rmat20", "k_peel_loop(3,4)"): 6.8875e+12,
+        ("rmat20", "k_count34"): 1.1411e+12,
     },
 }
 
