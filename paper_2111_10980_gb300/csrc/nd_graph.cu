@@ -288,13 +288,22 @@ __global__ void k_dup_check(GraphView g, int64_t nnz, int64_t seg, const int32_t
 }
 
 // The three kernels that write the lists give every warp a tile of up to 32 edges at a time, fewer where there would
-// not be four tiles for every resident warp. A tile is edge k0 of every m / tile, because the edges of a hub, whose
+// not be four tiles for every resident warp. A tile's edges lie 1,024 apart, because the edges of a hub, whose
 // rows and lists are the longest, are neighbours, and a warp takes long lists one after another: with 32
-// consecutive edges the index of R-MAT 2^12 took 0.94 ms and of R-MAT 2^18 with 0.9 M edges 4.0, now 0.30 and 1.7
-// (one edge per warp 0.28 and 2.4); of a Chung-Lu graph with 15 M edges 12.7, now 9.4 (27.9).
-__device__ __forceinline__ int64_t tile_edge(const GraphView& g, int64_t k0, int64_t apart, int lane, int tile) {
-    return lane < tile ? lane * apart + k0 : g.m;
-}
+// consecutive edges the index of R-MAT 2^12 took 0.94 ms and of R-MAT 2^18 with 0.9 M edges 4.0, now 0.30 and 1.8
+// (one edge per warp 0.28 and 2.4); of a Chung-Lu graph with 15 M edges 12.7, now 9.2 (27.9). They lie no further
+// apart, so that neighbouring warps stay in the same part of a large graph: 1,365 graphs in one, 41 M edges, 21 ms
+// with consecutive edges, 23 so, 30 with m / 32 in between.
+constexpr int64_t kTileSpan = 1024;  // tiles
+struct EdgeTile {
+    int64_t first, apart;
+    __device__ __forceinline__ EdgeTile(int64_t m, int64_t k, int64_t tiles, int tile) {
+        const int64_t span = k / kTileSpan * kTileSpan;
+        apart = tiles - span < kTileSpan ? (m - span * tile + tile - 1) / tile : kTileSpan;
+        first = span * tile + (k - span);
+    }
+    __device__ __forceinline__ int64_t edge(int lane) const { return first + lane * apart; }
+};
 
 // Lists of up to kShortList entries are not intersected out of the two rows, which are far longer, but
 // gathered: a second listing of the triangles over DG appends every triangle to the short lists among
@@ -307,10 +316,11 @@ __device__ __forceinline__ int64_t tile_edge(const GraphView& g, int64_t k0, int
 constexpr int kShortList = 128;
 
 // *rows += the row entries that merging (or, 16 for each that is bisected, searching) the rows of the edges with short
-// lists would look at
-__global__ void k_row_work(GraphView g, const int32_t* __restrict__ sigma, unsigned long long* rows) {
+// lists would look at, estimated from 32 edges of every 32 * every
+__global__ void k_row_work(GraphView g, const int32_t* __restrict__ sigma, int64_t every, unsigned long long* rows) {
+    const int lane = threadIdx.x & 31;
     unsigned long long c = 0;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < g.m; e += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t e = gwarp() * 32 * every + lane; e < g.m; e += nwarps() * 32 * every) {
         const int32_t n = sigma[e];
         if (n == 0 || n > kShortList) continue;
         const int32_t a = g.eu[e], b = g.ev[e];
@@ -318,7 +328,7 @@ __global__ void k_row_work(GraphView g, const int32_t* __restrict__ sigma, unsig
         c += nd_prefer_merge(lo, hi) ? lo + hi : 16 * lo;
     }
     for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd(rows, c);
+    if (lane == 0 && c) atomicAdd(rows, c * every);
 }
 
 struct GatherSink {
@@ -371,9 +381,10 @@ __global__ void k_edge_order(GraphView g, const int64_t* __restrict__ et_rp, con
                              int32_t* __restrict__ tri_e, int32_t* __restrict__ tri_pos, int tile) {
     const int lane = threadIdx.x & 31;
     const unsigned full = 0xffffffffu;
-    const int64_t apart = (g.m + tile - 1) / tile;
-    for (int64_t k0 = gwarp(); k0 < apart; k0 += nwarps()) {
-        const int64_t e = tile_edge(g, k0, apart, lane, tile);
+    const int64_t tiles = (g.m + tile - 1) / tile;
+    for (int64_t k = gwarp(); k < tiles; k += nwarps()) {
+        const EdgeTile T(g.m, k, tiles, tile);
+        const int64_t e = lane < tile ? T.edge(lane) : g.m;
         int64_t lo = 0, tb = 0;
         int32_t n = 0, low = 0;
         if (e < g.m) {
@@ -409,7 +420,7 @@ __global__ void k_edge_order(GraphView g, const int64_t* __restrict__ et_rp, con
             if (at >= olow) {
                 const int64_t tid = otb + (at - olow);
                 et_t[b + at] = (int32_t)tid;
-                tri_e[3 * tid + 0] = (int32_t)(own * apart + k0);
+                tri_e[3 * tid + 0] = (int32_t)T.edge(own);
                 tri_e[3 * tid + 1] = p_in[b + k];
                 tri_e[3 * tid + 2] = q_in[b + k];
                 tri_pos[3 * tid + 0] = at;
@@ -430,10 +441,11 @@ __global__ void k_edge_fill(GraphView g, const int64_t* __restrict__ et_rp, cons
                             int32_t* __restrict__ tri_pos, int64_t above, int tile) {
     const int lane = threadIdx.x & 31;
     const unsigned full = 0xffffffffu;
-    const int64_t apart = (g.m + tile - 1) / tile;
-    for (int64_t k0 = gwarp(); k0 < apart; k0 += nwarps()) {
+    const int64_t tiles = (g.m + tile - 1) / tile;
+    for (int64_t k = gwarp(); k < tiles; k += nwarps()) {
+        const EdgeTile T(g.m, k, tiles, tile);
         // each lane looks one edge over and sets it up; those with triangles are then taken one after another
-        const int64_t el = tile_edge(g, k0, apart, lane, tile);
+        const int64_t el = lane < tile ? T.edge(lane) : g.m;
         int32_t la = 0, lb = 0;
         int64_t lab = 0, lae = 0, lbb = 0, lbe = 0, lout = 0, lsig = 0, ltb = 0, lup = 0;
         if (el < g.m) {
@@ -448,7 +460,7 @@ __global__ void k_edge_fill(GraphView g, const int64_t* __restrict__ et_rp, cons
         }
         for (unsigned todo = __ballot_sync(full, lsig != 0); todo; todo &= todo - 1) {
             const int src = __ffs(todo) - 1;
-            const int64_t e = src * apart + k0;
+            const int64_t e = T.edge(src);
             const int32_t b = __shfl_sync(full, lb, src);
             const int64_t ab = __shfl_sync(full, lab, src), ae = __shfl_sync(full, lae, src);
             const int64_t bb = __shfl_sync(full, lbb, src), be = __shfl_sync(full, lbe, src);
@@ -512,9 +524,10 @@ __global__ void k_edge_fill(GraphView g, const int64_t* __restrict__ et_rp, cons
 __global__ void k_edge_fill_tid(GraphView g, int32_t* __restrict__ et_t, int32_t* __restrict__ tri_pos, int tile) {
     const int lane = threadIdx.x & 31;
     const unsigned full = 0xffffffffu;
-    const int64_t apart = (g.m + tile - 1) / tile;
-    for (int64_t k0 = gwarp(); k0 < apart; k0 += nwarps()) {
-        const int64_t e = tile_edge(g, k0, apart, lane, tile);
+    const int64_t tiles = (g.m + tile - 1) / tile;
+    for (int64_t k = gwarp(); k < tiles; k += nwarps()) {
+        const EdgeTile T(g.m, k, tiles, tile);
+        const int64_t e = lane < tile ? T.edge(lane) : g.m;
         int64_t lo = 0, low = 0;
         int32_t a = 0, b = 0;
         if (e < g.m) {
@@ -811,7 +824,8 @@ void nd_dup_check(const GraphView& g, const int32_t* sigma, int* err, cudaStream
 
 void nd_row_work(const GraphView& g, const int32_t* sigma, unsigned long long* rows, cudaStream_t st) {
     if (g.m <= 0) return;
-    ND_K(k_row_work<<<blocks_for_threads(g.m), kThreads, 0, st>>>(g, sigma, rows));
+    const int64_t every = g.m >= 1 << 20 ? 16 : 1;
+    ND_K(k_row_work<<<blocks_for_threads(g.m / every), kThreads, 0, st>>>(g, sigma, every, rows));
 }
 
 bool nd_gather_pays(int64_t n3, unsigned long long rows) { return n3 >= 1 << 16 && rows > 40 * (unsigned long long)n3; }
